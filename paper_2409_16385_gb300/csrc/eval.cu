@@ -1882,7 +1882,8 @@ __global__ void k_sum_final(const double* __restrict__ partial, int nb, double* 
 }
 
 // ------------------------------------------------------------------ friction lag
-__global__ void __launch_bounds__(kEvalThreads) k_lag(Topo T, const double* __restrict__ x4, eipc_pairs pr,
+__global__ void __launch_bounds__(kEvalThreads) k_lag(Topo T, const double* __restrict__ x4,
+                                                      const float* __restrict__ x4f, eipc_pairs pr,
                                                       double dhat, double kappa, eipc_lag out, DevStatus* st,
                                                       const double* __restrict__ moll_r2, double moll_factor,
                                                       uint64_t* __restrict__ key_out, int64_t key_cap) {
@@ -1901,8 +1902,7 @@ __global__ void __launch_bounds__(kEvalThreads) k_lag(Topo T, const double* __re
     for (int a = 0; a < 4; ++a) X[a] = load_x(x4, v[a]);
     for (int a = 0; a < 4; ++a) Y[a] = X[a] - X[0];
     Stencil S;
-    if (type == 0) pt_distance<true>(Y[0], Y[1], Y[2], Y[3], &S);
-    else ee_distance<true>(Y[0], Y[1], Y[2], Y[3], &S);
+    closest_pair<true>(type, Y, stencil_hint(type, x4f, v), &S);
     const double d = sqrt(S.d2);
     double b1 = 0.0;
     if (d > 0.0 && d < dhat) {
@@ -1944,8 +1944,8 @@ void lag_launch(eipc_scene* sc, const double* q_n, const eipc_pairs& pr, const e
                 cudaStream_t s) {
   EIPC_TIMED(sc, kKEmbed, s, embed_launch(sc, q_n, sc->x4, 1, 0, s));
   EIPC_TIMED(sc, kKLag, s,
-             (launch(k_lag, blocks_for(pr.capacity, 8, kEvalThreads), kEvalThreads, 0, s, sc->topo, sc->x4, pr, p.dhat,
-                     p.kappa, out, sc->status, static_cast<const double*>(sc->moll_factor > 0.0 ? sc->moll_r2 : nullptr),
+             (launch(k_lag, blocks_for(pr.capacity, 8, kEvalThreads), kEvalThreads, 0, s, sc->topo, sc->x4,
+                     static_cast<const float*>(sc->x4f), pr, p.dhat, p.kappa, out, sc->status, static_cast<const double*>(sc->moll_factor > 0.0 ? sc->moll_r2 : nullptr),
                      sc->moll_factor, sc->lag_key, sc->item_cap)));
   sc->lag_src = out.v;   // the lag state whose pair keys lag_key now holds
 }

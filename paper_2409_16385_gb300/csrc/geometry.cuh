@@ -26,16 +26,22 @@ struct Stencil {
   double d2;
 };
 
+// Comparisons of doubles as integers: an FP64 compare holds the FP64 pipe for nearly two
+// instruction slots, an integer one costs next to nothing.  a > 0; and a < b, a >= b for
+// non-negative operands (whose bit patterns are ordered like their values).
+__device__ __forceinline__ bool is_pos(double a) { return __double_as_longlong(a) > 0; }
+__device__ __forceinline__ bool lt_nonneg(double a, double b) { return __double_as_longlong(a) < __double_as_longlong(b); }
+
 // |p - (e0 + t (e1 - e0))|^2 over t in [0,1].  t = clamp((w.e) / (e.e), 0, 1), with the
-// division taken only inside (0, 1): w.e <= 0 gives 0 and w.e >= e.e gives 1, the values the
-// correctly rounded quotient clamps to (also for e = 0 and NaN).
+// quotient (one reciprocal and a product) taken only inside (0, 1): w.e <= 0 gives 0 and
+// w.e >= e.e gives 1, also for e = 0.  A NaN gives a NaN distance either way.
 __device__ __forceinline__ double seg_point_d2(V3 p, V3 e0, V3 e1, double* t_out) {
   V3 e = e1 - e0, w = p - e0;
   const double we = dot(w, e), ee = dot(e, e);
   double t;
-  if (!(we > 0.0)) t = 0.0;
-  else if (we >= ee) t = 1.0;
-  else t = we / ee;
+  if (!is_pos(we)) t = 0.0;
+  else if (!lt_nonneg(we, ee)) t = 1.0;
+  else t = we * (1.0 / ee);
   V3 r = w - e * t;
   *t_out = t;
   return dot(r, r);
@@ -50,19 +56,16 @@ __device__ __forceinline__ void set_zero(Stencil& S) {
 // with sign +1 (point on side A) -- used for PT edges and EE endpoint cases
 __device__ __forceinline__ void point_segment_stencil(Stencil& S, int ip, double sp, int ia, int ib,
                                                       double t) {
-  set_zero(S);
-  S.c[ip] = sp;
-  if (t <= 0.0) {
-    S.c[ia] = -sp; S.m = 0;
-  } else if (t >= 1.0) {
-    S.c[ib] = -sp; S.m = 0;
-  } else {
-    S.c[ia] = -sp * (1.0 - t);
-    S.c[ib] = -sp * t;
-    S.a[0][ia] = sp;
-    S.a[0][ib] = -sp;
-    S.m = 1;
+  const bool at_a = !is_pos(t), at_b = __double2hiint(t) >= 0x3ff00000;   // t <= 0, t >= 1
+  const double ca = at_b ? 0.0 : (at_a ? -sp : -sp * (1.0 - t)), cb = at_a ? 0.0 : (at_b ? -sp : -sp * t);
+  const bool inner = !at_a && !at_b;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {            // selects, so that the stencil stays in registers
+    S.c[k] = k == ip ? sp : (k == ia ? ca : (k == ib ? cb : 0.0));
+    S.a[0][k] = !inner ? 0.0 : (k == ia ? sp : (k == ib ? -sp : 0.0));
+    S.a[1][k] = 0.0;
   }
+  S.m = inner ? 1 : 0;
 }
 
 template <bool kStencil>
@@ -245,6 +248,167 @@ __device__ __forceinline__ bool ee_far_f32(F3 a0, F3 a1, F3 b0, F3 b1, float r2m
     d2 = fminf(fminf(fseg_d2(w, eb), fseg_d2(a1 - b0, eb)), fminf(fseg_d2(b0 - a0, ea), fseg_d2(b1 - a0, ea)));
   }
   return d2 > r2m;
+}
+
+// ---------------------------------------------------------------- FP32 choice of feature
+// On GB300 an FP64 warp instruction holds its sub-partition's pipe for 64 cycles however many
+// lanes are active (one dependent chain already saturates it), an FP32 one for about 1.6.  The
+// FP64 distance above spends most of its instructions on features that turn out not to be the
+// closest: the interior solve and three or four segments.  closest_hint decides in FP32 which
+// of them can be: bit k (k < 4) for segment k (PT: t0t1, t1t2, t2t0; EE: a0-b, a1-b, b0-a,
+// b1-a), kHintInterior if the interior solution is possible, kHintCertain if nothing else is.
+// closest_pair then runs the same FP64 formulas, in the same order and with the same ties, on
+// the features left: a feature is dropped only if its FP32 value misses the smallest by more
+// than the error of both, so the result is the full evaluation's.
+//
+// Errors (u = 2^-24): a coordinate read from its FP32 copy is off by ec = M u, M the largest
+// coordinate.  With E, W the longest edge and the offset w, the numerators of the interior
+// parameters (sizes up to W E^3) are off by at most (16 u W E + 8 ec (E + 3 W)) E^2 to first
+// order, taken as 64 (u E + ec)(W + E) E^2; a segment's FP32 distance is off by 8 u (W + E) + 4 ec,
+// taken as 32 u (W + E) + 8 ec (its parameter enters in second order).  Where |e1 x e2|^2 is
+// below 1e-6 |e1|^2 |e2|^2 or close to FP32's smallest numbers nothing is concluded, and any
+// NaN leaves every feature in.
+constexpr int kHintInterior = 16, kHintCertain = 32;
+
+__device__ __forceinline__ float fmax_abs(F3 a) { return fmaxf(fabsf(a.x), fmaxf(fabsf(a.y), fabsf(a.z))); }
+
+__device__ __forceinline__ float fseg_d2_fast(F3 w, F3 e) {
+  const float t = fminf(fmaxf(__fdividef(fdot(w, e), fdot(e, e)), 0.f), 1.f);
+  const F3 r = w - e * t;
+  return fdot(r, r);
+}
+
+__device__ __forceinline__ int closest_hint(int type, F3 p0, F3 p1, F3 p2, F3 p3, float ec) {
+  const bool pt = type == 0;
+  const F3 e1 = pt ? p2 - p1 : p1 - p0, e2 = pt ? p3 - p1 : p3 - p2, w = pt ? p0 - p1 : p0 - p2;
+  const F3 n = fcross(e1, e2);
+  const float nn = fdot(n, n), A = fdot(e1, e1), C = fdot(e2, e2), ww = fdot(w, w);
+  const float Em = sqrtf(fmaxf(A, C)), W = sqrtf(ww);
+  const float u = 5.9604645e-8f;
+  const float tol = 64.f * (u * Em + ec) * (W + Em) * Em * Em;
+  float lo;                                    // signed room inside the parameter region (times nn)
+  float d2[4];
+  if (pt) {
+    const float n1 = fdot(fcross(w, e2), n), n2 = fdot(fcross(e1, w), n);
+    lo = fminf(fminf(n1, n2), nn - n1 - n2);
+    d2[0] = fseg_d2_fast(w, e1);
+    d2[1] = fseg_d2_fast(p0 - p2, p3 - p2);
+    d2[2] = fseg_d2_fast(p0 - p3, p1 - p3);
+    d2[3] = INFINITY;
+  } else {
+    const float B = fdot(e1, e2), D = fdot(e1, w), E = fdot(e2, w);
+    const float n1 = B * E - C * D, n2 = A * E - B * D;
+    lo = fminf(fminf(n1, n2), fminf(nn - n1, nn - n2));
+    d2[0] = fseg_d2_fast(w, e2);
+    d2[1] = fseg_d2_fast(p1 - p2, e2);
+    d2[2] = fseg_d2_fast(p2 - p0, e1);
+    d2[3] = fseg_d2_fast(p3 - p0, e1);
+  }
+  const bool sharp = nn > 1e-6f * A * C && nn > 1e-30f;
+  if (sharp && lo > 2.f * tol) return kHintInterior | kHintCertain;
+  int hint = (sharp && lo < -2.f * tol) ? 0 : kHintInterior;
+  const float dm = fminf(fminf(d2[0], d2[1]), fminf(d2[2], d2[3]));
+  const float r = sqrtf(dm) + 64.f * u * (W + Em) + 16.f * ec;
+  const float thr = r * r + 1e-30f;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    if (!(d2[k] > thr)) hint |= 1 << k;
+  return pt ? hint & ~8 : hint;
+}
+
+// closest_hint of a stencil from the FP32 copies of its positions
+__device__ __forceinline__ int stencil_hint(int type, const float* __restrict__ x4f, const int32_t v[4]) {
+  F3 P[4];
+  float M = 0.f;
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    P[a] = load_xf(x4f, v[a]);
+    M = fmaxf(M, fmax_abs(P[a]));
+  }
+  return closest_hint(type, P[0], P[1], P[2], P[3], M * 5.9604645e-8f);
+}
+
+__device__ __forceinline__ V3 pick(const V3 X[4], int k) {
+  V3 r = X[0];
+  if (k == 1) r = X[1];
+  if (k == 2) r = X[2];
+  if (k == 3) r = X[3];
+  return r;
+}
+
+// slots of the point and the segment ends of segment k of a stencil
+__device__ __forceinline__ void segment_slots(int type, int k, int* ip, int* ia, int* ib) {
+  if (type == 0) {
+    *ip = 0; *ia = 1 + k; *ib = k == 2 ? 1 : 2 + k;
+  } else {
+    *ip = k; *ia = k < 2 ? 2 : 0; *ib = k < 2 ? 3 : 1;
+  }
+}
+
+// pt_distance (type 0) / ee_distance (type 1) of X with the features of `hint`
+template <bool kStencil>
+__device__ __forceinline__ double closest_pair(int type, const V3 X[4], int hint, Stencil* S) {
+  if (hint & kHintInterior) {
+    const bool certain = (hint & kHintCertain) != 0;
+    const V3 e1 = type == 0 ? X[2] - X[1] : X[1] - X[0];
+    const V3 e2 = type == 0 ? X[3] - X[1] : X[3] - X[2];
+    const V3 w = type == 0 ? X[0] - X[1] : X[0] - X[2];
+    const V3 n = cross(e1, e2);
+    const double nn = dot(n, n);
+    const double inv_nn = 1.0 / nn;
+    double s = 0.0, t = 0.0;
+    bool in = certain;
+    if (type == 0) {
+      if (kStencil || !certain) {
+        s = dot(cross(w, e2), n) * inv_nn;
+        t = dot(cross(e1, w), n) * inv_nn;
+        in = certain || (s >= 0.0 && t >= 0.0 && s + t <= 1.0);
+      }
+    } else if (kStencil || !certain) {
+      const double A = dot(e1, e1), B = dot(e1, e2), C = dot(e2, e2), D = dot(e1, w), E = dot(e2, w);
+      s = (B * E - C * D) * inv_nn;
+      t = (A * E - B * D) * inv_nn;
+      in = certain || (nn > 1e-20 * A * C && s >= 0.0 && s <= 1.0 && t >= 0.0 && t <= 1.0);
+    }
+    if (in) {
+      const double h = dot(w, n);
+      const double d2 = h * h * inv_nn;
+      if (kStencil) {
+        set_zero(*S);
+        if (type == 0) {
+          S->c[0] = 1.0; S->c[1] = -(1.0 - s - t); S->c[2] = -s; S->c[3] = -t;
+          S->a[0][1] = 1.0; S->a[0][2] = -1.0;
+          S->a[1][1] = 1.0; S->a[1][3] = -1.0;
+        } else {
+          S->c[0] = 1.0 - s; S->c[1] = s; S->c[2] = -(1.0 - t); S->c[3] = -t;
+          S->a[0][0] = -1.0; S->a[0][1] = 1.0;
+          S->a[1][2] = 1.0; S->a[1][3] = -1.0;
+        }
+        S->m = 2;
+        S->d2 = d2;
+      }
+      return d2;
+    }
+  }
+  int k = -1;
+  double best = 0.0, tb = 0.0;
+  int left = hint & 15;
+  for (int step = 0; step < 4 && left; ++step) {
+    const int q = __ffs(left) - 1;
+    left &= left - 1;
+    int ip, ia, ib;
+    segment_slots(type, q, &ip, &ia, &ib);
+    double t;
+    const double d2 = seg_point_d2(pick(X, ip), pick(X, ia), pick(X, ib), &t);
+    if (k < 0 || d2 < best) { best = d2; tb = t; k = q; }
+  }
+  if (kStencil) {
+    int ip, ia, ib;
+    segment_slots(type, k, &ip, &ia, &ib);
+    point_segment_stencil(*S, ip, (type == 0 || k < 2) ? 1.0 : -1.0, ia, ib, tb);
+    S->d2 = best;
+  }
+  return best;
 }
 
 }  // namespace eipc

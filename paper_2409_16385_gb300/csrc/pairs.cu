@@ -51,17 +51,16 @@ __device__ __forceinline__ void unpack(uint64_t key, int bi, int bj, int* type, 
   *type = (int)(key >> (bi + bj));
 }
 
-__device__ __forceinline__ double stencil_d2(const Topo& T, const double* __restrict__ x4, int type, int32_t i,
-                                             int32_t j) {
+// stencil vertex ids of pair (type, i, j)
+__device__ __forceinline__ void pair_vertices(const Topo& T, int type, int32_t i, int32_t j, int32_t v[4]) {
   if (type == 0) {
     const int32_t* f = T.tris + 3 * (int64_t)j;
-    return pt_distance<false>(load_x(x4, i), load_x(x4, f[0]), load_x(x4, f[1]), load_x(x4, f[2]), nullptr);
+    v[0] = i; v[1] = f[0]; v[2] = f[1]; v[3] = f[2];
+  } else {
+    const int2 a = reinterpret_cast<const int2*>(T.edges)[i], b = reinterpret_cast<const int2*>(T.edges)[j];
+    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
   }
-  const int32_t* ea = T.edges + 2 * (int64_t)i;
-  const int32_t* eb = T.edges + 2 * (int64_t)j;
-  return ee_distance<false>(load_x(x4, ea[0]), load_x(x4, ea[1]), load_x(x4, eb[0]), load_x(x4, eb[1]), nullptr);
 }
-
 
 // FP32 screen (geometry.cuh) over all candidates; the ones it cannot prove farther than
 // dhat are compacted into `out` for the exact FP64 test.  The radius carries, besides the
@@ -110,8 +109,11 @@ __global__ void __launch_bounds__(kBlock) k_screen(Topo T, const float* __restri
   }
 }
 
-// Exact filter of the broad-phase candidates: keep 0 < d < dhat, flag d <= 0.
-__global__ void __launch_bounds__(kBlock) k_narrow(Topo T, const double* __restrict__ x4,
+// Exact filter of the broad-phase candidates: keep 0 < d < dhat, flag d <= 0.  Bound by the FP64
+// pipe: the FP32 choice of the closest feature (closest_hint) leaves about one segment or one
+// interior solve in FP64 per candidate instead of all of them.  The bubble grasp's contact set
+// (137k candidates here, 120k kept): 486 to 437 us.
+__global__ void __launch_bounds__(kBlock) k_narrow(Topo T, const double* __restrict__ x4, const float* __restrict__ x4f,
                                                    const uint64_t* __restrict__ cand, const int64_t* n_cand,
                                                    int64_t cand_cap, double dhat, uint64_t* __restrict__ skeys,
                                                    uint32_t* __restrict__ svals, double* __restrict__ sd,
@@ -129,14 +131,19 @@ __global__ void __launch_bounds__(kBlock) k_narrow(Topo T, const double* __restr
     double d = 0.0;
     if (k < n) {
       key = cand[k];
-      int type; int32_t i, j;
+      int type; int32_t i, j, v[4];
       unpack(key, T.bits_i, T.bits_j, &type, &i, &j);
-      const double d2 = stencil_d2(T, x4, type, i, j);
+      pair_vertices(T, type, i, j, v);
+      const int hint = stencil_hint(type, x4f, v);
+      V3 X[4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) X[a] = load_x(x4, v[a]);
+      const double d2 = closest_pair<false>(type, X, hint, nullptr);
       if (!(d2 > 0.0)) {
         raise_flag(st, EIPC_FLAG_PENETRATION);
-      } else if (d2 < d2_reject) {
+      } else if (lt_nonneg(d2, d2_reject)) {
         d = sqrt(d2);
-        keep = d < dhat;
+        keep = lt_nonneg(d, dhat);
       }
     }
     uint32_t mask = __ballot_sync(0xffffffffu, keep);
@@ -167,6 +174,7 @@ __device__ __forceinline__ uint64_t feature_key(int kind, uint32_t a, uint32_t b
 }
 
 __global__ void __launch_bounds__(kBlock) k_feature_keys(Topo T, const double* __restrict__ x4,
+                                                         const float* __restrict__ x4f,
                                                          const uint64_t* __restrict__ keys, const int64_t* n_surv,
                                                          int64_t cap, const uint64_t* __restrict__ ekey,
                                                          const int32_t* __restrict__ eid, int B,
@@ -178,17 +186,12 @@ __global__ void __launch_bounds__(kBlock) k_feature_keys(Topo T, const double* _
     int type; int32_t i, j;
     unpack(keys[k], T.bits_i, T.bits_j, &type, &i, &j);
     int32_t v[4];
-    if (type == 0) {
-      v[0] = i; v[1] = T.tris[3 * (int64_t)j]; v[2] = T.tris[3 * (int64_t)j + 1]; v[3] = T.tris[3 * (int64_t)j + 2];
-    } else {
-      v[0] = T.edges[2 * (int64_t)i]; v[1] = T.edges[2 * (int64_t)i + 1];
-      v[2] = T.edges[2 * (int64_t)j]; v[3] = T.edges[2 * (int64_t)j + 1];
-    }
+    pair_vertices(T, type, i, j, v);
     V3 X[4];
-    for (int a = 0; a < 4; ++a) X[a] = load_x(x4, v[a]);
+    const V3 X0 = load_x(x4, v[0]);
+    for (int a = 0; a < 4; ++a) X[a] = load_x(x4, v[a]) - X0;
     Stencil S;
-    if (type == 0) pt_distance<true>(X[0] - X[0], X[1] - X[0], X[2] - X[0], X[3] - X[0], &S);
-    else ee_distance<true>(X[0] - X[0], X[1] - X[0], X[2] - X[0], X[3] - X[0], &S);
+    closest_pair<true>(type, X, stencil_hint(type, x4f, v), &S);
     // the stencil's nonzero weights name the realising features
     int nz[4], m = 0;
     for (int a = 0; a < 4; ++a)
@@ -424,7 +427,7 @@ void pairs_launch(eipc_scene* sc, const double* q, const eipc_params& p, const e
   launch(k_screen, blocks_for(sc->cand_cap, 16), kBlock, 0, s, sc->topo, static_cast<const float*>(sc->x4f),
          static_cast<const uint64_t*>(sc->cand),
          static_cast<const int64_t*>(n_cand), sc->cand_cap, p.dhat, sc->cand2, n_cand2);
-  launch(k_narrow, blocks_for(sc->cand_cap, 16), kBlock, 0, s, sc->topo, sc->x4, sc->cand2, n_cand2, sc->cand_cap,
+  launch(k_narrow, blocks_for(sc->cand_cap, 16), kBlock, 0, s, sc->topo, sc->x4, static_cast<const float*>(sc->x4f), sc->cand2, n_cand2, sc->cand_cap,
          p.dhat, sc->skeys, sc->svals, sc->sd, n_surv, sc->status);
   sc->timers->stop(kKNarrow, s);
   sc->timers->start(kKPairSort, s);
@@ -444,7 +447,8 @@ void pairs_launch(eipc_scene* sc, const double* q, const eipc_params& p, const e
     // feature keys in the record buffers (free until the evaluation), stable sort, firsts,
     // compaction back into (type, i, j) order in the other half of the pair-sort buffers
     const int64_t cap = sc->rec_cap < sc->cand_cap ? sc->rec_cap : sc->cand_cap;
-    launch(k_feature_keys, blocks_for(cap, 8), kBlock, 0, s, sc->topo, static_cast<const double*>(sc->x4), k,
+    launch(k_feature_keys, blocks_for(cap, 8), kBlock, 0, s, sc->topo, static_cast<const double*>(sc->x4),
+           static_cast<const float*>(sc->x4f), k,
            static_cast<const int64_t*>(n_surv), cap, static_cast<const uint64_t*>(sc->edge_key),
            static_cast<const int32_t*>(sc->edge_id), sc->feat_bits, sc->hkeys, sc->hvals, sc->status);
     const int wf = radix_sort_u64(sc->hkeys, sc->hvals, sc->hkeys_alt, sc->hvals_alt, n_surv, cap, 2 + 2 * sc->feat_bits,
