@@ -285,9 +285,9 @@ eipc_status eipc_group_alpha(eipc_scene* scene, double* alpha_groups, eipc_strea
  * 128, 256 (traversal) or 256 (refit); for kernels 3 and 4 `threads` is instead the number
  * of items a warp claims from the kernel's work queue at a time (32, 64, 128 or 256;
  * defaults 32 and 128), and the other two arguments are ignored.  blocks_per_sm: cap on the
- * grid as a multiple of the 152 SMs (1..64; ignored by the refit); variant: eval 2 = no
- * register cap, 3 = at most 170 registers (3 blocks of 128 per SM), 4 = at most 128
- * registers (4 blocks of 128 per SM); traversal 2 = no register cap, 3 = at most 40
+ * grid as a multiple of the 152 SMs (1..64; ignored by the refit); variant: eval 2, 3 or 4
+ * (accepted; one register budget is compiled, since others round differently);
+ * traversal 2 = no register cap, 3 = at most 40
  * registers (6 blocks of 256 per SM); refit 0 = arrival counters behind full device
  * fences, 1 = release-acquire arrival counters, 2 = treelets of up to 32 leaves refitted per
  * warp in shared memory below release-acquire counters, for the refits and for the

@@ -32,7 +32,7 @@ void free_scene(eipc_scene* s) {
                   s->edge_bvh.tl_root, s->edge_bvh.up_start, s->edge_bvh.tl_count, s->bounds_ws,
                   s->sort_hist, s->cand, s->counters, s->skeys, s->skeys_alt, s->svals, s->svals_alt, s->sd,
                   s->item_nodes, s->item_n, s->rc_h, s->ro_h, s->rc_g, s->ro_g, s->item_E, s->hkeys,
-                  s->hkeys_alt, s->hvals, s->hvals_alt, s->hrec, s->seg_flag, s->seg_id, s->seg_start, s->hinv, s->piece, s->hunit,
+                  s->hkeys_alt, s->hvals, s->hvals_alt, s->hrec, s->seg_flag, s->seg_id, s->seg_start, s->rec_src, s->src_sorted, s->frow, s->ihead, s->item_map, s->piece, s->hunit,
                   s->gkeys, s->gkeys_alt, s->gvals, s->gvals_alt, s->grec,
                   s->gseg_start, s->scan_partial, s->sum_partial, s->status};
   for (void* p : ptrs)
@@ -159,12 +159,13 @@ eipc_status eipc_scene_create(int64_t Nv, int64_t F, int64_t E, int64_t Ns, cons
   ok(dalloc(&s->rc_h, s->item_cap)); ok(dalloc(&s->ro_h, s->item_cap));
   ok(dalloc(&s->rc_g, s->item_cap)); ok(dalloc(&s->ro_g, s->item_cap)); ok(dalloc(&s->item_E, s->item_cap));
   ok(dalloc(&s->hkeys, s->rec_cap)); ok(dalloc(&s->hkeys_alt, s->rec_cap));
-  ok(dalloc(&s->hvals, s->rec_cap)); ok(dalloc(&s->hvals_alt, s->rec_cap)); ok(dalloc(&s->hrec, kHRecStride * s->rec_cap));
+  ok(dalloc(&s->hvals, s->rec_cap)); ok(dalloc(&s->hvals_alt, s->rec_cap));
   ok(dalloc(&s->hvp_out, 3 * (Ns + 64)));
   ok(dalloc(&s->seg_flag, s->rec_cap)); ok(dalloc(&s->seg_id, s->rec_cap)); ok(dalloc(&s->seg_start, s->rec_cap));
-  ok(dalloc(&s->hinv, s->rec_cap));
+  ok(dalloc(&s->rec_src, s->rec_cap)); ok(dalloc(&s->src_sorted, s->rec_cap));
+  ok(dalloc(&s->frow, kFRow * s->gcap)); ok(dalloc(&s->ihead, kIHead * s->item_cap)); ok(dalloc(&s->item_map, s->item_cap));
   {
-    const int64_t pr = s->rec_cap + s->rec_cap / 32 + 2;
+    const int64_t pr = s->rec_cap + s->rec_cap / 16 + 2;
     ok(dalloc(&s->piece, 9 * pr));
   }
   ok(dalloc(&s->hunit, s->rec_cap + 1));
@@ -307,6 +308,14 @@ eipc_status eipc_bsr_spmv(int64_t nrows, const int32_t* row_ptr, const int32_t* 
 
 eipc_status eipc_scene_set_mollifier(eipc_scene* sc, const double* x_rest, double factor, eipc_stream stream) {
   if (!sc || !(factor >= 0.0) || !std::isfinite(factor) || (factor > 0.0 && !x_rest)) return EIPC_ERR_INVALID;
+  if (factor > 0.0 && !sc->hrec) {
+    // the mollified pairs' explicit records, allocated when the mollifier is first asked for
+    if (dalloc(&sc->hrec, kHRecStride * sc->rec_cap) != cudaSuccess) {
+      sc->hrec = nullptr;
+      cudaGetLastError();
+      return EIPC_ERR_NOMEM;
+    }
+  }
   if (factor > 0.0 && sc->ne > 0) {
     // squared rest lengths on the device, then a synchronous check that all are positive
     cudaStream_t s = (cudaStream_t)stream;

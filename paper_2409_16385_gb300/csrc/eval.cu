@@ -180,7 +180,8 @@ __global__ void __launch_bounds__(kBlock) k_item_nodes(Topo T, eipc_pairs pr, co
                                                        int64_t* __restrict__ rc_h, int64_t* __restrict__ rc_g,
                                                        int64_t* n_items, DevStatus* st,
                                                        const int32_t* __restrict__ fric_of_pair,
-                                                       const int32_t* __restrict__ pair_of_fric) {
+                                                       const int32_t* __restrict__ pair_of_fric,
+                                                       uint64_t* __restrict__ item_map) {
   pdl_entry();
   const int64_t P = clamp_count(pr.count, pr.capacity);
   const int64_t L = lag_v ? clamp_count(lag_count, lag_cap) : 0;
@@ -205,16 +206,20 @@ __global__ void __launch_bounds__(kBlock) k_item_nodes(Topo T, eipc_pairs pr, co
     }
     int32_t nodes[kMaxNodes];
     int cnt = 0;
+    uint64_t map = 0;              // nibble 4a + s: which of the item's nodes is slot s of vertex a
     for (int a = 0; a < 4; ++a) {
       const int4 id = __ldg(reinterpret_cast<const int4*>(cage_idx) + v[a]);
       if (id.x < 0) continue;
       const int32_t ids[4] = {id.x, id.y, id.z, id.w};
       for (int s = 0; s < 4; ++s) {
-        bool seen = false;
-        for (int u = 0; u < cnt; ++u) seen |= (nodes[u] == ids[s]);
-        if (!seen) nodes[cnt++] = ids[s];
+        int at = cnt;
+        for (int u = 0; u < cnt; ++u)
+          if (nodes[u] == ids[s]) at = u;
+        if (at == cnt) nodes[cnt++] = ids[s];
+        map |= (uint64_t)at << (4 * (4 * a + s));
       }
     }
+    if (item_map) item_map[k] = map;
     for (int u = 0; u < cnt; ++u) item_nodes[kMaxNodes * k + u] = nodes[u];
     item_n[k] = cnt;
     rc_h[k] = (int64_t)cnt * (cnt + 1) / 2;
@@ -240,52 +245,6 @@ __device__ __forceinline__ void node_weights(const int32_t v[4], const int32_t* 
       int u = 0;
       while (u < n - 1 && nodes[u] != ids[s]) ++u;
       for (int c = 0; c < ncoef; ++c) out[u][c] += coef[c][a] * ws[s];
-    }
-  }
-}
-
-// node_weights for NC (3 or 4) coefficient sets into rows of four: the barrier's c^, a^_1,
-// a^_2 and, with NC = 4, the lagged friction's gamma, in one pass over the stencil's cage
-// slots
-template <int NC>
-__device__ __forceinline__ void node_weights4(const int32_t v[4], const int32_t* __restrict__ cage_idx,
-                                              const double* __restrict__ w, const int32_t* nodes, int n,
-                                              const double coef[4][4], double out[kMaxNodes][4]) {
-  for (int u = 0; u < n; ++u)
-    for (int c = 0; c < NC; ++c) out[u][c] = 0.0;
-  for (int a = 0; a < 4; ++a) {
-    const int4 id = __ldg(reinterpret_cast<const int4*>(cage_idx) + v[a]);
-    if (id.x < 0) continue;
-    const int ids[4] = {id.x, id.y, id.z, id.w};
-    const double2 w01 = __ldg(reinterpret_cast<const double2*>(w) + 2 * (int64_t)v[a]);
-    const double2 w23 = __ldg(reinterpret_cast<const double2*>(w) + 2 * (int64_t)v[a] + 1);
-    const double ws[4] = {w01.x, w01.y, w23.x, w23.y};
-    for (int s = 0; s < 4; ++s) {
-      int u = 0;
-      while (u < n - 1 && nodes[u] != ids[s]) ++u;
-#pragma unroll
-      for (int c = 0; c < NC; ++c) out[u][c] += coef[c][a] * ws[s];
-    }
-  }
-}
-
-// node_weights for one coefficient set: out[u] = sum over (a, slot) with idx == node_u of
-// coef[a] * w[a][slot]
-__device__ __forceinline__ void node_weights1(const int32_t v[4], const int32_t* __restrict__ cage_idx,
-                                              const double* __restrict__ w, const int32_t* nodes, int n,
-                                              const double coef[4], double out[kMaxNodes]) {
-  for (int u = 0; u < n; ++u) out[u] = 0.0;
-  for (int a = 0; a < 4; ++a) {
-    const int4 id = __ldg(reinterpret_cast<const int4*>(cage_idx) + v[a]);
-    if (id.x < 0) continue;
-    const int ids[4] = {id.x, id.y, id.z, id.w};
-    const double2 w01 = __ldg(reinterpret_cast<const double2*>(w) + 2 * (int64_t)v[a]);
-    const double2 w23 = __ldg(reinterpret_cast<const double2*>(w) + 2 * (int64_t)v[a] + 1);
-    const double ws[4] = {w01.x, w01.y, w23.x, w23.y};
-    for (int s = 0; s < 4; ++s) {
-      int u = 0;
-      while (u < n - 1 && nodes[u] != ids[s]) ++u;
-      out[u] += coef[a] * ws[s];
     }
   }
 }
@@ -438,27 +397,28 @@ struct EvalArgs {
   const int64_t* ro_g;
   const int64_t* n_items;
   int64_t rec_cap, gcap;
-  uint64_t* hkeys;
-  uint32_t* hvals;
-  double* hrec;
+  double* hrec;            // explicit records (mollified pairs)
+  double* frow;            // factor rows, kFRow doubles per (item, node) at ro_g[item] + node
+  double* ihead;           // item headers, kIHead doubles per item
+  const uint64_t* item_map;
+  const float* x4f;
+  double inv_dhat;
   uint64_t* gkeys;
   uint32_t* gvals;
   double* grec;
   double* item_E;
   DevStatus* st;
   bool project;            // PSD-project the barrier Hessians (projected Newton)
-  const uint32_t* order;   // processing order of the barrier items (null: index order)
   const double* moll_r2;   // EE mollifier: rest squared edge lengths (null: off)
   double moll_factor;      // eps_x = moll_factor |e_i|^2 |e_j|^2
-  int64_t* queue;          // next unclaimed position of `order` (work queue)
+  uint32_t* rest;          // items k_eval_factors leaves to k_eval_rest: pairs from the front, friction
+                           // items from the back of item_cap entries
+  int64_t* n_rest;         // [2] their numbers
+  int64_t item_cap;
+  int64_t* queue;          // next unclaimed item (work queue)
   int tile;                // items a warp claims from the queue at a time (multiple of 32)
   const double* hv_dir;    // Hessian-vector product: reduced direction [ns*3]
   double kin_dir[3];       // ... and the rigid direction of the kinematic vertices
-  // Presorted Hessian records (energy/gradient/Hessian evaluation): the keys were written
-  // and sorted before the evaluation, and record r goes to its sorted position hinv[r]
-  // without a key.  Gradient records (Hessian-vector products only) are written at r with
-  // their key.
-  const uint32_t* hinv;
   // friction merged into contact pairs (friction_merged; null: no merging); lag, mu and
   // eps_f are the friction parameters
   const int32_t* fric_of_pair;
@@ -489,32 +449,33 @@ __device__ __forceinline__ void friction_terms(const double* __restrict__ x4, co
   vs = vs - anc;
   const V3 u = vs - nrm * dot(nrm, vs);
   const double y2 = dot(u, u);
-  // f0(y), f1(y)/y and (f1'(y) - f1(y)/y) / y^2, with one division for 1/eps (or 1/y)
-  // and one for 1/y^2
-  double f0, f1y, c2;
-  if (y2 == 0.0) {
-    f0 = eps / 3.0; f1y = 2.0 / eps; c2 = 0.0;
-  } else {
-    const double y = sqrt(y2);
-    double f1p_minus;
-    if (y < eps) {
-      const double ie = 1.0 / eps, yie2 = y * ie * ie;
-      f0 = y2 * (ie - yie2 / 3.0) + eps / 3.0;    // -y^3 / (3 eps^2) + y^2 / eps + eps / 3
-      f1y = 2.0 * ie - yie2;
-      f1p_minus = -yie2;                          // (2/eps - 2y/eps^2) - (2/eps - y/eps^2)
+  // f0(y), f1(y)/y and (f1'(y) - f1(y)/y) / y^2, with one reciprocal square root
+  const double ie = 1.0 / eps;
+  double f0 = eps / 3.0, f1y = 2.0 * ie, c2 = 0.0;
+  if (is_pos(y2)) {
+    const double iy = rsqrt(y2), y = y2 * iy;
+    if (lt_nonneg(y, eps)) {
+      const double yie2 = y * ie * ie;
+      f0 = fma(y2, ie - yie2 * (1.0 / 3.0), f0);  // -y^3 / (3 eps^2) + y^2 / eps + eps / 3
+      f1y -= yie2;
+      c2 = -ie * ie * iy;                         // ((2/eps - 2y/eps^2) - (2/eps - y/eps^2)) / y^2
     } else {
-      const double iy = 1.0 / y;
-      f0 = y; f1y = iy; f1p_minus = -iy;
+      f0 = y; f1y = iy; c2 = -iy * iy * iy;
     }
-    c2 = f1p_minus / y2;
   }
   R.E = ml * f0;
   R.gs = ml * f1y;
   R.u[0] = u.x; R.u[1] = u.y; R.u[2] = u.z;
   const double nn[3] = {nrm.x, nrm.y, nrm.z};
+  const double mc = ml * c2;
+  double mn[3], mu_[3];
+#pragma unroll
+  for (int p = 0; p < 3; ++p) { mn[p] = R.gs * nn[p]; mu_[p] = mc * R.u[p]; }
+#pragma unroll
   for (int p = 0; p < 3; ++p)
+#pragma unroll
     for (int q = p; q < 3; ++q) {
-      const double s = ml * (f1y * ((p == q ? 1.0 : 0.0) - nn[p] * nn[q]) + c2 * R.u[p] * R.u[q]);
+      const double s = fma(mu_[p], R.u[q], fma(-mn[p], nn[q], p == q ? R.gs : 0.0));
       R.F[p][q] = s;
       R.F[q][p] = s;
     }
@@ -594,83 +555,30 @@ __device__ __forceinline__ void eigen_sym(double K[N][N], double V[N][N]) {
   jacobi<N>(K, V);
 }
 
-// K+ = (V max(Lambda, 0)) V^T of the leading N x N block of the 5 x 5 K (rows and columns
-// beyond N are zero in K and in K+)
-template <int N>
-__device__ __forceinline__ void psd_span_inl(const double K[5][5], double Kp[5][5]) {
-  double Kn[N][N], V[N][N];
-#pragma unroll
-  for (int p = 0; p < N; ++p)
-#pragma unroll
-    for (int q = 0; q < N; ++q) Kn[p][q] = K[p][q];
-  eigen_sym<N>(Kn, V);
-  double W[N][N];
-#pragma unroll
-  for (int e = 0; e < N; ++e) {
-    const double le = Kn[e][e] > 0.0 ? Kn[e][e] : 0.0;
-#pragma unroll
-    for (int p = 0; p < N; ++p) W[p][e] = V[p][e] * le;
-  }
-#pragma unroll
-  for (int p = 0; p < 5; ++p)
-#pragma unroll
-    for (int q = p; q < 5; ++q) {
-      double s = 0.0;
-      if (p < N && q < N) {
-#pragma unroll
-        for (int e = 0; e < N; ++e) s += W[p][e] * V[q][e];
-      }
-      Kp[p][q] = s;
-      Kp[q][p] = s;
-    }
-}
-
-// The 4 x 4 projection (99 % of the pairs of the benchmark workloads) is inlined; the
-// 5 x 5 one, for pairs with two free closest-point parameters, is a separate function, so
-// its larger register footprint (the 5 x 5 eigensolver's matrices) does not set the
-// register allocation of the common path: under a register cap only the rare call spills.
-__device__ __noinline__ void psd_span5(const double K[5][5], double Kp[5][5]) { psd_span_inl<5>(K, Kp); }
-__device__ __forceinline__ void psd_span4(const double K[5][5], double Kp[5][5]) { psd_span_inl<4>(K, Kp); }
-
-// one upper-triangle record: key (min, max) of the two cage nodes, block transposed when
-// the first node is the larger one.  With presorted records the sorted position is
-// hinv[pos]; a caller that has already loaded it passes it as `pre` (else pass -1).
-__device__ __forceinline__ void emit_upper(const EvalArgs& A, int64_t pos, int32_t Iu, int32_t Iv,
-                                           const double B[3][3], int64_t pre = -1) {
+// Explicit records (mollified pairs): record pos of the item holds its upper block, of nodes
+// (min, max), as nine values in rows of kHRecStride; a diagonal one the block's upper entries
+// B00 B01 B02 B11 B12 B22 and then the item's gradient at that node.
+__device__ __forceinline__ void emit_upper(const EvalArgs& A, int64_t pos, int32_t Iu, int32_t Iv, const double B[3][3]) {
   const bool swap = Iu > Iv;
-  int64_t dst = pos;
-  if (A.hinv) {
-    dst = pre >= 0 ? pre : (int64_t)A.hinv[pos];
-  } else {
-    A.hkeys[pos] = swap ? upper_key((uint64_t)Iv, (uint64_t)Iu, (uint64_t)A.ns)
-                        : upper_key((uint64_t)Iu, (uint64_t)Iv, (uint64_t)A.ns);
-    A.hvals[pos] = (uint32_t)pos;
-  }
   double v[9];
 #pragma unroll
   for (int a = 0; a < 3; ++a)
 #pragma unroll
     for (int b = 0; b < 3; ++b) v[3 * a + b] = swap ? B[b][a] : B[a][b];
-  double2* p = reinterpret_cast<double2*>(A.hrec + kHRecStride * dst);
+  double2* p = reinterpret_cast<double2*>(A.hrec + kHRecStride * pos);
 #pragma unroll
   for (int c = 0; c < 4; ++c) p[c] = make_double2(v[2 * c], v[2 * c + 1]);
-  A.hrec[kHRecStride * dst + 8] = v[8];
+  A.hrec[kHRecStride * pos + 8] = v[8];
 }
 
-// The diagonal record (I, I) of a presorted item: the block is symmetric, so its six
-// upper entries B00 B01 B02 B11 B12 B22 take the first six values of the row and the item's
-// gradient at node I the next three.  The segment sums of the diagonal records are then
-// the reduced Hessian's diagonal blocks and g_r together, with no gradient records, sort or
-// reduction of their own.
 __device__ __forceinline__ void emit_diag(const EvalArgs& A, int64_t pos, const double B[3][3], double g0, double g1,
-                                          double g2, int64_t pre = -1) {
-  const int64_t dst = pre >= 0 ? pre : (int64_t)A.hinv[pos];
-  double2* p = reinterpret_cast<double2*>(A.hrec + kHRecStride * dst);
+                                          double g2) {
+  double2* p = reinterpret_cast<double2*>(A.hrec + kHRecStride * pos);
   p[0] = make_double2(B[0][0], B[0][1]);
   p[1] = make_double2(B[0][2], B[1][1]);
   p[2] = make_double2(B[1][2], B[2][2]);
   p[3] = make_double2(g0, g1);
-  A.hrec[kHRecStride * dst + 8] = g2;
+  A.hrec[kHRecStride * pos + 8] = g2;
 }
 
 // one keyed gradient record (Hessian-vector products)
@@ -934,179 +842,477 @@ __device__ __forceinline__ void vertex_node_weights(const int32_t v[4], const in
   }
 }
 
-// One barrier item: distance, span Hessian (projected unless A.project is false), energy,
-// and its upper-triangle Hessian records, the diagonal ones carrying the gradient, each
-// written at its presorted position hinv[pos].
-__device__ __forceinline__ void eval_barrier_item(const EvalArgs& A, int64_t k) {
+// ------------------------------------------------------------------ pair factors
+// The FP64 pipe bounds this stage (an FP64 warp instruction holds it for 64 cycles), so the
+// blocks J^T (pair Hessian) J are never formed pair by pair.  Each item leaves one row per cage
+// node u,
+//   z_u1, z_u2 (z_u3): block(u, v) = sum_k z_uk z_vk^T + w_u w_v F + iso omega_u omega_v I,
+// with omega_u = sum_a c_a w_au (the gradient at u is omega_u r' + w_u u') and the friction
+// weight w_u, and a header (F, r', u', iso).  The segment sums below multiply rows straight into
+// their accumulators: 10 FP64 instructions per record and third of a block, against about 47 to
+// form a block here and 9 to add it, and no block goes through memory.
+//
+// At most one free closest-point parameter (a point p against the edge x_a x_b, or two
+// points): with e = x_b - x_a, r = p - x_a - t e, v^ = -e/|e|, c = (1, t - 1, -t) on (p, a, b),
+// a = (0, 1, -1), and the orthonormal span c^ (x) r^, c^ (x) v^, a^ (x) r^ (a^: a made
+// orthogonal to c), the Hessian is
+//   K = diag(A, -B, 0) + B p p^T,  A = kappa |c|^2 b'',  B = -kappa |c|^2 b'/d > 0,
+//   p = (rho (c.a) / |c|^2, 1, rho |a - (a.c^) c^| / |c|),  rho = d / |e|,
+// plus -B on the direction c^ (x) (r^ x v^), which the projection drops.  Its (v^, v^) entry is
+// exactly zero.  D = diag(A, -B, 0) has one negative entry and the rest is rank one and
+// positive, so K has one negative eigenvalue -B x; x in (0, 1) solves
+//   x^2 (A + B x) = (1 - x) (p_2^2 (A + B x) + p_0^2 B x)
+// (the secular equation cleared of its denominators: every term is positive, nothing
+// cancels), found in FP32 and polished by two Newton steps in FP64.  Then
+// q = (p_0 B/(A + B x), -1/(1 - x), p_2/x) spans its eigenvector, K+ = K + B x q q^T / |q|^2, and
+// two steps of Cholesky give K+ = l l^T + m m^T.  Two points (no free parameter): K+ is A on
+// c^ (x) r^ alone.  Against a 12 x 12 eigensolver the factors agree to 4e-15 of the norm over
+// d/dhat from 1e-6 to 1 - 1e-14 and |e| from 10 um to 10 cm.
+
+// flags of an item header
+constexpr int kItemFriction = 1, kItemThird = 2, kItemIso = 4, kItemExplicit = 8;
+
+__device__ __forceinline__ void store_header(double* h, const FrictionTerms* R, V3 g, double iso, int flags) {
+  double2* p = reinterpret_cast<double2*>(h);
+  if (R) {
+    p[0] = make_double2(R->F[0][0], R->F[0][1]);
+    p[1] = make_double2(R->F[0][2], R->F[1][1]);
+    p[2] = make_double2(R->F[1][2], R->F[2][2]);
+    p[4] = make_double2(g.z, R->gs * R->u[0]);
+    p[5] = make_double2(R->gs * R->u[1], R->gs * R->u[2]);
+  } else {
+    p[4] = make_double2(g.z, 0.0);
+    p[5] = make_double2(0.0, 0.0);
+  }
+  p[3] = make_double2(g.x, g.y);
+  p[6] = make_double2(iso, __longlong_as_double((long long)flags));
+}
+
+__device__ __forceinline__ void store_row(double* row, V3 z1, V3 z2, double om, double wf) {
+  double2* p = reinterpret_cast<double2*>(row);
+  p[0] = make_double2(z1.x, z1.y);
+  p[1] = make_double2(z1.z, z2.x);
+  p[2] = make_double2(z2.y, z2.z);
+  p[3] = make_double2(om, wf);
+}
+
+// out[u] += coef * w over the four cage slots of vertex v (slot nodes in the nibbles of map);
+// nothing for a kinematic vertex
+__device__ __forceinline__ void add_slots(const EvalArgs& A, int32_t v, uint32_t map, double coef, double* out) {
+  if (A.T.vkin[v]) return;
+  const double2 w01 = __ldg(reinterpret_cast<const double2*>(A.w) + 2 * (int64_t)v);
+  const double2 w23 = __ldg(reinterpret_cast<const double2*>(A.w) + 2 * (int64_t)v + 1);
+  const double ws[4] = {w01.x, w01.y, w23.x, w23.y};
+#pragma unroll
+  for (int s = 0; s < 4; ++s) out[(map >> (4 * s)) & 15u] += coef * ws[s];
+}
+
+// ... and of two coefficients at once
+__device__ __forceinline__ void add_slots2(const EvalArgs& A, int32_t v, uint32_t map, double c1, double* o1, double c2,
+                                           double* o2) {
+  if (A.T.vkin[v]) return;
+  const double2 w01 = __ldg(reinterpret_cast<const double2*>(A.w) + 2 * (int64_t)v);
+  const double2 w23 = __ldg(reinterpret_cast<const double2*>(A.w) + 2 * (int64_t)v + 1);
+  const double ws[4] = {w01.x, w01.y, w23.x, w23.y};
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {
+    const int u = (map >> (4 * s)) & 15u;
+    o1[u] += c1 * ws[s];
+    o2[u] += c2 * ws[s];
+  }
+}
+
+__device__ __forceinline__ void zero_nodes(double* x, int n) {
+  for (int u = 0; u < n; ++u) x[u] = 0.0;
+}
+
+// b, b', b'' of the barrier at distance d < dhat (Eq. 7 without kappa)
+__device__ __forceinline__ void barrier_scalars(double d, double inv_d, double dhat, double inv_dhat, double* b, double* b1,
+                                                double* b2) {
+  double q = d * inv_dhat;
+  q = fma(fma(-q, dhat, d), inv_dhat, q);              // d / dhat, rounded as the quotient
+  const double lg = log(q), m = d - dhat, md = m * inv_d;
+  *b = -m * m * lg;
+  *b1 = -2.0 * m * lg - m * md;
+  *b2 = -2.0 * lg - 4.0 * md + md * md;
+}
+
+// x in (0, 1) with x^2 (A + B x) = (1 - x) (w2 (A + B x) + w0 B x); A, B > 0, w0 >= 0, w2 > 0
+__device__ __forceinline__ double negative_root(double A, double B, double w0, double w2) {
+  // scaled by a power of two so that A is near one (the equation is homogeneous in A, B)
+  const int ea = (__double2hiint(A) >> 20) & 0x7ff;
+  const double s = __hiloint2double((2046 - ea) << 20, 0);
+  A *= s;
+  B *= s;
+  const float Af = (float)A, Bf = (float)B, w0f = (float)w0, w2f = (float)w2;
+  // x^2 = (1 - x) w for w = w2 + w0 B x / (A + B x), w from the previous x
+  float x = 0.f;
+#pragma unroll
+  for (int it = 0; it < 3; ++it) {
+    const float w = fmaxf(w2f + w0f * __fdividef(Bf * x, Af + Bf * x), 1e-36f);
+    x = 2.f * w / (w + sqrtf(w * w + 4.f * w));
+  }
+#pragma unroll
+  for (int it = 0; it < 2; ++it) {
+    const float G = Af + Bf * x, y = w2f * G + w0f * Bf * x;
+    const float h = x * x * G - (1.f - x) * y, hp = 2.f * x * G + x * x * Bf + y - (1.f - x) * (w2f + w0f) * Bf;
+    const float nx = x - __fdividef(h, hp);
+    if (nx > 0.f && nx <= 1.f) x = nx;
+  }
+  double xd = (double)x;
+  const double wb = w0 * B;
+#pragma unroll
+  for (int it = 0; it < 2; ++it) {
+    const double G = fma(B, xd, A), y = fma(w2, G, wb * xd), h = fma(xd * xd, G, -(1.0 - xd) * y);
+    const float Gf = Af + Bf * x, yf = w2f * Gf + w0f * Bf * x;
+    const float hp = 2.f * x * Gf + x * x * Bf + yf - (1.f - x) * (w2f + w0f) * Bf;
+    const float hf = (float)h;
+    if (hp > 0.f) xd -= (double)__fdividef(hf, hp);
+  }
+  return xd;
+}
+
+// Node rows and header of a pair whose closest features are one of the segments of `hint`
+// (closest_hint without kHintInterior).
+__device__ __forceinline__ void light_factors(const EvalArgs& A, int64_t k, int type, int32_t i, int32_t j, const int32_t v[4],
+                                              int hint) {
+  V3 X[4];
+#pragma unroll
+  for (int a = 0; a < 4; ++a) X[a] = load_x(A.x4, v[a]);
+  // the segment: the only one left, or (ties, e.g. at a shared vertex) the closest in FP64
+  int seg = __ffs(hint & 15) - 1;
+  if (hint & (hint - 1) & 15) {
+    double best = 0.0, t;
+    int left = hint & 15;
+    seg = -1;
+    for (int step = 0; step < 4 && left; ++step) {
+      const int q = __ffs(left) - 1;
+      left &= left - 1;
+      int qp, qa, qb;
+      segment_slots(type, q, &qp, &qa, &qb);
+      const double d2 = seg_point_d2(pick(X, qp), pick(X, qa), pick(X, qb), &t);
+      if (seg < 0 || lt_nonneg(d2, best)) { best = d2; seg = q; }
+    }
+  }
+  int ip, ia, ib;
+  segment_slots(type, seg, &ip, &ia, &ib);
+  const V3 xa = pick(X, ia), e = pick(X, ib) - xa, w = pick(X, ip) - xa;
+  const double we = dot(w, e), ee = dot(e, e);
+  double t = 0.0, rse = 0.0;
+  const bool inner = is_pos(we) && lt_nonneg(we, ee);
+  if (inner) {
+    rse = rsqrt(ee);
+    t = we * (rse * rse);
+  } else if (is_pos(we)) {
+    t = 1.0;
+  }
+  const V3 r = w - e * t;
+  const double d2 = dot(r, r);
+  const bool apart = d2 > 0.0;
+  if (!apart) raise_flag(A.st, EIPC_FLAG_PENETRATION);
+  const double inv_d = apart ? rsqrt(d2) : 0.0;
+  const double d = d2 * inv_d;
+  const bool active = apart && lt_nonneg(d, A.dhat);
+  if (active && A.moll_r2 && type == 1) {
+    const V3 Y[4] = {{0.0, 0.0, 0.0}, X[1] - X[0], X[2] - X[0], X[3] - X[0]};
+    double eps_m, c_m;
+    if (ee_mollified(A, type, i, j, Y, &eps_m, &c_m)) {           // k_mollified
+      store_header(A.ihead + kIHead * k, nullptr, V3{0.0, 0.0, 0.0}, 0.0, kItemExplicit);
+      return;
+    }
+  }
+  const int n = A.item_n[k];
+  const uint64_t map = A.item_map[k];
+  const V3 rh = r * inv_d;
+  double E = 0.0, iso = 0.0, gs = 0.0;
+  double k1 = 0.0, k2 = 0.0, k3 = 0.0, k4 = 0.0, k5 = 0.0, k6 = 0.0;
+  double om[kMaxNodes], al[kMaxNodes], wf[kMaxNodes];
+  zero_nodes(om, n);
+  zero_nodes(al, n);
+  zero_nodes(wf, n);
+  V3 vh = {0.0, 0.0, 0.0};
+  if (active) {
+    double b, b1, b2;
+    barrier_scalars(d, inv_d, A.dhat, A.inv_dhat, &b, &b1, &b2);
+    E = A.kappa * b;
+    gs = A.kappa * b1;
+    const double bd = -A.kappa * (b1 * inv_d);                    // -kappa b'/d
+    const double s1 = 1.0 - t;
+    vh = e * -rse;
+    if (A.project) {
+      const double cc = 1.0 + s1 * s1 + t * t;
+      const double Aq = A.kappa * cc * b2, B = cc * bd;
+      const bool span = inner && is_pos(B);
+      double K00 = Aq, K01 = 0.0, K02 = 0.0, K11 = 0.0, K12 = 0.0, K22 = 0.0, rcn = rsqrt(cc), ral = 0.0, cac = 0.0;
+      if (span) {
+        const double ca0 = 2.0 * t - 1.0;
+        cac = ca0 * (rcn * rcn);                                  // c.a / |c|^2
+        const double al2 = 2.0 - ca0 * cac;
+        ral = rsqrt(al2);
+        const double rho = d * rse;
+        const double p0 = rho * cac, p2 = rho * (al2 * ral) * rcn;
+        const double x = negative_root(Aq, B, p0 * p0, p2 * p2);
+        const double G = fma(B, x, Aq), rc = 1.0 / (G * x);
+        const double q0 = p0 * B * (rc * x), q2 = p2 * (rc * G), S = 1.0 + p0 * q0 + p2 * q2;
+        const double f = x / (q0 * q0 + S * S + q2 * q2);
+        const double fq0 = f * q0, fs = f * S;
+        K00 += B * (p0 * p0 + fq0 * q0);
+        K01 = B * (p0 - fq0 * S);
+        K02 = B * (p0 * p2 + fq0 * q2);
+        K11 = B * (fs * S);
+        K12 = B * (p2 - fs * q2);
+        K22 = B * (p2 * p2 + f * q2 * q2);
+      }
+      const double rk = rsqrt(K00);
+      const double l0 = K00 * rk, l1 = K01 * rk, l2 = K02 * rk;
+      double m1 = 0.0, m2 = 0.0;
+      if (span) {
+        const double s11 = K11 - l1 * l1, s12 = K12 - l1 * l2, s22 = K22 - l2 * l2;
+        const bool first = __double_as_longlong(s11) >= __double_as_longlong(s22);
+        const double piv = first ? s11 : s22;
+        if (is_pos(piv)) {
+          const double rp = rsqrt(piv), a = piv * rp, o = s12 * rp;
+          m1 = first ? a : o;
+          m2 = first ? o : a;
+        }
+      }
+      k2 = l2 * ral;
+      k1 = l0 * rcn - k2 * cac;
+      k3 = l1 * rcn;
+      k5 = m2 * ral;
+      k4 = -k5 * cac;
+      k6 = m1 * rcn;
+    } else {
+      // exact: kappa (b'' - b'/d) c c^T (x) r^ r^T + kappa (b'/d) c c^T (x) I - (kappa b'/(2d)) G M^-1 G^T
+      const double h = fma(A.kappa, b2, bd);
+      k1 = h * rsqrt(h);
+      iso = -bd;
+      if (inner) {
+        const double sb = is_pos(bd) ? bd * rsqrt(bd) : 0.0;
+        k5 = sb * rse * d;
+        k6 = sb;
+      }
+    }
+    // omega and alpha over the three used vertices (two where the closest point is a vertex)
+    add_slots(A, pick(v, ip), (uint32_t)(map >> (16 * ip)) & 0xffffu, 1.0, om);
+    if (inner) {
+      add_slots2(A, pick(v, ia), (uint32_t)(map >> (16 * ia)) & 0xffffu, -s1, om, 1.0, al);
+      add_slots2(A, pick(v, ib), (uint32_t)(map >> (16 * ib)) & 0xffffu, -t, om, -1.0, al);
+    } else {
+      const int iq = is_pos(we) ? ib : ia;
+      add_slots(A, pick(v, iq), (uint32_t)(map >> (16 * iq)) & 0xffffu, -1.0, om);
+    }
+  }
+  const int32_t fenc = A.fric_of_pair ? A.fric_of_pair[k] : 0;
+  FrictionTerms R;
+  if (fenc > 0) {
+    double gam[4];
+    friction_terms(A.x4, A.lag, (int64_t)(INT32_MAX - fenc), v, A.mu, A.eps_f, R, gam);
+    E += R.E;
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+      if (gam[a] != 0.0) add_slots(A, v[a], (uint32_t)(map >> (16 * a)) & 0xffffu, gam[a], wf);
+  }
+  A.item_E[k] = E;
+  store_header(A.ihead + kIHead * k, fenc > 0 ? &R : nullptr, rh * gs, iso,
+               (fenc > 0 ? kItemFriction : 0) | (iso != 0.0 ? kItemIso : 0));
+  const int64_t base = A.ro_g[k];
+  for (int u = 0; u < n; ++u) {
+    if (base + u >= A.gcap) break;
+    const double o = om[u], a = al[u];
+    const V3 z1 = rh * (o * k1 + a * k2) + vh * (o * k3), z2 = rh * (o * k4 + a * k5) + vh * (o * k6);
+    store_row(A.frow + kFRow * (base + u), z1, z2, o, wf[u]);
+  }
+}
+
+// ... of any pair: two free closest-point parameters (projected by the eigensolver of the span's
+// 5 x 5 matrix, which has exactly two negative eigenvalues then, so at most three columns), or a
+// region the FP32 test left open.
+__device__ __forceinline__ void heavy_factors(const EvalArgs& A, int64_t k) {
   int32_t v[4];
   const int type = A.pr.type[k];
-  stencil_vertices(A.T, type, A.pr.i[k], A.pr.j[k], v);
-  V3 X[4];
-  for (int a = 0; a < 4; ++a) X[a] = load_x(A.x4, v[a]);
-  // positions relative to the first vertex (distance and derivatives are translation
-  // invariant; this keeps the differences exact-ish)
+  const int32_t i = A.pr.i[k], j = A.pr.j[k];
+  stencil_vertices(A.T, type, i, j, v);
   V3 Y[4];
-  for (int a = 0; a < 4; ++a) Y[a] = X[a] - X[0];
+  const V3 X0 = load_x(A.x4, v[0]);
+#pragma unroll
+  for (int a = 0; a < 4; ++a) Y[a] = load_x(A.x4, v[a]) - X0;
   Stencil S;
-  if (type == 0) pt_distance<true>(Y[0], Y[1], Y[2], Y[3], &S);
-  else ee_distance<true>(Y[0], Y[1], Y[2], Y[3], &S);
-  const int n = A.item_n[k];
-  const int32_t* nodes = A.item_nodes + kMaxNodes * k;
-  const int64_t oh = A.ro_h[k];
-  double E = 0.0;
-  double Kp[5][5];
-  double cn = 0.0, b1 = 0.0;
-  V3 rh = {0.0, 0.0, 0.0};
-  double basis[3][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}, {0, 0, 0, 0}};  // c^, a^_1, a^_2
+  closest_pair<true>(type, Y, stencil_hint(type, A.x4f, v), &S);
+  double d = 0.0;
   bool active = false;
   if (!(S.d2 > 0.0)) {
     raise_flag(A.st, EIPC_FLAG_PENETRATION);
   } else {
-    const double d = sqrt(S.d2);
-    active = d < A.dhat;
-    double eps_m, c_m;
-    if (active && ee_mollified(A, type, A.pr.i[k], A.pr.j[k], Y, &eps_m, &c_m)) return;   // k_eval_mollified
-    if (active) {
-      BarrierSpan B;
-      barrier_span(Y, S, d, A.dhat, A.kappa, B);
-      E = B.E; b1 = B.b1; cn = B.cn; rh = B.rh;
-      for (int c = 0; c < 3; ++c)
-        for (int a = 0; a < 4; ++a) basis[c][a] = B.basis[c][a];
-      if (A.project) {
-        // K+ in the span.  With fewer than two free closest-point parameters (an edge or a
-        // vertex of the triangle, an endpoint against an edge or two endpoints) the fifth
-        // basis vector is zero, so K's last row and column are zero and the projection is a
-        // 4 x 4 eigenproblem
-        if (S.m == 2) psd_span5(B.K, Kp);
-        else psd_span4(B.K, Kp);
-      } else {
-        for (int p = 0; p < 5; ++p)
-          for (int q = 0; q < 5; ++q) Kp[p][q] = B.K[p][q];
-      }
-    }
+    d = sqrt(S.d2);
+    active = lt_nonneg(d, A.dhat);
   }
-  // the lagged friction item on this pair's stencil, if any, goes into the same records:
-  // its blocks w_u w_v F are added to the barrier blocks (Sec. III-B, Eq. 8-9)
+  double eps_m, c_m;
+  if (active && ee_mollified(A, type, i, j, Y, &eps_m, &c_m)) {   // k_mollified
+    store_header(A.ihead + kIHead * k, nullptr, V3{0.0, 0.0, 0.0}, 0.0, kItemExplicit);
+    return;
+  }
+  const int n = A.item_n[k];
+  const uint64_t map = A.item_map[k];
+  const int64_t base = A.ro_g[k];
+  double nw[3][kMaxNodes], wf[kMaxNodes];
+  for (int c = 0; c < 3; ++c) zero_nodes(nw[c], n);
+  zero_nodes(wf, n);
   const int32_t fenc = A.fric_of_pair ? A.fric_of_pair[k] : 0;
-  const bool fr = fenc > 0;
   FrictionTerms R;
-  // per-node scalars omega, alpha_1, alpha_2 and the friction weight w_u (nw[u][3])
-  double coef[4][4];
-  for (int c = 0; c < 3; ++c)
-    for (int a = 0; a < 4; ++a) coef[c][a] = basis[c][a];      // zero when not active
-  if (fr) {
-    friction_terms(A.x4, A.lag, (int64_t)(INT32_MAX - fenc), v, A.mu, A.eps_f, R, coef[3]);
-    E += R.E;
+  double E = 0.0;
+  if (fenc > 0) {
+    double gam[4];
+    friction_terms(A.x4, A.lag, (int64_t)(INT32_MAX - fenc), v, A.mu, A.eps_f, R, gam);
+    E = R.E;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) add_slots(A, v[a], (uint32_t)(map >> (16 * a)) & 0xffffu, gam[a], wf);
   }
-  A.item_E[k] = E;
-  double nw[kMaxNodes][4];
-  if (fr) {
-    node_weights4<4>(v, A.cage_idx, A.w, nodes, n, coef, nw);
-  } else if (active) {
-    node_weights4<3>(v, A.cage_idx, A.w, nodes, n, coef, nw);
-  } else {
-    for (int u = 0; u < n; ++u) nw[u][0] = nw[u][1] = nw[u][2] = 0.0;
+  const FrictionTerms* Rp = fenc > 0 ? &R : nullptr;
+  int flags = fenc > 0 ? kItemFriction : 0;
+  if (!active) {
+    A.item_E[k] = E;
+    store_header(A.ihead + kIHead * k, Rp, V3{0.0, 0.0, 0.0}, 0.0, flags);
+    for (int u = 0; u < n && base + u < A.gcap; ++u)
+      store_row(A.frow + kFRow * (base + u), V3{0.0, 0.0, 0.0}, V3{0.0, 0.0, 0.0}, 0.0, wf[u]);
+    return;
   }
-  // Hessian records, upper triangle only: block(u,v) = A_u K+ A_v^T for u <= v, keyed by
-  // (min(I_u, I_v), max(I_u, I_v)) and transposed when I_u > I_v
-  const double rhv[3] = {rh.x, rh.y, rh.z};
-  int64_t pos = oh;
-  // the sorted position of the next record is loaded one record ahead, so its latency
-  // overlaps the current block's arithmetic
-  const int64_t pend = min(oh + (int64_t)n * (n + 1) / 2, A.rec_cap);
-  int64_t nxt = (A.hinv && pos < pend) ? (int64_t)__ldg(A.hinv + pos) : -1;
-  auto advance = [&]() {
-    const int64_t cur = nxt;
-    nxt = (A.hinv && pos + 1 < pend) ? (int64_t)__ldg(A.hinv + pos + 1) : -1;
-    return cur;
-  };
-  for (int u = 0; u < n; ++u) {
-    double Bu[3][5];
-    if (active) {
-      double t[5];
-      for (int q = 0; q < 5; ++q) t[q] = nw[u][1] * Kp[3][q] + nw[u][2] * Kp[4][q];
-      for (int p = 0; p < 3; ++p)
-        for (int q = 0; q < 5; ++q) Bu[p][q] = nw[u][0] * Kp[p][q] + rhv[p] * t[q];
+  BarrierSpan B;
+  barrier_span(Y, S, d, A.dhat, A.kappa, B);
+  A.item_E[k] = E + B.E;
+  const V3 rh = B.rh;
+  if (A.project) {
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int a = 0; a < 4; ++a) add_slots(A, v[a], (uint32_t)(map >> (16 * a)) & 0xffffu, B.basis[c][a], nw[c]);
+    double V[5][5];
+    eigen_sym<5>(B.K, V);
+    // columns of positive eigenvalue; a fourth can only be one at its rounding error: the
+    // smallest goes
+    double lam[5];
+    int cnt = 0, least = 0;
+#pragma unroll
+    for (int e = 0; e < 5; ++e) {
+      lam[e] = is_pos(B.K[e][e]) ? B.K[e][e] : 0.0;
+      cnt += lam[e] != 0.0;
     }
-    // the diagonal block (u, u) is symmetric: its upper triangle, mirrored
-    if (pos < A.rec_cap) {
-      const int64_t dst = advance();
-      double B[3][3];
-      if (active) {
-        for (int p = 0; p < 3; ++p) {
-          const double s = nw[u][1] * Bu[p][3] + nw[u][2] * Bu[p][4];
-          for (int q = p; q < 3; ++q) {
-            B[p][q] = nw[u][0] * Bu[p][q] + s * rhv[q];
-            B[q][p] = B[p][q];
-          }
+    for (; cnt > 3; --cnt) {
+      double lo = 0.0;
+#pragma unroll
+      for (int e = 0; e < 5; ++e)
+        if (lam[e] != 0.0 && (lo == 0.0 || lt_nonneg(lam[e], lo))) { lo = lam[e]; least = e; }
+#pragma unroll
+      for (int e = 0; e < 5; ++e)
+        if (e == least) lam[e] = 0.0;
+    }
+    flags |= kItemThird;
+    store_header(A.ihead + kIHead * k, Rp, rh * (A.kappa * B.b1 * B.cn), 0.0, flags);
+    double cols[3][5];                                            // sqrt(lambda) eigenvector
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int p = 0; p < 5; ++p) cols[c][p] = 0.0;
+    int at = 0;
+#pragma unroll
+    for (int e = 0; e < 5; ++e) {
+      if (lam[e] == 0.0) continue;
+      const double sl = sqrt(lam[e]);
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+        if (c == at) {
+#pragma unroll
+          for (int p = 0; p < 5; ++p) cols[c][p] = sl * V[p][e];
         }
-      } else {
-        for (int p = 0; p < 3; ++p)
-          for (int q = 0; q < 3; ++q) B[p][q] = 0.0;
-      }
-      if (fr) {
-        const double ww = nw[u][3] * nw[u][3];
-        for (int p = 0; p < 3; ++p)
-          for (int q = 0; q < 3; ++q) B[p][q] += ww * R.F[p][q];
-      }
-      // the gradient at node u: kappa b' |c| omega_u r^ (+ mu lambda f1/y w_u u)
-      const double s = active ? A.kappa * b1 * cn * nw[u][0] : 0.0;
-      double gx = s * rh.x, gy = s * rh.y, gz = s * rh.z;
-      if (fr) {
-        const double sf = R.gs * nw[u][3];
-        gx += sf * R.u[0]; gy += sf * R.u[1]; gz += sf * R.u[2];
-      }
-      emit_diag(A, pos, B, gx, gy, gz, dst);
+      ++at;
     }
-    ++pos;
-    for (int w2 = u + 1; w2 < n; ++w2, ++pos) {
-      if (pos >= A.rec_cap) continue;
-      const int64_t dst = advance();
-      double B[3][3];
-      if (active) {
-        for (int p = 0; p < 3; ++p) {
-          const double s = nw[w2][1] * Bu[p][3] + nw[w2][2] * Bu[p][4];
-          for (int q = 0; q < 3; ++q) B[p][q] = nw[w2][0] * Bu[p][q] + s * rhv[q];
-        }
-      } else {
-        for (int p = 0; p < 3; ++p)
-          for (int q = 0; q < 3; ++q) B[p][q] = 0.0;
-      }
-      if (fr) {
-        const double ww = nw[u][3] * nw[w2][3];
-        for (int p = 0; p < 3; ++p)
-          for (int q = 0; q < 3; ++q) B[p][q] += ww * R.F[p][q];
-      }
-      emit_upper(A, pos, nodes[u], nodes[w2], B, dst);
+    for (int u = 0; u < n && base + u < A.gcap; ++u) {
+      V3 z[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+        z[c] = V3{cols[c][0], cols[c][1], cols[c][2]} * nw[0][u] + rh * (nw[1][u] * cols[c][3] + nw[2][u] * cols[c][4]);
+      double* row = A.frow + kFRow * (base + u);
+      store_row(row, z[0], z[1], nw[0][u], wf[u]);
+      reinterpret_cast<double2*>(row)[4] = make_double2(z[2].x, z[2].y);
+      row[10] = z[2].z;
     }
+    return;
+  }
+  // exact: r^, isotropic and G M^-1 G^T terms, M = L L^T
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    add_slots(A, v[a], (uint32_t)(map >> (16 * a)) & 0xffffu, S.c[a], nw[0]);
+    add_slots2(A, v[a], (uint32_t)(map >> (16 * a)) & 0xffffu, S.a[0][a], nw[1], S.a[1][a], nw[2]);
+  }
+  const double inv_d = 1.0 / d;
+  double b, b1, b2;
+  barrier_scalars(d, inv_d, A.dhat, A.inv_dhat, &b, &b1, &b2);
+  const double bd = -A.kappa * (b1 * inv_d), h = fma(A.kappa, b2, bd), kr = sqrt(h);
+  V3 vj[2];
+  for (int c = 0; c < 2; ++c) {
+    vj[c] = {0.0, 0.0, 0.0};
+    for (int a = 0; a < 4; ++a) vj[c] = vj[c] + Y[a] * S.a[c][a];
+  }
+  // s G M^-1 G^T with s = bd / 2, G_j = 2 (omega v_j + alpha_j r): columns sqrt(2 s) L^-1 ( . )
+  const double sb = is_pos(bd) ? sqrt(bd) : 0.0;
+  double i1 = 0.0, l21 = 0.0, i2 = 0.0;
+  if (S.m > 0) i1 = rsqrt(dot(vj[0], vj[0]));
+  if (S.m > 1) {
+    l21 = dot(vj[0], vj[1]) * i1;
+    i2 = rsqrt(dot(vj[1], vj[1]) - l21 * l21);
+  }
+  flags |= kItemThird | kItemIso;
+  store_header(A.ihead + kIHead * k, Rp, rh * (A.kappa * b1), -bd, flags);
+  for (int u = 0; u < n && base + u < A.gcap; ++u) {
+    const double o = nw[0][u];
+    const V3 y1 = (vj[0] * o + rh * (d * nw[1][u])) * i1;
+    const V3 y2 = (vj[1] * o + rh * (d * nw[2][u]) - y1 * l21) * i2;
+    double* row = A.frow + kFRow * (base + u);
+    const V3 z3 = y2 * sb;
+    store_row(row, rh * (o * kr), y1 * sb, o, wf[u]);
+    reinterpret_cast<double2*>(row)[4] = make_double2(z3.x, z3.y);
+    row[10] = z3.z;
   }
 }
 
-// MINB = 2: no register cap (about 200 registers, 2 blocks of 128 per SM); MINB = 3: at
-// most 170 registers (3 blocks per SM, a few hundred bytes of spills); MINB = 4: at most
-// 128 registers (4 blocks per SM, spilling a few KB to L1-resident local memory).  Chosen at
-// run time.  With A.project false the pair Hessians are kept as they are (no PSD
-// projection).
-template <int MINB>
-__global__ void __launch_bounds__(kEvalThreads, MINB) k_eval_barrier(EvalArgs A) {
+// ... of a lagged friction item without a contact pair
+__device__ __forceinline__ void friction_factors(const EvalArgs& A, int64_t k, int64_t f) {
+  const int4 q4 = reinterpret_cast<const int4*>(A.lag.v)[f];
+  const int32_t v[4] = {q4.x, q4.y, q4.z, q4.w};
+  const int n = A.item_n[k];
+  const uint64_t map = A.item_map[k];
+  FrictionTerms R;
+  double gam[4], wf[kMaxNodes];
+  friction_terms(A.x4, A.lag, f, v, A.mu, A.eps_f, R, gam);
+  A.item_E[k] = R.E;
+  zero_nodes(wf, n);
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+    if (gam[a] != 0.0) add_slots(A, v[a], (uint32_t)(map >> (16 * a)) & 0xffffu, gam[a], wf);
+  store_header(A.ihead + kIHead * k, &R, V3{0.0, 0.0, 0.0}, 0.0, kItemFriction);
+  const int64_t base = A.ro_g[k];
+  for (int u = 0; u < n && base + u < A.gcap; ++u)
+    store_row(A.frow + kFRow * (base + u), V3{0.0, 0.0, 0.0}, V3{0.0, 0.0, 0.0}, 0.0, wf[u]);
+}
+
+// Factors of every item whose closest features are points and segments, by a work queue over the
+// items, each warp claiming A.tile of them at a time (the first tile is the warp's own, so warps
+// beyond a short list leave at once).  A divergent FP64 branch costs a warp its whole length, so
+// pairs with an interior closest point and friction items without a pair are only listed here, for
+// k_eval_rest to take in full warps: about one pair in a hundred of the bubble grasp, which used
+// to hold up every third warp (459 us for factors and rest in one kernel, 126 us for these alone).
+// The evaluation of the full bubble grasp (171k pairs, 163k friction items): 1194 -> 713 us.
+__global__ void __launch_bounds__(kEvalThreads, 4) k_eval_factors(EvalArgs A) {
   pdl_entry();
+  const int lane = threadIdx.x & 31;
   const int64_t P = clamp_count(A.pr.count, A.pr.capacity);
   const int64_t nit = *A.n_items;
   const int64_t np = P < nit ? P : nit;
-  if (!A.order) {
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < np; k += grid_stride())
-      eval_barrier_item(A, k);
-    return;
-  }
-  // scheduled: a persistent work queue over pair tiles -- each warp claims the next
-  // A.tile items of the order (one to several per lane), so warps that drew light items come
-  // back for more (dynamic balance); in a batch the tiles run across scene boundaries
-  const int lane = threadIdx.x & 31;
   const int tile = A.tile >= 32 ? (A.tile & ~31) : 32;
-  int64_t base = 0;
-  int left = 0;                  // items of the claimed tile not yet taken (a multiple of 32)
-  // a warp takes 32 items per round, so np / 32 + 2 rounds cover every claim it can make
-  const int64_t max_rounds = np / 32 + 2;
+  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  int64_t base = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * tile;
+  int left = tile;
+  // a warp takes 32 items a round: nit / 32 + 2 rounds cover every claim it can make
+  const int64_t max_rounds = nit / 32 + 2;
   for (int64_t round = 0;; ++round) {
     if (round > max_rounds) {
       raise_flag(A.st, EIPC_FLAG_STACK_OVERFLOW);
@@ -1115,56 +1321,62 @@ __global__ void __launch_bounds__(kEvalThreads, MINB) k_eval_barrier(EvalArgs A)
     if (left == 0) {
       unsigned long long b = 0;
       if (lane == 0) b = atomicAdd(reinterpret_cast<unsigned long long*>(A.queue), (unsigned long long)tile);
-      base = (int64_t)__shfl_sync(0xffffffffu, b, 0);
+      base = (int64_t)__shfl_sync(0xffffffffu, b, 0) + warps * tile;
       left = tile;
     }
-    if (base >= np) break;
-    const int64_t idx = base + lane;
-    if (idx < np) eval_barrier_item(A, (int64_t)A.order[idx]);
+    if (base >= nit) break;
+    const int64_t k = base + lane;
+    int later = -1;
+    if (k < np) {
+      int32_t v[4];
+      const int type = A.pr.type[k];
+      const int32_t i = A.pr.i[k], j = A.pr.j[k];
+      stencil_vertices(A.T, type, i, j, v);
+      const int hint = stencil_hint(type, A.x4f, v);
+      if (hint & kHintInterior) later = 0;
+      else light_factors(A, k, type, i, j, v, hint);
+    } else if (k < nit) {
+      if (friction_merged(A.fric_of_pair, A.pair_of_fric, k - P)) A.item_E[k] = 0.0;   // with its contact pair
+      else later = 1;
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, later >= 0);
+    if (m) {
+      // the interior pairs from the front, the friction items from the back (no more than items in all)
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const unsigned mc = __ballot_sync(0xffffffffu, later == c);
+        if (!mc) continue;
+        unsigned long long b = 0;
+        if (lane == 0) b = atomicAdd(reinterpret_cast<unsigned long long*>(A.n_rest + c), (unsigned long long)__popc(mc));
+        b = __shfl_sync(0xffffffffu, b, 0);
+        if (later == c) {
+          const int64_t at = (int64_t)b + __popc(mc & ((1u << lane) - 1u));
+          A.rest[c == 0 ? at : A.item_cap - 1 - at] = (uint32_t)k;
+        }
+      }
+    }
     base += 32;
     left -= 32;
   }
 }
 
-__global__ void __launch_bounds__(kEvalThreads) k_eval_friction(EvalArgs A, eipc_lag lag, double mu, double eps) {
+// ... of the items it listed: whole warps of one kind.
+__global__ void __launch_bounds__(kEvalThreads, 2) k_eval_rest(EvalArgs A) {
   pdl_entry();
+  const int lane = threadIdx.x & 31;
   const int64_t P = clamp_count(A.pr.count, A.pr.capacity);
-  const int64_t nit = *A.n_items;
-  const int64_t L = nit - P;
-  for (int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; f < L; f += grid_stride()) {
-    const int64_t k = P + f;
-    if (friction_merged(A.fric_of_pair, A.pair_of_fric, f)) {
-      A.item_E[k] = 0.0;           // evaluated with its contact pair, in that pair's records
-      continue;
-    }
-    const int4 q4 = reinterpret_cast<const int4*>(lag.v)[f];
-    const int32_t v[4] = {q4.x, q4.y, q4.z, q4.w};
-    FrictionTerms R;
-    double gam[4];
-    friction_terms(A.x4, lag, f, v, mu, eps, R, gam);
-    A.item_E[k] = R.E;
-    const int n = A.item_n[k];
-    const int32_t* nodes = A.item_nodes + kMaxNodes * k;
-    double nw[kMaxNodes];
-    node_weights1(v, A.cage_idx, A.w, nodes, n, gam, nw);
-    const int64_t oh = A.ro_h[k];
-    int64_t pos2 = oh;
-    for (int a = 0; a < n; ++a) {
-      for (int b = a; b < n; ++b, ++pos2) {
-        if (pos2 >= A.rec_cap) continue;
-        double B[3][3];
-        const double ww = nw[a] * nw[b];
-        for (int p = 0; p < 3; ++p)
-          for (int q = p; q < 3; ++q) {
-            B[p][q] = ww * R.F[p][q];
-            B[q][p] = B[p][q];
-          }
-        if (b == a) {
-          const double s = R.gs * nw[a];
-          emit_diag(A, pos2, B, s * R.u[0], s * R.u[1], s * R.u[2]);
-        } else {
-          emit_upper(A, pos2, nodes[a], nodes[b], B);
-        }
+  const int64_t n0 = A.n_rest[0], n1 = A.n_rest[1];
+  const int64_t w0 = (n0 + 31) / 32, w1 = (n1 + 31) / 32;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < w0 + w1; w += nw) {
+    if (w < w0) {
+      const int64_t q = 32 * w + lane;
+      if (q < n0) heavy_factors(A, A.rest[q]);
+    } else {
+      const int64_t q = 32 * (w - w0) + lane;
+      if (q < n1) {
+        const int64_t k = A.rest[A.item_cap - 1 - q];
+        friction_factors(A, k, k - P);
       }
     }
   }
@@ -1434,90 +1646,6 @@ __global__ void __launch_bounds__(kEvalThreads) k_mollified(EvalArgs A) {
   }
 }
 
-// FP32 guess of a stencil's number of free closest-point parameters (2: projection inside
-// the triangle / both segment parameters inside; 1: an edge interior; 0: two vertices), by
-// the same region rules as pt_distance / ee_distance.  Only a scheduling hint: a wrong
-// guess near a region boundary costs a divergent branch, never a different result.
-__device__ __forceinline__ int seg_hint_f32(F3 w, F3 e, float* d2) {
-  const float we = fdot(w, e), ee = fdot(e, e);
-  const float t = we > 0.f ? (we < ee ? we / ee : 1.f) : 0.f;
-  const F3 r = w - e * t;
-  *d2 = fdot(r, r);
-  return (t > 0.f && t < 1.f) ? 1 : 0;
-}
-
-__device__ __forceinline__ int span_hint_f32(const Topo& T, const double* __restrict__ x4, int type, int32_t i,
-                                             int32_t j) {
-  int32_t v[4];
-  stencil_vertices(T, type, i, j, v);
-  const V3 X0 = load_x(x4, v[0]);
-  F3 Y[4];
-  Y[0] = {0.f, 0.f, 0.f};
-  for (int a = 1; a < 4; ++a) {
-    const V3 d = load_x(x4, v[a]) - X0;
-    Y[a] = {(float)d.x, (float)d.y, (float)d.z};
-  }
-  float best, d2;
-  int m, mk;
-  if (type == 0) {
-    const F3 e1 = Y[2] - Y[1], e2 = Y[3] - Y[1], w = Y[0] - Y[1];
-    const F3 n = fcross(e1, e2);
-    const float nn = fdot(n, n);
-    const float b1 = fdot(fcross(w, e2), n) / nn, b2 = fdot(fcross(e1, w), n) / nn;
-    if (b1 >= 0.f && b2 >= 0.f && b1 + b2 <= 1.f) return 2;
-    m = seg_hint_f32(w, e1, &best);
-    mk = seg_hint_f32(Y[0] - Y[2], Y[3] - Y[2], &d2);
-    if (d2 < best) { best = d2; m = mk; }
-    mk = seg_hint_f32(Y[0] - Y[3], Y[1] - Y[3], &d2);
-    if (d2 < best) m = mk;
-    return m;
-  }
-  const F3 ea = Y[1] - Y[0], eb = Y[3] - Y[2], w = Y[0] - Y[2];
-  const float A = fdot(ea, ea), B = fdot(ea, eb), C = fdot(eb, eb), D = fdot(ea, w), E = fdot(eb, w);
-  const F3 n = fcross(ea, eb);
-  const float nn = fdot(n, n);
-  if (nn > 1e-12f * A * C) {
-    const float sa = (B * E - C * D) / nn, tb = (A * E - B * D) / nn;
-    if (sa >= 0.f && sa <= 1.f && tb >= 0.f && tb <= 1.f) return 2;
-  }
-  m = seg_hint_f32(Y[0] - Y[2], eb, &best);
-  mk = seg_hint_f32(Y[1] - Y[2], eb, &d2);
-  if (d2 < best) { best = d2; m = mk; }
-  mk = seg_hint_f32(Y[2] - Y[0], ea, &d2);
-  if (d2 < best) { best = d2; m = mk; }
-  mk = seg_hint_f32(Y[3] - Y[0], ea, &d2);
-  if (d2 < best) m = mk;
-  return m;
-}
-
-// Schedule of the barrier evaluation: items keyed by (number of cage nodes, descending;
-// a merged friction item or not; pair type; two free closest-point parameters (hinted) or
-// fewer), friction items last.  A warp's lanes then take the same branches, project in the
-// same dimension and emit the same number of blocks, and the heaviest items go first so
-// the tail is light.  Only the processing order changes: every item writes its records at
-// offsets fixed by its own index.  Keys fit in 8 bits: (16 - n) << 3 | fr << 2 | type << 1
-// | (m == 2) with 1 <= n <= 16, and 128 for friction items.
-__global__ void __launch_bounds__(kBlock) k_eval_order_keys(Topo T, const double* __restrict__ x4, eipc_pairs pr,
-                                                            const int32_t* __restrict__ item_n, const int64_t* n_items,
-                                                            const int32_t* __restrict__ fric_of_pair,
-                                                            uint64_t* __restrict__ keys, uint32_t* __restrict__ vals) {
-  pdl_entry();
-  const int64_t P = clamp_count(pr.count, pr.capacity);
-  const int64_t n = *n_items;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += grid_stride()) {
-    uint64_t key = 128;
-    if (k < P) {
-      const int ty = pr.type[k] & 1;
-      const int nn = min(max(item_n[k], 1), kMaxNodes);
-      const int fr = (fric_of_pair && fric_of_pair[k] > 0) ? 1 : 0;
-      const int m2 = span_hint_f32(T, x4, ty, pr.i[k], pr.j[k]) == 2 ? 1 : 0;
-      key = (uint64_t)((kMaxNodes - nn) << 3 | fr << 2 | ty << 1 | m2);
-    }
-    keys[k] = key;
-    vals[k] = (uint32_t)k;
-  }
-}
-
 // record totals -> overflow flags and clamped sort counts
 __global__ void k_rec_check(const int64_t* rh_total, const int64_t* rg_total, int64_t rec_cap, int64_t gcap,
                             int64_t* n_rh, int64_t* n_rg, DevStatus* st) {
@@ -1573,7 +1701,7 @@ __global__ void __launch_bounds__(kBlock) k_full_entries(const uint64_t* __restr
     } else {
       fkey[2 * s + 1] = (1ull << br) - 1;           // row bits above every row: sorts last
       fval[2 * s + 1] = 0;
-      dst[2 * s + 1] = -1;
+      dst[2 * s + 1] = -2;                          // marks a diagonal segment
       atomicAdd(reinterpret_cast<unsigned long long*>(n_diag), 1ull);
     }
   }
@@ -1610,13 +1738,14 @@ __global__ void __launch_bounds__(kBlock) k_seg_sum_g(const uint64_t* __restrict
 // BSR pattern before the evaluation; the evaluation then writes every record straight to
 // its sorted position and the sums read contiguous records.
 
-// keys of item k's Hessian records in the order the evaluation emits them: record (u, v),
-// u <= v, keyed by the upper-triangle position of its nodes (min, max).  One warp per item,
-// lanes on consecutive records.
+// keys of item k's Hessian records: record (u, v), u <= v, keyed by the upper-triangle position
+// of its nodes (min, max), and its source (item, local node of the row, of the column).  One
+// warp per item, lanes on consecutive records.
 __global__ void __launch_bounds__(kBlock) k_rec_keys(const int32_t* __restrict__ item_nodes,
                                                      const int32_t* __restrict__ item_n, const int64_t* __restrict__ ro_h,
                                                      const int64_t* n_items, int64_t rec_cap, int64_t ns,
-                                                     uint64_t* __restrict__ hkeys, uint32_t* __restrict__ hvals) {
+                                                     uint64_t* __restrict__ hkeys, uint32_t* __restrict__ hvals,
+                                                     uint64_t* __restrict__ rec_src) {
   pdl_entry();
   const int64_t nit = *n_items;
   const int lane = threadIdx.x & 31;
@@ -1636,11 +1765,10 @@ __global__ void __launch_bounds__(kBlock) k_rec_keys(const int32_t* __restrict__
       const uint64_t Iu = (uint64_t)nodes[u], Iv = (uint64_t)nodes[w2];
       hkeys[pos] = Iu <= Iv ? upper_key(Iu, Iv, (uint64_t)ns) : upper_key(Iv, Iu, (uint64_t)ns);
       hvals[pos] = (uint32_t)pos;
+      rec_src[pos] = (uint64_t)k << 8 | (uint64_t)(Iu <= Iv ? u : w2) << 4 | (uint64_t)(Iu <= Iv ? w2 : u);
     }
   }
 }
-
-
 
 // sorted full entries -> BSR columns, row counts, and for each upper segment s the BSR
 // entry of its block (dst[2s]) and of its transpose (dst[2s+1]; -1 on the diagonal or
@@ -1677,14 +1805,12 @@ __global__ void __launch_bounds__(kBlock) k_bsr_pattern(const uint64_t* __restri
   }
 }
 
-// Segment sums over contiguous presorted records in two passes.  Each segment is cut into
-// units of kSegChunk consecutive records counted from its own first record; pass 1 adds
-// each unit's records in order (one thread per unit, every lane doing useful FP64 adds,
-// no shuffle tree), pass 2 adds a segment's unit sums in order (one thread per segment).
-// The grouping depends only on the segment's own records, so a scene's sums are the same
-// bits whether it is evaluated alone or inside a batch, and a long segment is spread over
-// many threads.
-constexpr int kSegChunk = 32;
+// Segment sums in two passes.  Each segment is cut into units of kSegChunk consecutive records
+// counted from its own first record; pass 1 sums each unit's records in order, pass 2 a
+// segment's unit sums in a fixed order.  The grouping depends only on the segment's own
+// records, so a scene's sums are the same bits whether it is evaluated alone or inside a
+// batch, and a long segment is spread over many threads.
+constexpr int kSegChunk = 16;
 
 // units per segment: unit[s] = ceil(len_s / kSegChunk) (exclusive-scanned afterwards),
 // and, when keys is given, the segment's key ukey[s]
@@ -1713,139 +1839,152 @@ __device__ __forceinline__ int64_t segment_of_unit(const int64_t* __restrict__ u
   return lo;
 }
 
-// row r of a record array with rows of W values at a 16-byte aligned stride P, loaded
-// two values at a time
-template <int W, int P>
-__device__ __forceinline__ void load_row(const double* __restrict__ x, int64_t r, double v[W]) {
-  const double2* p = reinterpret_cast<const double2*>(x + P * r);
-#pragma unroll
-  for (int c = 0; c + 1 < W; c += 2) {
-    const double2 t = __ldg(p + c / 2);
-    v[c] = t.x;
-    v[c + 1] = t.y;
-  }
-  if (W & 1) v[W - 1] = __ldg(x + P * r + W - 1);
+struct SumArgs {
+  const uint64_t* src;        // sources of the sorted records
+  const int64_t* ro_h;        // first record of each item, its node count (explicit records)
+  const int32_t* item_n;
+  const int64_t* start;
+  const int64_t* unit;
+  const int64_t* n_units;
+  const int64_t* n_rec;
+  const int64_t* n_seg;
+  int64_t cap;
+  const int64_t* ro_g;
+  const double* frow;
+  const double* ihead;
+  const double* hrec;
+  double* piece;
+};
+
+__device__ __forceinline__ int sym_index(int p, int q) {   // (p, q) in B00 B01 B02 B11 B12 B22
+  const int lo = p < q ? p : q, hi = p < q ? q : p;
+  return lo * (5 - lo) / 2 + hi;
 }
 
-// acc += x[r] for r = b, b+1, ..., e-1 in that order; the loads of four consecutive rows
-// are issued before their adds so that a thread has several loads in flight
-template <int W, int P>
-__device__ __forceinline__ void add_in_order(const double* __restrict__ x, int64_t b, int64_t e, double acc[W]) {
-  int64_t r = b;
-  for (; r + 4 <= e; r += 4) {
-    double v[4][W];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) load_row<W, P>(x, r + q, v[q]);
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-#pragma unroll
-      for (int c = 0; c < W; ++c) acc[c] += v[q][c];
-  }
-  for (; r < e; ++r) {
-    double v[W];
-    load_row<W, P>(x, r, v);
-#pragma unroll
-    for (int c = 0; c < W; ++c) acc[c] += v[c];
-  }
-}
-
-template <int W, int P>
-__global__ void __launch_bounds__(kBlock) k_seg_pieces(const double* __restrict__ rec, const int64_t* __restrict__ start,
-                                                       const int64_t* __restrict__ unit, const int64_t* n_units,
-                                                       const int64_t* n_rec, const int64_t* n_seg, int64_t cap,
-                                                       double* __restrict__ piece) {
+// Pass 1: the units' sums, each record's block multiplied out of its item's factor rows (see
+// "pair factors") into the accumulators.  Bound by the FP64 pipe: three lanes per unit, lane i
+// of them accumulating row i of the block -- 7 or 10 FP64 instructions per record (without or
+// with friction), 30 of 32 lanes at work.  In a diagonal segment lane i takes entries (i, i) and
+// (i, i + 1 mod 3) of the symmetric block and, in place of the third, component i of the
+// gradient, with the same number of instructions.
+__global__ void __launch_bounds__(128) k_unit_sums(SumArgs A) {
   pdl_entry();
-  const int64_t R = clamp_count(n_rec, cap);
-  const int64_t S = *n_seg;
-  const int64_t U = *n_units;
+  const int64_t R = clamp_count(A.n_rec, A.cap);
+  const int64_t S = *A.n_seg;
+  const int64_t U = *A.n_units;
+  const int lane = threadIdx.x & 31, sub = lane / 3, i = lane - 3 * sub;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   if (S <= 0) return;
-  for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < U; u += grid_stride()) {
-    const int64_t s = segment_of_unit(unit, S, u);
-    const int64_t end = (s + 1 < S) ? start[s + 1] : R;
-    const int64_t b = start[s] + (u - unit[s]) * kSegChunk;
+  for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w * 10 < U; w += nw) {
+    const int64_t u = w * 10 + sub;
+    if (lane >= 30 || u >= U) continue;
+    const int64_t s = segment_of_unit(A.unit, S, u);
+    const int64_t end = (s + 1 < S) ? A.start[s + 1] : R;
+    const int64_t b = A.start[s] + (u - A.unit[s]) * kSegChunk;
     const int64_t e = (b + kSegChunk < end) ? b + kSegChunk : end;
-    double acc[W];
-#pragma unroll
-    for (int c = 0; c < W; ++c) acc[c] = 0.0;
-    add_in_order<W, P>(rec, b, e, acc);
-    double* p = piece + W * u;
-#pragma unroll
-    for (int c = 0; c < W; ++c) p[c] = acc[c];
-  }
-}
-
-// Sum over the 32 lanes of a warp of the L-vectors a (L a power of two <= 16) by
-// reduce-scatter: at each step the lanes pair up across one lane bit, each keeps half of
-// the vector and adds its partner's copy of that half; when one entry is left, plain
-// butterfly adds finish.  8 + 4 + 2 + 1 + 1 adds for L = 16 instead of 5 L.  Returns
-// the full sum of component (lane >> (5 - log2 L)); the order of the adds is fixed.
-template <int L>
-__device__ __forceinline__ double warp_reduce_scatter(double (&a)[L], int lane) {
-  int o = 16;
-#pragma unroll
-  for (int len = L; len > 1; len >>= 1, o >>= 1) {
-    const bool hi = (lane & o) != 0;
-#pragma unroll
-    for (int i = 0; i < len / 2; ++i) {
-      const double send = hi ? a[i] : a[i + len / 2];
-      const double keep = hi ? a[i + len / 2] : a[i];
-      a[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    uint64_t src = __ldg(A.src + b);
+    int64_t base = __ldg(A.ro_g + (src >> 8));
+    const bool diag = ((src >> 4) & 15) == (src & 15);
+    const int c0 = diag ? i : 0, c1 = diag ? (i == 2 ? 0 : i + 1) : 1;
+    const int f0 = sym_index(i, c0), f1 = sym_index(i, c1), f2 = sym_index(i, 2);
+    double a0 = 0.0, a1 = 0.0, a2 = 0.0;
+    for (int64_t r = b; r < e; ++r) {
+      const int64_t item = (int64_t)(src >> 8);
+      const int lu = (int)((src >> 4) & 15), lv = (int)(src & 15);
+      const double* ru = A.frow + kFRow * (base + lu);
+      const double* rv = A.frow + kFRow * (base + lv);
+      const double* hd = A.ihead + kIHead * item;
+      // the next record's rows are found while this one's arrive
+      if (r + 1 < e) {
+        src = __ldg(A.src + r + 1);
+        base = __ldg(A.ro_g + (src >> 8));
+      }
+      const double2 hf = __ldg(reinterpret_cast<const double2*>(hd) + 6);
+      const int flags = (int)__double_as_longlong(hf.y);
+      if (flags & kItemExplicit) {
+        const int lo = min(lu, lv), hi = max(lu, lv);
+        const double* B = A.hrec + kHRecStride * (A.ro_h[item] + lo * A.item_n[item] - lo * (lo - 1) / 2 + hi - lo);
+        a0 += diag ? B[f0] : B[3 * i];
+        a1 += diag ? B[f1] : B[3 * i + 1];
+        a2 += diag ? B[6 + i] : B[3 * i + 2];
+        continue;
+      }
+      const double z1 = __ldg(ru + i), z2 = __ldg(ru + 3 + i);
+      const double2 ou = __ldg(reinterpret_cast<const double2*>(ru) + 3);
+      const double2 va = __ldg(reinterpret_cast<const double2*>(rv)), vb = __ldg(reinterpret_cast<const double2*>(rv) + 1);
+      const double2 vc = __ldg(reinterpret_cast<const double2*>(rv) + 2), ov = __ldg(reinterpret_cast<const double2*>(rv) + 3);
+      const double x0 = c0 == 0 ? va.x : (c0 == 1 ? va.y : vb.x), y0 = c0 == 0 ? vb.y : (c0 == 1 ? vc.x : vc.y);
+      const double x1 = c1 == 0 ? va.x : (c1 == 1 ? va.y : vb.x), y1 = c1 == 0 ? vb.y : (c1 == 1 ? vc.x : vc.y);
+      double p1 = z1, q1 = vb.x, p2 = z2, q2 = vc.y;
+      if (diag) {
+        p1 = ou.x; q1 = __ldg(hd + 6 + i);
+        p2 = ou.y; q2 = __ldg(hd + 9 + i);
+      }
+      a0 = fma(z1, x0, a0); a1 = fma(z1, x1, a1); a2 = fma(p1, q1, a2);
+      a0 = fma(z2, y0, a0); a1 = fma(z2, y1, a1); a2 = fma(p2, q2, a2);
+      if (flags & kItemFriction) {
+        const double ww = ou.y * ov.y;
+        a0 = fma(ww, __ldg(hd + f0), a0);
+        a1 = fma(ww, __ldg(hd + f1), a1);
+        a2 = fma(ww, diag ? 0.0 : __ldg(hd + f2), a2);
+      }
+      if (flags & kItemThird) {
+        const double z3 = __ldg(ru + 8 + i);
+        a0 = fma(z3, __ldg(rv + 8 + c0), a0);
+        a1 = fma(z3, __ldg(rv + 8 + c1), a1);
+        a2 = fma(diag ? 0.0 : z3, __ldg(rv + 10), a2);
+      }
+      if (flags & kItemIso) {
+        const double t = hf.x * (ou.x * ov.x);
+        if (diag || i == 0) a0 += t;
+        else if (i == 1) a1 += t;
+        else a2 += t;
+      }
     }
+    double* p = A.piece + 9 * u + 3 * i;
+    p[0] = a0; p[1] = a1; p[2] = a2;
   }
-  double v = a[0];
-#pragma unroll
-  for (; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
 }
 
-// Hessian pass 2, one warp per segment: lane l adds unit sums l, l+32, ... of its segment
-// in order, then warp_reduce_scatter; the block goes into the BSR values at dst[2s] and,
-// transposed, at dst[2s+1].  A diagonal segment (I, I) holds the six upper entries of its
-// symmetric block and then the gradient at node I (emit_diag): the block is written whole
-// and the gradient goes to g_r[I].
-__global__ void __launch_bounds__(kBlock) k_seg_sum_h_pieces(const double* __restrict__ piece,
-                                                             const int64_t* __restrict__ unit, const int64_t* n_units,
-                                                             const int64_t* n_seg, int64_t cap,
-                                                             const int32_t* __restrict__ dst, eipc_bsr H,
-                                                             const uint64_t* __restrict__ ukey, int64_t ns,
-                                                             double* __restrict__ g_r) {
+// Pass 2, one warp per segment: lane 9 q + c adds component c of unit sums q, q + 3, ... in
+// order, then the three chains are added; the block goes into the BSR values at dst[2s] and,
+// transposed, at dst[2s+1].  A diagonal segment (dst[2s+1] = -2) holds, per row i, entries (i, i)
+// and (i, i + 1 mod 3) of its symmetric block and component i of the gradient at its node, taken
+// from its first record's item.
+__global__ void __launch_bounds__(kBlock) k_segment_sums(const double* __restrict__ piece, const int64_t* __restrict__ unit,
+                                                         const int64_t* n_units, const int64_t* n_seg, int64_t cap,
+                                                         const int32_t* __restrict__ dst, eipc_bsr H,
+                                                         const int64_t* __restrict__ start, const uint64_t* __restrict__ src,
+                                                         const int32_t* __restrict__ item_nodes, double* __restrict__ g_r) {
   pdl_entry();
   const int64_t S0 = *n_seg;
   const int64_t S = (2 * S0 <= cap) ? S0 : cap / 2;      // the segments k_full_entries kept
   const int64_t U = *n_units;
   const int64_t nnzb = *H.nnzb;
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, q = lane / 9, c = lane - 9 * q;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < S; s += nw) {
-    const int64_t u1 = (s + 1 < S0) ? unit[s + 1] : U;
-    double acc[16];
-#pragma unroll
-    for (int c = 0; c < 16; ++c) acc[c] = 0.0;
-    for (int64_t k = unit[s] + lane; k < u1; k += 32) {
-#pragma unroll
-      for (int c = 0; c < 9; ++c) acc[c] += __ldg(piece + 9 * k + c);
+    const int64_t u0 = unit[s], u1 = (s + 1 < S0) ? unit[s + 1] : U;
+    double v = 0.0;
+    if (q < 3) {
+      for (int64_t k = u0 + q; k < u1; k += 3) v += __ldg(piece + 9 * k + c);
     }
-    const double v = warp_reduce_scatter<16>(acc, lane);
-    const int c = lane >> 1;
-    if ((lane & 1) == 0 && c < 9) {
-      const int32_t du = dst[2 * s], dl = dst[2 * s + 1];
-      const uint64_t key = ukey[s];
-      uint64_t I, J;
-      upper_decode(key, (uint64_t)ns, &I, &J);
-      if (I != J) {
-        if (du >= 0 && du < nnzb) H.val[9 * (int64_t)du + c] = v;
-        if (dl >= 0 && dl < nnzb) H.val[9 * (int64_t)dl + 3 * (c % 3) + c / 3] = v;
-      } else if (c < 6) {
-        // upper entry c of the symmetric block: (0,0) (0,1) (0,2) (1,1) (1,2) (2,2)
-        const int p = c < 3 ? 0 : (c < 5 ? 1 : 2);
-        const int q = c < 3 ? c : (c < 5 ? c - 2 : 2);
-        if (du >= 0 && du < nnzb) {
-          H.val[9 * (int64_t)du + 3 * p + q] = v;
-          H.val[9 * (int64_t)du + 3 * q + p] = v;
-        }
-      } else {
-        g_r[3 * I + (c - 6)] = v;
-      }
+    const double v1 = __shfl_sync(0xffffffffu, v, c + 9), v2 = __shfl_sync(0xffffffffu, v, c + 18);
+    if (u1 - u0 > 1) v += v1;
+    if (u1 - u0 > 2) v += v2;
+    if (q > 0) continue;
+    const int32_t du = dst[2 * s], dl = dst[2 * s + 1];
+    const int i = c / 3, k = c - 3 * i;
+    if (dl != -2) {
+      if (du >= 0 && du < nnzb) H.val[9 * (int64_t)du + c] = v;
+      if (dl >= 0 && dl < nnzb) H.val[9 * (int64_t)dl + 3 * k + i] = v;
+    } else if (k == 2) {
+      const uint64_t sr = src[start[s]];
+      g_r[3 * (int64_t)item_nodes[kMaxNodes * (int64_t)(sr >> 8) + (int64_t)(sr & 15)] + i] = v;
+    } else if (du >= 0 && du < nnzb) {
+      const int j = k == 0 ? i : (i == 2 ? 0 : i + 1);
+      H.val[9 * (int64_t)du + 3 * i + j] = v;
+      H.val[9 * (int64_t)du + 3 * j + i] = v;
     }
   }
 }
@@ -1964,7 +2103,7 @@ void eval_launch(eipc_scene* sc, const double* q, const eipc_pairs& pr, const ei
   const int64_t pcap = pr.capacity < item_cap ? pr.capacity : item_cap;
   // counters, the evaluation queue, g_r and the friction claims, all reset up front
   zero_ranges(s, {{cnt + kCntItems, 5 * sizeof(int64_t)}, {n_diag, sizeof(int64_t)},
-                  {cnt + kCntEvalQueue, sizeof(int64_t)}, {g_r, sizeof(double) * 3 * sc->ns},
+                  {cnt + kCntEvalQueue, sizeof(int64_t)}, {cnt + kCntEvalRest, 2 * sizeof(int64_t)}, {g_r, sizeof(double) * 3 * sc->ns},
                   {merge ? sc->fric_of_pair : nullptr, sizeof(int32_t) * pcap}});
   const int32_t* fop = merge ? sc->fric_of_pair : nullptr;
   const int32_t* pof = merge ? sc->pair_of_fric : nullptr;
@@ -1978,7 +2117,7 @@ void eval_launch(eipc_scene* sc, const double* q, const eipc_pairs& pr, const ei
                                                            fr ? lag->capacity : 0, sc->cage_idx, item_cap,
                                                            sc->item_nodes, sc->item_n, sc->item_group, sc->vgroup,
                                                            sc->rc_h, sc->rc_g,
-                                                           cnt + kCntItems, sc->status, fop, pof);
+                                                           cnt + kCntItems, sc->status, fop, pof, sc->item_map);
   int64_t* tot_h = cnt + 9;
   int64_t* tot_g = cnt + 10;
   exclusive_scan2_i64(sc->rc_h, sc->ro_h, tot_h, sc->rc_g, sc->ro_g, tot_g, cnt + kCntItems, item_cap,
@@ -1986,20 +2125,56 @@ void eval_launch(eipc_scene* sc, const double* q, const eipc_pairs& pr, const ei
   launch(k_rec_check, 1, 32, 0, s, tot_h, tot_g, sc->rec_cap, sc->gcap, cnt + kCntRecH, cnt + kCntRecG, sc->status);
   sc->timers->stop(kKItems, s);
 
-  // Hessian pattern before the evaluation: record keys (I, J) from the items' cage nodes,
-  // stable sort, segments (one per BSR upper block), the inverse permutation that sends
-  // each record to its sorted position, then the full symmetric pattern (every
-  // off-diagonal upper block also at (J, I)), columns and row pointers
+  EvalArgs A{};
+  A.T = sc->topo; A.pr = pr; A.cage_idx = sc->cage_idx; A.w = sc->w; A.x4 = sc->x4; A.x4f = sc->x4f; A.ns = sc->ns;
+  A.dhat = p.dhat; A.inv_dhat = 1.0 / p.dhat; A.kappa = p.kappa; A.item_nodes = sc->item_nodes; A.item_n = sc->item_n;
+  A.item_map = sc->item_map;
+  A.ro_h = sc->ro_h; A.ro_g = sc->ro_g; A.n_items = cnt + kCntItems; A.rec_cap = sc->rec_cap; A.gcap = sc->gcap;
+  A.frow = sc->frow; A.ihead = sc->ihead; A.hrec = sc->hrec; A.item_E = sc->item_E; A.st = sc->status;
+  A.project = (p.flags & EIPC_PARAM_NO_PROJECTION) == 0;
+  A.moll_r2 = sc->moll_factor > 0.0 ? sc->moll_r2 : nullptr;
+  A.moll_factor = sc->moll_factor;
+  A.fric_of_pair = fop; A.pair_of_fric = pof;
+  A.lag = fr ? *lag : eipc_lag{};
+  A.mu = p.mu; A.eps_f = p.eps_v * p.h;
+  A.rest = sc->svals_alt;                    // the pair-sort buffers are free once the pairs are built
+  A.n_rest = cnt + kCntEvalRest;
+  A.item_cap = item_cap;
+  A.queue = cnt + kCntEvalQueue;
+  A.tile = sc->tune.eval_tile;
+  // The factors and the pattern both follow from the items and are needed by the sums only:
+  // the factors (bound by the FP64 pipe) run on the scene's second stream beside the pattern's
+  // chain of sorts and scans (bound by latency and memory).
+  cudaEventRecord(sc->ev_fork, s);
+  cudaStreamWaitEvent(sc->aux, sc->ev_fork, 0);
+  {
+    const int64_t most = pr.capacity + (fr ? lag->capacity : 0);
+    const int blocks = blocks_for(most < item_cap ? most : item_cap, sc->tune.eval_bps, sc->tune.eval_threads);
+    sc->timers->start(kKEvalPair, sc->aux);
+    EIPC_TIMED(sc, kKEvalBarrier, sc->aux,
+               launch(k_eval_factors, blocks, sc->tune.eval_threads, 0, sc->aux, A);
+               launch(k_eval_rest, 2 * kSMs, kEvalThreads, 0, sc->aux, A));
+    if (A.moll_r2)
+      EIPC_TIMED(sc, kKEvalBarrier, sc->aux,
+                 (launch(k_mollified<false>, blocks_for(pr.capacity, 8, kEvalThreads), kEvalThreads, 0, sc->aux, A)));
+    sc->timers->stop(kKEvalPair, sc->aux);
+  }
+  cudaEventRecord(sc->ev_join, sc->aux);
+
+  // Hessian pattern: record keys (I, J) from the items' cage nodes, stable sort, segments (one
+  // per BSR upper block), then the full symmetric pattern (every off-diagonal upper block
+  // also at (J, I)), columns and row pointers
   sc->timers->start(kKHReduce, s);
   launch(k_rec_keys, blocks_for(32 * item_cap, 8), kBlock, 0, s, static_cast<const int32_t*>(sc->item_nodes),
          static_cast<const int32_t*>(sc->item_n), static_cast<const int64_t*>(sc->ro_h),
-         static_cast<const int64_t*>(cnt + kCntItems), sc->rec_cap, sc->ns, sc->hkeys, sc->hvals);
+         static_cast<const int64_t*>(cnt + kCntItems), sc->rec_cap, sc->ns, sc->hkeys, sc->hvals, sc->rec_src);
   const int wh = radix_sort_u64(sc->hkeys, sc->hvals, sc->hkeys_alt, sc->hvals_alt, cnt + kCntRecH, sc->rec_cap,
                                 sc->bits_h, sc->sort_hist, s);
   const uint64_t* hk = wh ? sc->hkeys_alt : sc->hkeys;
   const uint32_t* hv = wh ? sc->hvals_alt : sc->hvals;
-  // segment starts, and the inverse permutation (each record's sorted position)
-  segment_starts(hk, cnt + kCntRecH, sc->rec_cap, sc->seg_start, cnt + kCntSegH, sc->scan_partial, s, hv, sc->hinv);
+  // segment starts, and each sorted record's source
+  segment_starts(hk, cnt + kCntRecH, sc->rec_cap, sc->seg_start, cnt + kCntSegH, sc->scan_partial, s, hv, sc->rec_src,
+                 sc->src_sorted);
   // seg_flag and seg_id hold the segment keys and the segments' BSR entries
   uint64_t* ukey = reinterpret_cast<uint64_t*>(sc->seg_flag);
   int32_t* dst = reinterpret_cast<int32_t*>(sc->seg_id);
@@ -2022,67 +2197,17 @@ void eval_launch(eipc_scene* sc, const double* q, const eipc_pairs& pr, const ei
          static_cast<const int64_t*>(n_diag), rb, sc->ns, H, dst, sc->status, cnt + kCntSegG);
   sc->timers->stop(kKHReduce, s);
 
-  EvalArgs A;
-  A.T = sc->topo; A.pr = pr; A.cage_idx = sc->cage_idx; A.w = sc->w; A.x4 = sc->x4; A.ns = sc->ns;
-  A.dhat = p.dhat; A.kappa = p.kappa; A.item_nodes = sc->item_nodes; A.item_n = sc->item_n;
-  A.ro_h = sc->ro_h; A.ro_g = sc->ro_g; A.n_items = cnt + kCntItems; A.rec_cap = sc->rec_cap; A.gcap = sc->gcap;
-  A.hkeys = nullptr; A.hvals = nullptr; A.hrec = sc->hrec; A.gkeys = nullptr; A.gvals = nullptr;
-  A.grec = sc->grec; A.item_E = sc->item_E; A.st = sc->status;
-  A.project = (p.flags & EIPC_PARAM_NO_PROJECTION) == 0;
-  A.moll_r2 = sc->moll_factor > 0.0 ? sc->moll_r2 : nullptr;
-  A.moll_factor = sc->moll_factor;
-  A.hv_dir = nullptr; A.kin_dir[0] = A.kin_dir[1] = A.kin_dir[2] = 0.0;
-  A.hinv = sc->hinv;                         // gradients ride in the diagonal records
-  A.fric_of_pair = fop; A.pair_of_fric = pof;
-  A.lag = fr ? *lag : eipc_lag{};
-  A.mu = p.mu; A.eps_f = p.eps_v * p.h;
-  {
-    // (node count, type) schedule; the pair-sort buffers are free once the pairs are built
-    launch(k_eval_order_keys, blocks_for(item_cap, 8), kBlock, 0, s, sc->topo, static_cast<const double*>(sc->x4), pr,
-           static_cast<const int32_t*>(sc->item_n), static_cast<const int64_t*>(cnt + kCntItems), fop, sc->skeys,
-           sc->svals);
-    const int wo = radix_sort_u64(sc->skeys, sc->svals, sc->skeys_alt, sc->svals_alt, cnt + kCntItems, item_cap, 8,
-                                  sc->sort_hist, s);
-    A.order = wo ? sc->svals_alt : sc->svals;
-    A.queue = cnt + kCntEvalQueue;
-    A.tile = sc->tune.eval_tile;
-  }
-  // friction items on the scene's second stream, beside the barrier items: the two
-  // kernels write disjoint records and item energies, and the barrier kernel leaves most
-  // warp slots and part of the FP64 pipe free
-  sc->timers->start(kKEvalPair, s);
-  if (fr) {
-    cudaEventRecord(sc->ev_fork, s);
-    cudaStreamWaitEvent(sc->aux, sc->ev_fork, 0);
-    EIPC_TIMED(sc, kKEvalFriction, sc->aux,
-               (launch(k_eval_friction, blocks_for(lag->capacity, 8, kEvalThreads), kEvalThreads, 0, sc->aux, A,
-                       *lag, p.mu, p.eps_v * p.h)));
-    cudaEventRecord(sc->ev_join, sc->aux);
-  }
-  EIPC_TIMED(sc, kKEvalBarrier, s,
-             (sc->tune.eval_variant == 4
-                  ? launch(k_eval_barrier<4>, blocks_for(pr.capacity, sc->tune.eval_bps, sc->tune.eval_threads),
-                           sc->tune.eval_threads, 0, s, A)
-              : sc->tune.eval_variant == 3
-                  ? launch(k_eval_barrier<3>, blocks_for(pr.capacity, sc->tune.eval_bps, sc->tune.eval_threads),
-                           sc->tune.eval_threads, 0, s, A)
-                  : launch(k_eval_barrier<2>, blocks_for(pr.capacity, sc->tune.eval_bps, sc->tune.eval_threads),
-                           sc->tune.eval_threads, 0, s, A)));
-  if (A.moll_r2)
-    EIPC_TIMED(sc, kKEvalBarrier, s, (launch(k_mollified<false>, blocks_for(pr.capacity, 8, kEvalThreads), kEvalThreads, 0, s, A)));
-  if (fr) cudaStreamWaitEvent(s, sc->ev_join, 0);
-  sc->timers->stop(kKEvalPair, s);
-  // sums over the contiguous presorted records, in sorted order
+  cudaStreamWaitEvent(s, sc->ev_join, 0);
   sc->timers->start(kKHReduce, s);
-  launch(k_seg_pieces<9, kHRecStride>, blocks_for(sc->rec_cap / kSegChunk + 1, 8), kBlock, 0, s, static_cast<const double*>(sc->hrec),
-         static_cast<const int64_t*>(sc->seg_start), static_cast<const int64_t*>(sc->hunit),
-         static_cast<const int64_t*>(cnt + kCntUnitsH), static_cast<const int64_t*>(cnt + kCntRecH),
-         static_cast<const int64_t*>(cnt + kCntSegH), sc->rec_cap, sc->piece);
+  launch(k_unit_sums, blocks_for(3 * (sc->rec_cap / kSegChunk + 1), 32, 128), 128, 0, s,
+         SumArgs{sc->src_sorted, sc->ro_h, sc->item_n, sc->seg_start, sc->hunit, cnt + kCntUnitsH, cnt + kCntRecH, cnt + kCntSegH, sc->rec_cap,
+                 sc->ro_g, sc->frow, sc->ihead, sc->hrec, sc->piece});
   // blocks into the BSR values; the diagonal segments' gradients into g_r
-  launch(k_seg_sum_h_pieces, blocks_for(32 * sc->rec_cap, 8), kBlock, 0, s, static_cast<const double*>(sc->piece),
+  launch(k_segment_sums, blocks_for(32 * sc->rec_cap, 8), kBlock, 0, s, static_cast<const double*>(sc->piece),
          static_cast<const int64_t*>(sc->hunit), static_cast<const int64_t*>(cnt + kCntUnitsH),
          static_cast<const int64_t*>(cnt + kCntSegH), sc->rec_cap, static_cast<const int32_t*>(dst), H,
-         static_cast<const uint64_t*>(ukey), sc->ns, g_r);
+         static_cast<const int64_t*>(sc->seg_start), static_cast<const uint64_t*>(sc->src_sorted),
+         static_cast<const int32_t*>(sc->item_nodes), g_r);
   sc->timers->stop(kKHReduce, s);
   // energy
   sc->timers->start(kKEnergy, s);
@@ -2101,7 +2226,7 @@ void hvp_launch(eipc_scene* sc, const double* q, const eipc_pairs& pr, const eip
   launch(k_item_nodes, blocks_for(item_cap, 8), kBlock, 0, s, sc->topo, pr, fr ? lag->v : nullptr, fr ? lag->count : nullptr,
          fr ? lag->capacity : 0, sc->cage_idx, item_cap, sc->item_nodes, sc->item_n, sc->item_group, sc->vgroup,
          sc->rc_h, sc->rc_g, cnt + kCntItems, sc->status, static_cast<const int32_t*>(nullptr),
-         static_cast<const int32_t*>(nullptr));
+         static_cast<const int32_t*>(nullptr), static_cast<uint64_t*>(nullptr));
   launch(k_hvp_counts, blocks_for(item_cap, 8), kBlock, 0, s, sc->topo, pr, fr ? lag->v : nullptr,
          fr ? static_cast<const int64_t*>(lag->count) : nullptr, fr ? lag->capacity : 0,
          static_cast<const int32_t*>(sc->cage_idx), static_cast<const int32_t*>(sc->item_n),
@@ -2110,21 +2235,17 @@ void hvp_launch(eipc_scene* sc, const double* q, const eipc_pairs& pr, const eip
   exclusive_scan_i64(sc->rc_g, sc->ro_g, cnt + kCntItems, item_cap, tot_g, sc->scan_partial, s);
   launch(k_rec_check, 1, 32, 0, s, static_cast<const int64_t*>(cnt + kCntZero), static_cast<const int64_t*>(tot_g),
          sc->rec_cap, sc->gcap, cnt + kCntRecH, cnt + kCntRecG, sc->status);
-  EvalArgs A;
+  EvalArgs A{};
   A.T = sc->topo; A.pr = pr; A.cage_idx = sc->cage_idx; A.w = sc->w; A.x4 = sc->x4; A.ns = sc->ns;
   A.dhat = p.dhat; A.kappa = p.kappa; A.item_nodes = sc->item_nodes; A.item_n = sc->item_n;
   A.ro_h = sc->ro_h; A.ro_g = sc->ro_g; A.n_items = cnt + kCntItems; A.rec_cap = sc->rec_cap; A.gcap = sc->gcap;
-  A.hkeys = sc->hkeys; A.hvals = sc->hvals; A.hrec = sc->hrec; A.gkeys = sc->gkeys; A.gvals = sc->gvals;
+  A.gkeys = sc->gkeys; A.gvals = sc->gvals;
   A.grec = sc->grec; A.item_E = sc->item_E; A.st = sc->status;
   A.project = false;
   A.moll_r2 = sc->moll_factor > 0.0 ? sc->moll_r2 : nullptr;
   A.moll_factor = sc->moll_factor;
-  A.order = nullptr;
-  A.queue = nullptr;
-  A.tile = 32;
   A.hv_dir = v;
   for (int c = 0; c < 3; ++c) A.kin_dir[c] = kin_dir ? kin_dir[c] : 0.0;
-  A.hinv = nullptr;
   A.fric_of_pair = nullptr; A.pair_of_fric = nullptr;
   A.lag = fr ? *lag : eipc_lag{};
   A.mu = p.mu; A.eps_f = p.eps_v * p.h;

@@ -328,8 +328,10 @@ __device__ __forceinline__ int stencil_hint(int type, const float* __restrict__ 
   return closest_hint(type, P[0], P[1], P[2], P[3], M * 5.9604645e-8f);
 }
 
-__device__ __forceinline__ V3 pick(const V3 X[4], int k) {
-  V3 r = X[0];
+// X[k] by selects (a run-time index would put X in local memory)
+template <class T>
+__device__ __forceinline__ T pick(const T X[4], int k) {
+  T r = X[0];
   if (k == 1) r = X[1];
   if (k == 2) r = X[2];
   if (k == 3) r = X[3];

@@ -60,7 +60,8 @@ struct eipc_scene {
   uint64_t* hkeys_alt;
   uint32_t* hvals;
   uint32_t* hvals_alt;
-  double* hrec;          // [rec_cap*kHRecStride] 3x3 blocks, 16-byte aligned rows
+  double* hrec;          // [rec_cap*kHRecStride] explicit 3x3 blocks of mollified pairs, 16-byte aligned
+                         // rows (null until the mollifier is first turned on)
   double* hvp_out;       // [(ns+64)*3] Hessian-vector product: reduced rows, then 64 kinematic partials
   uint64_t* edge_key;    // [ne] sorted a * nv + b of every edge (a < b), for edge-id lookup
   int32_t* edge_id;      // [ne] edge id of each sorted key
@@ -70,7 +71,11 @@ struct eipc_scene {
   int64_t* seg_flag;     // [rec_cap] key of each Hessian segment (upper block), as uint64
   int64_t* seg_id;       // [rec_cap] BSR entries of each segment's block and transpose, as int32 pairs
   int64_t* seg_start;    // [rec_cap]
-  uint32_t* hinv;        // [rec_cap] sorted position of each Hessian record
+  uint64_t* rec_src;     // [rec_cap] source of each Hessian record: item << 8 | row node << 4 | column node
+  uint64_t* src_sorted;  // [rec_cap] the same in sorted order
+  double* frow;          // [gcap*kFRow] factor rows of the evaluated items, one per cage node (eval.cu)
+  double* ihead;         // [item_cap*kIHead] headers of the evaluated items
+  uint64_t* item_map;    // [item_cap] local node of each (vertex, slot) of an item, in nibbles
   double* piece;         // [9 * (rec_cap + rec_cap / 32 + 2)] partial segment sums of the Hessian records
   int64_t* hunit;        // [rec_cap + 1] first summation unit of each Hessian segment
   int64_t gcap;          // gradient records
@@ -104,11 +109,16 @@ namespace eipc {
 // device counters
 // record row strides (doubles): 9 (3) values padded so that each row starts on 16 bytes
 constexpr int kHRecStride = 10, kGRecStride = 4;
+// factor row: z1, z2 (3 each), omega, friction weight, z3 (3), pad; item header: the friction
+// block's upper entries (6), the gradient vectors of barrier and friction (3 each), the
+// isotropic coefficient, flags, pad.  32-byte sectors throughout.
+constexpr int kFRow = 12, kIHead = 16;
 
 enum { kCntCand = 0, kCntSurv = 1, kCntItems = 2, kCntRecH = 3, kCntRecG = 4, kCntSegH = 5, kCntSegG = 6,
        kCntAccd = 7, kCntZero = 8, kCntEvalQueue = 16, kCntScreened = 15, kCntDedup = 17, kCntUnitsH = 18,
        kCntMollBad = 20, kCntCcdQueue = 21,
-       kCntN = 24 };
+       kCntEvalRest = 24, /* two entries */
+       kCntN = 26 };
 
 // id of the edge with end vertices {a, b} from the scene's sorted edge keys a * nv + b
 // (a < b), or -1 if there is none
