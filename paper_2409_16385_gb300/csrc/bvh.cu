@@ -62,37 +62,6 @@ __device__ __forceinline__ uint32_t spread10(uint32_t v) {
   return v;
 }
 
-// Per-vertex FP32 boxes, rounded outward from the FP64 positions (swept over x + dx when
-// dx4 is given): vbox[8v..8v+5] = lo xyz, hi xyz (rows of 8 floats), and vbox_pad the same
-// grown by pad in FP64 before rounding.  Outward rounding and the pad subtraction are
-// monotone, so the min / max over a primitive's vertices of these boxes is bit for bit the
-// box made from the primitive's FP64 positions (FP64 min / max, padded, rounded outward):
-// the hierarchy and traversal read these instead of recomputing FP64 minima per primitive.
-__global__ void __launch_bounds__(kBlock) k_vertex_boxes(int64_t nv, const double* __restrict__ x4,
-                                                         const double* __restrict__ dx4, double pad,
-                                                         float* __restrict__ vbox, float* __restrict__ vbox_pad) {
-  pdl_entry();
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < nv; v += grid_stride()) {
-    const V3 p = load_x(x4, (int32_t)v);
-    double lo[3] = {p.x, p.y, p.z}, hi[3] = {p.x, p.y, p.z};
-    if (dx4) {
-      const V3 d = load_x(dx4, (int32_t)v);
-      const double e[3] = {p.x + d.x, p.y + d.y, p.z + d.z};
-      for (int k = 0; k < 3; ++k) { lo[k] = fmin(lo[k], e[k]); hi[k] = fmax(hi[k], e[k]); }
-    }
-    float4* o = reinterpret_cast<float4*>(vbox + 8 * v);
-    o[0] = make_float4(__double2float_rd(lo[0]), __double2float_rd(lo[1]), __double2float_rd(lo[2]),
-                       __double2float_ru(hi[0]));
-    o[1] = make_float4(__double2float_ru(hi[1]), __double2float_ru(hi[2]), 0.f, 0.f);
-    if (vbox_pad) {
-      float4* op = reinterpret_cast<float4*>(vbox_pad + 8 * v);
-      op[0] = make_float4(__double2float_rd(__dsub_rd(lo[0], pad)), __double2float_rd(__dsub_rd(lo[1], pad)),
-                          __double2float_rd(__dsub_rd(lo[2], pad)), __double2float_ru(__dadd_ru(hi[0], pad)));
-      op[1] = make_float4(__double2float_ru(__dadd_ru(hi[1], pad)), __double2float_ru(__dadd_ru(hi[2], pad)), 0.f, 0.f);
-    }
-  }
-}
-
 // box of up to three vertices from the per-vertex boxes (ids < 0 are skipped)
 __device__ __forceinline__ void verts_box(const float* __restrict__ vbox, int32_t a, int32_t b, int32_t c,
                                           float lo[3], float hi[3]) {
@@ -644,12 +613,6 @@ __global__ void __launch_bounds__(256, MINB) k_query(Bvh tt, Bvh te, Topo T, con
 }
 
 }  // namespace
-
-void vertex_boxes(const Topo& topo, const double* x4, const double* dx4, double pad, float* vbox, float* vbox_pad,
-                  cudaStream_t s) {
-  if (topo.nv <= 0) return;
-  launch(k_vertex_boxes, blocks_for(topo.nv), kBlock, 0, s, topo.nv, x4, dx4, pad, vbox, vbox_pad);
-}
 
 void bvh_build(Bvh& t, PrimKind kind, const Topo& topo, const double* x4, const double* dx4, const float* vbox,
                int32_t* bounds_ws, uint32_t* sort_hist, cudaStream_t s, int refit_variant) {

@@ -60,13 +60,6 @@ __host__ __device__ __forceinline__ uint64_t pair_key(int type, uint32_t i, uint
   return ((uint64_t)type << (bi + bj)) | ((uint64_t)i << bj) | (uint64_t)j;
 }
 
-// Per-vertex FP32 boxes of the positions x4 (padded), swept over x + dx when dx4 is given,
-// rounded outward: vbox[8 nv] unpadded and, when vbox_pad is not null, vbox_pad[8 nv] grown
-// by pad.  The leaf and query boxes below are taken from these; they are bit for bit the
-// boxes computed from the positions primitive by primitive.
-void vertex_boxes(const Topo& topo, const double* x4, const double* dx4, double pad, float* vbox, float* vbox_pad,
-                  cudaStream_t s);
-
 // Build the tree over primitives of `kind`: scene bounds from positions x4 (padded),
 // optionally swept by dx4 (CCD), leaf boxes from the matching per-vertex boxes vbox;
 // `bounds_ws` holds 6 ints of scratch.  Enqueued on stream s.

@@ -32,6 +32,35 @@ struct Stencil {
 __device__ __forceinline__ bool is_pos(double a) { return __double_as_longlong(a) > 0; }
 __device__ __forceinline__ bool lt_nonneg(double a, double b) { return __double_as_longlong(a) < __double_as_longlong(b); }
 
+// x to FP32, rounded to nearest (mode 0), down (-1) or up (+1), by integer instructions: the
+// conversion instruction holds the FP64 pipe like an FP64 operation.  Results of FP32's normal
+// range and zeros; anything else takes the instruction.
+template <int mode>
+__device__ __forceinline__ float to_float(double x) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  if (((hi << 1) | lo) == 0) return __int_as_float(hi);
+  const int e = ((hi >> 20) & 0x7ff) - 896;            // biased FP32 exponent
+  if (e >= 1 && e <= 253) {
+    const unsigned mag = ((unsigned)e << 23) | ((unsigned)(hi & 0xfffff) << 3) | ((unsigned)lo >> 29);
+    const unsigned rest = (unsigned)lo & 0x1fffffffu;
+    const bool up = mode == 0 ? (rest > 0x10000000u || (rest == 0x10000000u && (mag & 1u)))
+                              : (rest != 0u && (mode < 0) == (hi < 0));
+    return __int_as_float((int)((unsigned)(hi & 0x80000000) | (mag + (up ? 1u : 0u))));
+  }
+  return mode == 0 ? __double2float_rn(x) : (mode < 0 ? __double2float_rd(x) : __double2float_ru(x));
+}
+__device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+
+// Per-vertex FP32 box of [lo, hi], rounded outward from the FP64 positions, in rows of 8 floats (lo
+// xyz, hi xyz).  Outward rounding is monotone, so the min / max over a primitive's vertices of
+// these boxes is bit for bit the box made from the primitive's FP64 positions: the hierarchy
+// and the traversal read these instead of recomputing FP64 minima per primitive.
+__device__ __forceinline__ void store_box(float* row, const double lo[3], const double hi[3]) {
+  float4* o = reinterpret_cast<float4*>(row);
+  o[0] = make_float4(to_float<-1>(lo[0]), to_float<-1>(lo[1]), to_float<-1>(lo[2]), to_float<1>(hi[0]));
+  o[1] = make_float4(to_float<1>(hi[1]), to_float<1>(hi[2]), 0.f, 0.f);
+}
+
 // |p - (e0 + t (e1 - e0))|^2 over t in [0,1].  t = clamp((w.e) / (e.e), 0, 1), with the
 // quotient (one reciprocal and a product) taken only inside (0, 1): w.e <= 0 gives 0 and
 // w.e >= e.e gives 1, also for e = 0.  A NaN gives a NaN distance either way.

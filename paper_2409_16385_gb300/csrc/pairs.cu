@@ -9,12 +9,22 @@ namespace {
 
 // x_k = sum_j w_kj q_{idx_kj}; kinematic rows take x_kin (or 0 for a displacement).
 // One thread per vertex; writes either the padded internal layout or a caller [Nv,3] array.
+// With vbox (contact set) also the vertex's FP32 box and the same grown by pad in FP64 before
+// rounding, and thread 0 zeroes the counters of `zero`: one pass over the vertices and one
+// launch instead of three.  Bound by the FP64 pipe where it is not by latency (12 products and
+// sums per vertex, 6 for the padding; the conversions are integer work).
 __global__ void __launch_bounds__(kBlock) k_embed(int64_t nv, const int32_t* __restrict__ idx,
                                                   const double* __restrict__ w, const double* __restrict__ xk4,
                                                   const double* __restrict__ q, double* __restrict__ out,
                                                   int padded, int displacement, float* __restrict__ outf,
-                                                  DevStatus* st) {
+                                                  DevStatus* st, float* __restrict__ vbox, float* __restrict__ vbox_pad,
+                                                  double pad, CounterList zero) {
   pdl_entry();
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+#pragma unroll
+    for (int c = 0; c < kCounterList; ++c)
+      if (zero.p[c]) *zero.p[c] = 0;
+  }
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < nv; v += grid_stride()) {
     const int4 id = __ldg(reinterpret_cast<const int4*>(idx) + v);
     double r[3];
@@ -31,14 +41,19 @@ __global__ void __launch_bounds__(kBlock) k_embed(int64_t nv, const int32_t* __r
         for (int j = 0; j < 4; ++j) s += ws[j] * __ldg(q + 3 * (int64_t)ids[j] + k);
         r[k] = s;
       }
-      if (!(isfinite(r[0]) && isfinite(r[1]) && isfinite(r[2]))) raise_flag(st, EIPC_FLAG_NONFINITE);
+      if (!(finite_bits(r[0]) && finite_bits(r[1]) && finite_bits(r[2]))) raise_flag(st, EIPC_FLAG_NONFINITE);
     }
     if (padded) {
       reinterpret_cast<double2*>(out)[2 * v] = make_double2(r[0], r[1]);
       reinterpret_cast<double2*>(out)[2 * v + 1] = make_double2(r[2], 0.0);
       if (outf)
-        reinterpret_cast<float4*>(outf)[v] =
-            make_float4(__double2float_rn(r[0]), __double2float_rn(r[1]), __double2float_rn(r[2]), 0.f);
+        reinterpret_cast<float4*>(outf)[v] = make_float4(to_float<0>(r[0]), to_float<0>(r[1]), to_float<0>(r[2]), 0.f);
+      if (vbox) {
+        store_box(vbox + 8 * v, r, r);
+        const double lo[3] = {__dsub_rd(r[0], pad), __dsub_rd(r[1], pad), __dsub_rd(r[2], pad)};
+        const double hi[3] = {__dadd_ru(r[0], pad), __dadd_ru(r[1], pad), __dadd_ru(r[2], pad)};
+        store_box(vbox_pad + 8 * v, lo, hi);
+      }
     } else {
       for (int k = 0; k < 3; ++k) out[3 * v + k] = r[k];
     }
@@ -328,7 +343,7 @@ void embed_launch(const eipc_scene* sc, const double* q, double* out, int out_pa
                   cudaStream_t s) {
   float* outf = (out_padded && out == sc->x4) ? sc->x4f : nullptr;   // FP32 copy for the screen
   launch(k_embed, blocks_for(sc->nv), kBlock, 0, s, sc->nv, sc->cage_idx, sc->w, sc->x_kin4, q, out, out_padded,
-         displacement, outf, sc->status);
+         displacement, outf, sc->status, static_cast<float*>(nullptr), static_cast<float*>(nullptr), 0.0, CounterList{});
 }
 
 namespace {
@@ -396,18 +411,18 @@ void set_kinematic_launch(eipc_scene* sc, const double* x_kin, cudaStream_t s) {
 }
 
 void pairs_launch(eipc_scene* sc, const double* q, const eipc_params& p, const eipc_pairs& out, cudaStream_t s) {
-  EIPC_TIMED(sc, kKEmbed, s, embed_launch(sc, q, sc->x4, 1, 0, s));
   int64_t* n_cand = sc->counters + kCntCand;
   int64_t* n_surv = sc->counters + kCntSurv;
   int64_t* n_cand2 = sc->counters + kCntScreened;
-  zero_ranges(s, {{sc->counters + kCntCand, 2 * sizeof(int64_t)}, {n_cand2, sizeof(int64_t)}});
+  // positions, per-vertex boxes (unpadded for the leaves, grown by dhat for the queries), counters
+  EIPC_TIMED(sc, kKEmbed, s,
+             (launch(k_embed, blocks_for(sc->nv), kBlock, 0, s, sc->nv, sc->cage_idx, sc->w, sc->x_kin4, q, sc->x4, 1, 0,
+                     sc->x4f, sc->status, sc->vbox, sc->vbox_pad, p.dhat, CounterList{{n_cand, n_surv, n_cand2, nullptr}})));
   // LBVHs over triangles and edges, then one traversal: vertex boxes grown by dhat against
   // the triangle tree (PT) and edge boxes grown by dhat against the edge tree (EE, j > i)
   // full rebuild every `rebuild_interval` calls, refit of the same hierarchy in between (the
   // candidate set is exact for any hierarchy; only traversal cost depends on its quality)
   const bool rebuild = !sc->tri_bvh.built || !sc->edge_bvh.built || sc->contact_refits + 1 >= sc->rebuild_interval;
-  // per-vertex boxes: unpadded for the leaves, grown by dhat for the queries
-  EIPC_TIMED(sc, kKBvh, s, vertex_boxes(sc->topo, sc->x4, nullptr, p.dhat, sc->vbox, sc->vbox_pad, s));
   if (rebuild) {
     EIPC_TIMED(sc, kKBvh, s, bvh_build(sc->tri_bvh, kTri, sc->topo, sc->x4, nullptr, sc->vbox, sc->bounds_ws, sc->sort_hist, s,
                                       sc->tune.refit_variant));

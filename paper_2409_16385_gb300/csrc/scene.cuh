@@ -29,7 +29,8 @@ struct eipc_scene {
   // positions (padded, 4 doubles per vertex)
   double* x4;
   double* dx4;
-  float* x4f;            // [nv*4] FP32 copy of x4 for the narrow-phase screen
+  float* x4f;            // [nv*4] FP32 copy of x4 for the FP32 screens
+  float* dx4f;           // [nv*4] FP32 copy of dx4
   float* vbox;           // [nv*8] per-vertex FP32 boxes of the last call (contact or swept)
   float* vbox_pad;       // [nv*8] the contact ones grown by dhat (the query boxes)
   // broad phase
@@ -116,9 +117,15 @@ constexpr int kFRow = 12, kIHead = 16;
 
 enum { kCntCand = 0, kCntSurv = 1, kCntItems = 2, kCntRecH = 3, kCntRecG = 4, kCntSegH = 5, kCntSegG = 6,
        kCntAccd = 7, kCntZero = 8, kCntEvalQueue = 16, kCntScreened = 15, kCntDedup = 17, kCntUnitsH = 18,
-       kCntMollBad = 20, kCntCcdQueue = 21,
+       kCntMollBad = 20, kCntCcdQueue = 21, kCntCcdList = 22,
        kCntEvalRest = 24, /* two entries */
        kCntN = 26 };
+
+// device counters a kernel zeroes before the launches that count (null: none)
+constexpr int kCounterList = 4;
+struct CounterList {
+  int64_t* p[kCounterList];
+};
 
 // id of the edge with end vertices {a, b} from the scene's sorted edge keys a * nv + b
 // (a < b), or -1 if there is none
