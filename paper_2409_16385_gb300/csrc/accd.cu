@@ -314,25 +314,11 @@ void accd_launch(eipc_scene* sc, const double* x, const double* dx, const eipc_p
              (launch(k_ccd_begin, blocks_for(sc->nv > sc->n_groups ? sc->nv : sc->n_groups), kBlock, 0, s, x, dx, sc->nv, sc->x4,
                      sc->dx4, sc->x4f, sc->dx4f, sc->vbox, sc->status, CounterList{{n_cand, n_adv, queue, n_list}}, abits,
                      sc->group_alpha_bits, sc->n_groups)));
-  if (sc->tri_bvh.built && sc->edge_bvh.built) {
-    EIPC_TIMED(sc, kKBvh, s, bvh_refit_pair(sc->tri_bvh, kTri, sc->edge_bvh, kEdge, sc->topo, sc->vbox, s,
-                                           sc->tune.refit_variant));
-  } else {
-    if (sc->tri_bvh.built)
-      EIPC_TIMED(sc, kKBvh, s, bvh_refit(sc->tri_bvh, kTri, sc->topo, sc->vbox, s, sc->tune.refit_variant));
-    else
-      EIPC_TIMED(sc, kKBvh, s, bvh_build(sc->tri_bvh, kTri, sc->topo, sc->x4, sc->dx4, sc->vbox, sc->bounds_ws, sc->sort_hist, s,
-                                        sc->tune.refit_variant));
-    if (sc->edge_bvh.built)
-      EIPC_TIMED(sc, kKBvh, s, bvh_refit(sc->edge_bvh, kEdge, sc->topo, sc->vbox, s, sc->tune.refit_variant));
-    else
-      EIPC_TIMED(sc, kKBvh, s, bvh_build(sc->edge_bvh, kEdge, sc->topo, sc->x4, sc->dx4, sc->vbox, sc->bounds_ws, sc->sort_hist, s,
-                                        sc->tune.refit_variant));
-  }
+  if (sc->broad.built) EIPC_TIMED(sc, kKBvh, s, bvh_refit(sc->broad, sc->vbox, s));
+  else EIPC_TIMED(sc, kKBvh, s, bvh_build(sc->broad, sc->topo, sc->vbox, sc->sort_hist, s));
   EIPC_TIMED(sc, kKQuery, s,
-             bvh_query(sc->tri_bvh, sc->edge_bvh, sc->topo, sc->vbox, sc->cand, n_cand, sc->cand_cap,
-                       sc->status, s, sc->tune.query_threads, sc->tune.query_bps,
-                       sc->tune.query_variant));
+             bvh_query(sc->broad, sc->topo, sc->vbox, sc->cand, n_cand, sc->cand_cap, sc->status, s,
+                       sc->tune.query_threads, sc->tune.query_bps));
   // cand2 is free here (the contact search's screened list)
   sc->timers->start(kKCa, s);
   launch(k_ccd_screen, blocks_for(sc->cand_cap, 8), kBlock, 0, s, sc->topo, static_cast<const double*>(sc->x4),

@@ -23,13 +23,11 @@ cudaError_t dalloc(T** p, int64_t n) {
 void free_scene(eipc_scene* s) {
   if (!s) return;
   void* ptrs[] = {s->tris, s->edges, s->cage_idx, s->w, s->x_kin4, s->hvp_out, s->edge_key, s->edge_id, s->moll_r2, s->vkin, s->ekin, s->fkin, s->vgroup, s->group_alpha_bits, s->group_count, s->item_group, s->fric_of_pair, s->pair_of_fric, s->lag_key, s->x4, s->dx4, s->x4f, s->dx4f, s->vbox, s->vbox_pad, s->cand2,
-                  s->tri_bvh.n_dev, s->tri_bvh.nodes, s->tri_bvh.parent, s->tri_bvh.leaf_prim, s->tri_bvh.leaf_info,
-                  s->tri_bvh.leaf_box, s->tri_bvh.refit_flag, s->tri_bvh.keys, s->tri_bvh.vals,
-                  s->tri_bvh.keys_alt, s->tri_bvh.vals_alt, s->tri_bvh.range, s->tri_bvh.tl_root, s->tri_bvh.up_start,
-                  s->tri_bvh.tl_count, s->edge_bvh.n_dev, s->edge_bvh.nodes, s->edge_bvh.leaf_info,
-                  s->edge_bvh.parent, s->edge_bvh.leaf_prim, s->edge_bvh.leaf_box, s->edge_bvh.refit_flag,
-                  s->edge_bvh.keys, s->edge_bvh.vals, s->edge_bvh.keys_alt, s->edge_bvh.vals_alt, s->edge_bvh.range,
-                  s->edge_bvh.tl_root, s->edge_bvh.up_start, s->edge_bvh.tl_count, s->bounds_ws,
+                  s->broad.tri.nodes, s->broad.tri.parent, s->broad.tri.leaf_info, s->broad.tri.leaf_box, s->broad.tri.flag,
+                  s->broad.tri.treelet, s->broad.tri.n_treelets, s->broad.tri.treelet_box, s->broad.edge.treelet_box, s->broad.edge.nodes, s->broad.edge.parent,
+                  s->broad.edge.leaf_info, s->broad.edge.leaf_box, s->broad.edge.flag, s->broad.edge.treelet,
+                  s->broad.edge.n_treelets, s->broad.keys, s->broad.keys_alt, s->broad.vals, s->broad.vals_alt,
+                  s->broad.n_dev, s->broad.bounds,
                   s->sort_hist, s->cand, s->counters, s->skeys, s->skeys_alt, s->svals, s->svals_alt, s->sd,
                   s->item_nodes, s->item_n, s->rc_h, s->ro_h, s->rc_g, s->ro_g, s->item_E, s->hkeys,
                   s->hkeys_alt, s->hvals, s->hvals_alt, s->hrec, s->seg_flag, s->seg_id, s->seg_start, s->rec_src, s->src_sorted, s->frow, s->ihead, s->item_map, s->piece, s->hunit,
@@ -51,22 +49,28 @@ cudaError_t alloc_bvh(Bvh& t, int64_t n) {
   t.n = n;
   cudaError_t e = cudaSuccess;
   auto ok = [&](cudaError_t r) { if (r != cudaSuccess && e == cudaSuccess) e = r; };
-  ok(dalloc(&t.n_dev, 1));
   ok(dalloc(&t.nodes, n > 1 ? n - 1 : 1));
   ok(dalloc(&t.parent, 2 * n));
-  ok(dalloc(&t.leaf_prim, n));
   ok(dalloc(&t.leaf_info, n));
-  ok(dalloc(&t.leaf_box, 6 * n));
-  ok(dalloc(&t.refit_flag, n));
-  ok(dalloc(&t.keys, n));
-  ok(dalloc(&t.vals, n));
-  ok(dalloc(&t.keys_alt, n));
-  ok(dalloc(&t.vals_alt, n));
-  ok(dalloc(&t.range, n > 1 ? n - 1 : 1));
-  ok(dalloc(&t.tl_root, n));
-  ok(dalloc(&t.up_start, n));
-  ok(dalloc(&t.tl_count, 2));
-  if (e == cudaSuccess) e = cudaMemcpy(t.n_dev, &n, sizeof(int64_t), cudaMemcpyHostToDevice);
+  ok(dalloc(&t.leaf_box, 8 * n));
+  ok(dalloc(&t.flag, n));
+  ok(dalloc(&t.treelet, n));
+  ok(dalloc(&t.treelet_box, 8 * n));
+  ok(dalloc(&t.n_treelets, 1));
+  return e;
+}
+
+cudaError_t alloc_broad(Broad& b, int64_t nf, int64_t ne, int64_t nv) {
+  const int64_t n = nf + ne + nv;
+  cudaError_t e = cudaSuccess;
+  auto ok = [&](cudaError_t r) { if (r != cudaSuccess && e == cudaSuccess) e = r; };
+  ok(alloc_bvh(b.tri, nf));
+  ok(alloc_bvh(b.edge, ne));
+  ok(dalloc(&b.keys, n)); ok(dalloc(&b.keys_alt, n));
+  ok(dalloc(&b.vals, n)); ok(dalloc(&b.vals_alt, n));
+  ok(dalloc(&b.n_dev, 1));
+  ok(dalloc(&b.bounds, 6));
+  if (e == cudaSuccess) e = cudaMemcpy(b.n_dev, &n, sizeof(int64_t), cudaMemcpyHostToDevice);
   return e;
 }
 
@@ -143,9 +147,7 @@ eipc_status eipc_scene_create(int64_t Nv, int64_t F, int64_t E, int64_t Ns, cons
   ok(dalloc(&s->vgroup, Nv)); ok(dalloc(&s->group_alpha_bits, 1)); ok(dalloc(&s->group_count, 4));
   ok(dalloc(&s->x4, 4 * Nv)); ok(dalloc(&s->dx4, 4 * Nv)); ok(dalloc(&s->x4f, 4 * Nv)); ok(dalloc(&s->dx4f, 4 * Nv));
   ok(dalloc(&s->vbox, 8 * Nv)); ok(dalloc(&s->vbox_pad, 8 * Nv));
-  ok(alloc_bvh(s->tri_bvh, F));
-  ok(alloc_bvh(s->edge_bvh, E));
-  ok(dalloc(&s->bounds_ws, 8));
+  ok(alloc_broad(s->broad, F, E, Nv));
   ok(dalloc(&s->sort_hist, (int64_t)sort_hist_entries()));
   ok(dalloc(&s->cand, s->cand_cap));
   ok(dalloc(&s->cand2, s->cand_cap));
@@ -434,7 +436,7 @@ eipc_status eipc_scene_set_groups(eipc_scene* sc, const int32_t* vertex_group, i
   sc->group_alpha_bits = gb;
   sc->group_count = gc;
   sc->n_groups = n_groups;
-  sc->tri_bvh.built = sc->edge_bvh.built = false;   // leaf records carry the group
+  sc->broad.built = false;   // leaf records carry the group
   return EIPC_OK;
 }
 

@@ -1,49 +1,41 @@
-// LBVH build (Morton sort, Karras hierarchy, bottom-up refit) and traversal.
+// LBVH build (one Morton sort, Karras hierarchies, treelets), refit and traversal.
 #include "bvh.cuh"
 #include "sort.cuh"
 
 namespace eipc {
 namespace {
 
-// order-preserving map float -> int for atomic min / max
+// order-preserving map float -> int for integer min / max
 __device__ __forceinline__ int32_t f2ord(float f) {
   int32_t i = __float_as_int(f);
   return i >= 0 ? i : i ^ 0x7fffffff;
 }
 __device__ __forceinline__ float ord2f(int32_t i) { return __int_as_float(i >= 0 ? i : i ^ 0x7fffffff); }
 
-__global__ void k_bounds_init(int32_t* b) {
+__device__ __forceinline__ float warp_min(float x) { return ord2f(__reduce_min_sync(0xffffffffu, f2ord(x))); }
+__device__ __forceinline__ float warp_max(float x) { return ord2f(__reduce_max_sync(0xffffffffu, f2ord(x))); }
+
+__global__ void k_bounds_init(int32_t* b, int32_t* n_tri, int32_t* n_edge) {
   pdl_entry();
   if (threadIdx.x < 3) b[threadIdx.x] = 0x7fffffff;
   else if (threadIdx.x < 6) b[threadIdx.x] = (int32_t)0x80000000;
+  else if (threadIdx.x == 6) *n_tri = 0;
+  else if (threadIdx.x == 7) *n_edge = 0;
 }
 
-// scene box over all vertex positions (and their swept ends)
-__global__ void __launch_bounds__(kBlock) k_bounds(const double* __restrict__ x4, const double* __restrict__ dx4,
-                                                   int64_t nv, int32_t* __restrict__ b) {
+// scene box over all per-vertex boxes
+__global__ void __launch_bounds__(kBlock) k_bounds(const float* __restrict__ vbox, int64_t nv, int32_t* __restrict__ b) {
   pdl_entry();
   float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < nv; v += grid_stride()) {
-    V3 p = load_x(x4, (int32_t)v);
-    double c[3] = {p.x, p.y, p.z};
-    for (int k = 0; k < 3; ++k) {
-      lo[k] = fminf(lo[k], __double2float_rd(c[k]));
-      hi[k] = fmaxf(hi[k], __double2float_ru(c[k]));
-    }
-    if (dx4) {
-      V3 d = load_x(dx4, (int32_t)v);
-      double e[3] = {p.x + d.x, p.y + d.y, p.z + d.z};
-      for (int k = 0; k < 3; ++k) {
-        lo[k] = fminf(lo[k], __double2float_rd(e[k]));
-        hi[k] = fmaxf(hi[k], __double2float_ru(e[k]));
-      }
-    }
+    const float4 p = __ldg(reinterpret_cast<const float4*>(vbox + 8 * v));
+    const float4 q = __ldg(reinterpret_cast<const float4*>(vbox + 8 * v) + 1);
+    lo[0] = fminf(lo[0], p.x); lo[1] = fminf(lo[1], p.y); lo[2] = fminf(lo[2], p.z);
+    hi[0] = fmaxf(hi[0], p.w); hi[1] = fmaxf(hi[1], q.x); hi[2] = fmaxf(hi[2], q.y);
   }
   for (int k = 0; k < 3; ++k) {
-    for (int o = 16; o > 0; o >>= 1) {
-      lo[k] = fminf(lo[k], __shfl_xor_sync(0xffffffffu, lo[k], o));
-      hi[k] = fmaxf(hi[k], __shfl_xor_sync(0xffffffffu, hi[k], o));
-    }
+    lo[k] = warp_min(lo[k]);
+    hi[k] = warp_max(hi[k]);
   }
   if ((threadIdx.x & 31) == 0) {
     for (int k = 0; k < 3; ++k) {
@@ -67,6 +59,7 @@ __device__ __forceinline__ void verts_box(const float* __restrict__ vbox, int32_
                                           float lo[3], float hi[3]) {
   for (int k = 0; k < 3; ++k) { lo[k] = INFINITY; hi[k] = -INFINITY; }
   const int32_t v[3] = {a, b, c};
+#pragma unroll
   for (int s = 0; s < 3; ++s) {
     if (v[s] < 0) continue;
     const float4 p = __ldg(reinterpret_cast<const float4*>(vbox + 8 * (int64_t)v[s]));
@@ -76,18 +69,10 @@ __device__ __forceinline__ void verts_box(const float* __restrict__ vbox, int32_
   }
 }
 
-// box of one primitive from the per-vertex boxes
-__device__ __forceinline__ void prim_box_v(PrimKind kind, int64_t i, const Topo& T, const float* __restrict__ vbox,
-                                           float lo[3], float hi[3]) {
-  if (kind == kVertex) verts_box(vbox, (int32_t)i, -1, -1, lo, hi);
-  else if (kind == kEdge) verts_box(vbox, T.edges[2 * i], T.edges[2 * i + 1], -1, lo, hi);
-  else verts_box(vbox, T.tris[3 * i], T.tris[3 * i + 1], T.tris[3 * i + 2], lo, hi);
-}
-
-__global__ void __launch_bounds__(kBlock) k_leaves(PrimKind kind, int64_t n, Topo T, const float* __restrict__ vbox,
-                                                   const int32_t* __restrict__ b,
-                                                   float* __restrict__ leaf_box, uint64_t* __restrict__ keys,
-                                                   uint32_t* __restrict__ vals) {
+// Sort keys of every triangle, edge and vertex: kind (0, 1, 2) above the Morton code of the box
+// centre, so that one sort orders all three.
+__global__ void __launch_bounds__(kBlock) k_morton_keys(Topo T, const float* __restrict__ vbox, const int32_t* __restrict__ b,
+                                                        uint64_t* __restrict__ keys, uint32_t* __restrict__ vals) {
   pdl_entry();
   float blo[3], bext[3];
   for (int k = 0; k < 3; ++k) {
@@ -95,19 +80,23 @@ __global__ void __launch_bounds__(kBlock) k_leaves(PrimKind kind, int64_t n, Top
     float e = ord2f(b[3 + k]) - blo[k];
     bext[k] = e > 0.f ? e : 1.f;
   }
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += grid_stride()) {
+  const int64_t n = T.nf + T.ne + T.nv;
+  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n; g += grid_stride()) {
+    const int kind = g < T.nf ? 0 : (g < T.nf + T.ne ? 1 : 2);
+    const int64_t i = kind == 0 ? g : (kind == 1 ? g - T.nf : g - T.nf - T.ne);
     float lo[3], hi[3];
-    prim_box_v(kind, i, T, vbox, lo, hi);
+    if (kind == 0) verts_box(vbox, T.tris[3 * i], T.tris[3 * i + 1], T.tris[3 * i + 2], lo, hi);
+    else if (kind == 1) verts_box(vbox, T.edges[2 * i], T.edges[2 * i + 1], -1, lo, hi);
+    else verts_box(vbox, (int32_t)i, -1, -1, lo, hi);
     uint32_t code = 0;
     for (int k = 0; k < 3; ++k) {
       float c = (0.5f * (lo[k] + hi[k]) - blo[k]) / bext[k];
       c = fminf(fmaxf(c, 0.f), 1.f);
-      uint32_t q = (uint32_t)fminf(c * 1024.f, 1023.f);
+      const uint32_t q = (uint32_t)fminf(c * 1024.f, 1023.f);
       code |= spread10(q) << (2 - k);
     }
-    for (int k = 0; k < 3; ++k) { leaf_box[6 * i + k] = lo[k]; leaf_box[6 * i + 3 + k] = hi[k]; }
-    keys[i] = code;
-    vals[i] = (uint32_t)i;
+    keys[g] = (uint64_t)kind << 30 | code;
+    vals[g] = (uint32_t)i;
   }
 }
 
@@ -118,330 +107,191 @@ __device__ __forceinline__ int delta(const uint64_t* __restrict__ k, int64_t n, 
   return __clzll((unsigned long long)(a ^ b));
 }
 
+// What building and refitting need of one tree; n = 0 marks an absent tree.
+struct TreeView {
+  int64_t n;
+  const uint64_t* keys;      // this tree's sorted keys (build only)
+  const uint32_t* prim;
+  BvhNode* nodes;
+  int32_t* parent;
+  int4* leaf_info;
+  float* leaf_box;
+  int32_t* flag;
+  int4* treelet;
+  float* treelet_box;
+  int32_t* n_treelets;
+};
+
 // Karras 2012: internal node i covers a key range; its split is the highest differing bit.
-__global__ void __launch_bounds__(kBlock) k_internal(const uint64_t* __restrict__ keys, int64_t n,
-                                                     BvhNode* __restrict__ nodes, int32_t* __restrict__ parent,
-                                                     int2* __restrict__ range) {
+__device__ __forceinline__ void internal_node(const TreeView& T, int64_t i) {
+  const uint64_t* keys = T.keys;
+  const int64_t n = T.n;
+  int dir = (delta(keys, n, i, i + 1) - delta(keys, n, i, i - 1)) >= 0 ? 1 : -1;
+  int dmin = delta(keys, n, i, i - dir);
+  int64_t lmax = 2;
+  while (delta(keys, n, i, i + lmax * dir) > dmin) lmax *= 2;
+  int64_t l = 0;
+  for (int64_t t = lmax / 2; t >= 1; t /= 2)
+    if (delta(keys, n, i, i + (l + t) * dir) > dmin) l += t;
+  int64_t j = i + l * dir;
+  int dnode = delta(keys, n, i, j);
+  int64_t s = 0;
+  for (int64_t div = 2;; div *= 2) {
+    int64_t t = (l + div - 1) / div;
+    if (delta(keys, n, i, i + (s + t) * dir) > dnode) s += t;
+    if (t == 1) break;
+  }
+  const int64_t split = i + s * dir + (dir < 0 ? -1 : 0);
+  const int64_t lo = i < j ? i : j, hi = i < j ? j : i;
+  int4* tail = reinterpret_cast<int4*>(&T.nodes[i].first);
+  *tail = make_int4((int32_t)lo, (int32_t)hi, 0, (int32_t)split);
+  T.flag[i] = 0;
+  T.parent[lo == split ? n - 1 + split : split] = (int32_t)(i << 1);
+  T.parent[hi == split + 1 ? n + split : split + 1] = (int32_t)(i << 1) | 1;
+}
+
+__global__ void __launch_bounds__(kBlock) k_internal(TreeView A, TreeView B) {
   pdl_entry();
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n - 1; i += grid_stride()) {
-    int dir = (delta(keys, n, i, i + 1) - delta(keys, n, i, i - 1)) >= 0 ? 1 : -1;
-    int dmin = delta(keys, n, i, i - dir);
-    int64_t lmax = 2;
-    while (delta(keys, n, i, i + lmax * dir) > dmin) lmax *= 2;
-    int64_t l = 0;
-    for (int64_t t = lmax / 2; t >= 1; t /= 2)
-      if (delta(keys, n, i, i + (l + t) * dir) > dmin) l += t;
-    int64_t j = i + l * dir;
-    int dnode = delta(keys, n, i, j);
-    int64_t s = 0;
-    for (int64_t div = 2;; div *= 2) {
-      int64_t t = (l + div - 1) / div;
-      if (delta(keys, n, i, i + (s + t) * dir) > dnode) s += t;
-      if (t == 1) break;
+  const int64_t nA = A.n > 1 ? A.n - 1 : 0, nB = B.n > 1 ? B.n - 1 : 0;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nA + nB; i += grid_stride()) {
+    if (i < nA) internal_node(A, i);
+    else internal_node(B, i - nA);
+  }
+}
+
+// Leaf records, and the treelets: the largest subtrees of at most kTreelet leaves (single leaves
+// directly under a larger node among them).  Their order in the list has no meaning.
+__device__ __forceinline__ void treelet_lists(const TreeView& T, PrimKind kind, const Topo& topo, int64_t wbase) {
+  const int lane = threadIdx.x & 31;
+  const int64_t n = T.n, i = wbase + lane;
+  bool is = false;
+  int4 en = make_int4(0, 0, -1, 0);
+  auto size_of = [&](int32_t node) { return T.nodes[node].last - T.nodes[node].first + 1; };
+  if (i < n) {                                    // leaf i
+    const int64_t p = T.prim[i];
+    if (kind == kTri) {
+      const int32_t v0 = topo.tris[3 * p];
+      T.leaf_info[i] = make_int4(v0, topo.tris[3 * p + 1], topo.tris[3 * p + 2], topo.fkin[p] | (topo.vgroup[v0] << 1));
+    } else {
+      const int32_t v0 = topo.edges[2 * p];
+      T.leaf_info[i] = make_int4(v0, topo.edges[2 * p + 1], -1, topo.ekin[p] | (topo.vgroup[v0] << 1));
     }
-    int64_t gamma = i + s * dir + (dir < 0 ? -1 : 0);
-    int64_t lo = i < j ? i : j, hi = i < j ? j : i;
-    int32_t c0 = (lo == gamma) ? ~(int32_t)gamma : (int32_t)gamma;
-    int32_t c1 = (hi == gamma + 1) ? ~(int32_t)(gamma + 1) : (int32_t)(gamma + 1);
-    nodes[i].c0 = c0;
-    nodes[i].c1 = c1;
-    nodes[i].split = (int32_t)gamma;   // last leaf position under child 0
-    range[i] = make_int2((int32_t)lo, (int32_t)hi);
-    parent[c0 >= 0 ? c0 : (n - 1 + ~c0)] = (int32_t)(i << 1);
-    parent[c1 >= 0 ? c1 : (n - 1 + ~c1)] = (int32_t)(i << 1) | 1;
+    const int32_t ps = n > 1 ? T.parent[n - 1 + i] : -1;
+    if (ps < 0 || size_of(ps >> 1) > kTreelet) {
+      is = true;
+      en = make_int4((int32_t)i, 1, ps, 0);
+    }
+  } else if (i < 2 * n - 1) {                     // internal node i - n
+    const int32_t node = (int32_t)(i - n);
+    const int32_t size = size_of(node);
+    if (size <= kTreelet) {
+      const int32_t ps = node == 0 ? -1 : T.parent[node];
+      if (ps < 0 || size_of(ps >> 1) > kTreelet) {
+        is = true;
+        en = make_int4(T.nodes[node].first, size, ps, 0);
+      }
+    }
+  }
+  const unsigned m = __ballot_sync(0xffffffffu, is);
+  if (m) {
+    int base = 0;
+    if (lane == 0) base = atomicAdd(T.n_treelets, __popc(m));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (is) T.treelet[base + __popc(m & ((1u << lane) - 1u))] = en;
   }
 }
 
-__device__ __forceinline__ uint8_t prim_kin(PrimKind kind, const Topo& T, int64_t p) {
-  return kind == kTri ? T.fkin[p] : (kind == kEdge ? T.ekin[p] : T.vkin[p]);
-}
-
-// The per-leaf records of a build, in leaf (Morton) order for the traversal: the primitive,
-// and its vertex ids with (kinematic flag | scene group << 1).  Returns the kinematic flag.
-__device__ __forceinline__ int write_leaf_record(PrimKind kind, const Topo& T, int32_t prim, int64_t l,
-                                                 int32_t* __restrict__ leaf_prim, int4* __restrict__ leaf_info) {
-  leaf_prim[l] = prim;
-  const int kin = prim_kin(kind, T, prim);
-  if (kind == kTri) {
-    const int32_t v0 = T.tris[3 * (int64_t)prim];
-    leaf_info[l] = make_int4(v0, T.tris[3 * (int64_t)prim + 1], T.tris[3 * (int64_t)prim + 2], kin | (T.vgroup[v0] << 1));
-  } else {
-    const int32_t v0 = T.edges[2 * (int64_t)prim];
-    leaf_info[l] = make_int4(v0, T.edges[2 * (int64_t)prim + 1], -1, kin | (T.vgroup[v0] << 1));
+__global__ void __launch_bounds__(kBlock) k_treelet_lists(TreeView A, TreeView B, Topo topo) {
+  pdl_entry();
+  // whole warps per tree
+  const int64_t nA = (2 * A.n + 30) / 32, nB = (2 * B.n + 30) / 32;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < nA + nB; w += nw) {
+    if (w < nA) treelet_lists(A, kTri, topo, 32 * w);
+    else treelet_lists(B, kEdge, topo, 32 * (w - nA));
   }
-  return kin;
-}
-
-template <bool first>
-__device__ __forceinline__ void write_child(BvhNode* nd, int slot, const float lo[3], const float hi[3], int kin) {
-  float* l = slot ? nd->lo1 : nd->lo0;
-  float* h = slot ? nd->hi1 : nd->hi0;
-  for (int k = 0; k < 3; ++k) { __stcg(&l[k], lo[k]); __stcg(&h[k], hi[k]); }
-  if (first && kin) atomicOr(&nd->kin, 1 << slot);
 }
 
 // Arrival counter of the bottom-up refit with release-acquire semantics at device scope:
 // the child box a thread stored before its increment is visible to the thread whose
-// increment comes second, which then reads both boxes.
-__device__ __forceinline__ int32_t arrive_acq_rel(int32_t* f) {
+// increment comes second, which then reads the sibling's box.  A refit brings two arrivals
+// to every node, so the counter's parity tells first from second and it is never reset.
+__device__ __forceinline__ bool arrive_first(int32_t* f) {
   int32_t old;
   asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(old) : "l"(f) : "memory");
-  return old;
+  return (old & 1) == 0;
 }
 
-template <bool fences>
-__device__ __forceinline__ int32_t arrive(int32_t* f) {
-  if (fences) {
-    __threadfence();
-    return atomicAdd(f, 1);
-  }
-  return arrive_acq_rel(f);
-}
-
-// leaf boxes in leaf order, for refitting an existing hierarchy; the leaf's vertex ids
-// come from its leaf record (coalesced) rather than the primitive tables
-// FP32 box of one leaf from the per-vertex boxes of its leaf record's vertex ids
-__device__ __forceinline__ void leaf_box_of(int4 li, const float* __restrict__ vbox, float lo[3], float hi[3]) {
-  verts_box(vbox, li.x, li.y, li.z, lo, hi);
-}
-
-__global__ void __launch_bounds__(kBlock) k_leaf_boxes(int64_t n, const int4* __restrict__ leaf_info,
-                                                       const float* __restrict__ vbox, float* __restrict__ leaf_box) {
+// Refit of both trees in two launches.  Leaves: one warp per treelet, a lane per leaf taking the
+// leaf's box from the per-vertex boxes and storing it, and six warp reductions giving the
+// treelet's box.  Nothing is kept below the treelets: the traversal reads their leaf boxes
+// directly.  Climb: a thread per treelet carries its box upward, the second child to arrive at a
+// node taking the union on; no thread waits on another.  (One kernel for both, lane 0 climbing,
+// took twice as long on the 256-scene batch: the climbs' round trips stood between a warp's
+// treelets.)  On a build (`first`) the kinematic bits climb with the boxes.  The first is bound by
+// memory (16 B record and 32 B box per leaf), the second by dependent L2 round trips.  256-scene
+// batch (10.5 M leaves): 211 + 150 us per refit, where treelets refitted node by node in shared
+// memory and the same climb took 533 + 224 us; bubble grasp 11 + 33 us, before 28 + 34 us.
+__global__ void __launch_bounds__(kBlock) k_refit_leaves(TreeView A, TreeView B, const float* __restrict__ vbox) {
   pdl_entry();
-  for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < n; l += grid_stride()) {
-    float lo[3], hi[3];
-    leaf_box_of(leaf_info[l], vbox, lo, hi);
-    float2* o = reinterpret_cast<float2*>(leaf_box + 6 * l);
-    o[0] = make_float2(lo[0], lo[1]);
-    o[1] = make_float2(lo[2], hi[0]);
-    o[2] = make_float2(hi[1], hi[2]);
-  }
-}
-
-// Bottom-up refit: the second child to finish a node unions both child boxes and
-// carries on upward; the first one stops.  No thread ever waits on another.  On a build
-// (`first`) it also writes the per-leaf records and the kinematic bits, which a refit of
-// the same hierarchy leaves as they are.  Leaf boxes are indexed by primitive on a build
-// (written by the Morton pass) and by leaf on a refit (k_leaf_boxes).
-template <bool first, bool fences>
-__global__ void __launch_bounds__(kBlock) k_refit(PrimKind kind, int64_t n, Topo T, const uint32_t* __restrict__ sorted,
-                                                  const float* __restrict__ leaf_box, BvhNode* nodes,
-                                                  const int32_t* __restrict__ parent, int32_t* leaf_prim,
-                                                  int4* __restrict__ leaf_info, int32_t* flag) {
-  pdl_entry();
-  for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < n; l += grid_stride()) {
-    int kin = 0;
-    float lo[3], hi[3];
-    if (first) {
-      const int32_t prim = (int32_t)sorted[l];
-      kin = write_leaf_record(kind, T, prim, l, leaf_prim, leaf_info);
-      for (int k = 0; k < 3; ++k) { lo[k] = leaf_box[6 * prim + k]; hi[k] = leaf_box[6 * prim + 3 + k]; }
-    } else {
-      const float2* b = reinterpret_cast<const float2*>(leaf_box + 6 * l);
-      const float2 a0 = b[0], a1 = b[1], a2 = b[2];
-      lo[0] = a0.x; lo[1] = a0.y; lo[2] = a1.x; hi[0] = a1.y; hi[1] = a2.x; hi[2] = a2.y;
-    }
-    if (n == 1) continue;
-    int32_t ps = parent[n - 1 + l];
-    int32_t node = ps >> 1;
-    write_child<first>(&nodes[node], ps & 1, lo, hi, kin);
-    int32_t up = node ? parent[node] : 0;       // fetched before the arrival, not after it
-    if (arrive<fences>(&flag[node]) == 0) continue;
-    for (int64_t step = 0; step < n; ++step) {   // a root path has at most n-1 nodes
-      if (fences) __threadfence();
-      const BvhNode* nd = &nodes[node];
-      for (int k = 0; k < 3; ++k) {
-        lo[k] = fminf(__ldcg(&nd->lo0[k]), __ldcg(&nd->lo1[k]));
-        hi[k] = fmaxf(__ldcg(&nd->hi0[k]), __ldcg(&nd->hi1[k]));
-      }
-      if (first) kin = (__ldcg(&nd->kin) & 3) == 3;
-      if (node == 0) break;
-      ps = up;
-      node = ps >> 1;
-      write_child<first>(&nodes[node], ps & 1, lo, hi, kin);
-      up = node ? parent[node] : 0;
-      if (arrive<fences>(&flag[node]) == 0) break;
-    }
-  }
-}
-
-// ---------------------------------------------------------------- two-phase refit
-// Every subtree covers a contiguous leaf range and its internal nodes carry indices inside
-// that range.  At build time the tree is cut into treelets: subtrees of at most kTreelet
-// leaves whose parent covers more.  A refit then (A) refits each treelet with one warp:
-// its leaf boxes, leaf parents and node links are loaded coalesced into shared memory and
-// the bottom-up union runs on shared-memory arrival counters, with no dependent global
-// loads; and (B) climbs from the treelet roots (and the few leaves hanging directly off
-// larger nodes) with the release-acquire counters.  Box unions are exact, so the boxes
-// are those of any other refit order.
-
-// On a build refitted by treelets (leaf_prim not null) it also writes the leaf records,
-// which both refit phases read.
-__global__ void __launch_bounds__(kBlock) k_treelet_lists(int64_t n, const int2* __restrict__ range,
-                                                          const int32_t* __restrict__ parent, int32_t* __restrict__ tl_root,
-                                                          int32_t* __restrict__ up_start, int32_t* __restrict__ count,
-                                                          PrimKind kind, Topo T, const uint32_t* __restrict__ sorted,
-                                                          int32_t* __restrict__ leaf_prim, int4* __restrict__ leaf_info) {
-  pdl_entry();
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < 2 * n - 1; i += grid_stride()) {
-    if (i < n - 1) {                              // internal node i
-      const int2 r = range[i];
-      const int64_t size = (int64_t)r.y - r.x + 1;
-      const int64_t psize = (i == 0) ? INT64_MAX : (int64_t)range[parent[i] >> 1].y - range[parent[i] >> 1].x + 1;
-      if (size <= kTreelet && psize > kTreelet) {
-        tl_root[atomicAdd(&count[0], 1)] = (int32_t)i;
-        up_start[atomicAdd(&count[1], 1)] = (int32_t)i;
-      }
-    } else {                                      // leaf l = i - (n - 1)
-      const int64_t l = i - (n - 1);
-      if (leaf_prim) write_leaf_record(kind, T, (int32_t)sorted[l], l, leaf_prim, leaf_info);
-      const int32_t p = parent[i] >> 1;
-      if ((int64_t)range[p].y - range[p].x + 1 > kTreelet) up_start[atomicAdd(&count[1], 1)] = ~(int32_t)l;
-    }
-  }
-}
-
-constexpr int kTreeletWarps = kBlock / 32;
-
-// What the two-phase refit needs of one tree; n <= 1 marks an absent tree.
-struct RefitView {
-  int64_t n;
-  const int32_t* tl_root;
-  const int32_t* up_start;
-  const int32_t* count;      // [2]: treelet roots, upper starts
-  const int2* range;
-  const int32_t* parent;
-  const int4* leaf_info;
-  BvhNode* nodes;
-  int32_t* flag;
-};
-
-__host__ __device__ __forceinline__ RefitView refit_view(const Bvh& t) {
-  return RefitView{t.n, t.tl_root, t.up_start, t.tl_count, t.range, t.parent, t.leaf_info, t.nodes, t.refit_flag};
-}
-
-// Phase A of the refit of up to two trees in one launch: one warp per treelet, lane l
-// computing leaf l's box from the positions and climbing in shared memory.  The grid also
-// clears both trees' arrival counters for phase B.  On a build (`first`) it also sets each
-// node's kinematic bits (bit s: every primitive under child s is kinematic), which a refit
-// leaves as they are.
-template <bool first>
-__global__ void __launch_bounds__(kBlock) k_treelet_refit(RefitView A, RefitView B, const float* __restrict__ vbox) {
-  pdl_entry();
-  __shared__ float sbox[kTreeletWarps][kTreelet][2][6];
-  __shared__ int scnt[kTreeletWarps][kTreelet];
-  __shared__ int spar[kTreeletWarps][kTreelet];
-  __shared__ int skin[kTreeletWarps][kTreelet];
-  const int nA = A.n > 1 ? (int)A.n : 0, nB = B.n > 1 ? (int)B.n : 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (int64_t)nA + nB; i += grid_stride()) {
-    if (i < nA) A.flag[i] = 0;
-    else B.flag[i - nA] = 0;
-  }
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  const int64_t nA = A.n > 0 ? *A.n_treelets : 0, nB = B.n > 0 ? *B.n_treelets : 0;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t ntA = nA ? A.count[0] : 0, ntB = nB ? B.count[0] : 0;
-  for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < ntA + ntB; w += nw) {
-    const bool inA = w < ntA;
-    const RefitView T = inA ? A : B;
-    const int64_t n = T.n;
-    const int32_t root = T.tl_root[inA ? w : w - ntA];
-    const int2 rg = T.range[root];
-    const int lo = rg.x, m = rg.y - rg.x + 1;           // m <= kTreelet leaves, m - 1 internal nodes
-    // parent links (parent << 1 | slot) of the indices lo .. hi (the treelet's internal
-    // nodes are among them)
-    if (lane < m && lo + lane < n - 1) spar[wib][lane] = T.parent[lo + lane];
-    scnt[wib][lane] = 0;
-    if (first) skin[wib][lane] = 0;
-    __syncwarp();
-    if (lane < m) {
-      const int32_t l = lo + lane;
-      float b[6];
-      const int4 li = T.leaf_info[l];
-      leaf_box_of(li, vbox, b, b + 3);
-      int kin = li.w & 1;
-      int32_t ps = T.parent[n - 1 + l];
-      for (int step = 0; step < kTreelet; ++step) {  // a treelet is at most kTreelet - 1 deep
-        const int32_t node = ps >> 1;
-        const int off = node - lo, slot = ps & 1;
-        if (off < 0 || off >= m) break;              // (a subtree's nodes lie in its leaf range)
-        float* dl = slot ? T.nodes[node].lo1 : T.nodes[node].lo0;
-        float* dh = slot ? T.nodes[node].hi1 : T.nodes[node].hi0;
-        for (int k = 0; k < 3; ++k) { __stcg(&dl[k], b[k]); __stcg(&dh[k], b[3 + k]); }
-        for (int k = 0; k < 6; ++k) sbox[wib][off][slot][k] = b[k];
-        if (first && kin) atomicOr(&skin[wib][off], 1 << slot);
-        __threadfence_block();
-        if (atomicAdd(&scnt[wib][off], 1) == 0) break;   // the sibling finishes this node
-        __threadfence_block();
-        for (int k = 0; k < 3; ++k) {
-          b[k] = fminf(sbox[wib][off][0][k], sbox[wib][off][1][k]);
-          b[3 + k] = fmaxf(sbox[wib][off][0][3 + k], sbox[wib][off][1][3 + k]);
-        }
-        if (first) {                                 // both children's bits are in
-          const int kb = skin[wib][off];
-          T.nodes[node].kin = kb;
-          kin = kb == 3;
-        }
-        if (node == root) break;                     // its box goes up in phase B
-        ps = spar[wib][off];
-      }
+  for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < nA + nB; w += nw) {
+    const bool inA = w < nA;
+    const int4 en = __ldg(inA ? A.treelet + w : B.treelet + (w - nA));
+    const int64_t l = en.x + (int64_t)lane;
+    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+    int kin = 1;
+    if (lane < en.y) {
+      const int4 li = __ldg((inA ? A.leaf_info : B.leaf_info) + l);
+      verts_box(vbox, li.x, li.y, li.z, lo, hi);
+      kin = li.w & 1;
+      float4* o = reinterpret_cast<float4*>((inA ? A.leaf_box : B.leaf_box) + 8 * l);
+      o[0] = make_float4(lo[0], lo[1], lo[2], hi[0]);
+      o[1] = make_float4(hi[1], hi[2], 0.f, 0.f);
     }
-    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 3; ++k) { lo[k] = warp_min(lo[k]); hi[k] = warp_max(hi[k]); }
+    kin = __all_sync(0xffffffffu, kin);
+    if (lane == 0) {
+      float4* o = reinterpret_cast<float4*>(inA ? A.treelet_box + 8 * w : B.treelet_box + 8 * (w - nA));
+      o[0] = make_float4(lo[0], lo[1], lo[2], hi[0]);
+      o[1] = make_float4(hi[1], hi[2], __int_as_float(kin), 0.f);
+    }
   }
 }
 
-// Phase B for up to two trees: one thread per upper start (a treelet root, or a leaf
-// directly under a larger node, its box from the positions) climbs with release-acquire
-// arrival counters; the two trees' climbs run side by side.  On a build (`first`) the
-// kinematic bits climb with the boxes.
 template <bool first>
-__global__ void __launch_bounds__(kBlock) k_upper_refit(RefitView A, RefitView B, const float* __restrict__ vbox) {
+__global__ void __launch_bounds__(kBlock) k_refit_climb(TreeView A, TreeView B) {
   pdl_entry();
-  const int64_t nuA = A.n > 1 ? A.count[1] : 0, nuB = B.n > 1 ? B.count[1] : 0;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nuA + nuB; k += grid_stride()) {
-    const bool inA = k < nuA;
-    const RefitView T = inA ? A : B;
-    const int64_t n = T.n;
-    const int32_t st = T.up_start[inA ? k : k - nuA];
-    float lo[3], hi[3];
-    int32_t ps;                                      // parent << 1 | slot of the climbing box
-    int kin = 0;                                     // (first) every primitive below is kinematic
-    if (st >= 0) {                                   // a treelet root: its box from its children
-      const BvhNode* nd = &T.nodes[st];
-      for (int q = 0; q < 3; ++q) {
-        lo[q] = fminf(__ldcg(&nd->lo0[q]), __ldcg(&nd->lo1[q]));
-        hi[q] = fmaxf(__ldcg(&nd->hi0[q]), __ldcg(&nd->hi1[q]));
-      }
-      if (first) kin = (__ldcg(&nd->kin) & 3) == 3;
-      if (st == 0) continue;                         // the whole tree was one treelet
-      ps = __ldg(T.parent + st);
-    } else {                                         // a leaf under a larger node
-      const int32_t l = ~st;
-      const int4 li = T.leaf_info[l];
-      leaf_box_of(li, vbox, lo, hi);
-      if (first) kin = li.w & 1;
-      ps = __ldg(T.parent + n - 1 + l);
-    }
-    // Per level: store this box into its slot, arrive, and (second arrival) take the union
-    // with the sibling's box.  The slot comes with the parent link, and the next link is
-    // fetched before the arrival, so the climb waits on the arrival and the sibling's box
-    // only.
+  const int64_t nA = A.n > 0 ? *A.n_treelets : 0, nB = B.n > 0 ? *B.n_treelets : 0;
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nA + nB; k += grid_stride()) {
+    const bool inA = k < nA;
+    int32_t ps = (inA ? A.treelet + k : B.treelet + (k - nA))->z;
+    if (ps < 0) continue;                            // the whole tree is this treelet
+    const float4* tb = reinterpret_cast<const float4*>(inA ? A.treelet_box + 8 * k : B.treelet_box + 8 * (k - nA));
+    const float4 t0 = __ldg(tb), t1 = __ldg(tb + 1);
+    float lo[3] = {t0.x, t0.y, t0.z}, hi[3] = {t0.w, t1.x, t1.y};
+    int kin = __float_as_int(t1.z);
+    BvhNode* nodes = inA ? A.nodes : B.nodes;
+    const int32_t* parent = inA ? A.parent : B.parent;
+    int32_t* flag = inA ? A.flag : B.flag;
+    const int64_t n = inA ? A.n : B.n;
     for (int64_t step = 0; step < n; ++step) {       // a root path has at most n-1 nodes
       const int32_t node = ps >> 1, slot = ps & 1;
-      BvhNode* nd = &T.nodes[node];
-      float* dl = slot ? nd->lo1 : nd->lo0;
-      float* dh = slot ? nd->hi1 : nd->hi0;
-      for (int q = 0; q < 3; ++q) { __stcg(&dl[q], lo[q]); __stcg(&dh[q], hi[q]); }
-      if (first && kin) atomicOr(&nd->kin, 1 << slot);
-      const int32_t up = node ? __ldg(T.parent + node) : 0;
-      if (arrive<false>(&T.flag[node]) == 0) break;
-      const float* sl = slot ? nd->lo0 : nd->lo1;
-      const float* sh = slot ? nd->hi0 : nd->hi1;
-      for (int q = 0; q < 3; ++q) {                // operands in slot order, as in the build
-        const float a = __ldcg(&sl[q]), b = __ldcg(&sh[q]);
-        lo[q] = slot ? fminf(a, lo[q]) : fminf(lo[q], a);
-        hi[q] = slot ? fmaxf(b, hi[q]) : fmaxf(hi[q], b);
-      }
-      if (first) kin = (__ldcg(&nd->kin) & 3) == 3;
+      float2* mine = reinterpret_cast<float2*>(nodes[node].box[slot]);
+      __stcg(mine, make_float2(lo[0], lo[1]));
+      __stcg(mine + 1, make_float2(lo[2], hi[0]));
+      __stcg(mine + 2, make_float2(hi[1], hi[2]));
+      if (first && kin) atomicOr(&nodes[node].kin, 1 << slot);
+      const int32_t up = node ? __ldg(parent + node) : 0;      // fetched before the arrival
+      if (arrive_first(&flag[node])) break;
+      const float2* sib = reinterpret_cast<const float2*>(nodes[node].box[slot ^ 1]);
+      const float2 a = __ldcg(sib), b = __ldcg(sib + 1), c = __ldcg(sib + 2);
+      lo[0] = fminf(lo[0], a.x); lo[1] = fminf(lo[1], a.y); lo[2] = fminf(lo[2], b.x);
+      hi[0] = fmaxf(hi[0], b.y); hi[1] = fmaxf(hi[1], c.x); hi[2] = fmaxf(hi[2], c.y);
+      if (first) kin = (__ldcg(&nodes[node].kin) & 3) == 3;
       if (node == 0) break;
       ps = up;
     }
@@ -453,256 +303,236 @@ __device__ __forceinline__ bool box_overlap(const float* lo, const float* hi, co
            qlo[2] > hi[2]);
 }
 
-__device__ __forceinline__ void emit(uint64_t key, uint64_t* cand, int64_t* n_cand, int64_t cap, DevStatus* st) {
-  uint32_t mask = __activemask();
-  int lane = threadIdx.x & 31;
-  int leader = __ffs(mask) - 1;
-  unsigned long long base = 0;
-  if (lane == leader) base = atomicAdd(reinterpret_cast<unsigned long long*>(n_cand), (unsigned long long)__popc(mask));
-  base = __shfl_sync(mask, base, leader);
-  int64_t pos = (int64_t)base + __popc(mask & ((1u << lane) - 1u));
-  if (pos < cap) {
-    cand[pos] = key;
-  } else {
-    raise_flag(st, EIPC_FLAG_CAND_OVERFLOW);
-    raise_need(st, &st->need_cand, pos + 1);
-  }
-}
+// ---------------------------------------------------------------- traversal
+// A warp answers 32 queries that are neighbours in Morton order.  (1) It walks the nodes above the
+// treelets once for all of them, depth first: the node is one 64-byte broadcast read, each lane
+// tests its own query against both children, and a child is followed if any lane meets it.  33
+// nodes per warp on the 256-scene batch, where a walk per query visited 31 and a warp of such
+// walks took 47 steps with 13 of 32 lanes active.  Stack and treelet list are spread over the
+// lanes' registers.  (2) Each treelet reached is tested a lane per leaf: its leaf boxes arrive in
+// one coalesced read, fetched one treelet ahead, and each query that met the treelet is compared
+// with all its leaves at once.  Candidates go to a buffer of the warp and out with one global
+// atomic per flush.  Contact
+// set of the bubble grasp: 180 us, with a walk per query 215 us.
+constexpr int kQueryBuf = 128;         // candidates; flushed when a treelet's 32 might not fit
 
-// Candidates found during one round of a warp's queries are appended to the warp's own
-// slice of shared memory (a shared-memory atomic per candidate) and written out when the
-// round ends: one global atomic per warp per round reserves their positions, and the
-// copy is coalesced.  A round's candidates beyond the slice's capacity go straight to
-// global memory through emit().  Without this, every leaf hit waited for a global
-// atomic's returned position.
-constexpr int kQueryWarpBuf = 256;
+struct QueryWarp {
+  float4 box[32][2];                   // lo xyz, hi x | hi yz, id, -
+  int4 info[32];                       // vertices a, b (PT: both the vertex), own leaf position, kin | group << 1
+  uint64_t cand[kQueryBuf];
+};
 
-__device__ __forceinline__ void flush_warp_candidates(uint64_t* buf, int* count, uint64_t* cand, int64_t* n_cand,
-                                                      int64_t cap, DevStatus* st, int lane) {
+__device__ __forceinline__ void flush_candidates(QueryWarp& W, int count, uint64_t* cand, int64_t* n_cand, int64_t cap,
+                                                 DevStatus* st, int lane) {
   __syncwarp();
-  int c = *count;
-  if (c > kQueryWarpBuf) c = kQueryWarpBuf;
-  if (c > 0) {
+  if (count > 0) {
     unsigned long long base = 0;
-    if (lane == 0) base = atomicAdd(reinterpret_cast<unsigned long long*>(n_cand), (unsigned long long)c);
+    if (lane == 0) base = atomicAdd(reinterpret_cast<unsigned long long*>(n_cand), (unsigned long long)count);
     base = __shfl_sync(0xffffffffu, base, 0);
-    for (int k = lane; k < c; k += 32) {
+    for (int k = lane; k < count; k += 32) {
       const int64_t pos = (int64_t)base + k;
-      if (pos < cap) cand[pos] = buf[k];
+      if (pos < cap) cand[pos] = W.cand[k];
     }
-    if (lane == 0 && (int64_t)base + c > cap) {
+    if (lane == 0 && (int64_t)base + count > cap) {
       raise_flag(st, EIPC_FLAG_CAND_OVERFLOW);
-      raise_need(st, &st->need_cand, (int64_t)base + c);
+      raise_need(st, &st->need_cand, (int64_t)base + count);
     }
   }
   __syncwarp();
-  if (lane == 0) *count = 0;
-  __syncwarp();
 }
 
-// One launch for both query sets: threads [0, nv) run vertex boxes against the triangle
-// tree (PT), threads [nv, nv + ne) run edge boxes against the edge tree (EE, j > i), the
-// edges in that tree's Morton order so neighbouring threads take similar paths.  A warp's
-// 32 lanes take rounds of 32 consecutive queries together (lanes past the end idle), so
-// the warp can write out its round's candidates at the round's end.  MINB is the minimum
-// number of 256-thread blocks per SM the register allocation must allow: the walk is
-// latency-bound (dependent node fetches), so more resident warps hide more of it; 4 leaves
-// the compiler free (48 registers), 6 caps it at 40 registers.  Dynamic shared memory:
-// kQueryWarpBuf 8-byte keys per warp.
-template <int MINB>
-__global__ void __launch_bounds__(256, MINB) k_query(Bvh tt, Bvh te, Topo T, const float* __restrict__ vbox_q,
-                                                     uint64_t* cand, int64_t* n_cand, int64_t cap, DevStatus* st) {
+__global__ void __launch_bounds__(256, 4) k_query(Bvh tt, Bvh te, Topo T, const uint32_t* __restrict__ vertex_order,
+                                               const float* __restrict__ vbox_q, uint64_t* cand, int64_t* n_cand,
+                                               int64_t cap, DevStatus* st) {
   pdl_entry();
-  extern __shared__ uint64_t qbuf[];
-  __shared__ int qcount[8];
-  const int64_t nq = (tt.n > 0 ? T.nv : 0) + (te.n > 0 ? T.ne : 0);
-  const int64_t nv_q = tt.n > 0 ? T.nv : 0;
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  uint64_t* wbuf = qbuf + (size_t)wib * kQueryWarpBuf;
-  int* wcount = qcount + wib;
-  if (lane == 0) *wcount = 0;
-  __syncwarp();
-  const int64_t wstride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t wbase = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); wbase < nq; wbase += wstride) {
-    const int64_t qi = wbase + lane;
-    if (qi < nq) {
-      const bool is_pt = qi < nv_q;
-      const Bvh& t = is_pt ? tt : te;
-      const PrimKind qkind = is_pt ? kVertex : kEdge;
-      const int64_t qpos = is_pt ? -1 : qi - nv_q;     // EE: the query's own leaf position
-      const int64_t q = is_pt ? qi : (int64_t)te.leaf_prim[qpos];
-      float qlo[3], qhi[3];
-      prim_box_v(qkind, q, T, vbox_q, qlo, qhi);
-      int32_t qa, qb;
-      if (is_pt) { qa = (int32_t)q; qb = (int32_t)q; }
-      else { qa = T.edges[2 * q]; qb = T.edges[2 * q + 1]; }
-      const bool qkin = prim_kin(qkind, T, q);
-      const int32_t qgroup = T.vgroup[qa];   // primitives of different scenes never pair
-      auto put = [&](uint64_t key) {
-        const int slot = atomicAdd(wcount, 1);
-        if (slot < kQueryWarpBuf) wbuf[slot] = key;
-        else emit(key, cand, n_cand, cap, st);
-      };
-      auto leaf = [&](int32_t lpos) {
-        const int4 info = __ldg(t.leaf_info + lpos);
-        if (is_pt) {
-          if (info.x == qa || info.y == qa || info.z == qa) return;
-          if ((qkin && (info.w & 1)) || (info.w >> 1) != qgroup) return;
-          const int32_t p = t.leaf_prim[lpos];
-          put(pair_key(0, (uint32_t)q, (uint32_t)p, T.bits_i, T.bits_j));
-        } else {
-          // each EE pair is found once, from the edge earlier in Morton order
-          if (lpos <= qpos) return;
-          if (info.x == qa || info.x == qb || info.y == qa || info.y == qb) return;
-          if ((qkin && (info.w & 1)) || (info.w >> 1) != qgroup) return;
-          const int32_t p = t.leaf_prim[lpos];
-          const uint32_t lo = (uint32_t)(p < q ? p : q), hi = (uint32_t)(p < q ? q : p);
-          put(pair_key(1, lo, hi, T.bits_i, T.bits_j));
+  extern __shared__ __align__(16) unsigned char query_smem[];
+  QueryWarp& W = reinterpret_cast<QueryWarp*>(query_smem)[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
+  const int64_t pt_warps = tt.n > 0 ? (T.nv + 31) / 32 : 0, ee_warps = te.n > 0 ? (T.ne + 31) / 32 : 0;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < pt_warps + ee_warps; w += nw) {
+    const bool pt = w < pt_warps;
+    const BvhNode* nodes = pt ? tt.nodes : te.nodes;
+    const float* leaf_box = pt ? tt.leaf_box : te.leaf_box;
+    const int4* leaf_info = pt ? tt.leaf_info : te.leaf_info;
+    const uint32_t* leaf_prim = pt ? tt.prim : te.prim;
+    const int32_t n_leaves = (int32_t)(pt ? tt.n : te.n);
+    const int64_t qi = 32 * (pt ? w : w - pt_warps) + lane;
+    // the lane's query; a lane past the end has an empty box
+    float qlo[3] = {INFINITY, INFINITY, INFINITY}, qhi[3] = {-INFINITY, -INFINITY, -INFINITY};
+    int32_t qpos = INT32_MAX;
+    bool kin = true;
+    if (qi < (pt ? T.nv : T.ne)) {
+      const int32_t id = (int32_t)(pt ? vertex_order[qi] : leaf_prim[qi]);
+      int32_t a = id, b = id;
+      if (pt) {
+        kin = T.vkin[id];
+        qpos = -1;
+      } else {
+        const int2 e = reinterpret_cast<const int2*>(T.edges)[id];
+        a = e.x; b = e.y;
+        kin = T.ekin[id];
+        qpos = (int32_t)qi;                // each EE pair is found once, from the edge earlier in Morton order
+      }
+      verts_box(vbox_q, a, pt ? -1 : b, -1, qlo, qhi);
+      W.info[lane] = make_int4(a, b, qpos, (kin ? 1 : 0) | (T.vgroup[a] << 1));
+      W.box[lane][0] = make_float4(qlo[0], qlo[1], qlo[2], qhi[0]);
+      W.box[lane][1] = make_float4(qhi[1], qhi[2], __int_as_float(id), 0.f);
+    }
+    __syncwarp();
+    int kept = 0;                            // candidates in the buffer (the same in all lanes)
+    int listed = 0, l_first = 0, l_count = 0;      // treelet t of the list is lane t's
+    unsigned l_mask = 0;
+    auto list = [&](int first, int count, unsigned mask) {
+      if (lane == listed) { l_first = first; l_count = count; l_mask = mask; }
+      ++listed;
+    };
+    // the listed treelets, their leaf boxes fetched one ahead
+    auto handle = [&]() {
+      float4 nb0 = make_float4(0.f, 0.f, 0.f, 0.f), nb1 = nb0;
+      int nfirst = __shfl_sync(0xffffffffu, l_first, 0), ncount = __shfl_sync(0xffffffffu, l_count, 0);
+      auto fetch = [&]() {
+        if (lane < ncount) {
+          const float4* p = reinterpret_cast<const float4*>(leaf_box + 8 * ((int64_t)nfirst + lane));
+          nb0 = __ldg(p);
+          nb1 = __ldg(p + 1);
         }
       };
-      if (t.n == 1) {
-        const float* b = t.leaf_box + 6 * (int64_t)t.leaf_prim[0];
-        if (box_overlap(b, b + 3, qlo, qhi)) leaf(0);
-      } else {
-        // Depth-first walk that descends into an overlapping child directly and pushes only
-        // the second child when both overlap, so a descent costs one node fetch and no stack
-        // round trip; leaves are handled where they are found.  The stack holds (node, last
-        // leaf position under it); EE queries skip subtrees that lie entirely at or before
-        // their own leaf.
-        int32_t stack[64], smax[64];
-        int sp = 0;
-        int32_t node = 0;
-        int32_t nmax = (int32_t)(t.n - 1);
-        // a tree of n leaves has n-1 internal nodes, each fetched at most once
-        int64_t visits = 0;
-        while (true) {
-          if (++visits > t.n) {
-            raise_flag(st, EIPC_FLAG_STACK_OVERFLOW);
-            break;
+      if (listed > 0) fetch();
+      for (int t = 0; t < listed; ++t) {
+        const float llo[3] = {nb0.x, nb0.y, nb0.z}, lhi[3] = {nb0.w, nb1.x, nb1.y};
+        const int32_t m = ncount, lpos = nfirst + lane;
+        unsigned mask = __shfl_sync(0xffffffffu, l_mask, t);
+        if (t + 1 < listed) {
+          nfirst = __shfl_sync(0xffffffffu, l_first, t + 1);
+          ncount = __shfl_sync(0xffffffffu, l_count, t + 1);
+          fetch();
+        }
+        int4 li = make_int4(0, 0, 0, 0);
+        bool loaded = false;
+        while (mask) {
+          const int q = __ffs(mask) - 1;
+          mask &= mask - 1;
+          const float4 q0 = W.box[q][0], q1 = W.box[q][1];
+          const float blo[3] = {q0.x, q0.y, q0.z}, bhi[3] = {q0.w, q1.x, q1.y};
+          const int4 qn = W.info[q];
+          bool hit = lane < m && lpos > qn.z && box_overlap(llo, lhi, blo, bhi);
+          if (!__any_sync(0xffffffffu, hit)) continue;
+          if (!loaded) {
+            loaded = true;
+            if (lane < m) li = __ldg(leaf_info + lpos);
           }
-          const float4* np = reinterpret_cast<const float4*>(&t.nodes[node]);
-          const float4 f0 = __ldg(np), f1 = __ldg(np + 1), f2 = __ldg(np + 2);
-          const int4 f3 = __ldg(reinterpret_cast<const int4*>(np + 3));
-          const float lo0[3] = {f0.x, f0.y, f0.z}, hi0[3] = {f0.w, f1.x, f1.y};
-          const float lo1[3] = {f1.z, f1.w, f2.x}, hi1[3] = {f2.y, f2.z, f2.w};
-          const int32_t c0 = f3.x, c1 = f3.y, kin = f3.z, split = f3.w;
-          bool o0 = box_overlap(lo0, hi0, qlo, qhi) && !(qkin && (kin & 1)) && (split > qpos);
-          bool o1 = box_overlap(lo1, hi1, qlo, qhi) && !(qkin && (kin & 2)) && (nmax > qpos);
-          if (o0 && c0 < 0) { leaf(~c0); o0 = false; }
-          if (o1 && c1 < 0) { leaf(~c1); o1 = false; }
-          if (o0) {
-            if (o1) {
-              if (sp < 64) { stack[sp] = c1; smax[sp++] = nmax; }
-              else raise_flag(st, EIPC_FLAG_STACK_OVERFLOW);
-            }
-            node = c0;
-            nmax = split;
-          } else if (o1) {
-            node = c1;
-          } else {
-            if (sp == 0) break;
-            --sp;
-            node = stack[sp];
-            nmax = smax[sp];
+          hit = hit && li.x != qn.x && li.y != qn.x && li.z != qn.x && li.x != qn.y && li.y != qn.y && li.z != qn.y &&
+                !(qn.w & li.w & 1) && (qn.w >> 1) == (li.w >> 1);
+          const unsigned mh = __ballot_sync(0xffffffffu, hit);
+          if (!mh) continue;
+          if (hit) {
+            const uint32_t id = (uint32_t)__float_as_int(q1.z), prim = __ldg(leaf_prim + lpos);
+            const uint32_t lo32 = pt ? id : (id < prim ? id : prim), hi32 = pt ? prim : (id < prim ? prim : id);
+            W.cand[kept + __popc(mh & below)] = pair_key(pt ? 0 : 1, lo32, hi32, T.bits_i, T.bits_j);
+          }
+          kept += __popc(mh);
+          if (kept > kQueryBuf - 32) {
+            flush_candidates(W, kept, cand, n_cand, cap, st, lane);
+            kept = 0;
           }
         }
       }
+      listed = 0;
+    };
+    if (n_leaves <= kTreelet) {
+      list(0, n_leaves, __ballot_sync(0xffffffffu, qpos != INT32_MAX));
+    } else {
+      int32_t node = 0, stack0 = 0, stack1 = 0;     // entries 0-31 and 32-63, one per lane
+      int held = 0;
+      int64_t visits = 0;                    // a tree of n leaves has n-1 internal nodes, each fetched at most once
+      while (true) {
+        if (++visits > n_leaves) {
+          if (lane == 0) raise_flag(st, EIPC_FLAG_STACK_OVERFLOW);
+          break;
+        }
+        const float4* np = reinterpret_cast<const float4*>(&nodes[node]);
+        const float4 f0 = __ldg(np), f1 = __ldg(np + 1), f2 = __ldg(np + 2);
+        const int4 tail = __ldg(reinterpret_cast<const int4*>(np + 3));      // first, last, kin, split
+        const float lo0[3] = {f0.x, f0.y, f0.z}, hi0[3] = {f0.w, f1.x, f1.y};
+        const float lo1[3] = {f1.z, f1.w, f2.x}, hi1[3] = {f2.y, f2.z, f2.w};
+        const unsigned m0 = __ballot_sync(0xffffffffu, box_overlap(lo0, hi0, qlo, qhi) && tail.w > qpos && !(kin && (tail.z & 1)));
+        const unsigned m1 = __ballot_sync(0xffffffffu, box_overlap(lo1, hi1, qlo, qhi) && tail.y > qpos && !(kin && (tail.z & 2)));
+        const int n0 = tail.w - tail.x + 1, n1 = tail.y - tail.w;
+        int32_t next = -1;
+        if (m0) {
+          if (n0 <= kTreelet) list(tail.x, n0, m0);
+          else next = tail.w;
+        }
+        if (m1) {
+          if (n1 <= kTreelet) {
+            list(tail.w + 1, n1, m1);
+          } else if (next < 0) {
+            next = tail.w + 1;
+          } else if (held < 64) {
+            if (lane == (held & 31)) {
+              if (held < 32) stack0 = tail.w + 1;
+              else stack1 = tail.w + 1;
+            }
+            ++held;
+          } else if (lane == 0) {
+            raise_flag(st, EIPC_FLAG_STACK_OVERFLOW);
+          }
+        }
+        if (listed > 30) handle();
+        if (next >= 0) {
+          node = next;
+        } else {
+          if (held == 0) break;
+          --held;
+          node = __shfl_sync(0xffffffffu, held < 32 ? stack0 : stack1, held & 31);
+        }
+      }
     }
-    flush_warp_candidates(wbuf, wcount, cand, n_cand, cap, st, lane);
+    handle();
+    flush_candidates(W, kept, cand, n_cand, cap, st, lane);
   }
+}
+
+TreeView view(const Bvh& t, const uint64_t* keys) {
+  return TreeView{t.n, keys, t.prim, t.nodes, t.parent, t.leaf_info, t.leaf_box, t.flag, t.treelet, t.treelet_box, t.n_treelets};
 }
 
 }  // namespace
 
-void bvh_build(Bvh& t, PrimKind kind, const Topo& topo, const double* x4, const double* dx4, const float* vbox,
-               int32_t* bounds_ws, uint32_t* sort_hist, cudaStream_t s, int refit_variant) {
-  if (t.n <= 0) return;
-  zero_ranges(s, {{t.nodes, sizeof(BvhNode) * (t.n > 1 ? t.n - 1 : 1)}, {t.refit_flag, sizeof(int32_t) * t.n},
-                  {t.n > 1 ? t.tl_count : nullptr, 2 * sizeof(int32_t)}});
-  launch(k_bounds_init, 1, 32, 0, s, bounds_ws);
-  launch(k_bounds, blocks_for(topo.nv, 4), kBlock, 0, s, x4, dx4, topo.nv, bounds_ws);
-  launch(k_leaves, blocks_for(t.n), kBlock, 0, s, kind, t.n, topo, vbox, static_cast<const int32_t*>(bounds_ws),
-         t.leaf_box, t.keys, t.vals);
-  int which = radix_sort_u64(t.keys, t.vals, t.keys_alt, t.vals_alt, t.n_dev, t.n, 30, sort_hist, s);
-  const uint64_t* sk = which ? t.keys_alt : t.keys;
-  const uint32_t* sv = which ? t.vals_alt : t.vals;
-  t.sorted = sv;
-  if (t.n > 1) launch(k_internal, blocks_for(t.n - 1), kBlock, 0, s, sk, t.n, t.nodes, t.parent, t.range);
-  if (refit_variant == 2 && t.n > 1) {
-    // the treelet lists first (with the leaf records), then both refit phases with the
-    // kinematic bits
-    launch(k_treelet_lists, blocks_for(2 * t.n), kBlock, 0, s, t.n, static_cast<const int2*>(t.range),
-           static_cast<const int32_t*>(t.parent), t.tl_root, t.up_start, t.tl_count, kind, topo, sv, t.leaf_prim,
-           t.leaf_info);
-    const RefitView A = refit_view(t);
-    const RefitView none{0, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-    launch(k_treelet_refit<true>, blocks_for(t.n, 8), kBlock, 0, s, A, none, vbox);
-    launch(k_upper_refit<true>, blocks_for(t.n), kBlock, 0, s, A, none, vbox);
-    t.built = true;
-    return;
-  }
-  if (refit_variant == 0)
-    launch(k_refit<true, true>, blocks_for(t.n), kBlock, 0, s, kind, t.n, topo, sv,
-           static_cast<const float*>(t.leaf_box), t.nodes, static_cast<const int32_t*>(t.parent), t.leaf_prim,
-           t.leaf_info, t.refit_flag);
-  else
-    launch(k_refit<true, false>, blocks_for(t.n), kBlock, 0, s, kind, t.n, topo, sv,
-           static_cast<const float*>(t.leaf_box), t.nodes, static_cast<const int32_t*>(t.parent), t.leaf_prim,
-           t.leaf_info, t.refit_flag);
-  if (t.n > 1) {
-    launch(k_treelet_lists, blocks_for(2 * t.n), kBlock, 0, s, t.n, static_cast<const int2*>(t.range),
-           static_cast<const int32_t*>(t.parent), t.tl_root, t.up_start, t.tl_count, kind, topo, sv,
-           static_cast<int32_t*>(nullptr), static_cast<int4*>(nullptr));
-  }
-  t.built = true;
+void bvh_build(Broad& b, const Topo& topo, const float* vbox, uint32_t* sort_hist, cudaStream_t s) {
+  const int64_t n = topo.nf + topo.ne + topo.nv;
+  launch(k_bounds_init, 1, 32, 0, s, b.bounds, b.tri.n_treelets, b.edge.n_treelets);
+  launch(k_bounds, blocks_for(topo.nv, 4), kBlock, 0, s, vbox, topo.nv, b.bounds);
+  launch(k_morton_keys, blocks_for(n), kBlock, 0, s, topo, vbox, static_cast<const int32_t*>(b.bounds), b.keys, b.vals);
+  const int which = radix_sort_u64(b.keys, b.vals, b.keys_alt, b.vals_alt, b.n_dev, n, 32, sort_hist, s);
+  const uint64_t* sk = which ? b.keys_alt : b.keys;
+  const uint32_t* sv = which ? b.vals_alt : b.vals;
+  b.tri.prim = sv;
+  b.edge.prim = sv + topo.nf;
+  b.vertex_order = sv + topo.nf + topo.ne;
+  const TreeView A = view(b.tri, sk), B = view(b.edge, sk + topo.nf);
+  launch(k_internal, blocks_for(topo.nf + topo.ne), kBlock, 0, s, A, B);
+  launch(k_treelet_lists, blocks_for(2 * (topo.nf + topo.ne)), kBlock, 0, s, A, B, topo);
+  launch(k_refit_leaves, blocks_for(topo.nf + topo.ne), kBlock, 0, s, A, B, vbox);
+  launch(k_refit_climb<true>, blocks_for((topo.nf + topo.ne) / 8), kBlock, 0, s, A, B);
+  b.built = true;
 }
 
-// both phases of the treelet refit for one or two trees (b may be null)
-static void treelet_refit(Bvh& a, Bvh* b, const float* vbox, cudaStream_t s) {
-  RefitView A = refit_view(a);
-  RefitView Bv = b ? refit_view(*b) : RefitView{0, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-  const int64_t n = a.n + (b ? b->n : 0);
-  launch(k_treelet_refit<false>, blocks_for(n, 8), kBlock, 0, s, A, Bv, vbox);
-  launch(k_upper_refit<false>, blocks_for(n), kBlock, 0, s, A, Bv, vbox);
+void bvh_refit(Broad& b, const float* vbox, cudaStream_t s) {
+  const TreeView A = view(b.tri, nullptr), B = view(b.edge, nullptr);
+  launch(k_refit_leaves, blocks_for(A.n + B.n), kBlock, 0, s, A, B, vbox);
+  launch(k_refit_climb<false>, blocks_for((A.n + B.n) / 8), kBlock, 0, s, A, B);
 }
 
-void bvh_refit_pair(Bvh& a, PrimKind ka, Bvh& b, PrimKind kb, const Topo& topo, const float* vbox, cudaStream_t s,
-                    int refit_variant) {
-  if (refit_variant == 2 && a.n > 1 && b.n > 1) {
-    treelet_refit(a, &b, vbox, s);
-    return;
-  }
-  bvh_refit(a, ka, topo, vbox, s, refit_variant);
-  bvh_refit(b, kb, topo, vbox, s, refit_variant);
-}
-
-void bvh_refit(Bvh& t, PrimKind kind, const Topo& topo, const float* vbox, cudaStream_t s, int refit_variant) {
-  if (t.n <= 0) return;
-  if (refit_variant == 2 && t.n > 1) {
-    treelet_refit(t, nullptr, vbox, s);
-    return;
-  }
-  launch(k_leaf_boxes, blocks_for(t.n), kBlock, 0, s, t.n, static_cast<const int4*>(t.leaf_info), vbox, t.leaf_box);
-  zero_ranges(s, {{t.refit_flag, sizeof(int32_t) * t.n}});
-  if (refit_variant == 0)
-    launch(k_refit<false, true>, blocks_for(t.n), kBlock, 0, s, kind, t.n, topo, t.sorted,
-           static_cast<const float*>(t.leaf_box), t.nodes, static_cast<const int32_t*>(t.parent), t.leaf_prim,
-           t.leaf_info, t.refit_flag);
-  else
-    launch(k_refit<false, false>, blocks_for(t.n), kBlock, 0, s, kind, t.n, topo, t.sorted,
-           static_cast<const float*>(t.leaf_box), t.nodes, static_cast<const int32_t*>(t.parent), t.leaf_prim,
-           t.leaf_info, t.refit_flag);
-}
-
-void bvh_query(const Bvh& tri, const Bvh& edge, const Topo& topo, const float* vbox_q, uint64_t* cand,
-               int64_t* n_cand, int64_t cap, DevStatus* st, cudaStream_t s, int threads, int bps, int variant) {
-  const int64_t nq = (tri.n > 0 ? topo.nv : 0) + (edge.n > 0 ? topo.ne : 0);
-  if (nq <= 0) return;
-  const size_t smem = (size_t)(threads / 32) * kQueryWarpBuf * sizeof(uint64_t);
-  if (variant == 3)
-    launch(k_query<6>, blocks_for(nq, bps, threads), threads, smem, s, tri, edge, topo, vbox_q, cand, n_cand, cap, st);
-  else
-    launch(k_query<4>, blocks_for(nq, bps, threads), threads, smem, s, tri, edge, topo, vbox_q, cand, n_cand, cap, st);
+void bvh_query(const Broad& b, const Topo& topo, const float* vbox_q, uint64_t* cand, int64_t* n_cand, int64_t cap,
+               DevStatus* st, cudaStream_t s, int threads, int bps) {
+  const int64_t warps = (b.tri.n > 0 ? (topo.nv + 31) / 32 : 0) + (b.edge.n > 0 ? (topo.ne + 31) / 32 : 0);
+  if (warps <= 0) return;
+  const size_t smem = (size_t)(threads / 32) * sizeof(QueryWarp);
+  launch(k_query, blocks_for(32 * warps, bps, threads), threads, smem, s, b.tri, b.edge, topo, b.vertex_order, vbox_q, cand,
+         n_cand, cap, st);
 }
 
 }  // namespace eipc

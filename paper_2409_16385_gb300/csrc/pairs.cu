@@ -422,22 +422,17 @@ void pairs_launch(eipc_scene* sc, const double* q, const eipc_params& p, const e
   // the triangle tree (PT) and edge boxes grown by dhat against the edge tree (EE, j > i)
   // full rebuild every `rebuild_interval` calls, refit of the same hierarchy in between (the
   // candidate set is exact for any hierarchy; only traversal cost depends on its quality)
-  const bool rebuild = !sc->tri_bvh.built || !sc->edge_bvh.built || sc->contact_refits + 1 >= sc->rebuild_interval;
+  const bool rebuild = !sc->broad.built || sc->contact_refits + 1 >= sc->rebuild_interval;
   if (rebuild) {
-    EIPC_TIMED(sc, kKBvh, s, bvh_build(sc->tri_bvh, kTri, sc->topo, sc->x4, nullptr, sc->vbox, sc->bounds_ws, sc->sort_hist, s,
-                                      sc->tune.refit_variant));
-    EIPC_TIMED(sc, kKBvh, s, bvh_build(sc->edge_bvh, kEdge, sc->topo, sc->x4, nullptr, sc->vbox, sc->bounds_ws, sc->sort_hist, s,
-                                      sc->tune.refit_variant));
+    EIPC_TIMED(sc, kKBvh, s, bvh_build(sc->broad, sc->topo, sc->vbox, sc->sort_hist, s));
     sc->contact_refits = 0;
   } else {
-    EIPC_TIMED(sc, kKBvh, s,
-               bvh_refit_pair(sc->tri_bvh, kTri, sc->edge_bvh, kEdge, sc->topo, sc->vbox, s, sc->tune.refit_variant));
+    EIPC_TIMED(sc, kKBvh, s, bvh_refit(sc->broad, sc->vbox, s));
     ++sc->contact_refits;
   }
   EIPC_TIMED(sc, kKQuery, s,
-             bvh_query(sc->tri_bvh, sc->edge_bvh, sc->topo, sc->vbox_pad, sc->cand, n_cand, sc->cand_cap,
-                       sc->status, s, sc->tune.query_threads, sc->tune.query_bps,
-                       sc->tune.query_variant));
+             bvh_query(sc->broad, sc->topo, sc->vbox_pad, sc->cand, n_cand, sc->cand_cap, sc->status, s,
+                       sc->tune.query_threads, sc->tune.query_bps));
   sc->timers->start(kKNarrow, s);
   launch(k_screen, blocks_for(sc->cand_cap, 16), kBlock, 0, s, sc->topo, static_cast<const float*>(sc->x4f),
          static_cast<const uint64_t*>(sc->cand),

@@ -34,8 +34,7 @@ struct eipc_scene {
   float* vbox;           // [nv*8] per-vertex FP32 boxes of the last call (contact or swept)
   float* vbox_pad;       // [nv*8] the contact ones grown by dhat (the query boxes)
   // broad phase
-  eipc::Bvh tri_bvh, edge_bvh;
-  int32_t* bounds_ws;
+  eipc::Broad broad;
   uint32_t* sort_hist;
   int64_t cand_cap;
   uint64_t* cand;
