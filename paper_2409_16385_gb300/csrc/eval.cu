@@ -411,6 +411,8 @@ struct EvalArgs {
   bool project;            // PSD-project the barrier Hessians (projected Newton)
   const double* moll_r2;   // EE mollifier: rest squared edge lengths (null: off)
   double moll_factor;      // eps_x = moll_factor |e_i|^2 |e_j|^2
+  uint32_t* moll_list;     // mollified pairs found by the factor kernel, their number
+  int64_t* n_moll;
   uint32_t* rest;          // items k_eval_factors leaves to k_eval_rest: pairs from the front, friction
                            // items from the back of item_cap entries
   int64_t* n_rest;         // [2] their numbers
@@ -777,54 +779,6 @@ __device__ __noinline__ void mollified_local(const V3* Y, const Stencil& S, doub
     }
 }
 
-// cyclic Jacobi on an N x N symmetric matrix in memory, then A <- V max(Lambda, 0) V^T
-__device__ __noinline__ void psd_project_mem(double* A, int N) {
-  double V[144];
-  for (int i = 0; i < N * N; ++i) V[i] = (i / N == i % N) ? 1.0 : 0.0;
-  double fro = 0.0;
-  for (int i = 0; i < N * N; ++i) fro += A[i] * A[i];
-  const double tol = 1e-28 * fro;
-  for (int sweep = 0; sweep < 30; ++sweep) {
-    double off = 0.0;
-    for (int p = 0; p < N; ++p)
-      for (int q = p + 1; q < N; ++q) off += A[p * N + q] * A[p * N + q];
-    if (off <= tol) break;
-    for (int p = 0; p < N; ++p)
-      for (int q = p + 1; q < N; ++q) {
-        const double apq = A[p * N + q];
-        if (apq == 0.0) continue;
-        const double theta = (A[q * N + q] - A[p * N + p]) / (2.0 * apq);
-        const double at = fabs(theta);
-        double t = at > 1e150 ? 0.5 / at : 1.0 / (at + sqrt(at * at + 1.0));
-        t = theta < 0.0 ? -t : t;
-        const double cs = rsqrt(t * t + 1.0), sn = t * cs;
-        for (int k = 0; k < N; ++k) {
-          const double akp = A[k * N + p], akq = A[k * N + q];
-          A[k * N + p] = cs * akp - sn * akq;
-          A[k * N + q] = sn * akp + cs * akq;
-        }
-        for (int k = 0; k < N; ++k) {
-          const double apk = A[p * N + k], aqk = A[q * N + k];
-          A[p * N + k] = cs * apk - sn * aqk;
-          A[q * N + k] = sn * apk + cs * aqk;
-        }
-        for (int k = 0; k < N; ++k) {
-          const double vkp = V[k * N + p], vkq = V[k * N + q];
-          V[k * N + p] = cs * vkp - sn * vkq;
-          V[k * N + q] = sn * vkp + cs * vkq;
-        }
-      }
-  }
-  double lam[12];
-  for (int e = 0; e < N; ++e) lam[e] = A[e * N + e] > 0.0 ? A[e * N + e] : 0.0;
-  for (int p = 0; p < N; ++p)
-    for (int q = 0; q < N; ++q) {
-      double acc = 0.0;
-      for (int e = 0; e < N; ++e) acc += V[p * N + e] * lam[e] * V[q * N + e];
-      A[p * N + q] = acc;
-    }
-}
-
 // weight of each stencil vertex on each of the item's cage nodes (0 for kinematic)
 __device__ __forceinline__ void vertex_node_weights(const int32_t v[4], const int32_t* __restrict__ cage_idx,
                                                     const double* __restrict__ w, const int32_t* nodes, int n,
@@ -894,6 +848,12 @@ __device__ __forceinline__ void store_row(double* row, V3 z1, V3 z2, double om, 
   p[1] = make_double2(z1.z, z2.x);
   p[2] = make_double2(z2.y, z2.z);
   p[3] = make_double2(om, wf);
+}
+
+// a mollified pair: its records come from k_mollified_eval
+__device__ __forceinline__ void list_mollified(const EvalArgs& A, int64_t k) {
+  store_header(A.ihead + kIHead * k, nullptr, V3{0.0, 0.0, 0.0}, 0.0, kItemExplicit);
+  A.moll_list[atomicAdd(reinterpret_cast<unsigned long long*>(A.n_moll), 1ull)] = (uint32_t)k;
 }
 
 // out[u] += coef * w over the four cage slots of vertex v (slot nodes in the nibbles of map);
@@ -1017,7 +977,7 @@ __device__ __forceinline__ void light_factors(const EvalArgs& A, int64_t k, int 
     const V3 Y[4] = {{0.0, 0.0, 0.0}, X[1] - X[0], X[2] - X[0], X[3] - X[0]};
     double eps_m, c_m;
     if (ee_mollified(A, type, i, j, Y, &eps_m, &c_m)) {           // k_mollified
-      store_header(A.ihead + kIHead * k, nullptr, V3{0.0, 0.0, 0.0}, 0.0, kItemExplicit);
+      list_mollified(A, k);
       return;
     }
   }
@@ -1149,7 +1109,7 @@ __device__ __forceinline__ void heavy_factors(const EvalArgs& A, int64_t k) {
   }
   double eps_m, c_m;
   if (active && ee_mollified(A, type, i, j, Y, &eps_m, &c_m)) {   // k_mollified
-    store_header(A.ihead + kIHead * k, nullptr, V3{0.0, 0.0, 0.0}, 0.0, kItemExplicit);
+    list_mollified(A, k);
     return;
   }
   const int n = A.item_n[k];
@@ -1382,6 +1342,262 @@ __global__ void __launch_bounds__(kEvalThreads, 2) k_eval_rest(EvalArgs A) {
   }
 }
 
+// Mollified EE pairs in the evaluation (the factor kernel lists them): explicit records.
+//
+// Nine lanes per pair, three pairs per warp.  The pair's Hessian vanishes on translations, so it
+// is taken in the nine directions u_i (x) e_k with the orthonormal u_1 = (1,-1,0,0)/sqrt 2,
+// u_2 = (0,0,1,-1)/sqrt 2, u_3 = (1,1,-1,-1)/2; lane j holds column j.  The projection is a cyclic
+// two-sided Jacobi in which each round's four disjoint rotations run at once (round r pairs i
+// and j with i + j = r mod 9): a lane fetches its partner's column by shuffles and every lane
+// applies the four row rotations to its own.  A rotation by any angle is exact, so the angle's
+// tangent is taken in FP32 (the entry left is 1e-7 of the one removed) and only c = 1/sqrt(1 +
+// t^2) in FP64.  One thread per pair, with its 12 x 12 matrices in local memory, kept 174 warps
+// busy with 70,000 FP64 instructions each: 4.2 ms for the 2.5k mollified pairs of two
+// 16 x 16-cell sheets.
+constexpr int kMollWarps = 2;
+struct MollShared {
+  double H[81];                // the (projected) Hessian, column-major
+  double HW[kMaxNodes][27];    // H times the node's weights: rows j, component k
+  double W[3][kMaxNodes];      // the nodes' weights in the basis u_1, u_2, u_3
+  double g[9];
+};
+
+__device__ __forceinline__ double shfl_d(double x, int src) { return __shfl_sync(0xffffffffu, x, src); }
+
+template <int N>
+__device__ __forceinline__ double select_d(const double (&x)[N], int k) {
+  double r = x[0];
+#pragma unroll
+  for (int i = 1; i < N; ++i)
+    if (k == i) r = x[i];
+  return r;
+}
+
+// one round of rotations on the columns T, V of lane `me` of the nine from lane `first` on
+template <int R>
+__device__ __forceinline__ void jacobi9_round(double (&T)[9], double (&V)[9], int me, int first) {
+  int other = R - me;
+  if (other < 0) other += 9;
+  const bool bye = other == me;
+  const bool low = me < other;
+  const int lp = first + (low ? me : other), lo = first + other;
+  const double dg = select_d(T, me), off = shfl_d(select_d(T, other), lp), dgo = shfl_d(dg, lo);
+  const double gap = low ? dgo - dg : dg - dgo;          // a_qq - a_pp
+  const float gf = (float)gap, of = (float)off;
+  float tf = 0.f;
+  if (fabsf(of) > 0.f) {
+    const float th = gf / (2.f * of), at = fabsf(th);
+    tf = at > 1e18f ? 0.5f / at : 1.f / (at + sqrtf(at * at + 1.f));
+    tf = th < 0.f ? -tf : tf;
+  }
+  if (bye) tf = 0.f;
+  const double t = (double)tf, c = rsqrt(fma(t, t, 1.0)), s = t * c, sg = low ? -s : s;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const double a = shfl_d(T[k], lo), b = shfl_d(V[k], lo);
+    T[k] = fma(c, T[k], bye ? 0.0 : sg * a);
+    V[k] = fma(c, V[k], bye ? 0.0 : sg * b);
+  }
+#pragma unroll
+  for (int p = 0; p < 9; ++p) {
+    const int q = (R - p + 9) % 9;
+    if (q <= p) continue;
+    const double cp = shfl_d(c, first + p), sp = shfl_d(s, first + p);
+    const double tp = T[p], tq = T[q];
+    T[p] = fma(cp, tp, -sp * tq);
+    T[q] = fma(cp, tq, sp * tp);
+  }
+}
+
+__global__ void __launch_bounds__(32 * kMollWarps) k_mollified_eval(EvalArgs A, const uint32_t* __restrict__ list,
+                                                                    const int64_t* n_list) {
+  pdl_entry();
+  __shared__ MollShared shared[kMollWarps][3];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const int grp = lane / 9 < 3 ? lane / 9 : 2, me = lane - 9 * (lane / 9), first = 9 * grp;
+  const bool live_lane = lane < 27;
+  MollShared& sh = shared[wib][grp];
+  const int64_t n_list_v = *n_list;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t w0 = 3 * (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); w0 < n_list_v; w0 += 3 * nw) {
+    // idle groups and lanes repeat the last pair's work without writing, so that the shuffles stay
+    // whole
+    const bool live = live_lane && w0 + grp < n_list_v;
+    const int64_t k = list[w0 + grp < n_list_v ? w0 + grp : n_list_v - 1];
+    const int m_e = me < 9 ? me : 8;
+    int32_t v[4];
+    const int32_t i = A.pr.i[k], j = A.pr.j[k];
+    stencil_vertices(A.T, 1, i, j, v);
+    V3 Y[4];
+    const V3 X0 = load_x(A.x4, v[0]);
+#pragma unroll
+    for (int a = 0; a < 4; ++a) Y[a] = load_x(A.x4, v[a]) - X0;
+    double eps, c;
+    ee_mollified(A, 1, i, j, Y, &eps, &c);
+    Stencil S;
+    closest_pair<true>(1, Y, stencil_hint(1, A.x4f, v), &S);
+    const double d = sqrt(S.d2);
+    BarrierSpan B;
+    barrier_span(Y, S, d, A.dhat, A.kappa, B);
+    const double ie = 1.0 / eps;
+    const double m = c * (2.0 * ie - c * ie * ie), m1 = 2.0 * ie - 2.0 * c * ie * ie, m2 = -2.0 * ie * ie;
+    const double kb = B.E;                               // kappa b
+    // the span's vectors in the basis u_1, u_2, u_3
+    const double r2 = 0.70710678118654752440;
+    double ub[3][3];                                     // [c^, a^_1, a^_2][u]
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      ub[q][0] = (B.basis[q][0] - B.basis[q][1]) * r2;
+      ub[q][1] = (B.basis[q][2] - B.basis[q][3]) * r2;
+      ub[q][2] = 0.5 * (B.basis[q][0] + B.basis[q][1] - B.basis[q][2] - B.basis[q][3]);
+    }
+    const V3 e0 = Y[1] - Y[0], e1 = Y[3] - Y[2];
+    const double s00 = dot(e0, e0), s11 = dot(e1, e1), s01 = dot(e0, e1);
+    const double E0[3] = {e0.x, e0.y, e0.z}, E1[3] = {e1.x, e1.y, e1.z};
+    const double rh[3] = {B.rh.x, B.rh.y, B.rh.z};
+    // gradients of c and of kappa b, component (u, k) at 3 u + k (e_0 = -sqrt 2 of the u_1 motion,
+    // e_1 of u_2)
+    double gc[9], gb[9];
+    const double gs = A.kappa * B.b1 * B.cn;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      gc[q] = -4.0 * r2 * (s11 * E0[q] - s01 * E1[q]);
+      gc[3 + q] = -4.0 * r2 * (s00 * E1[q] - s01 * E0[q]);
+      gc[6 + q] = 0.0;
+#pragma unroll
+      for (int u = 0; u < 3; ++u) gb[3 * u + q] = gs * ub[0][u] * rh[q];
+    }
+    // column me of m H_b + kb (m2 gc gc^T + m1 H_c) + m1 (gb gc^T + gc gb^T)
+    const int mu = m_e / 3, mk = m_e - 3 * mu;
+    const double cu = mu == 0 ? ub[0][0] : (mu == 1 ? ub[0][1] : ub[0][2]);
+    const double a1u = mu == 0 ? ub[1][0] : (mu == 1 ? ub[1][1] : ub[1][2]);
+    const double a2u = mu == 0 ? ub[2][0] : (mu == 1 ? ub[2][1] : ub[2][2]);
+    const double rk = select_d(rh, mk), gcm = select_d(gc, m_e), gbm = select_d(gb, m_e);
+    const double E0m = select_d(E0, mk), E1m = select_d(E1, mk);
+    double y[5];
+#pragma unroll
+    for (int p = 0; p < 5; ++p) {
+      const double kp = mk == 0 ? B.K[p][0] : (mk == 1 ? B.K[p][1] : B.K[p][2]);
+      y[p] = kp * cu + (B.K[p][3] * a1u + B.K[p][4] * a2u) * rk;
+    }
+    double T[9], V[9];
+#pragma unroll
+    for (int u = 0; u < 3; ++u) {
+      const double yr = ub[1][u] * y[3] + ub[2][u] * y[4];
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        double hc = 0.0;                                 // second derivatives of c, in (e_0, e_1)
+        const double dl = q == mk ? 1.0 : 0.0;
+        if (u < 2 && mu < 2) {
+          if (u == 0) hc = mu == 0 ? 2.0 * (s11 * dl - E1[q] * E1m) : 4.0 * E0[q] * E1m - 2.0 * E1[q] * E0m - 2.0 * s01 * dl;
+          else hc = mu == 1 ? 2.0 * (s00 * dl - E0[q] * E0m) : 4.0 * E1[q] * E0m - 2.0 * E0[q] * E1m - 2.0 * s01 * dl;
+          hc *= 2.0;
+        }
+        const int r = 3 * u + q;
+        const double hb = ub[0][u] * y[q] + rh[q] * yr;
+        T[r] = m * hb + kb * (m2 * gc[r] * gcm + m1 * hc) + m1 * (gb[r] * gcm + gc[r] * gbm);
+        V[r] = r == m_e ? 1.0 : 0.0;
+      }
+    }
+    if (A.project) {
+      double fro = 0.0;
+#pragma unroll
+      for (int r = 0; r < 9; ++r) fro += T[r] * T[r];
+      double tot = 0.0;
+#pragma unroll
+      for (int q = 0; q < 9; ++q) tot += shfl_d(fro, first + q);
+      const double tol = 1e-28 * tot;
+      for (int sweep = 0; sweep < 30; ++sweep) {
+        double off = 0.0;
+#pragma unroll
+        for (int r = 0; r < 9; ++r) off += r == m_e ? 0.0 : T[r] * T[r];
+        double all = 0.0;
+#pragma unroll
+        for (int q = 0; q < 9; ++q) all += shfl_d(off, first + q);
+        if (!__any_sync(0xffffffffu, 0.5 * all > tol)) break;
+        jacobi9_round<0>(T, V, m_e, first); jacobi9_round<1>(T, V, m_e, first); jacobi9_round<2>(T, V, m_e, first);
+        jacobi9_round<3>(T, V, m_e, first); jacobi9_round<4>(T, V, m_e, first); jacobi9_round<5>(T, V, m_e, first);
+        jacobi9_round<6>(T, V, m_e, first); jacobi9_round<7>(T, V, m_e, first); jacobi9_round<8>(T, V, m_e, first);
+      }
+      // column me of V max(Lambda, 0) V^T: sum over e of V[:, e] lambda_e V[me][e]
+      const double lam = select_d(T, m_e), lp = lam > 0.0 ? lam : 0.0;
+      __syncwarp();
+      if (live_lane) {
+#pragma unroll
+        for (int r = 0; r < 9; ++r) sh.H[9 * m_e + r] = V[r];
+        sh.g[m_e] = lp;
+      }
+      __syncwarp();
+#pragma unroll
+      for (int r = 0; r < 9; ++r) T[r] = 0.0;
+#pragma unroll
+      for (int q = 0; q < 9; ++q) {
+        const double s = sh.g[q] * sh.H[9 * q + m_e];
+#pragma unroll
+        for (int r = 0; r < 9; ++r) T[r] = fma(s, sh.H[9 * q + r], T[r]);
+      }
+    }
+    __syncwarp();
+    const int n = A.item_n[k];
+    const int32_t* nodes = A.item_nodes + kMaxNodes * k;
+    const uint64_t map = A.item_map[k];
+    if (live_lane) {
+#pragma unroll
+      for (int r = 0; r < 9; ++r) sh.H[9 * m_e + r] = T[r];
+      sh.g[m_e] = m * gbm + kb * m1 * gcm;
+      for (int u = m_e; u < n; u += 9) {
+        double wa[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          wa[a] = 0.0;
+          if (A.T.vkin[v[a]]) continue;
+          for (int q = 0; q < 4; ++q)
+            if ((int)((map >> (16 * a + 4 * q)) & 15u) == u) wa[a] += __ldg(A.w + 4 * (int64_t)v[a] + q);
+        }
+        sh.W[0][u] = (wa[0] - wa[1]) * r2;
+        sh.W[1][u] = (wa[2] - wa[3]) * r2;
+        sh.W[2][u] = 0.5 * (wa[0] + wa[1] - wa[2] - wa[3]);
+      }
+    }
+    __syncwarp();
+    if (live_lane) {
+      for (int u = 0; u < n; ++u)                        // row me of H times node u's weights
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+          sh.HW[u][3 * m_e + q] = sh.W[0][u] * sh.H[9 * q + m_e] + sh.W[1][u] * sh.H[9 * (3 + q) + m_e] +
+                                  sh.W[2][u] * sh.H[9 * (6 + q) + m_e];
+    }
+    __syncwarp();
+    if (live) {
+      if (m_e == 0) A.item_E[k] = m * kb;
+      const int64_t oh = A.ro_h[k];
+      const int nrec = n * (n + 1) / 2;
+      for (int l = m_e; l < nrec; l += 9) {
+        int u = 0, before = 0;
+        while (before + (n - u) <= l) { before += n - u; ++u; }
+        const int w2 = u + (l - before);
+        if (oh + l >= A.rec_cap) break;
+        double Bk[3][3];
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+#pragma unroll
+          for (int q = 0; q < 3; ++q)
+            Bk[p][q] = sh.W[0][u] * sh.HW[w2][3 * p + q] + sh.W[1][u] * sh.HW[w2][3 * (3 + p) + q] +
+                       sh.W[2][u] * sh.HW[w2][3 * (6 + p) + q];
+        if (w2 == u) {
+          double gr[3];                                  // the diagonal record carries the gradient at node u
+#pragma unroll
+          for (int q = 0; q < 3; ++q) gr[q] = sh.W[0][u] * sh.g[q] + sh.W[1][u] * sh.g[3 + q] + sh.W[2][u] * sh.g[6 + q];
+          emit_diag(A, oh + l, Bk, gr[0], gr[1], gr[2]);
+        } else {
+          emit_upper(A, oh + l, nodes[u], nodes[w2], Bk);
+        }
+      }
+    }
+    __syncwarp();
+  }
+}
+
 // ------------------------------------------------------------------ Hessian-vector product
 // y = H u for the unprojected contact Hessian H and the full-space direction u = J v on the
 // embedded vertices, u = kin_dir on the kinematic ones.  Each item emits one record per
@@ -1559,11 +1775,9 @@ __global__ void __launch_bounds__(kEvalThreads) k_hvp_friction(EvalArgs A, eipc_
   }
 }
 
-// Mollified EE pairs (the main kernels skip them): the full 12 x 12 path, one thread per
-// item, launched only when the mollifier is on.  The records go to the item's own offsets,
-// as for every other item.
-template <bool hvp>
-__global__ void __launch_bounds__(kEvalThreads) k_mollified(EvalArgs A) {
+// Mollified EE pairs of a Hessian-vector product (the main kernel skips them): the full 12 x 12
+// path, one thread per item, launched only when the mollifier is on.
+__global__ void __launch_bounds__(kEvalThreads) k_hvp_mollified(EvalArgs A) {
   pdl_entry();
   const int64_t P = clamp_count(A.pr.count, A.pr.capacity);
   const int64_t nit = *A.n_items;
@@ -1591,58 +1805,31 @@ __global__ void __launch_bounds__(kEvalThreads) k_mollified(EvalArgs A) {
     mollified_local(Y, S, d, A.dhat, A.kappa, eps_m, c_m, &Em, g12, H12);
     double W[4][kMaxNodes];
     vertex_node_weights(v, A.cage_idx, A.w, nodes, n, W);
-    if (hvp) {
-      double u12[12], y12[12];
-      bool kin = false;
-      for (int a = 0; a < 4; ++a) {
-        const bool ka = __ldg(A.cage_idx + 4 * (int64_t)v[a]) < 0;
-        kin |= ka;
-        V3 ua = ka ? kd : V3{0.0, 0.0, 0.0};
-        for (int u = 0; u < n; ++u) ua = ua + load_dir(A.hv_dir, nodes[u]) * W[a][u];
-        u12[3 * a] = ua.x; u12[3 * a + 1] = ua.y; u12[3 * a + 2] = ua.z;
-      }
-      for (int r = 0; r < 12; ++r) {
-        double acc = 0.0;
-        for (int q = 0; q < 12; ++q) acc += H12[12 * r + q] * u12[q];
-        y12[r] = acc;
-      }
-      for (int u = 0; u < n; ++u) {
-        V3 y = {0.0, 0.0, 0.0};
-        for (int a = 0; a < 4; ++a) y = y + V3{y12[3 * a], y12[3 * a + 1], y12[3 * a + 2]} * W[a][u];
-        emit_g(A, og + u, (uint64_t)nodes[u], y);
-      }
-      if (kin) {
-        V3 yk = {0.0, 0.0, 0.0};
-        for (int a = 0; a < 4; ++a)
-          if (__ldg(A.cage_idx + 4 * (int64_t)v[a]) < 0) yk = yk + V3{y12[3 * a], y12[3 * a + 1], y12[3 * a + 2]};
-        emit_g(A, og + n, (uint64_t)(A.ns + (k & (kKinSlots - 1))), yk);
-      }
-      continue;
+    double u12[12], y12[12];
+    bool kin = false;
+    for (int a = 0; a < 4; ++a) {
+      const bool ka = __ldg(A.cage_idx + 4 * (int64_t)v[a]) < 0;
+      kin |= ka;
+      V3 ua = ka ? kd : V3{0.0, 0.0, 0.0};
+      for (int u = 0; u < n; ++u) ua = ua + load_dir(A.hv_dir, nodes[u]) * W[a][u];
+      u12[3 * a] = ua.x; u12[3 * a + 1] = ua.y; u12[3 * a + 2] = ua.z;
     }
-    if (A.project) psd_project_mem(H12, 12);
-    A.item_E[k] = Em;
-    int64_t pos = A.ro_h[k];
-    for (int u = 0; u < n; ++u)
-      for (int w2 = u; w2 < n; ++w2, ++pos) {
-        if (pos >= A.rec_cap) continue;
-        double Bk[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-        for (int a = 0; a < 4; ++a)
-          for (int b = 0; b < 4; ++b) {
-            const double ww = W[a][u] * W[b][w2];
-            if (ww == 0.0) continue;
-            for (int p = 0; p < 3; ++p)
-              for (int q = 0; q < 3; ++q) Bk[p][q] += ww * H12[12 * (3 * a + p) + 3 * b + q];
-          }
-        if (w2 == u) {
-          // the diagonal record carries the gradient at node u
-          double y[3] = {0.0, 0.0, 0.0};
-          for (int a = 0; a < 4; ++a)
-            for (int c = 0; c < 3; ++c) y[c] += W[a][u] * g12[3 * a + c];
-          emit_diag(A, pos, Bk, y[0], y[1], y[2]);
-        } else {
-          emit_upper(A, pos, nodes[u], nodes[w2], Bk);
-        }
-      }
+    for (int r = 0; r < 12; ++r) {
+      double acc = 0.0;
+      for (int q = 0; q < 12; ++q) acc += H12[12 * r + q] * u12[q];
+      y12[r] = acc;
+    }
+    for (int u = 0; u < n; ++u) {
+      V3 y = {0.0, 0.0, 0.0};
+      for (int a = 0; a < 4; ++a) y = y + V3{y12[3 * a], y12[3 * a + 1], y12[3 * a + 2]} * W[a][u];
+      emit_g(A, og + u, (uint64_t)nodes[u], y);
+    }
+    if (kin) {
+      V3 yk = {0.0, 0.0, 0.0};
+      for (int a = 0; a < 4; ++a)
+        if (__ldg(A.cage_idx + 4 * (int64_t)v[a]) < 0) yk = yk + V3{y12[3 * a], y12[3 * a + 1], y12[3 * a + 2]};
+      emit_g(A, og + n, (uint64_t)(A.ns + (k & (kKinSlots - 1))), yk);
+    }
   }
 }
 
@@ -2101,9 +2288,10 @@ void eval_launch(eipc_scene* sc, const double* q, const eipc_pairs& pr, const ei
   int64_t* n_diag = cnt + 14;
   const int64_t item_cap = sc->item_cap;
   const int64_t pcap = pr.capacity < item_cap ? pr.capacity : item_cap;
+  int64_t* n_moll = sc->moll_factor > 0.0 ? cnt + kCntMollList : nullptr;
   // counters, the evaluation queue, g_r and the friction claims, all reset up front
   zero_ranges(s, {{cnt + kCntItems, 5 * sizeof(int64_t)}, {n_diag, sizeof(int64_t)},
-                  {cnt + kCntEvalQueue, sizeof(int64_t)}, {cnt + kCntEvalRest, 2 * sizeof(int64_t)}, {g_r, sizeof(double) * 3 * sc->ns},
+                  {cnt + kCntEvalQueue, sizeof(int64_t)}, {cnt + kCntEvalRest, 2 * sizeof(int64_t)}, {n_moll, sizeof(int64_t)}, {g_r, sizeof(double) * 3 * sc->ns},
                   {merge ? sc->fric_of_pair : nullptr, sizeof(int32_t) * pcap}});
   const int32_t* fop = merge ? sc->fric_of_pair : nullptr;
   const int32_t* pof = merge ? sc->pair_of_fric : nullptr;
@@ -2137,6 +2325,8 @@ void eval_launch(eipc_scene* sc, const double* q, const eipc_pairs& pr, const ei
   A.fric_of_pair = fop; A.pair_of_fric = pof;
   A.lag = fr ? *lag : eipc_lag{};
   A.mu = p.mu; A.eps_f = p.eps_v * p.h;
+  A.moll_list = sc->svals;                   // the pair-sort buffers are free once the pairs are built
+  A.n_moll = cnt + kCntMollList;
   A.rest = sc->svals_alt;                    // the pair-sort buffers are free once the pairs are built
   A.n_rest = cnt + kCntEvalRest;
   A.item_cap = item_cap;
@@ -2156,7 +2346,8 @@ void eval_launch(eipc_scene* sc, const double* q, const eipc_pairs& pr, const ei
                launch(k_eval_rest, 2 * kSMs, kEvalThreads, 0, sc->aux, A));
     if (A.moll_r2)
       EIPC_TIMED(sc, kKEvalBarrier, sc->aux,
-                 (launch(k_mollified<false>, blocks_for(pr.capacity, 8, kEvalThreads), kEvalThreads, 0, sc->aux, A)));
+                 (launch(k_mollified_eval, 8 * kSMs, 32 * kMollWarps, 0, sc->aux, A,
+                         static_cast<const uint32_t*>(A.moll_list), static_cast<const int64_t*>(A.n_moll))));
     sc->timers->stop(kKEvalPair, sc->aux);
   }
   cudaEventRecord(sc->ev_join, sc->aux);
@@ -2252,7 +2443,7 @@ void hvp_launch(eipc_scene* sc, const double* q, const eipc_pairs& pr, const eip
   EIPC_TIMED(sc, kKEvalBarrier, s,
              (launch(k_hvp_barrier, blocks_for(pr.capacity, 8, kEvalThreads), kEvalThreads, 0, s, A)));
   if (A.moll_r2)
-    EIPC_TIMED(sc, kKEvalBarrier, s, (launch(k_mollified<true>, blocks_for(pr.capacity, 8, kEvalThreads), kEvalThreads, 0, s, A)));
+    EIPC_TIMED(sc, kKEvalBarrier, s, (launch(k_hvp_mollified, blocks_for(pr.capacity, 8, kEvalThreads), kEvalThreads, 0, s, A)));
   if (fr)
     EIPC_TIMED(sc, kKEvalFriction, s,
                (launch(k_hvp_friction, blocks_for(lag->capacity, 8, kEvalThreads), kEvalThreads, 0, s, A, *lag, p.mu,

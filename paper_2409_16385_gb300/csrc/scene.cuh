@@ -116,7 +116,7 @@ constexpr int kFRow = 12, kIHead = 16;
 
 enum { kCntCand = 0, kCntSurv = 1, kCntItems = 2, kCntRecH = 3, kCntRecG = 4, kCntSegH = 5, kCntSegG = 6,
        kCntAccd = 7, kCntZero = 8, kCntEvalQueue = 16, kCntScreened = 15, kCntDedup = 17, kCntUnitsH = 18,
-       kCntMollBad = 20, kCntCcdQueue = 21, kCntCcdList = 22,
+       kCntMollBad = 20, kCntCcdQueue = 21, kCntCcdList = 22, kCntMollList = 23,
        kCntEvalRest = 24, /* two entries */
        kCntN = 26 };
 
