@@ -22,7 +22,7 @@ cudaError_t dalloc(T** p, int64_t n) {
 
 void free_scene(eipc_scene* s) {
   if (!s) return;
-  void* ptrs[] = {s->tris, s->edges, s->cage_idx, s->w, s->x_kin4, s->hvp_out, s->edge_key, s->edge_id, s->moll_r2, s->vkin, s->ekin, s->fkin, s->vgroup, s->group_alpha_bits, s->group_count, s->item_group, s->fric_of_pair, s->pair_of_fric, s->lag_key, s->x4, s->dx4, s->x4f, s->dx4f, s->vbox, s->vbox_pad, s->cand2,
+  void* ptrs[] = {s->tris, s->edges, s->cage_idx, s->w, s->x_kin4, s->inc_ptr, s->inc, s->hvp_part, s->edge_key, s->edge_id, s->moll_r2, s->vkin, s->ekin, s->fkin, s->vgroup, s->group_alpha_bits, s->group_count, s->item_group, s->fric_of_pair, s->pair_of_fric, s->lag_key, s->x4, s->dx4, s->x4f, s->dx4f, s->vbox, s->vbox_pad, s->cand2,
                   s->broad.tri.nodes, s->broad.tri.parent, s->broad.tri.leaf_info, s->broad.tri.leaf_box, s->broad.tri.flag,
                   s->broad.tri.treelet, s->broad.tri.n_treelets, s->broad.tri.treelet_box, s->broad.edge.treelet_box, s->broad.edge.nodes, s->broad.edge.parent,
                   s->broad.edge.leaf_info, s->broad.edge.leaf_box, s->broad.edge.flag, s->broad.edge.treelet,
@@ -31,8 +31,8 @@ void free_scene(eipc_scene* s) {
                   s->sort_hist, s->cand, s->counters, s->skeys, s->skeys_alt, s->svals, s->svals_alt, s->sd,
                   s->item_nodes, s->item_n, s->rc_h, s->ro_h, s->rc_g, s->ro_g, s->item_E, s->hkeys,
                   s->hkeys_alt, s->hvals, s->hvals_alt, s->hrec, s->seg_flag, s->seg_id, s->seg_start, s->rec_src, s->src_sorted, s->frow, s->ihead, s->item_map, s->piece, s->hunit,
-                  s->gkeys, s->gkeys_alt, s->gvals, s->gvals_alt, s->grec,
-                  s->gseg_start, s->scan_partial, s->sum_partial, s->status};
+                  s->gkeys, s->gkeys_alt, s->gvals, s->gvals_alt,
+                  s->scan_partial, s->sum_partial, s->status};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (s->timers) {
@@ -162,7 +162,7 @@ eipc_status eipc_scene_create(int64_t Nv, int64_t F, int64_t E, int64_t Ns, cons
   ok(dalloc(&s->rc_g, s->item_cap)); ok(dalloc(&s->ro_g, s->item_cap)); ok(dalloc(&s->item_E, s->item_cap));
   ok(dalloc(&s->hkeys, s->rec_cap)); ok(dalloc(&s->hkeys_alt, s->rec_cap));
   ok(dalloc(&s->hvals, s->rec_cap)); ok(dalloc(&s->hvals_alt, s->rec_cap));
-  ok(dalloc(&s->hvp_out, 3 * (Ns + 64)));
+  ok(dalloc(&s->inc_ptr, Ns + 2)); ok(dalloc(&s->inc, 4 * Nv)); ok(dalloc(&s->hvp_part, 3 * 64));
   ok(dalloc(&s->seg_flag, s->rec_cap)); ok(dalloc(&s->seg_id, s->rec_cap)); ok(dalloc(&s->seg_start, s->rec_cap));
   ok(dalloc(&s->rec_src, s->rec_cap)); ok(dalloc(&s->src_sorted, s->rec_cap));
   ok(dalloc(&s->frow, kFRow * s->gcap)); ok(dalloc(&s->ihead, kIHead * s->item_cap)); ok(dalloc(&s->item_map, s->item_cap));
@@ -172,8 +172,7 @@ eipc_status eipc_scene_create(int64_t Nv, int64_t F, int64_t E, int64_t Ns, cons
   }
   ok(dalloc(&s->hunit, s->rec_cap + 1));
   ok(dalloc(&s->gkeys, s->gcap)); ok(dalloc(&s->gkeys_alt, s->gcap));
-  ok(dalloc(&s->gvals, s->gcap)); ok(dalloc(&s->gvals_alt, s->gcap)); ok(dalloc(&s->grec, kGRecStride * s->gcap));
-  ok(dalloc(&s->gseg_start, s->gcap));
+  ok(dalloc(&s->gvals, s->gcap)); ok(dalloc(&s->gvals_alt, s->gcap));
   ok(dalloc(&s->edge_key, E > 0 ? E : 1)); ok(dalloc(&s->edge_id, E > 0 ? E : 1));
   ok(dalloc(&s->moll_r2, E > 0 ? E : 1));
   ok(dalloc(&s->scan_partial, 2 * (kScanBlocks + 1))); ok(dalloc(&s->sum_partial, kScanBlocks));
@@ -211,6 +210,7 @@ eipc_status eipc_scene_create(int64_t Nv, int64_t F, int64_t E, int64_t Ns, cons
       ok(cudaMemcpy(s->edge_id, ids.data(), sizeof(int32_t) * E, cudaMemcpyHostToDevice));
     }
   }
+  if (e == cudaSuccess) ok(incidence_build(s));
   ok(cudaMemset(s->counters, 0, sizeof(int64_t) * kCntN));
   ok(cudaMemset(s->status, 0, sizeof(DevStatus)));
   ok(cudaMemset(s->vgroup, 0, sizeof(int32_t) * Nv));

@@ -227,28 +227,6 @@ __global__ void __launch_bounds__(kBlock) k_item_nodes(Topo T, eipc_pairs pr, co
   }
 }
 
-// per-node weights of a stencil basis: out[u] = sum over (a, slot) with idx == node_u of
-// coef[a] * w[a][slot]
-__device__ __forceinline__ void node_weights(const int32_t v[4], const int32_t* __restrict__ cage_idx,
-                                             const double* __restrict__ w, const int32_t* nodes, int n,
-                                             const double coef[3][4], int ncoef, double out[kMaxNodes][3]) {
-  for (int u = 0; u < n; ++u)
-    for (int c = 0; c < 3; ++c) out[u][c] = 0.0;
-  for (int a = 0; a < 4; ++a) {
-    const int4 id = __ldg(reinterpret_cast<const int4*>(cage_idx) + v[a]);
-    if (id.x < 0) continue;
-    const int ids[4] = {id.x, id.y, id.z, id.w};
-    const double2 w01 = __ldg(reinterpret_cast<const double2*>(w) + 2 * (int64_t)v[a]);
-    const double2 w23 = __ldg(reinterpret_cast<const double2*>(w) + 2 * (int64_t)v[a] + 1);
-    const double ws[4] = {w01.x, w01.y, w23.x, w23.y};
-    for (int s = 0; s < 4; ++s) {
-      int u = 0;
-      while (u < n - 1 && nodes[u] != ids[s]) ++u;
-      for (int c = 0; c < ncoef; ++c) out[u][c] += coef[c][a] * ws[s];
-    }
-  }
-}
-
 // One Jacobi rotation J (c, s = t c in rows/columns p, q) of the symmetric A held in full,
 // A <- J^T A J, and V <- V J.  The entries outside rows and columns p, q are unchanged; the
 // (p, q) block takes the closed form of the rotation that zeroes a_pq (a_pp - t a_pq,
@@ -403,9 +381,6 @@ struct EvalArgs {
   const uint64_t* item_map;
   const float* x4f;
   double inv_dhat;
-  uint64_t* gkeys;
-  uint32_t* gvals;
-  double* grec;
   double* item_E;
   DevStatus* st;
   bool project;            // PSD-project the barrier Hessians (projected Newton)
@@ -419,8 +394,6 @@ struct EvalArgs {
   int64_t item_cap;
   int64_t* queue;          // next unclaimed item (work queue)
   int tile;                // items a warp claims from the queue at a time (multiple of 32)
-  const double* hv_dir;    // Hessian-vector product: reduced direction [ns*3]
-  double kin_dir[3];       // ... and the rigid direction of the kinematic vertices
   // friction merged into contact pairs (friction_merged; null: no merging); lag, mu and
   // eps_f are the friction parameters
   const int32_t* fric_of_pair;
@@ -581,14 +554,6 @@ __device__ __forceinline__ void emit_diag(const EvalArgs& A, int64_t pos, const 
   p[2] = make_double2(B[1][2], B[2][2]);
   p[3] = make_double2(g0, g1);
   A.hrec[kHRecStride * pos + 8] = g2;
-}
-
-// one keyed gradient record (Hessian-vector products)
-__device__ __forceinline__ void emit_grad(const EvalArgs& A, int64_t pos, uint64_t key, double y0, double y1, double y2) {
-  A.gkeys[pos] = key;
-  A.gvals[pos] = (uint32_t)pos;
-  *reinterpret_cast<double2*>(A.grec + kGRecStride * pos) = make_double2(y0, y1);
-  A.grec[kGRecStride * pos + 2] = y2;
 }
 
 // The barrier Hessian of one active pair in its span (Sec. III-B, Eq. 7; the 12 x 12
@@ -779,23 +744,6 @@ __device__ __noinline__ void mollified_local(const V3* Y, const Stencil& S, doub
     }
 }
 
-// weight of each stencil vertex on each of the item's cage nodes (0 for kinematic)
-__device__ __forceinline__ void vertex_node_weights(const int32_t v[4], const int32_t* __restrict__ cage_idx,
-                                                    const double* __restrict__ w, const int32_t* nodes, int n,
-                                                    double W[4][kMaxNodes]) {
-  for (int a = 0; a < 4; ++a) {
-    for (int u = 0; u < n; ++u) W[a][u] = 0.0;
-    const int4 id = __ldg(reinterpret_cast<const int4*>(cage_idx) + v[a]);
-    if (id.x < 0) continue;
-    const int ids[4] = {id.x, id.y, id.z, id.w};
-    for (int s2 = 0; s2 < 4; ++s2) {
-      int u = 0;
-      while (u < n - 1 && nodes[u] != ids[s2]) ++u;
-      W[a][u] += __ldg(w + 4 * (int64_t)v[a] + s2);
-    }
-  }
-}
-
 // ------------------------------------------------------------------ pair factors
 // The FP64 pipe bounds this stage (an FP64 warp instruction holds it for 64 cycles), so the
 // blocks J^T (pair Hessian) J are never formed pair by pair.  Each item leaves one row per cage
@@ -932,14 +880,18 @@ __device__ __forceinline__ double negative_root(double A, double B, double w0, d
   return xd;
 }
 
-// Node rows and header of a pair whose closest features are one of the segments of `hint`
-// (closest_hint without kHintInterior).
-__device__ __forceinline__ void light_factors(const EvalArgs& A, int64_t k, int type, int32_t i, int32_t j, const int32_t v[4],
-                                              int hint) {
-  V3 X[4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a) X[a] = load_x(A.x4, v[a]);
-  // the segment: the only one left, or (ties, e.g. at a shared vertex) the closest in FP64
+// The closest segment of a pair among those of `hint` (closest_hint without kHintInterior): point
+// slot ip against edge (ia, ib), e = x_b - x_a, parameter t in [0, 1] (inner: strictly inside),
+// r = x_p - x_a - t e, rse = 1/|e| (inner only).
+struct SegmentPair {
+  int ip, ia, ib;
+  bool inner;
+  double t, rse;
+  V3 e, r;
+};
+
+__device__ __forceinline__ SegmentPair closest_segment(int type, const V3 X[4], int hint) {
+  // the only one left, or (ties, e.g. at a shared vertex) the closest in FP64
   int seg = __ffs(hint & 15) - 1;
   if (hint & (hint - 1) & 15) {
     double best = 0.0, t;
@@ -954,19 +906,36 @@ __device__ __forceinline__ void light_factors(const EvalArgs& A, int64_t k, int 
       if (seg < 0 || lt_nonneg(d2, best)) { best = d2; seg = q; }
     }
   }
-  int ip, ia, ib;
-  segment_slots(type, seg, &ip, &ia, &ib);
-  const V3 xa = pick(X, ia), e = pick(X, ib) - xa, w = pick(X, ip) - xa;
-  const double we = dot(w, e), ee = dot(e, e);
-  double t = 0.0, rse = 0.0;
-  const bool inner = is_pos(we) && lt_nonneg(we, ee);
-  if (inner) {
-    rse = rsqrt(ee);
-    t = we * (rse * rse);
+  SegmentPair G;
+  segment_slots(type, seg, &G.ip, &G.ia, &G.ib);
+  const V3 xa = pick(X, G.ia), w = pick(X, G.ip) - xa;
+  G.e = pick(X, G.ib) - xa;
+  const double we = dot(w, G.e), ee = dot(G.e, G.e);
+  G.t = 0.0;
+  G.rse = 0.0;
+  G.inner = is_pos(we) && lt_nonneg(we, ee);
+  if (G.inner) {
+    G.rse = rsqrt(ee);
+    G.t = we * (G.rse * G.rse);
   } else if (is_pos(we)) {
-    t = 1.0;
+    G.t = 1.0;
   }
-  const V3 r = w - e * t;
+  G.r = w - G.e * G.t;
+  return G;
+}
+
+// Node rows and header of a pair whose closest features are one of the segments of `hint`
+// (closest_hint without kHintInterior).
+__device__ __forceinline__ void light_factors(const EvalArgs& A, int64_t k, int type, int32_t i, int32_t j, const int32_t v[4],
+                                              int hint) {
+  V3 X[4];
+#pragma unroll
+  for (int a = 0; a < 4; ++a) X[a] = load_x(A.x4, v[a]);
+  const SegmentPair Sg = closest_segment(type, X, hint);
+  const int ip = Sg.ip, ia = Sg.ia, ib = Sg.ib;
+  const bool inner = Sg.inner;
+  const double t = Sg.t, rse = Sg.rse;
+  const V3 e = Sg.e, r = Sg.r;
   const double d2 = dot(r, r);
   const bool apart = d2 > 0.0;
   if (!apart) raise_flag(A.st, EIPC_FLAG_PENETRATION);
@@ -976,7 +945,7 @@ __device__ __forceinline__ void light_factors(const EvalArgs& A, int64_t k, int 
   if (active && A.moll_r2 && type == 1) {
     const V3 Y[4] = {{0.0, 0.0, 0.0}, X[1] - X[0], X[2] - X[0], X[3] - X[0]};
     double eps_m, c_m;
-    if (ee_mollified(A, type, i, j, Y, &eps_m, &c_m)) {           // k_mollified
+    if (ee_mollified(A, type, i, j, Y, &eps_m, &c_m)) {           // k_mollified_eval
       list_mollified(A, k);
       return;
     }
@@ -1059,7 +1028,7 @@ __device__ __forceinline__ void light_factors(const EvalArgs& A, int64_t k, int 
       add_slots2(A, pick(v, ia), (uint32_t)(map >> (16 * ia)) & 0xffffu, -s1, om, 1.0, al);
       add_slots2(A, pick(v, ib), (uint32_t)(map >> (16 * ib)) & 0xffffu, -t, om, -1.0, al);
     } else {
-      const int iq = is_pos(we) ? ib : ia;
+      const int iq = is_pos(t) ? ib : ia;
       add_slots(A, pick(v, iq), (uint32_t)(map >> (16 * iq)) & 0xffffu, -1.0, om);
     }
   }
@@ -1598,237 +1567,417 @@ __global__ void __launch_bounds__(32 * kMollWarps) k_mollified_eval(EvalArgs A, 
   }
 }
 
+// sums over a warp by a fixed shuffle tree (the result in lane 0)
+template <int W>
+__device__ __forceinline__ void warp_tree_sum(double acc[W]) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int c = 0; c < W; ++c) acc[c] += __shfl_down_sync(0xffffffffu, acc[c], o);
+}
+
 // ------------------------------------------------------------------ Hessian-vector product
-// y = H u for the unprojected contact Hessian H and the full-space direction u = J v on the
-// embedded vertices, u = kin_dir on the kinematic ones.  Each item emits one record per
-// cage node of its stencil (J^T y restricted to the item) and, if it touches kinematic
-// vertices, one record holding the sum of y over them under key ns + (item mod 64); the
-// gradient reduction sums the records, and the 64 kinematic partials are added in order.
-constexpr int kKinSlots = 64;
-
-__device__ __forceinline__ bool item_has_kinematic(const Topo& T, const eipc_pairs& pr, int64_t P, const int32_t* lag_v,
-                                                   int64_t L, int64_t k, const int32_t* __restrict__ cage_idx) {
-  int32_t v[4];
-  item_vertices(T, pr, P, lag_v, L, k, v);
-  bool any = false;
-  for (int a = 0; a < 4; ++a) any |= __ldg(cage_idx + 4 * (int64_t)v[a]) < 0;
-  return any;
-}
-
-__global__ void k_hvp_counts(Topo T, eipc_pairs pr, const int32_t* lag_v, const int64_t* lag_count, int64_t lag_cap,
-                             const int32_t* __restrict__ cage_idx, const int32_t* __restrict__ item_n,
-                             const int64_t* n_items, int64_t cap, int64_t* __restrict__ rc_g) {
-  pdl_entry();
-  const int64_t n = clamp_count(n_items, cap);
-  const int64_t P = clamp_count(pr.count, pr.capacity);
-  const int64_t L = lag_v ? clamp_count(lag_count, lag_cap) : 0;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += grid_stride())
-    rc_g[k] = (int64_t)item_n[k] + (item_has_kinematic(T, pr, P, lag_v, L, k, cage_idx) ? 1 : 0);
-}
-
-__global__ void k_hvp_kin_sum(const double* __restrict__ rows, double* __restrict__ out_kin) {
-  pdl_entry();
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double a[3] = {0.0, 0.0, 0.0};
-    for (int s = 0; s < kKinSlots; ++s)
-      for (int c = 0; c < 3; ++c) a[c] += rows[3 * s + c];
-    for (int c = 0; c < 3; ++c) out_kin[c] = a[c];
-  }
-}
-
-// coefficient sums over the kinematic vertices of a stencil
-__device__ __forceinline__ void kinematic_sums(const int32_t v[4], const int32_t* __restrict__ cage_idx,
-                                               const double coef[3][4], int ncoef, double out[3]) {
-  for (int c = 0; c < 3; ++c) out[c] = 0.0;
-  for (int a = 0; a < 4; ++a) {
-    if (__ldg(cage_idx + 4 * (int64_t)v[a]) >= 0) continue;
-    for (int c = 0; c < ncoef; ++c) out[c] += coef[c][a];
-  }
-}
+// out = J^T H u for the unprojected contact Hessian H and the full-space direction u = J v on the
+// embedded vertices, u = kin_dir on the kinematic ones (Sec. III-D, Eq. 17).
+//
+// Each item's y = H_k u is twelve numbers on its four vertices, in closed form (no 12 x 12 matrix,
+// no eigensolve, about 110 FP64 instructions); they are added per vertex, and J^T is applied once
+// per vertex instead of once per item and cage node.  The sum over items has to be the same bits
+// on every run without sorting records: every vertex keeps the largest exponent E among its
+// contributions (an integer maximum), and each contribution is added to the vertex as a fixed-point
+// number of 80 bits below 2^(E+1), in two 64-bit integers of 40 bits each (headroom for 2^22
+// items).  Integer sums do not depend on their order, and 80 bits lose less than adding in FP64.
+// The sums then become doubles where the static lists of each node's vertices gather them, a
+// warp per node in a fixed order.  Before: 1.24 M keyed records of the bubble grasp written,
+// radix-sorted and summed, 23 launches, 443 us; now 6 launches, 162 us.
+constexpr int kKinSlots = 64;          // partial sums over the kinematic vertices
+constexpr int kFix = 34;               // bits per fixed-point limb
 
 __device__ __forceinline__ V3 load_dir(const double* __restrict__ v, int32_t node) {
   return {v[3 * (int64_t)node], v[3 * (int64_t)node + 1], v[3 * (int64_t)node + 2]};
 }
 
-__device__ __forceinline__ void emit_g(const EvalArgs& A, int64_t pos, uint64_t key, V3 y) {
-  if (pos >= A.gcap) return;
-  emit_grad(A, pos, key, y.x, y.y, y.z);
+// u = J v (kin on the kinematic vertices), padded, and the vertices' sums reset
+__global__ void __launch_bounds__(kBlock) k_hvp_direction(int64_t nv, const int32_t* __restrict__ idx,
+                                                          const double* __restrict__ w, const double* __restrict__ dir,
+                                                          V3 kin, double* __restrict__ u4, int32_t* __restrict__ vexp,
+                                                          unsigned long long* __restrict__ hi, unsigned long long* __restrict__ lo,
+                                                          CounterList zero) {
+  pdl_entry();
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+#pragma unroll
+    for (int c = 0; c < kCounterList; ++c)
+      if (zero.p[c]) *zero.p[c] = 0;
+  }
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < nv; v += grid_stride()) {
+    const int4 id = __ldg(reinterpret_cast<const int4*>(idx) + v);
+    V3 r = kin;
+    if (id.x >= 0) {
+      const double2 w01 = __ldg(reinterpret_cast<const double2*>(w) + 2 * v);
+      const double2 w23 = __ldg(reinterpret_cast<const double2*>(w) + 2 * v + 1);
+      r = load_dir(dir, id.x) * w01.x + load_dir(dir, id.y) * w01.y + load_dir(dir, id.z) * w23.x + load_dir(dir, id.w) * w23.y;
+    }
+    reinterpret_cast<double2*>(u4)[2 * v] = make_double2(r.x, r.y);
+    reinterpret_cast<double2*>(u4)[2 * v + 1] = make_double2(r.z, 0.0);
+    vexp[v] = 0;
+    reinterpret_cast<ulonglong2*>(hi)[2 * v] = make_ulonglong2(0, 0);
+    reinterpret_cast<ulonglong2*>(hi)[2 * v + 1] = make_ulonglong2(0, 0);
+    reinterpret_cast<ulonglong2*>(lo)[2 * v] = make_ulonglong2(0, 0);
+    reinterpret_cast<ulonglong2*>(lo)[2 * v + 1] = make_ulonglong2(0, 0);
+  }
 }
 
-__global__ void __launch_bounds__(kEvalThreads) k_hvp_barrier(EvalArgs A) {
-  pdl_entry();
-  const int64_t P = clamp_count(A.pr.count, A.pr.capacity);
-  const int64_t nit = *A.n_items;
-  const int64_t np = P < nit ? P : nit;
-  const V3 kd = {A.kin_dir[0], A.kin_dir[1], A.kin_dir[2]};
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < np; k += grid_stride()) {
-    int32_t v[4];
-    const int type = A.pr.type[k];
-    stencil_vertices(A.T, type, A.pr.i[k], A.pr.j[k], v);
-    V3 Y[4];
-    const V3 X0 = load_x(A.x4, v[0]);
-    for (int a = 0; a < 4; ++a) Y[a] = load_x(A.x4, v[a]) - X0;
-    Stencil S;
-    if (type == 0) pt_distance<true>(Y[0], Y[1], Y[2], Y[3], &S);
-    else ee_distance<true>(Y[0], Y[1], Y[2], Y[3], &S);
-    const int n = A.item_n[k];
-    const int32_t* nodes = A.item_nodes + kMaxNodes * k;
-    const int64_t og = A.ro_g[k];
-    bool active = false;
-    double t[5] = {0, 0, 0, 0, 0};
-    double nw[kMaxNodes][3];
-    double ks[3] = {0, 0, 0};
-    V3 rh = {0.0, 0.0, 0.0};
-    if (!(S.d2 > 0.0)) {
-      raise_flag(A.st, EIPC_FLAG_PENETRATION);
-    } else {
-      const double d = sqrt(S.d2);
-      active = d < A.dhat;
-      double eps_m, c_m;
-      if (active && ee_mollified(A, type, A.pr.i[k], A.pr.j[k], Y, &eps_m, &c_m)) continue;   // k_hvp_mollified
-      if (active) {
-        BarrierSpan B;
-        barrier_span(Y, S, d, A.dhat, A.kappa, B);
-        rh = B.rh;
-        node_weights(v, A.cage_idx, A.w, nodes, n, B.basis, 3, nw);
-        kinematic_sums(v, A.cage_idx, B.basis, 3, ks);
-        // the direction in the span: Q^T u
-        V3 uc = kd * ks[0];
-        double ur[2] = {ks[1] * dot(kd, rh), ks[2] * dot(kd, rh)};
-        for (int u = 0; u < n; ++u) {
-          const V3 vu = load_dir(A.hv_dir, nodes[u]);
-          uc = uc + vu * nw[u][0];
-          const double vr = dot(vu, rh);
-          ur[0] += nw[u][1] * vr;
-          ur[1] += nw[u][2] * vr;
-        }
-        const double in5[5] = {uc.x, uc.y, uc.z, ur[0], ur[1]};
-        for (int p = 0; p < 5; ++p) {
-          double acc = 0.0;
-          for (int q = 0; q < 5; ++q) acc += B.K[p][q] * in5[q];
-          t[p] = acc;
-        }
+struct HvpArgs {
+  Topo T;
+  eipc_pairs pr;
+  eipc_lag lag;
+  bool friction;
+  const double* x4;
+  const float* x4f;
+  const double* u4;
+  double dhat, inv_dhat, kappa, mu, eps_f;
+  const double* moll_r2;
+  double moll_factor;
+  int64_t item_cap;
+  double* y;                 // [12 * items]
+  int32_t* vexp;             // [nv] largest biased exponent of the vertex's contributions
+  unsigned long long* hi;    // [4 nv] fixed-point sums, upper and lower limbs
+  unsigned long long* lo;
+  uint32_t* rest;            // pairs left to k_hvp_rest, mollified pairs left to k_hvp_mollified
+  int64_t* n_rest;
+  uint32_t* moll_list;
+  int64_t* n_moll;
+  DevStatus* st;
+};
+
+__device__ __forceinline__ int32_t exponent_of(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+
+__device__ __forceinline__ void hvp_store(const HvpArgs& A, int64_t k, int slot, int32_t v, V3 y) {
+  double* row = A.y + 12 * k + 3 * slot;
+  row[0] = y.x; row[1] = y.y; row[2] = y.z;
+  const int32_t e = max(exponent_of(y.x), max(exponent_of(y.y), exponent_of(y.z)));
+  if (e > 0 && e > __ldcg(A.vexp + v)) atomicMax(A.vexp + v, e);
+}
+
+// y of a pair whose closest feature is a segment of `hint`
+__device__ __forceinline__ void hvp_light(const HvpArgs& A, int64_t k, int type, const int32_t v[4], int hint) {
+  V3 X[4];
+#pragma unroll
+  for (int a = 0; a < 4; ++a) X[a] = load_x(A.x4, v[a]);
+  const SegmentPair G = closest_segment(type, X, hint);
+  const double d2 = dot(G.r, G.r);
+  const V3 zero = {0.0, 0.0, 0.0};
+  V3 fc = zero, fa = zero;
+  if (!(d2 > 0.0)) {
+    raise_flag(A.st, EIPC_FLAG_PENETRATION);
+  } else {
+    const double inv_d = rsqrt(d2), d = d2 * inv_d;
+    if (lt_nonneg(d, A.dhat)) {
+      double b, b1, b2;
+      barrier_scalars(d, inv_d, A.dhat, A.inv_dhat, &b, &b1, &b2);
+      const double bd = -A.kappa * (b1 * inv_d);               // -kappa b'/d
+      const V3 rh = G.r * inv_d;
+      const V3 up = load_x(A.u4, pick(v, G.ip)), ua = load_x(A.u4, pick(v, G.ia)), ub = load_x(A.u4, pick(v, G.ib));
+      const V3 ul = ua - ub, uc = up - ua + ul * G.t;          // sum alpha_a u_a, sum c_a u_a
+      fc = rh * (fma(A.kappa, b2, bd) * dot(rh, uc)) - uc * bd;
+      if (G.inner) {
+        // -(kappa b'/(2d)) G M^-1 G^T with G = 2 (c (x) v + alpha (x) r), v = -e, M = 2 |e|^2
+        const double s = bd * (G.rse * G.rse) * (dot(G.r, ul) - dot(G.e, uc));
+        fc = fc - G.e * s;
+        fa = G.r * s;
       }
     }
-    const V3 tc = {t[0], t[1], t[2]};
-    for (int u = 0; u < n; ++u) {
-      V3 y = {0.0, 0.0, 0.0};
-      if (active) y = tc * nw[u][0] + rh * (nw[u][1] * t[3] + nw[u][2] * t[4]);
-      emit_g(A, og + u, (uint64_t)nodes[u], y);
-    }
-    bool kin = false;
-    for (int a = 0; a < 4; ++a) kin |= __ldg(A.cage_idx + 4 * (int64_t)v[a]) < 0;
-    if (kin) {
-      V3 yk = {0.0, 0.0, 0.0};
-      if (active) yk = tc * ks[0] + rh * (ks[1] * t[3] + ks[2] * t[4]);
-      emit_g(A, og + n, (uint64_t)(A.ns + (k & (kKinSlots - 1))), yk);
-    }
+  }
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    V3 y = zero;
+    if (a == G.ip) y = fc;
+    if (a == G.ia) y = fa - fc * (1.0 - G.t);
+    if (a == G.ib) y = zero - fa - fc * G.t;
+    hvp_store(A, k, a, v[a], y);
   }
 }
 
-__global__ void __launch_bounds__(kEvalThreads) k_hvp_friction(EvalArgs A, eipc_lag lag, double mu, double eps) {
-  pdl_entry();
-  const int64_t P = clamp_count(A.pr.count, A.pr.capacity);
-  const int64_t nit = *A.n_items;
-  const int64_t L = nit - P;
-  const V3 kd = {A.kin_dir[0], A.kin_dir[1], A.kin_dir[2]};
-  for (int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; f < L; f += grid_stride()) {
-    const int64_t k = P + f;
-    const int4 q4 = reinterpret_cast<const int4*>(lag.v)[f];
-    const int32_t v[4] = {q4.x, q4.y, q4.z, q4.w};
-    double gam[4];
-    for (int a = 0; a < 4; ++a) gam[a] = lag.gamma[4 * f + a];
-    const V3 nrm = {lag.n[3 * f], lag.n[3 * f + 1], lag.n[3 * f + 2]};
-    const V3 anc = {lag.anchor[3 * f], lag.anchor[3 * f + 1], lag.anchor[3 * f + 2]};
-    const double ml = mu * lag.lambda[f];
-    V3 vs = {0.0, 0.0, 0.0};
-    for (int a = 0; a < 4; ++a) vs = vs + load_x(A.x4, v[a]) * gam[a];
-    vs = vs - anc;
-    const V3 u = vs - nrm * dot(nrm, vs);
-    const double y2 = dot(u, u);
-    double f1y, f1p_minus;   // f1(y)/y, f1'(y) - f1(y)/y
-    if (y2 == 0.0) {
-      f1y = 2.0 / eps; f1p_minus = 0.0;
-    } else {
-      const double y = sqrt(y2);
-      if (y < eps) { f1y = 2.0 / eps - y / (eps * eps); f1p_minus = -y / (eps * eps); }
-      else { f1y = 1.0 / y; f1p_minus = -1.0 / y; }
-    }
-    const int n = A.item_n[k];
-    const int32_t* nodes = A.item_nodes + kMaxNodes * k;
-    const double coef[3][4] = {{gam[0], gam[1], gam[2], gam[3]}, {0, 0, 0, 0}, {0, 0, 0, 0}};
-    double nw[kMaxNodes][3];
-    node_weights(v, A.cage_idx, A.w, nodes, n, coef, 1, nw);
-    double ks[3];
-    kinematic_sums(v, A.cage_idx, coef, 1, ks);
-    // s = sum_a gamma_a u_a, then F s with F = mu lambda [f1/y (I - n n^T) + (f1' - f1/y) u u^T / y^2]
-    V3 sd = kd * ks[0];
-    for (int a = 0; a < n; ++a) sd = sd + load_dir(A.hv_dir, nodes[a]) * nw[a][0];
-    const V3 sp = sd - nrm * dot(nrm, sd);
-    V3 Fs = sp * (ml * f1y);
-    if (y2 > 0.0) Fs = Fs + u * (ml * f1p_minus * dot(u, sd) / y2);
-    const int64_t og = A.ro_g[k];
-    for (int a = 0; a < n; ++a) emit_g(A, og + a, (uint64_t)nodes[a], Fs * nw[a][0]);
-    bool kin = false;
-    for (int a = 0; a < 4; ++a) kin |= __ldg(A.cage_idx + 4 * (int64_t)v[a]) < 0;
-    if (kin) emit_g(A, og + n, (uint64_t)(A.ns + (k & (kKinSlots - 1))), Fs * ks[0]);
+// ... of any pair
+__device__ __forceinline__ void hvp_heavy(const HvpArgs& A, int64_t k) {
+  int32_t v[4];
+  const int type = A.pr.type[k];
+  stencil_vertices(A.T, type, A.pr.i[k], A.pr.j[k], v);
+  V3 Y[4], u[4];
+  const V3 X0 = load_x(A.x4, v[0]);
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    Y[a] = load_x(A.x4, v[a]) - X0;
+    u[a] = load_x(A.u4, v[a]);
   }
+  Stencil S;
+  closest_pair<true>(type, Y, stencil_hint(type, A.x4f, v), &S);
+  const V3 zero = {0.0, 0.0, 0.0};
+  V3 fc = zero, fa[2] = {zero, zero};
+  if (!(S.d2 > 0.0)) {
+    raise_flag(A.st, EIPC_FLAG_PENETRATION);
+  } else {
+    const double inv_d = rsqrt(S.d2), d = S.d2 * inv_d;
+    if (lt_nonneg(d, A.dhat)) {
+      double b, b1, b2;
+      barrier_scalars(d, inv_d, A.dhat, A.inv_dhat, &b, &b1, &b2);
+      const double bd = -A.kappa * (b1 * inv_d);
+      V3 r = zero, uc = zero, ul[2] = {zero, zero}, vj[2] = {zero, zero};
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        r = r + Y[a] * S.c[a];
+        uc = uc + u[a] * S.c[a];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          ul[q] = ul[q] + u[a] * S.a[q][a];
+          vj[q] = vj[q] + Y[a] * S.a[q][a];
+        }
+      }
+      const V3 rh = r * inv_d;
+      fc = rh * (fma(A.kappa, b2, bd) * dot(rh, uc)) - uc * bd;
+      if (S.m > 0) {
+        // s_j of bd M'^-1 g with M' = [v_j . v_l], g_j = v_j . u_c + r . u_j
+        const double g0 = dot(vj[0], uc) + dot(r, ul[0]), g1 = dot(vj[1], uc) + dot(r, ul[1]);
+        const double m00 = dot(vj[0], vj[0]);
+        double s0 = 0.0, s1 = 0.0;
+        if (S.m == 1) {
+          s0 = bd * g0 / m00;
+        } else {
+          const double m01 = dot(vj[0], vj[1]), m11 = dot(vj[1], vj[1]);
+          const double q = bd / (m00 * m11 - m01 * m01);
+          s0 = q * (m11 * g0 - m01 * g1);
+          s1 = q * (m00 * g1 - m01 * g0);
+        }
+        fc = fc + vj[0] * s0 + vj[1] * s1;
+        fa[0] = r * s0;
+        fa[1] = r * s1;
+      }
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < 4; ++a) hvp_store(A, k, a, v[a], fc * S.c[a] + fa[0] * S.a[0][a] + fa[1] * S.a[1][a]);
 }
 
-// Mollified EE pairs of a Hessian-vector product (the main kernel skips them): the full 12 x 12
-// path, one thread per item, launched only when the mollifier is on.
-__global__ void __launch_bounds__(kEvalThreads) k_hvp_mollified(EvalArgs A) {
-  pdl_entry();
-  const int64_t P = clamp_count(A.pr.count, A.pr.capacity);
-  const int64_t nit = *A.n_items;
-  const int64_t np = P < nit ? P : nit;
-  const V3 kd = {A.kin_dir[0], A.kin_dir[1], A.kin_dir[2]};
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < np; k += grid_stride()) {
-    const int type = A.pr.type[k];
-    if (type != 1) continue;
-    int32_t v[4];
-    stencil_vertices(A.T, type, A.pr.i[k], A.pr.j[k], v);
-    V3 Y[4];
-    const V3 X0 = load_x(A.x4, v[0]);
-    for (int a = 0; a < 4; ++a) Y[a] = load_x(A.x4, v[a]) - X0;
-    double eps_m, c_m;
-    if (!ee_mollified(A, type, A.pr.i[k], A.pr.j[k], Y, &eps_m, &c_m)) continue;
-    Stencil S;
-    ee_distance<true>(Y[0], Y[1], Y[2], Y[3], &S);
-    if (!(S.d2 > 0.0)) continue;             // flagged by the main kernel
-    const double d = sqrt(S.d2);
-    if (!(d < A.dhat)) continue;
-    const int n = A.item_n[k];
-    const int32_t* nodes = A.item_nodes + kMaxNodes * k;
-    const int64_t og = A.ro_g[k];
-    double g12[12], H12[144], Em;
-    mollified_local(Y, S, d, A.dhat, A.kappa, eps_m, c_m, &Em, g12, H12);
-    double W[4][kMaxNodes];
-    vertex_node_weights(v, A.cage_idx, A.w, nodes, n, W);
-    double u12[12], y12[12];
-    bool kin = false;
-    for (int a = 0; a < 4; ++a) {
-      const bool ka = __ldg(A.cage_idx + 4 * (int64_t)v[a]) < 0;
-      kin |= ka;
-      V3 ua = ka ? kd : V3{0.0, 0.0, 0.0};
-      for (int u = 0; u < n; ++u) ua = ua + load_dir(A.hv_dir, nodes[u]) * W[a][u];
-      u12[3 * a] = ua.x; u12[3 * a + 1] = ua.y; u12[3 * a + 2] = ua.z;
-    }
-    for (int r = 0; r < 12; ++r) {
+__device__ __forceinline__ void hvp_friction(const HvpArgs& A, int64_t k, int64_t f) {
+  const int4 q4 = reinterpret_cast<const int4*>(A.lag.v)[f];
+  const int32_t v[4] = {q4.x, q4.y, q4.z, q4.w};
+  FrictionTerms R;
+  double gam[4];
+  friction_terms(A.x4, A.lag, f, v, A.mu, A.eps_f, R, gam);
+  V3 s = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int a = 0; a < 4; ++a) s = s + load_x(A.u4, v[a]) * gam[a];
+  const V3 Fs = {R.F[0][0] * s.x + R.F[0][1] * s.y + R.F[0][2] * s.z, R.F[1][0] * s.x + R.F[1][1] * s.y + R.F[1][2] * s.z,
+                 R.F[2][0] * s.x + R.F[2][1] * s.y + R.F[2][2] * s.z};
+#pragma unroll
+  for (int a = 0; a < 4; ++a) hvp_store(A, k, a, v[a], Fs * gam[a]);
+}
+
+// whether pair k is active and mollified (then Y, eps, c are its offsets and mollifier arguments)
+__device__ __forceinline__ bool hvp_is_mollified(const HvpArgs& A, int type, int32_t i, int32_t j, const int32_t v[4], V3 Y[4],
+                                                 double* eps, double* c) {
+  if (!A.moll_r2 || type != 1) return false;
+  const V3 X0 = load_x(A.x4, v[0]);
+#pragma unroll
+  for (int a = 0; a < 4; ++a) Y[a] = load_x(A.x4, v[a]) - X0;
+  const V3 nn = cross(Y[1] - Y[0], Y[3] - Y[2]);
+  *c = dot(nn, nn);
+  *eps = A.moll_factor * A.moll_r2[i] * A.moll_r2[j];
+  if (!(*c < *eps)) return false;
+  const double d2 = closest_pair<false>(1, Y, stencil_hint(1, A.x4f, v), nullptr);
+  return d2 > 0.0 && sqrt(d2) < A.dhat;
+}
+
+// a mollified EE pair: its full 12 x 12 Hessian
+__device__ __forceinline__ void hvp_mollified(const HvpArgs& A, int64_t k) {
+  int32_t v[4];
+  const int32_t i = A.pr.i[k], j = A.pr.j[k];
+  stencil_vertices(A.T, 1, i, j, v);
+  V3 Y[4];
+  double eps, c;
+  if (!hvp_is_mollified(A, 1, i, j, v, Y, &eps, &c)) return;
+  Stencil S;
+  ee_distance<true>(Y[0], Y[1], Y[2], Y[3], &S);
+  double g12[12], H12[144], E;
+  mollified_local(Y, S, sqrt(S.d2), A.dhat, A.kappa, eps, c, &E, g12, H12);
+  double u12[12];
+  for (int a = 0; a < 4; ++a) {
+    const V3 u = load_x(A.u4, v[a]);
+    u12[3 * a] = u.x; u12[3 * a + 1] = u.y; u12[3 * a + 2] = u.z;
+  }
+  for (int a = 0; a < 4; ++a) {
+    double y[3];
+    for (int q = 0; q < 3; ++q) {
       double acc = 0.0;
-      for (int q = 0; q < 12; ++q) acc += H12[12 * r + q] * u12[q];
-      y12[r] = acc;
+      for (int p = 0; p < 12; ++p) acc += H12[12 * (3 * a + q) + p] * u12[p];
+      y[q] = acc;
     }
-    for (int u = 0; u < n; ++u) {
-      V3 y = {0.0, 0.0, 0.0};
-      for (int a = 0; a < 4; ++a) y = y + V3{y12[3 * a], y12[3 * a + 1], y12[3 * a + 2]} * W[a][u];
-      emit_g(A, og + u, (uint64_t)nodes[u], y);
+    hvp_store(A, k, a, v[a], V3{y[0], y[1], y[2]});
+  }
+}
+
+// appends k to a list (one atomic per warp)
+__device__ __forceinline__ void list_append(bool mine, int64_t k, uint32_t* list, int64_t* n) {
+  const unsigned m = __ballot_sync(0xffffffffu, mine);
+  if (!m) return;
+  const int lane = threadIdx.x & 31;
+  unsigned long long b = 0;
+  if (lane == 0) b = atomicAdd(reinterpret_cast<unsigned long long*>(n), (unsigned long long)__popc(m));
+  b = __shfl_sync(0xffffffffu, b, 0);
+  if (mine) list[(int64_t)b + __popc(m & ((1u << lane) - 1u))] = (uint32_t)k;
+}
+
+// y of every item but the pairs it lists: those with an interior closest point (as in
+// k_eval_factors) and mollified ones
+__global__ void __launch_bounds__(kEvalThreads, 4) k_hvp_items(HvpArgs A) {
+  pdl_entry();
+  const int lane = threadIdx.x & 31;
+  const int64_t P = clamp_count(A.pr.count, A.pr.capacity);
+  const int64_t L = A.friction ? clamp_count(A.lag.count, A.lag.capacity) : 0;
+  const int64_t n = P + L < A.item_cap ? P + L : A.item_cap;
+  if (P + L > A.item_cap && blockIdx.x == 0 && threadIdx.x == 0) raise_flag(A.st, EIPC_FLAG_REC_OVERFLOW);
+  const int64_t np = P < n ? P : n;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t base = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
+    const int64_t k = base + lane;
+    bool rest = false, moll = false;
+    if (k < np) {
+      int32_t v[4];
+      const int type = A.pr.type[k];
+      const int32_t i = A.pr.i[k], j = A.pr.j[k];
+      stencil_vertices(A.T, type, i, j, v);
+      V3 Y[4];
+      double eps, c;
+      moll = hvp_is_mollified(A, type, i, j, v, Y, &eps, &c);
+      if (!moll) {
+        const int hint = stencil_hint(type, A.x4f, v);
+        if (hint & kHintInterior) rest = true;
+        else hvp_light(A, k, type, v, hint);
+      }
+    } else if (k < n) {
+      hvp_friction(A, k, k - P);
     }
+    list_append(rest, k, A.rest, A.n_rest);
+    if (A.n_moll) list_append(moll, k, A.moll_list, A.n_moll);
+  }
+}
+
+__global__ void __launch_bounds__(kEvalThreads) k_hvp_rest(HvpArgs A) {
+  pdl_entry();
+  const int64_t n = *A.n_rest;
+  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += grid_stride()) hvp_heavy(A, A.rest[q]);
+}
+
+__global__ void __launch_bounds__(kEvalThreads) k_hvp_mollified(HvpArgs A) {
+  pdl_entry();
+  const int64_t n = *A.n_moll;
+  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += grid_stride()) hvp_mollified(A, A.moll_list[q]);
+}
+
+// adds y / 2^(E - 1022) as a fixed-point number: kFix bits in hi, the next kFix in lo
+__device__ __forceinline__ void add_fixed(unsigned long long* hi, unsigned long long* lo, double y, int32_t E) {
+  const long long b = __double_as_longlong(y);
+  int32_t e = (int32_t)((b >> 52) & 0x7ff);
+  unsigned long long m = (unsigned long long)b & 0xfffffffffffffull;
+  if (e > 0) m |= 1ull << 52;
+  else e = 1;
+  if (m == 0) return;
+  const int sh = 2 * kFix - 53 - (E - e);      // value = m 2^sh in units of 2^(-2 kFix)
+  const int down = kFix - sh;
+  unsigned long long h = down < 64 ? m >> down : 0;
+  unsigned long long l = sh >= 0 ? m << sh : (sh > -64 ? m >> -sh : 0);
+  l &= (1ull << kFix) - 1;
+  if (b < 0) { h = 0ull - h; l = 0ull - l; }
+  if (h) atomicAdd(hi, h);
+  if (l) atomicAdd(lo, l);
+}
+
+__global__ void __launch_bounds__(kBlock) k_hvp_accumulate(HvpArgs A) {
+  pdl_entry();
+  const int64_t P = clamp_count(A.pr.count, A.pr.capacity);
+  const int64_t L = A.friction ? clamp_count(A.lag.count, A.lag.capacity) : 0;
+  const int64_t n = P + L < A.item_cap ? P + L : A.item_cap;
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < 4 * n; t += grid_stride()) {
+    const int64_t k = t >> 2;
+    const int a = (int)(t & 3);
+    int32_t v[4];
+    item_vertices(A.T, A.pr, P, A.lag.v, L, k, v);
+    const int32_t va = pick(v, a);
+    const double* y = A.y + 3 * t;
+    const double y0 = y[0], y1 = y[1], y2 = y[2];
+    const int32_t E = A.vexp[va];
+    if (E == 0 || E == 0x7ff) continue;        // nothing but zeros; a NaN or infinity (the gather says so)
+    add_fixed(A.hi + 4 * (int64_t)va, A.lo + 4 * (int64_t)va, y0, E);
+    add_fixed(A.hi + 4 * (int64_t)va + 1, A.lo + 4 * (int64_t)va + 1, y1, E);
+    add_fixed(A.hi + 4 * (int64_t)va + 2, A.lo + 4 * (int64_t)va + 2, y2, E);
+  }
+}
+
+// a fixed-point sum as a double
+__device__ __forceinline__ double from_fixed(long long hi, long long lo, double scale) {
+  const long long t = hi + (lo >> kFix), f = lo & ((1ll << kFix) - 1);
+  return fma((double)f, 1.0 / (double)(1ll << kFix), (double)t) * scale;
+}
+
+// Rows of J^T: warp r < ns gathers node r's vertices, the next kKinSlots warps a share of the
+// kinematic ones each (weight one); the last of these to finish adds the shares in order.
+__global__ void __launch_bounds__(kBlock) k_hvp_gather(int64_t ns, const int64_t* __restrict__ inc_ptr,
+                                                       const uint32_t* __restrict__ inc, const double* __restrict__ w,
+                                                       const int32_t* __restrict__ vexp, const long long* __restrict__ hi,
+                                                       const long long* __restrict__ lo, double* __restrict__ out_r,
+                                                       double* __restrict__ out_kin, double* part, int64_t* ticket) {
+  pdl_entry();
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  const int64_t rows = ns + (out_kin ? kKinSlots : 0);
+  for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < rows; r += nw) {
+    const bool kin = r >= ns;
+    int64_t b = inc_ptr[kin ? ns : r], e = inc_ptr[(kin ? ns : r) + 1];
     if (kin) {
-      V3 yk = {0.0, 0.0, 0.0};
-      for (int a = 0; a < 4; ++a)
-        if (__ldg(A.cage_idx + 4 * (int64_t)v[a]) < 0) yk = yk + V3{y12[3 * a], y12[3 * a + 1], y12[3 * a + 2]};
-      emit_g(A, og + n, (uint64_t)(A.ns + (k & (kKinSlots - 1))), yk);
+      const int64_t per = (e - b + kKinSlots - 1) / kKinSlots, b0 = b + per * (r - ns);
+      e = b0 + per < e ? b0 + per : e;
+      b = b0;
+    }
+    double a0 = 0.0, a1 = 0.0, a2 = 0.0;
+    for (int64_t q = b + lane; q < e; q += 32) {
+      const uint32_t t = inc[q];
+      const int64_t v = t >> 2;
+      const int32_t E = vexp[v];
+      if (E == 0) continue;
+      // 2^(E - 1022 - kFix), or NaN where a contribution was not finite
+      const double sc = E == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
+                                   : (E >= kFix ? __hiloint2double((E - kFix + 1) << 20, 0) : ldexp(1.0, E - 1022 - kFix));
+      const longlong2 h01 = *reinterpret_cast<const longlong2*>(hi + 4 * v), l01 = *reinterpret_cast<const longlong2*>(lo + 4 * v);
+      const double ww = kin ? 1.0 : w[t];
+      a0 = fma(ww, from_fixed(h01.x, l01.x, sc), a0);
+      a1 = fma(ww, from_fixed(h01.y, l01.y, sc), a1);
+      a2 = fma(ww, from_fixed(hi[4 * v + 2], lo[4 * v + 2], sc), a2);
+    }
+    if (__any_sync(0xffffffffu, a0 != 0.0 || a1 != 0.0 || a2 != 0.0)) {
+      double acc[3] = {a0, a1, a2};
+      warp_tree_sum<3>(acc);
+      a0 = acc[0]; a1 = acc[1]; a2 = acc[2];
+    }
+    if (!kin) {
+      if (lane == 0) { out_r[3 * r] = a0; out_r[3 * r + 1] = a1; out_r[3 * r + 2] = a2; }
+      continue;
+    }
+    int64_t done = 0;
+    if (lane == 0) {
+      double* p = part + 3 * (r - ns);
+      p[0] = a0; p[1] = a1; p[2] = a2;
+      __threadfence();
+      done = (int64_t)atomicAdd(reinterpret_cast<unsigned long long*>(ticket), 1ull);
+    }
+    done = __shfl_sync(0xffffffffu, done, 0);
+    if (done == kKinSlots - 1) {
+      __threadfence();
+      double acc[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) acc[c] = __ldcg(part + 3 * lane + c) + __ldcg(part + 3 * (lane + 32) + c);
+      warp_tree_sum<3>(acc);
+      if (lane == 0)
+        for (int c = 0; c < 3; ++c) out_kin[c] = acc[c];
     }
   }
 }
@@ -1846,16 +1995,6 @@ __global__ void k_rec_check(const int64_t* rh_total, const int64_t* rg_total, in
     *n_rh = a < rec_cap ? a : rec_cap;
     *n_rg = b < gcap ? b : gcap;
   }
-}
-
-// Segment sums, one warp per segment: lane l adds records b+l, b+l+32, ... in order and a
-// fixed shuffle tree combines the lanes, so the result depends only on the sorted order.
-template <int W>
-__device__ __forceinline__ void warp_tree_sum(double acc[W]) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-    for (int c = 0; c < W; ++c) acc[c] += __shfl_down_sync(0xffffffffu, acc[c], o);
 }
 
 // every upper block (I, J) becomes the full-pattern entry (I, J) and, off the diagonal,
@@ -1893,37 +2032,6 @@ __global__ void __launch_bounds__(kBlock) k_full_entries(const uint64_t* __restr
     }
   }
 }
-
-__global__ void __launch_bounds__(kBlock) k_seg_sum_g(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ vals,
-                                                      const double* __restrict__ rec, const int64_t* __restrict__ start,
-                                                      const int64_t* n_rec, const int64_t* n_seg, int64_t cap,
-                                                      double* __restrict__ g) {
-  pdl_entry();
-  const int64_t R = clamp_count(n_rec, cap);
-  const int64_t S = *n_seg;
-  const int lane = threadIdx.x & 31;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < S; s += nw) {
-    const int64_t b = start[s], e = (s + 1 < S) ? start[s + 1] : R;
-    double acc[3] = {0.0, 0.0, 0.0};
-    for (int64_t r = b + lane; r < e; r += 32) {
-      const double* p = rec + kGRecStride * (int64_t)vals[r];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) acc[c] += p[c];
-    }
-    warp_tree_sum<3>(acc);
-    if (lane == 0) {
-      const int64_t node = (int64_t)keys[b];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) g[3 * node + c] = acc[c];
-    }
-  }
-}
-
-// ---- presorted reduction: the record keys of the energy/gradient/Hessian evaluation
-// depend only on each item's cage nodes, so they are written, sorted and turned into the
-// BSR pattern before the evaluation; the evaluation then writes every record straight to
-// its sorted position and the sums read contiguous records.
 
 // keys of item k's Hessian records: record (u, v), u <= v, keyed by the upper-triangle position
 // of its nodes (min, max), and its source (item, local node of the row, of the column).  One
@@ -2409,58 +2517,95 @@ void eval_launch(eipc_scene* sc, const double* q, const eipc_pairs& pr, const ei
 
 void hvp_launch(eipc_scene* sc, const double* q, const eipc_pairs& pr, const eipc_lag* lag, const eipc_params& p,
                 const double* v, const double* kin_dir, double* out_r, double* out_kin, cudaStream_t s) {
-  EIPC_TIMED(sc, kKEmbed, s, embed_launch(sc, q, sc->x4, 1, 0, s));
   const bool fr = lag && p.mu > 0.0;
-  int64_t* cnt = sc->counters;
-  zero_ranges(s, {{cnt + kCntItems, 5 * sizeof(int64_t)}, {cnt + kCntZero, sizeof(int64_t)}});
-  const int64_t item_cap = sc->item_cap;
-  launch(k_item_nodes, blocks_for(item_cap, 8), kBlock, 0, s, sc->topo, pr, fr ? lag->v : nullptr, fr ? lag->count : nullptr,
-         fr ? lag->capacity : 0, sc->cage_idx, item_cap, sc->item_nodes, sc->item_n, sc->item_group, sc->vgroup,
-         sc->rc_h, sc->rc_g, cnt + kCntItems, sc->status, static_cast<const int32_t*>(nullptr),
-         static_cast<const int32_t*>(nullptr), static_cast<uint64_t*>(nullptr));
-  launch(k_hvp_counts, blocks_for(item_cap, 8), kBlock, 0, s, sc->topo, pr, fr ? lag->v : nullptr,
-         fr ? static_cast<const int64_t*>(lag->count) : nullptr, fr ? lag->capacity : 0,
-         static_cast<const int32_t*>(sc->cage_idx), static_cast<const int32_t*>(sc->item_n),
-         static_cast<const int64_t*>(cnt + kCntItems), item_cap, sc->rc_g);
-  int64_t* tot_g = cnt + 10;
-  exclusive_scan_i64(sc->rc_g, sc->ro_g, cnt + kCntItems, item_cap, tot_g, sc->scan_partial, s);
-  launch(k_rec_check, 1, 32, 0, s, static_cast<const int64_t*>(cnt + kCntZero), static_cast<const int64_t*>(tot_g),
-         sc->rec_cap, sc->gcap, cnt + kCntRecH, cnt + kCntRecG, sc->status);
-  EvalArgs A{};
-  A.T = sc->topo; A.pr = pr; A.cage_idx = sc->cage_idx; A.w = sc->w; A.x4 = sc->x4; A.ns = sc->ns;
-  A.dhat = p.dhat; A.kappa = p.kappa; A.item_nodes = sc->item_nodes; A.item_n = sc->item_n;
-  A.ro_h = sc->ro_h; A.ro_g = sc->ro_g; A.n_items = cnt + kCntItems; A.rec_cap = sc->rec_cap; A.gcap = sc->gcap;
-  A.gkeys = sc->gkeys; A.gvals = sc->gvals;
-  A.grec = sc->grec; A.item_E = sc->item_E; A.st = sc->status;
-  A.project = false;
+  const V3 kin = kin_dir ? V3{kin_dir[0], kin_dir[1], kin_dir[2]} : V3{0.0, 0.0, 0.0};
+  HvpArgs A{};
+  A.T = sc->topo; A.pr = pr; A.friction = fr;
+  if (fr) A.lag = *lag;
+  A.x4 = sc->x4; A.x4f = sc->x4f; A.u4 = sc->dx4;
+  A.dhat = p.dhat; A.inv_dhat = 1.0 / p.dhat; A.kappa = p.kappa; A.mu = p.mu; A.eps_f = p.eps_v * p.h;
   A.moll_r2 = sc->moll_factor > 0.0 ? sc->moll_r2 : nullptr;
   A.moll_factor = sc->moll_factor;
-  A.hv_dir = v;
-  for (int c = 0; c < 3; ++c) A.kin_dir[c] = kin_dir ? kin_dir[c] : 0.0;
-  A.fric_of_pair = nullptr; A.pair_of_fric = nullptr;
-  A.lag = fr ? *lag : eipc_lag{};
-  A.mu = p.mu; A.eps_f = p.eps_v * p.h;
-  EIPC_TIMED(sc, kKEvalBarrier, s,
-             (launch(k_hvp_barrier, blocks_for(pr.capacity, 8, kEvalThreads), kEvalThreads, 0, s, A)));
+  A.item_cap = sc->item_cap;
+  // scratch: the factor rows hold y, the search's per-vertex boxes the sums, the FP32
+  // displacements the exponents (every other call writes them anew before it reads them)
+  A.y = sc->frow;
+  A.vexp = reinterpret_cast<int32_t*>(sc->dx4f);
+  A.hi = reinterpret_cast<unsigned long long*>(sc->vbox);
+  A.lo = reinterpret_cast<unsigned long long*>(sc->vbox_pad);
+  A.st = sc->status;
+  int64_t* ticket = sc->counters + kCntHvpTicket;
+  EIPC_TIMED(sc, kKEmbed, s, embed_launch(sc, q, sc->x4, 1, 0, s);
+             launch(k_hvp_direction, blocks_for(sc->nv), kBlock, 0, s, sc->nv, static_cast<const int32_t*>(sc->cage_idx),
+                    static_cast<const double*>(sc->w), v, kin, sc->dx4, A.vexp, A.hi, A.lo,
+                    CounterList{{ticket, sc->counters + kCntEvalRest, sc->counters + kCntMollList, nullptr}}));
+  const int64_t want = pr.capacity + (fr ? lag->capacity : 0), most = want < sc->item_cap ? want : sc->item_cap;
+  A.rest = sc->svals; A.n_rest = sc->counters + kCntEvalRest;
+  A.moll_list = sc->svals_alt; A.n_moll = A.moll_r2 ? sc->counters + kCntMollList : nullptr;
+  EIPC_TIMED(sc, kKEvalBarrier, s, launch(k_hvp_items, blocks_for(most, 8, kEvalThreads), kEvalThreads, 0, s, A);
+             launch(k_hvp_rest, 2 * kSMs, kEvalThreads, 0, s, A));
   if (A.moll_r2)
-    EIPC_TIMED(sc, kKEvalBarrier, s, (launch(k_hvp_mollified, blocks_for(pr.capacity, 8, kEvalThreads), kEvalThreads, 0, s, A)));
-  if (fr)
-    EIPC_TIMED(sc, kKEvalFriction, s,
-               (launch(k_hvp_friction, blocks_for(lag->capacity, 8, kEvalThreads), kEvalThreads, 0, s, A, *lag, p.mu,
-                       p.eps_v * p.h)));
+    EIPC_TIMED(sc, kKEvalBarrier, s, (launch(k_hvp_mollified, 2 * kSMs, kEvalThreads, 0, s, A)));
   sc->timers->start(kKGReduce, s);
-  int wg = radix_sort_u64(sc->gkeys, sc->gvals, sc->gkeys_alt, sc->gvals_alt, cnt + kCntRecG, sc->gcap,
-                          bits_for((uint64_t)(sc->ns + kKinSlots)), sc->sort_hist, s);
-  const uint64_t* gk = wg ? sc->gkeys_alt : sc->gkeys;
-  const uint32_t* gv = wg ? sc->gvals_alt : sc->gvals;
-  segment_starts(gk, cnt + kCntRecG, sc->gcap, sc->gseg_start, cnt + kCntSegG, sc->scan_partial, s);
-  zero_ranges(s, {{sc->hvp_out, sizeof(double) * 3 * (sc->ns + kKinSlots)}});
-  launch(k_seg_sum_g, blocks_for(sc->gcap, 16), kBlock, 0, s, gk, gv, sc->grec, sc->gseg_start, cnt + kCntRecG,
-         cnt + kCntSegG, sc->gcap, sc->hvp_out);
-  cudaMemcpyAsync(out_r, sc->hvp_out, sizeof(double) * 3 * sc->ns, cudaMemcpyDeviceToDevice, s);
-  if (out_kin)
-    launch(k_hvp_kin_sum, 1, 32, 0, s, static_cast<const double*>(sc->hvp_out + 3 * sc->ns), out_kin);
+  launch(k_hvp_accumulate, blocks_for(4 * most, 8), kBlock, 0, s, A);
+  launch(k_hvp_gather, blocks_for(32 * (sc->ns + kKinSlots), 8), kBlock, 0, s, sc->ns, static_cast<const int64_t*>(sc->inc_ptr),
+         static_cast<const uint32_t*>(sc->inc), static_cast<const double*>(sc->w), static_cast<const int32_t*>(A.vexp),
+         reinterpret_cast<const long long*>(A.hi), reinterpret_cast<const long long*>(A.lo), out_r, out_kin, sc->hvp_part, ticket);
   sc->timers->stop(kKGReduce, s);
+}
+
+// Static lists for J^T: the embedded vertices' (vertex, slot) entries by cage node, then the
+// kinematic vertices; built once at scene creation on the default stream, by the stable radix
+// sort.
+namespace {
+__global__ void __launch_bounds__(kBlock) k_incidence_keys(int64_t nv, int64_t ns, const int32_t* __restrict__ idx,
+                                                           uint64_t* __restrict__ keys, uint32_t* __restrict__ vals) {
+  pdl_entry();
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < 4 * nv; t += grid_stride()) {
+    const int32_t id = idx[t];
+    keys[t] = (uint64_t)(id >= 0 ? id : ((t & 3) == 0 ? ns : ns + 1));     // a kinematic vertex counts once
+    vals[t] = (uint32_t)t;
+  }
+}
+
+__global__ void __launch_bounds__(kBlock) k_incidence_rows(int64_t ns, int64_t n, const uint64_t* __restrict__ keys,
+                                                           int64_t* __restrict__ ptr) {
+  pdl_entry();
+  for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < ns + 2; r += grid_stride()) {
+    int64_t lo = 0, hi = n;                  // first entry of row r
+    while (lo < hi) {
+      const int64_t mid = (lo + hi) >> 1;
+      if (keys[mid] < (uint64_t)r) lo = mid + 1;
+      else hi = mid;
+    }
+    ptr[r] = lo;
+  }
+}
+}  // namespace
+
+cudaError_t incidence_build(eipc_scene* sc) {
+  const int64_t n = 4 * sc->nv;
+  uint64_t *k = nullptr, *ka = nullptr;
+  uint32_t* va = nullptr;
+  int64_t* nd = nullptr;
+  cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&k), 8 * n);
+  if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&ka), 8 * n);
+  if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&va), 4 * n);
+  if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&nd), 8);
+  if (e == cudaSuccess) e = cudaMemcpy(nd, &n, 8, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) {
+    launch(k_incidence_keys, blocks_for(n), kBlock, 0, nullptr, sc->nv, sc->ns, static_cast<const int32_t*>(sc->cage_idx), k, sc->inc);
+    const int which = radix_sort_u64(k, sc->inc, ka, va, nd, n, bits_for((uint64_t)sc->ns + 1), sc->sort_hist, nullptr);
+    launch(k_incidence_rows, blocks_for(sc->ns + 2), kBlock, 0, nullptr, sc->ns, n, static_cast<const uint64_t*>(which ? ka : k),
+           sc->inc_ptr);
+    if (which) e = cudaMemcpyAsync(sc->inc, va, 4 * n, cudaMemcpyDeviceToDevice, nullptr);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+  }
+  if (k) cudaFree(k);
+  if (ka) cudaFree(ka);
+  if (va) cudaFree(va);
+  if (nd) cudaFree(nd);
+  return e;
 }
 
 }  // namespace eipc

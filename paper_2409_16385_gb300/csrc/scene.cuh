@@ -62,7 +62,9 @@ struct eipc_scene {
   uint32_t* hvals_alt;
   double* hrec;          // [rec_cap*kHRecStride] explicit 3x3 blocks of mollified pairs, 16-byte aligned
                          // rows (null until the mollifier is first turned on)
-  double* hvp_out;       // [(ns+64)*3] Hessian-vector product: reduced rows, then 64 kinematic partials
+  int64_t* inc_ptr;      // [ns + 2] J^T: first entry of each cage node's vertices, then of the kinematic ones
+  uint32_t* inc;         // [4 nv] entries 4 vertex + slot, by node (kinematic vertices last)
+  double* hvp_part;      // [3*64] partial sums over the kinematic vertices
   uint64_t* edge_key;    // [ne] sorted a * nv + b of every edge (a < b), for edge-id lookup
   int32_t* edge_id;      // [ne] edge id of each sorted key
   int feat_bits;         // bits per id in the feature keys of the deduplicated pair set
@@ -78,13 +80,11 @@ struct eipc_scene {
   uint64_t* item_map;    // [item_cap] local node of each (vertex, slot) of an item, in nibbles
   double* piece;         // [9 * (rec_cap + rec_cap / 32 + 2)] partial segment sums of the Hessian records
   int64_t* hunit;        // [rec_cap + 1] first summation unit of each Hessian segment
-  int64_t gcap;          // gradient records
+  int64_t gcap;          // factor rows; entries of the per-group energy sort
   uint64_t* gkeys;
   uint64_t* gkeys_alt;
   uint32_t* gvals;
   uint32_t* gvals_alt;
-  double* grec;          // [gcap*kGRecStride] 3-vectors, 16-byte aligned rows
-  int64_t* gseg_start;
   int64_t* scan_partial; // [2 (kScanBlocks+1)] scan partials (two arrays for exclusive_scan2_i64)
   double* sum_partial;   // [kScanBlocks]
   int bits_h, bits_g;    // key widths of the reduction sorts
@@ -107,8 +107,8 @@ struct eipc_scene {
 
 namespace eipc {
 // device counters
-// record row strides (doubles): 9 (3) values padded so that each row starts on 16 bytes
-constexpr int kHRecStride = 10, kGRecStride = 4;
+// record row stride (doubles): 9 values padded so that each row starts on 16 bytes
+constexpr int kHRecStride = 10;
 // factor row: z1, z2 (3 each), omega, friction weight, z3 (3), pad; item header: the friction
 // block's upper entries (6), the gradient vectors of barrier and friction (3 each), the
 // isotropic coefficient, flags, pad.  32-byte sectors throughout.
@@ -118,7 +118,8 @@ enum { kCntCand = 0, kCntSurv = 1, kCntItems = 2, kCntRecH = 3, kCntRecG = 4, kC
        kCntAccd = 7, kCntZero = 8, kCntEvalQueue = 16, kCntScreened = 15, kCntDedup = 17, kCntUnitsH = 18,
        kCntMollBad = 20, kCntCcdQueue = 21, kCntCcdList = 22, kCntMollList = 23,
        kCntEvalRest = 24, /* two entries */
-       kCntN = 26 };
+       kCntHvpTicket = 26,
+       kCntN = 28 };
 
 // device counters a kernel zeroes before the launches that count (null: none)
 constexpr int kCounterList = 4;
@@ -155,6 +156,7 @@ void lag_launch(eipc_scene* sc, const double* q_n, const eipc_pairs& pr, const e
 void eval_launch(eipc_scene* sc, const double* q, const eipc_pairs& pr, const eipc_lag* lag, const eipc_params& p,
                  double* E, double* g_r, const eipc_bsr& H, cudaStream_t s);
 int bits_for(uint64_t maxval);
+cudaError_t incidence_build(eipc_scene* sc);
 void group_energy_launch(eipc_scene* sc, double* E_groups, cudaStream_t s);
 void hvp_launch(eipc_scene* sc, const double* q, const eipc_pairs& pr, const eipc_lag* lag, const eipc_params& p,
                 const double* v, const double* kin_dir, double* out_r, double* out_kin, cudaStream_t s);
