@@ -30,7 +30,7 @@ void free_scene(eipc_scene* s) {
                   s->broad.n_dev, s->broad.bounds,
                   s->sort_hist, s->cand, s->counters, s->skeys, s->skeys_alt, s->svals, s->svals_alt, s->sd,
                   s->item_nodes, s->item_n, s->rc_h, s->ro_h, s->rc_g, s->ro_g, s->item_E, s->hkeys,
-                  s->hkeys_alt, s->hvals, s->hvals_alt, s->hrec, s->seg_flag, s->seg_id, s->seg_start, s->rec_src, s->src_sorted, s->frow, s->ihead, s->item_map, s->piece, s->hunit,
+                  s->hkeys_alt, s->hvals, s->hvals_alt, s->hrec, s->seg_flag, s->seg_id, s->seg_start, s->rec_src, s->group_start, s->frow, s->ihead, s->item_map, s->piece,
                   s->gkeys, s->gkeys_alt, s->gvals, s->gvals_alt,
                   s->scan_partial, s->sum_partial, s->status};
   for (void* p : ptrs)
@@ -40,6 +40,7 @@ void free_scene(eipc_scene* s) {
     delete s->timers;
   }
   if (s->ev_fork) cudaEventDestroy(s->ev_fork);
+  if (s->ev_mid) cudaEventDestroy(s->ev_mid);
   if (s->ev_join) cudaEventDestroy(s->ev_join);
   if (s->aux) cudaStreamDestroy(s->aux);
   delete s;
@@ -164,13 +165,9 @@ eipc_status eipc_scene_create(int64_t Nv, int64_t F, int64_t E, int64_t Ns, cons
   ok(dalloc(&s->hvals, s->rec_cap)); ok(dalloc(&s->hvals_alt, s->rec_cap));
   ok(dalloc(&s->inc_ptr, Ns + 2)); ok(dalloc(&s->inc, 4 * Nv)); ok(dalloc(&s->hvp_part, 3 * 64));
   ok(dalloc(&s->seg_flag, s->rec_cap)); ok(dalloc(&s->seg_id, s->rec_cap)); ok(dalloc(&s->seg_start, s->rec_cap));
-  ok(dalloc(&s->rec_src, s->rec_cap)); ok(dalloc(&s->src_sorted, s->rec_cap));
+  ok(dalloc(&s->rec_src, s->rec_cap)); ok(dalloc(&s->group_start, s->gcap));
   ok(dalloc(&s->frow, kFRow * s->gcap)); ok(dalloc(&s->ihead, kIHead * s->item_cap)); ok(dalloc(&s->item_map, s->item_cap));
-  {
-    const int64_t pr = s->rec_cap + s->rec_cap / 16 + 2;
-    ok(dalloc(&s->piece, 9 * pr));
-  }
-  ok(dalloc(&s->hunit, s->rec_cap + 1));
+  ok(dalloc(&s->piece, 9 * s->rec_cap));
   ok(dalloc(&s->gkeys, s->gcap)); ok(dalloc(&s->gkeys_alt, s->gcap));
   ok(dalloc(&s->gvals, s->gcap)); ok(dalloc(&s->gvals_alt, s->gcap));
   ok(dalloc(&s->edge_key, E > 0 ? E : 1)); ok(dalloc(&s->edge_id, E > 0 ? E : 1));
@@ -179,6 +176,7 @@ eipc_status eipc_scene_create(int64_t Nv, int64_t F, int64_t E, int64_t Ns, cons
   ok(dalloc(&s->status, 1));
   ok(cudaStreamCreateWithFlags(&s->aux, cudaStreamNonBlocking));
   ok(cudaEventCreateWithFlags(&s->ev_fork, cudaEventDisableTiming));
+  ok(cudaEventCreateWithFlags(&s->ev_mid, cudaEventDisableTiming));
   ok(cudaEventCreateWithFlags(&s->ev_join, cudaEventDisableTiming));
   if (e != cudaSuccess) {
     free_scene(s);

@@ -58,6 +58,17 @@ __device__ __forceinline__ void upper_decode(uint64_t key, uint64_t ns, uint64_t
   *J = key - upper_key((uint64_t)i, (uint64_t)i, ns) + (uint64_t)i;
 }
 
+// node I of a diagonal key (I, I): I ns - I (I - 1) / 2 = key, by bisection
+__device__ __forceinline__ int64_t diagonal_node(uint64_t key, uint64_t ns) {
+  uint64_t lo = 0, hi = ns - 1;
+  while (lo < hi) {
+    const uint64_t mid = (lo + hi + 1) >> 1;
+    if (upper_key(mid, mid, ns) <= key) lo = mid;
+    else hi = mid - 1;
+  }
+  return (int64_t)lo;
+}
+
 // stencil vertex ids of pair (type, i, j)
 __device__ __forceinline__ void stencil_vertices(const Topo& T, int type, int32_t i, int32_t j, int32_t v[4]) {
   if (type == 0) {
@@ -171,7 +182,13 @@ __global__ void __launch_bounds__(kBlock) k_fric_match(Topo T, eipc_pairs pr, ei
   }
 }
 
-// unique cage nodes of each item (kinematic vertices carry none), record counts
+// Unique cage nodes of each item in ascending order (kinematic vertices carry none), the node of
+// every (vertex, slot), record counts, and the key that brings items with the same nodes together:
+// the first node above a hash of the others' offsets from it.  Offsets, not ids, so that a
+// scene's items order alike alone and inside a batch, where its ids are shifted.  Items without
+// nodes get a key above all.
+constexpr int kHashBits = 7;   // the full grasp has about ten node sets per first node
+
 __global__ void __launch_bounds__(kBlock) k_item_nodes(Topo T, eipc_pairs pr, const int32_t* lag_v,
                                                        const int64_t* lag_count, int64_t lag_cap,
                                                        const int32_t* __restrict__ cage_idx, int64_t item_cap,
@@ -181,7 +198,8 @@ __global__ void __launch_bounds__(kBlock) k_item_nodes(Topo T, eipc_pairs pr, co
                                                        int64_t* n_items, DevStatus* st,
                                                        const int32_t* __restrict__ fric_of_pair,
                                                        const int32_t* __restrict__ pair_of_fric,
-                                                       uint64_t* __restrict__ item_map) {
+                                                       uint64_t* __restrict__ item_map, int key_bits,
+                                                       uint64_t* __restrict__ keys, uint32_t* __restrict__ vals) {
   pdl_entry();
   const int64_t P = clamp_count(pr.count, pr.capacity);
   const int64_t L = lag_v ? clamp_count(lag_count, lag_cap) : 0;
@@ -198,32 +216,53 @@ __global__ void __launch_bounds__(kBlock) k_item_nodes(Topo T, eipc_pairs pr, co
     int32_t v[4];
     item_vertices(T, pr, P, lag_v, L, k, v);
     item_group[k] = vgroup[v[0]];
-    if (k >= P && friction_merged(fric_of_pair, pair_of_fric, k - P)) {
-      item_n[k] = 0;               // evaluated in its contact pair's records
-      rc_h[k] = 0;
-      rc_g[k] = 0;
-      continue;
-    }
+    vals[k] = (uint32_t)k;
     int32_t nodes[kMaxNodes];
     int cnt = 0;
     uint64_t map = 0;              // nibble 4a + s: which of the item's nodes is slot s of vertex a
-    for (int a = 0; a < 4; ++a) {
-      const int4 id = __ldg(reinterpret_cast<const int4*>(cage_idx) + v[a]);
-      if (id.x < 0) continue;
-      const int32_t ids[4] = {id.x, id.y, id.z, id.w};
-      for (int s = 0; s < 4; ++s) {
-        int at = cnt;
-        for (int u = 0; u < cnt; ++u)
-          if (nodes[u] == ids[s]) at = u;
-        if (at == cnt) nodes[cnt++] = ids[s];
-        map |= (uint64_t)at << (4 * (4 * a + s));
+    // a merged friction item is evaluated in its contact pair's records
+    if (k < P || !friction_merged(fric_of_pair, pair_of_fric, k - P)) {
+      for (int a = 0; a < 4; ++a) {
+        const int4 id = __ldg(reinterpret_cast<const int4*>(cage_idx) + v[a]);
+        if (id.x < 0) continue;
+        const int32_t ids[4] = {id.x, id.y, id.z, id.w};
+        for (int s = 0; s < 4; ++s) {
+          int at = cnt;
+          for (int u = 0; u < cnt; ++u)
+            if (nodes[u] == ids[s]) at = u;
+          if (at == cnt) nodes[cnt++] = ids[s];
+          map |= (uint64_t)at << (4 * (4 * a + s));
+        }
       }
     }
-    if (item_map) item_map[k] = map;
-    for (int u = 0; u < cnt; ++u) item_nodes[kMaxNodes * k + u] = nodes[u];
     item_n[k] = cnt;
     rc_h[k] = (int64_t)cnt * (cnt + 1) / 2;
     rc_g[k] = cnt;
+    if (cnt == 0) {
+      keys[k] = (1ull << key_bits) - 1;
+      continue;
+    }
+    uint64_t rank = 0;             // nibble u: place of nodes[u] in ascending order
+    int32_t first = nodes[0];
+    for (int u = 0; u < cnt; ++u) {
+      int r = 0;
+      for (int w = 0; w < cnt; ++w) r += nodes[w] < nodes[u];
+      rank |= (uint64_t)r << (4 * u);
+      item_nodes[kMaxNodes * k + r] = nodes[u];
+      first = min(first, nodes[u]);
+    }
+    uint32_t h = (uint32_t)cnt;    // order-free over the nodes: a sum of mixed offsets
+    for (int u = 0; u < cnt; ++u) {
+      uint32_t x = (uint32_t)(nodes[u] - first) * 0x9e3779b1u;
+      x = (x ^ (x >> 15)) * 0x85ebca6bu;
+      h += x ^ (x >> 13);
+    }
+    h = (h ^ (h >> 16)) * 0xc2b2ae35u;
+    keys[k] = (uint64_t)(uint32_t)first << kHashBits | (h >> (32 - kHashBits));
+    uint64_t sorted_map = 0;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) sorted_map |= (rank >> (4 * ((map >> (4 * q)) & 15u)) & 15ull) << (4 * q);
+    item_map[k] = sorted_map;
   }
 }
 
@@ -2033,36 +2072,129 @@ __global__ void __launch_bounds__(kBlock) k_full_entries(const uint64_t* __restr
   }
 }
 
-// keys of item k's Hessian records: record (u, v), u <= v, keyed by the upper-triangle position
-// of its nodes (min, max), and its source (item, local node of the row, of the column).  One
-// warp per item, lanes on consecutive records.
-__global__ void __launch_bounds__(kBlock) k_rec_keys(const int32_t* __restrict__ item_nodes,
-                                                     const int32_t* __restrict__ item_n, const int64_t* __restrict__ ro_h,
-                                                     const int64_t* n_items, int64_t rec_cap, int64_t ns,
+// ---- records.  Items with the same nodes -- 171k of the full bubble grasp have 9.7k node sets
+// between them -- are summed together before anything is sorted by block: sorted by key, a run of
+// items with equal nodes is a group, cut into chunks of kChunk items from its own start; a record is
+// one upper block (u, v) of a chunk.  2.57 M item records become about 0.35 M.  Group and chunk
+// borders depend only on the scene's own items, so sums are the same bits alone or in a batch.
+constexpr int kChunk = 16;
+
+// whether sorted item i starts a group (two sets with one key and hash part here as well)
+__device__ __forceinline__ bool group_head(int64_t i, const uint64_t* __restrict__ keys, const uint32_t* __restrict__ vals,
+                                           const int32_t* __restrict__ item_n, const int32_t* __restrict__ item_nodes) {
+  if (i == 0 || keys[i] != keys[i - 1]) return true;
+  const int64_t a = vals[i], b = vals[i - 1];
+  const int n = item_n[a];
+  if (n != item_n[b]) return true;
+  const int4* p = reinterpret_cast<const int4*>(item_nodes + kMaxNodes * a);
+  const int4* q = reinterpret_cast<const int4*>(item_nodes + kMaxNodes * b);
+  for (int u = 0; u < n; u += 4) {
+    const int4 x = p[u / 4], y = q[u / 4];
+    if (x.x != y.x || (u + 1 < n && x.y != y.y) || (u + 2 < n && x.z != y.z) || (u + 3 < n && x.w != y.w)) return true;
+  }
+  return false;
+}
+
+__global__ void __launch_bounds__(256) k_group_count(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ vals,
+                                                     const int64_t* n_items, const int32_t* __restrict__ item_n,
+                                                     const int32_t* __restrict__ item_nodes, int64_t* __restrict__ partial) {
+  pdl_entry();
+  __shared__ int wsum[8];
+  const int64_t n = *n_items, per = (n + gridDim.x - 1) / gridDim.x, b = blockIdx.x * per, e = b + per < n ? b + per : n;
+  int c = 0;
+  for (int64_t i = b + threadIdx.x; i < e; i += blockDim.x) c += group_head(i, keys, vals, item_n, item_nodes);
+  c = __reduce_add_sync(0xffffffffu, c);
+  if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = c;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int t = 0;
+    for (int w = 0; w < 8; ++w) t += wsum[w];
+    partial[blockIdx.x] = t;
+  }
+}
+
+__global__ void __launch_bounds__(256) k_group_start(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ vals,
+                                                     const int64_t* n_items, const int32_t* __restrict__ item_n,
+                                                     const int32_t* __restrict__ item_nodes,
+                                                     const int64_t* __restrict__ partial, int64_t* __restrict__ start) {
+  pdl_entry();
+  __shared__ int32_t wsum[8];
+  const int64_t n = *n_items, per = (n + gridDim.x - 1) / gridDim.x, b = blockIdx.x * per, e = b + per < n ? b + per : n;
+  int64_t run = partial[blockIdx.x];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  for (int64_t tile = b; tile < e; tile += 256) {
+    const int64_t i = tile + t;
+    const bool h = i < e && group_head(i, keys, vals, item_n, item_nodes);
+    const unsigned m = __ballot_sync(0xffffffffu, h);
+    if (lane == 0) wsum[warp] = __popc(m);
+    __syncthreads();
+    int before = 0, all = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+      before += w < warp ? wsum[w] : 0;
+      all += wsum[w];
+    }
+    if (h) start[run + before + __popc(m & ((1u << lane) - 1u))] = i;
+    __syncthreads();
+    run += all;
+  }
+}
+
+// records per group (none for the items without nodes, which end the order)
+__global__ void __launch_bounds__(kBlock) k_group_records(const int64_t* __restrict__ start, const int64_t* n_groups,
+                                                          const int64_t* n_items, const uint32_t* __restrict__ vals,
+                                                          const int32_t* __restrict__ item_n, int64_t* __restrict__ count) {
+  pdl_entry();
+  const int64_t G = *n_groups, N = *n_items;
+  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < G; g += grid_stride()) {
+    const int64_t b = start[g], e = g + 1 < G ? start[g + 1] : N;
+    const int n = item_n[vals[b]];
+    count[g] = (e - b + kChunk - 1) / kChunk * (n * (n + 1) / 2);
+  }
+}
+
+// Keys of the chunk records, and their source: first sorted item of the chunk, items - 1, local
+// node of the row and of the column.  One warp per group.
+__global__ void __launch_bounds__(kBlock) k_rec_keys(const int64_t* __restrict__ start, const int64_t* n_groups,
+                                                     const int64_t* n_items, const uint32_t* __restrict__ vals,
+                                                     const int32_t* __restrict__ item_n, const int32_t* __restrict__ item_nodes,
+                                                     const int64_t* __restrict__ offset, int64_t rec_cap, int64_t ns,
                                                      uint64_t* __restrict__ hkeys, uint32_t* __restrict__ hvals,
                                                      uint64_t* __restrict__ rec_src) {
   pdl_entry();
-  const int64_t nit = *n_items;
+  const int64_t G = *n_groups, N = *n_items;
   const int lane = threadIdx.x & 31;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t k = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < nit; k += nw) {
-    const int n = item_n[k];
-    const int32_t* nodes = item_nodes + kMaxNodes * k;
-    const int64_t oh = ro_h[k];
+  for (int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < G; g += nw) {
+    const int64_t b = start[g], e = g + 1 < G ? start[g + 1] : N, oh = offset[g];
+    const int64_t item = vals[b];
+    const int n = item_n[item];
+    if (n == 0) continue;
+    const int32_t* nodes = item_nodes + kMaxNodes * item;
     const int nrec = n * (n + 1) / 2;
-    for (int l = lane; l < nrec; l += 32) {
-      // row u of the upper triangle holds n - u records
-      int u = 0, before = 0;
-      while (before + (n - u) <= l) { before += n - u; ++u; }
-      const int w2 = u + (l - before);
+    const int64_t all = (e - b + kChunk - 1) / kChunk * nrec;
+    for (int64_t l = lane; l < all; l += 32) {
+      const int64_t c = l / nrec;
+      const int r = (int)(l - c * nrec);
+      int u = 0, before = 0;                 // row u of the upper triangle holds n - u records
+      while (before + (n - u) <= r) { before += n - u; ++u; }
+      const int w2 = u + (r - before);
       const int64_t pos = oh + l;
       if (pos >= rec_cap) continue;
-      const uint64_t Iu = (uint64_t)nodes[u], Iv = (uint64_t)nodes[w2];
-      hkeys[pos] = Iu <= Iv ? upper_key(Iu, Iv, (uint64_t)ns) : upper_key(Iv, Iu, (uint64_t)ns);
+      const int64_t first = b + c * kChunk, left = e - first;
+      hkeys[pos] = upper_key((uint64_t)nodes[u], (uint64_t)nodes[w2], (uint64_t)ns);
       hvals[pos] = (uint32_t)pos;
-      rec_src[pos] = (uint64_t)k << 8 | (uint64_t)(Iu <= Iv ? u : w2) << 4 | (uint64_t)(Iu <= Iv ? w2 : u);
+      rec_src[pos] = (uint64_t)first << 16 | (uint64_t)((left < kChunk ? left : kChunk) - 1) << 8 | (uint64_t)u << 4 | (uint64_t)w2;
     }
   }
+}
+
+// key of each segment (block) of the sorted records
+__global__ void __launch_bounds__(kBlock) k_seg_keys(const int64_t* __restrict__ start, const int64_t* n_seg,
+                                                     const uint64_t* __restrict__ keys, uint64_t* __restrict__ ukey) {
+  pdl_entry();
+  const int64_t S = *n_seg;
+  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < S; s += grid_stride()) ukey[s] = keys[start[s]];
 }
 
 // sorted full entries -> BSR columns, row counts, and for each upper segment s the BSR
@@ -2100,50 +2232,13 @@ __global__ void __launch_bounds__(kBlock) k_bsr_pattern(const uint64_t* __restri
   }
 }
 
-// Segment sums in two passes.  Each segment is cut into units of kSegChunk consecutive records
-// counted from its own first record; pass 1 sums each unit's records in order, pass 2 a
-// segment's unit sums in a fixed order.  The grouping depends only on the segment's own
-// records, so a scene's sums are the same bits whether it is evaluated alone or inside a
-// batch, and a long segment is spread over many threads.
-constexpr int kSegChunk = 16;
-
-// units per segment: unit[s] = ceil(len_s / kSegChunk) (exclusive-scanned afterwards),
-// and, when keys is given, the segment's key ukey[s]
-__global__ void __launch_bounds__(kBlock) k_seg_units(const int64_t* __restrict__ start, const int64_t* n_rec,
-                                                      const int64_t* n_seg, int64_t cap, int64_t* __restrict__ unit,
-                                                      const uint64_t* __restrict__ keys, uint64_t* __restrict__ ukey) {
-  pdl_entry();
-  const int64_t R = clamp_count(n_rec, cap);
-  const int64_t S = *n_seg;
-  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < S; s += grid_stride()) {
-    const int64_t b = start[s];
-    const int64_t len = ((s + 1 < S) ? start[s + 1] : R) - b;
-    unit[s] = (len + kSegChunk - 1) / kSegChunk;
-    if (keys) ukey[s] = keys[b];
-  }
-}
-
-// the segment owning unit u: largest s with unit[s] <= u (unit exclusive-scanned, S >= 1)
-__device__ __forceinline__ int64_t segment_of_unit(const int64_t* __restrict__ unit, int64_t S, int64_t u) {
-  int64_t lo = 0, hi = S - 1;
-  while (lo < hi) {
-    const int64_t mid = (lo + hi + 1) >> 1;
-    if (unit[mid] <= u) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
-}
-
 struct SumArgs {
-  const uint64_t* src;        // sources of the sorted records
-  const int64_t* ro_h;        // first record of each item, its node count (explicit records)
-  const int32_t* item_n;
-  const int64_t* start;
-  const int64_t* unit;
-  const int64_t* n_units;
+  const uint64_t* src;        // sources of the records
   const int64_t* n_rec;
-  const int64_t* n_seg;
   int64_t cap;
+  const uint32_t* items;      // items in group order
+  const int64_t* ro_h;        // first explicit record of each item, its node count
+  const int32_t* item_n;
   const int64_t* ro_g;
   const double* frow;
   const double* ihead;
@@ -2156,49 +2251,41 @@ __device__ __forceinline__ int sym_index(int p, int q) {   // (p, q) in B00 B01 
   return lo * (5 - lo) / 2 + hi;
 }
 
-// Pass 1: the units' sums, each record's block multiplied out of its item's factor rows (see
-// "pair factors") into the accumulators.  Bound by the FP64 pipe: three lanes per unit, lane i
-// of them accumulating row i of the block -- 7 or 10 FP64 instructions per record (without or
-// with friction), 30 of 32 lanes at work.  In a diagonal segment lane i takes entries (i, i) and
-// (i, i + 1 mod 3) of the symmetric block and, in place of the third, component i of the
-// gradient, with the same number of instructions.
-__global__ void __launch_bounds__(128) k_unit_sums(SumArgs A) {
+// The records' sums over their chunk's items, each block multiplied out of the item's factor rows
+// (see "pair factors") into the accumulators.  Bound by the FP64 pipe: three lanes per record, lane
+// i of them accumulating row i of the block -- 7 or 10 FP64 instructions per item (without or
+// with friction), 30 of 32 lanes at work, neighbouring lanes on the same items.  In a diagonal
+// record lane i takes entries (i, i) and (i, i + 1 mod 3) of the symmetric block and, in place of
+// the third, component i of the gradient, with the same number of instructions.
+__global__ void __launch_bounds__(128) k_chunk_sums(SumArgs A) {
   pdl_entry();
   const int64_t R = clamp_count(A.n_rec, A.cap);
-  const int64_t S = *A.n_seg;
-  const int64_t U = *A.n_units;
   const int lane = threadIdx.x & 31, sub = lane / 3, i = lane - 3 * sub;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  if (S <= 0) return;
-  for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w * 10 < U; w += nw) {
-    const int64_t u = w * 10 + sub;
-    if (lane >= 30 || u >= U) continue;
-    const int64_t s = segment_of_unit(A.unit, S, u);
-    const int64_t end = (s + 1 < S) ? A.start[s + 1] : R;
-    const int64_t b = A.start[s] + (u - A.unit[s]) * kSegChunk;
-    const int64_t e = (b + kSegChunk < end) ? b + kSegChunk : end;
-    uint64_t src = __ldg(A.src + b);
-    int64_t base = __ldg(A.ro_g + (src >> 8));
-    const bool diag = ((src >> 4) & 15) == (src & 15);
+  for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w * 10 < R; w += nw) {
+    const int64_t r = w * 10 + sub;
+    if (lane >= 30 || r >= R) continue;
+    const uint64_t src = __ldg(A.src + r);
+    const int lu = (int)((src >> 4) & 15), lv = (int)(src & 15), m = (int)((src >> 8) & 255) + 1;
+    const uint32_t* items = A.items + (src >> 16);
+    const bool diag = lu == lv;
     const int c0 = diag ? i : 0, c1 = diag ? (i == 2 ? 0 : i + 1) : 1;
     const int f0 = sym_index(i, c0), f1 = sym_index(i, c1), f2 = sym_index(i, 2);
+    int64_t item = __ldg(items), base = __ldg(A.ro_g + item);
     double a0 = 0.0, a1 = 0.0, a2 = 0.0;
-    for (int64_t r = b; r < e; ++r) {
-      const int64_t item = (int64_t)(src >> 8);
-      const int lu = (int)((src >> 4) & 15), lv = (int)(src & 15);
+    for (int q = 0; q < m; ++q) {
       const double* ru = A.frow + kFRow * (base + lu);
       const double* rv = A.frow + kFRow * (base + lv);
       const double* hd = A.ihead + kIHead * item;
-      // the next record's rows are found while this one's arrive
-      if (r + 1 < e) {
-        src = __ldg(A.src + r + 1);
-        base = __ldg(A.ro_g + (src >> 8));
+      const int64_t cur = item;
+      if (q + 1 < m) {                       // the next item's rows are found while this one's arrive
+        item = __ldg(items + q + 1);
+        base = __ldg(A.ro_g + item);
       }
       const double2 hf = __ldg(reinterpret_cast<const double2*>(hd) + 6);
       const int flags = (int)__double_as_longlong(hf.y);
       if (flags & kItemExplicit) {
-        const int lo = min(lu, lv), hi = max(lu, lv);
-        const double* B = A.hrec + kHRecStride * (A.ro_h[item] + lo * A.item_n[item] - lo * (lo - 1) / 2 + hi - lo);
+        const double* B = A.hrec + kHRecStride * (A.ro_h[cur] + lu * A.item_n[cur] - lu * (lu - 1) / 2 + lv - lu);
         a0 += diag ? B[f0] : B[3 * i];
         a1 += diag ? B[f1] : B[3 * i + 1];
         a2 += diag ? B[6 + i] : B[3 * i + 2];
@@ -2236,37 +2323,44 @@ __global__ void __launch_bounds__(128) k_unit_sums(SumArgs A) {
         else a2 += t;
       }
     }
-    double* p = A.piece + 9 * u + 3 * i;
+    double* p = A.piece + 9 * r + 3 * i;
     p[0] = a0; p[1] = a1; p[2] = a2;
   }
 }
 
-// Pass 2, one warp per segment: lane 9 q + c adds component c of unit sums q, q + 3, ... in
-// order, then the three chains are added; the block goes into the BSR values at dst[2s] and,
-// transposed, at dst[2s+1].  A diagonal segment (dst[2s+1] = -2) holds, per row i, entries (i, i)
-// and (i, i + 1 mod 3) of its symmetric block and component i of the gradient at its node, taken
-// from its first record's item.
-__global__ void __launch_bounds__(kBlock) k_segment_sums(const double* __restrict__ piece, const int64_t* __restrict__ unit,
-                                                         const int64_t* n_units, const int64_t* n_seg, int64_t cap,
+// The blocks, one warp per segment of the sorted records: lane 9 q + c adds component c of records
+// q, q + 3, ... in order, then the three chains are added; the block goes into the BSR values at
+// dst[2s] and, transposed, at dst[2s+1].  A diagonal segment (dst[2s+1] = -2) holds, per row i,
+// entries (i, i) and (i, i + 1 mod 3) of its symmetric block and component i of the gradient at its
+// node.
+__global__ void __launch_bounds__(kBlock) k_segment_sums(const double* __restrict__ piece, const uint32_t* __restrict__ perm,
+                                                         const int64_t* __restrict__ start, const int64_t* n_rec,
+                                                         const int64_t* n_seg, int64_t cap,
                                                          const int32_t* __restrict__ dst, eipc_bsr H,
-                                                         const int64_t* __restrict__ start, const uint64_t* __restrict__ src,
-                                                         const int32_t* __restrict__ item_nodes, double* __restrict__ g_r) {
+                                                         const uint64_t* __restrict__ ukey, int64_t ns,
+                                                         double* __restrict__ g_r) {
   pdl_entry();
+  const int64_t R = clamp_count(n_rec, cap);
   const int64_t S0 = *n_seg;
   const int64_t S = (2 * S0 <= cap) ? S0 : cap / 2;      // the segments k_full_entries kept
-  const int64_t U = *n_units;
   const int64_t nnzb = *H.nnzb;
   const int lane = threadIdx.x & 31, q = lane / 9, c = lane - 9 * q;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < S; s += nw) {
-    const int64_t u0 = unit[s], u1 = (s + 1 < S0) ? unit[s + 1] : U;
+    const int64_t b = start[s], e = (s + 1 < S0) ? start[s + 1] : R;
     double v = 0.0;
     if (q < 3) {
-      for (int64_t k = u0 + q; k < u1; k += 3) v += __ldg(piece + 9 * k + c);
+      int64_t k = b + q;
+      for (; k + 9 < e; k += 12) {           // four gathers in flight
+        const double x0 = __ldg(piece + 9 * (int64_t)__ldg(perm + k) + c), x1 = __ldg(piece + 9 * (int64_t)__ldg(perm + k + 3) + c);
+        const double x2 = __ldg(piece + 9 * (int64_t)__ldg(perm + k + 6) + c), x3 = __ldg(piece + 9 * (int64_t)__ldg(perm + k + 9) + c);
+        v += x0; v += x1; v += x2; v += x3;
+      }
+      for (; k < e; k += 3) v += __ldg(piece + 9 * (int64_t)__ldg(perm + k) + c);
     }
     const double v1 = __shfl_sync(0xffffffffu, v, c + 9), v2 = __shfl_sync(0xffffffffu, v, c + 18);
-    if (u1 - u0 > 1) v += v1;
-    if (u1 - u0 > 2) v += v2;
+    if (e - b > 1) v += v1;
+    if (e - b > 2) v += v2;
     if (q > 0) continue;
     const int32_t du = dst[2 * s], dl = dst[2 * s + 1];
     const int i = c / 3, k = c - 3 * i;
@@ -2274,8 +2368,7 @@ __global__ void __launch_bounds__(kBlock) k_segment_sums(const double* __restric
       if (du >= 0 && du < nnzb) H.val[9 * (int64_t)du + c] = v;
       if (dl >= 0 && dl < nnzb) H.val[9 * (int64_t)dl + 3 * k + i] = v;
     } else if (k == 2) {
-      const uint64_t sr = src[start[s]];
-      g_r[3 * (int64_t)item_nodes[kMaxNodes * (int64_t)(sr >> 8) + (int64_t)(sr & 15)] + i] = v;
+      g_r[3 * diagonal_node(ukey[s], (uint64_t)ns) + i] = v;
     } else if (du >= 0 && du < nnzb) {
       const int j = k == 0 ? i : (i == 2 ? 0 : i + 1);
       H.val[9 * (int64_t)du + 3 * i + j] = v;
@@ -2401,6 +2494,9 @@ void eval_launch(eipc_scene* sc, const double* q, const eipc_pairs& pr, const ei
   zero_ranges(s, {{cnt + kCntItems, 5 * sizeof(int64_t)}, {n_diag, sizeof(int64_t)},
                   {cnt + kCntEvalQueue, sizeof(int64_t)}, {cnt + kCntEvalRest, 2 * sizeof(int64_t)}, {n_moll, sizeof(int64_t)}, {g_r, sizeof(double) * 3 * sc->ns},
                   {merge ? sc->fric_of_pair : nullptr, sizeof(int32_t) * pcap}});
+  // group keys: the first node above kHashBits of hash (a fixed number: a scene's items must fall
+  // into the same groups whatever the size of the batch around it)
+  const int key_bits = sc->bits_g + kHashBits;
   const int32_t* fop = merge ? sc->fric_of_pair : nullptr;
   const int32_t* pof = merge ? sc->pair_of_fric : nullptr;
   sc->timers->start(kKItems, s);
@@ -2413,7 +2509,8 @@ void eval_launch(eipc_scene* sc, const double* q, const eipc_pairs& pr, const ei
                                                            fr ? lag->capacity : 0, sc->cage_idx, item_cap,
                                                            sc->item_nodes, sc->item_n, sc->item_group, sc->vgroup,
                                                            sc->rc_h, sc->rc_g,
-                                                           cnt + kCntItems, sc->status, fop, pof, sc->item_map);
+                                                           cnt + kCntItems, sc->status, fop, pof, sc->item_map, key_bits,
+                                                           sc->skeys, sc->svals);
   int64_t* tot_h = cnt + 9;
   int64_t* tot_g = cnt + 10;
   exclusive_scan2_i64(sc->rc_h, sc->ro_h, tot_h, sc->rc_g, sc->ro_g, tot_g, cnt + kCntItems, item_cap,
@@ -2433,9 +2530,9 @@ void eval_launch(eipc_scene* sc, const double* q, const eipc_pairs& pr, const ei
   A.fric_of_pair = fop; A.pair_of_fric = pof;
   A.lag = fr ? *lag : eipc_lag{};
   A.mu = p.mu; A.eps_f = p.eps_v * p.h;
-  A.moll_list = sc->svals;                   // the pair-sort buffers are free once the pairs are built
+  A.moll_list = reinterpret_cast<uint32_t*>(sc->rc_g);    // the record counts have been scanned
   A.n_moll = cnt + kCntMollList;
-  A.rest = sc->svals_alt;                    // the pair-sort buffers are free once the pairs are built
+  A.rest = reinterpret_cast<uint32_t*>(sc->rc_h);
   A.n_rest = cnt + kCntEvalRest;
   A.item_cap = item_cap;
   A.queue = cnt + kCntEvalQueue;
@@ -2458,55 +2555,65 @@ void eval_launch(eipc_scene* sc, const double* q, const eipc_pairs& pr, const ei
                          static_cast<const uint32_t*>(A.moll_list), static_cast<const int64_t*>(A.n_moll))));
     sc->timers->stop(kKEvalPair, sc->aux);
   }
-  cudaEventRecord(sc->ev_join, sc->aux);
 
-  // Hessian pattern: record keys (I, J) from the items' cage nodes, stable sort, segments (one
-  // per BSR upper block), then the full symmetric pattern (every off-diagonal upper block
-  // also at (J, I)), columns and row pointers
+  // groups of items with the same nodes, their chunks' records, and the records' sums (after the
+  // factors, on their stream); beside those, the Hessian pattern: record keys (I, J), stable
+  // sort, segments (one per BSR upper block), then the full symmetric pattern (every
+  // off-diagonal upper block also at (J, I)), columns and row pointers
   sc->timers->start(kKHReduce, s);
-  launch(k_rec_keys, blocks_for(32 * item_cap, 8), kBlock, 0, s, static_cast<const int32_t*>(sc->item_nodes),
-         static_cast<const int32_t*>(sc->item_n), static_cast<const int64_t*>(sc->ro_h),
-         static_cast<const int64_t*>(cnt + kCntItems), sc->rec_cap, sc->ns, sc->hkeys, sc->hvals, sc->rec_src);
-  const int wh = radix_sort_u64(sc->hkeys, sc->hvals, sc->hkeys_alt, sc->hvals_alt, cnt + kCntRecH, sc->rec_cap,
-                                sc->bits_h, sc->sort_hist, s);
+  const int wi = radix_sort_u64(sc->skeys, sc->svals, sc->skeys_alt, sc->svals_alt, cnt + kCntItems, item_cap, key_bits,
+                                sc->sort_hist, s);
+  const uint64_t* ik = wi ? sc->skeys_alt : sc->skeys;
+  const uint32_t* iv = wi ? sc->svals_alt : sc->svals;
+  const int64_t* n_items = cnt + kCntItems;
+  const int64_t* n_groups = cnt + kCntGroups;
+  const int64_t* n_rec = cnt + kCntRecords;
+  launch(k_group_count, kScanBlocks, 256, 0, s, ik, iv, n_items, static_cast<const int32_t*>(sc->item_n),
+         static_cast<const int32_t*>(sc->item_nodes), sc->scan_partial);
+  scan_partials(sc->scan_partial, cnt + kCntGroups, s);
+  launch(k_group_start, kScanBlocks, 256, 0, s, ik, iv, n_items, static_cast<const int32_t*>(sc->item_n),
+         static_cast<const int32_t*>(sc->item_nodes), static_cast<const int64_t*>(sc->scan_partial), sc->group_start);
+  int64_t* gcount = reinterpret_cast<int64_t*>(sc->gkeys);
+  int64_t* goffset = reinterpret_cast<int64_t*>(sc->gkeys_alt);
+  launch(k_group_records, blocks_for(item_cap, 8), kBlock, 0, s, static_cast<const int64_t*>(sc->group_start), n_groups, n_items,
+         iv, static_cast<const int32_t*>(sc->item_n), gcount);
+  exclusive_scan_i64(gcount, goffset, n_groups, item_cap, cnt + kCntRecords, sc->scan_partial, s);
+  launch(k_rec_keys, blocks_for(32 * item_cap, 8), kBlock, 0, s, static_cast<const int64_t*>(sc->group_start), n_groups, n_items,
+         iv, static_cast<const int32_t*>(sc->item_n), static_cast<const int32_t*>(sc->item_nodes),
+         static_cast<const int64_t*>(goffset), sc->rec_cap, sc->ns, sc->hkeys, sc->hvals, sc->rec_src);
+  cudaEventRecord(sc->ev_mid, s);
+  cudaStreamWaitEvent(sc->aux, sc->ev_mid, 0);
+  launch(k_chunk_sums, blocks_for(3 * sc->rec_cap, 32, 128), 128, 0, sc->aux,
+         SumArgs{sc->rec_src, n_rec, sc->rec_cap, iv, sc->ro_h, sc->item_n, sc->ro_g, sc->frow, sc->ihead, sc->hrec, sc->piece});
+  cudaEventRecord(sc->ev_join, sc->aux);
+  const int wh = radix_sort_u64(sc->hkeys, sc->hvals, sc->hkeys_alt, sc->hvals_alt, n_rec, sc->rec_cap, sc->bits_h,
+                                sc->sort_hist, s);
   const uint64_t* hk = wh ? sc->hkeys_alt : sc->hkeys;
   const uint32_t* hv = wh ? sc->hvals_alt : sc->hvals;
-  // segment starts, and each sorted record's source
-  segment_starts(hk, cnt + kCntRecH, sc->rec_cap, sc->seg_start, cnt + kCntSegH, sc->scan_partial, s, hv, sc->rec_src,
-                 sc->src_sorted);
+  segment_starts(hk, n_rec, sc->rec_cap, sc->seg_start, cnt + kCntSegH, sc->scan_partial, s);
   // seg_flag and seg_id hold the segment keys and the segments' BSR entries
   uint64_t* ukey = reinterpret_cast<uint64_t*>(sc->seg_flag);
   int32_t* dst = reinterpret_cast<int32_t*>(sc->seg_id);
-  launch(k_seg_units, blocks_for(sc->rec_cap), kBlock, 0, s, static_cast<const int64_t*>(sc->seg_start),
-         static_cast<const int64_t*>(cnt + kCntRecH), static_cast<const int64_t*>(cnt + kCntSegH), sc->rec_cap, sc->hunit,
-         hk, ukey);
-  exclusive_scan_i64(sc->hunit, sc->hunit, cnt + kCntSegH, sc->rec_cap, cnt + kCntUnitsH, sc->scan_partial, s);
+  launch(k_seg_keys, blocks_for(sc->rec_cap), kBlock, 0, s, static_cast<const int64_t*>(sc->seg_start),
+         static_cast<const int64_t*>(cnt + kCntSegH), hk, ukey);
   // row field: bits_g rounded up to whole radix digits (the sort passes cover whole bytes,
   // so the column must start on a byte); 2^bits_g > ns, so the all-ones row of the
-  // diagonal twins is above every row
+  // diagonal twins is above every row.  The group buffers are free here.
   const int rb = ((sc->bits_g + 7) / 8) * 8;
   launch(k_full_entries, blocks_for(sc->rec_cap), kBlock, 0, s, static_cast<const uint64_t*>(ukey),
-         static_cast<const int64_t*>(cnt + kCntSegH), sc->ns, rb, sc->rec_cap, sc->hkeys, sc->hvals, n_full, n_diag,
+         static_cast<const int64_t*>(cnt + kCntSegH), sc->ns, rb, sc->rec_cap, sc->gkeys, sc->gvals, n_full, n_diag,
          sc->status, dst);
-  const int wf = radix_sort_u64(sc->hkeys, sc->hvals, sc->hkeys_alt, sc->hvals_alt, n_full, sc->rec_cap, rb,
+  const int wf = radix_sort_u64(sc->gkeys, sc->gvals, sc->gkeys_alt, sc->gvals_alt, n_full, sc->rec_cap, rb,
                                 sc->sort_hist, s);
-  const uint64_t* fk = wf ? sc->hkeys_alt : sc->hkeys;
-  const uint32_t* fv = wf ? sc->hvals_alt : sc->hvals;
+  const uint64_t* fk = wf ? sc->gkeys_alt : sc->gkeys;
+  const uint32_t* fv = wf ? sc->gvals_alt : sc->gvals;
   launch(k_bsr_pattern, blocks_for(sc->rec_cap), kBlock, 0, s, fk, fv, static_cast<const int64_t*>(n_full),
          static_cast<const int64_t*>(n_diag), rb, sc->ns, H, dst, sc->status, cnt + kCntSegG);
-  sc->timers->stop(kKHReduce, s);
-
   cudaStreamWaitEvent(s, sc->ev_join, 0);
-  sc->timers->start(kKHReduce, s);
-  launch(k_unit_sums, blocks_for(3 * (sc->rec_cap / kSegChunk + 1), 32, 128), 128, 0, s,
-         SumArgs{sc->src_sorted, sc->ro_h, sc->item_n, sc->seg_start, sc->hunit, cnt + kCntUnitsH, cnt + kCntRecH, cnt + kCntSegH, sc->rec_cap,
-                 sc->ro_g, sc->frow, sc->ihead, sc->hrec, sc->piece});
   // blocks into the BSR values; the diagonal segments' gradients into g_r
-  launch(k_segment_sums, blocks_for(32 * sc->rec_cap, 8), kBlock, 0, s, static_cast<const double*>(sc->piece),
-         static_cast<const int64_t*>(sc->hunit), static_cast<const int64_t*>(cnt + kCntUnitsH),
-         static_cast<const int64_t*>(cnt + kCntSegH), sc->rec_cap, static_cast<const int32_t*>(dst), H,
-         static_cast<const int64_t*>(sc->seg_start), static_cast<const uint64_t*>(sc->src_sorted),
-         static_cast<const int32_t*>(sc->item_nodes), g_r);
+  launch(k_segment_sums, blocks_for(32 * sc->rec_cap, 8), kBlock, 0, s, static_cast<const double*>(sc->piece), hv,
+         static_cast<const int64_t*>(sc->seg_start), n_rec, static_cast<const int64_t*>(cnt + kCntSegH), sc->rec_cap,
+         static_cast<const int32_t*>(dst), H, static_cast<const uint64_t*>(ukey), sc->ns, g_r);
   sc->timers->stop(kKHReduce, s);
   // energy
   sc->timers->start(kKEnergy, s);

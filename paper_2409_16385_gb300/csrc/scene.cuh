@@ -73,13 +73,12 @@ struct eipc_scene {
   int64_t* seg_flag;     // [rec_cap] key of each Hessian segment (upper block), as uint64
   int64_t* seg_id;       // [rec_cap] BSR entries of each segment's block and transpose, as int32 pairs
   int64_t* seg_start;    // [rec_cap]
-  uint64_t* rec_src;     // [rec_cap] source of each Hessian record: item << 8 | row node << 4 | column node
-  uint64_t* src_sorted;  // [rec_cap] the same in sorted order
+  uint64_t* rec_src;     // [rec_cap] source of each record: first sorted item << 16 | items - 1 << 8 | nodes
+  int64_t* group_start;  // [gcap] first sorted item of each group of items with the same nodes
   double* frow;          // [gcap*kFRow] factor rows of the evaluated items, one per cage node (eval.cu)
   double* ihead;         // [item_cap*kIHead] headers of the evaluated items
   uint64_t* item_map;    // [item_cap] local node of each (vertex, slot) of an item, in nibbles
-  double* piece;         // [9 * (rec_cap + rec_cap / 32 + 2)] partial segment sums of the Hessian records
-  int64_t* hunit;        // [rec_cap + 1] first summation unit of each Hessian segment
+  double* piece;         // [9 * rec_cap] sums of the records
   int64_t gcap;          // factor rows; entries of the per-group energy sort
   uint64_t* gkeys;
   uint64_t* gkeys_alt;
@@ -102,7 +101,7 @@ struct eipc_scene {
   // barrier evaluation (they write disjoint records), forked from and joined back to the
   // caller's stream with two events, which also works inside a graph capture
   cudaStream_t aux;
-  cudaEvent_t ev_fork, ev_join;
+  cudaEvent_t ev_fork, ev_mid, ev_join;
 };
 
 namespace eipc {
@@ -115,10 +114,11 @@ constexpr int kHRecStride = 10;
 constexpr int kFRow = 12, kIHead = 16;
 
 enum { kCntCand = 0, kCntSurv = 1, kCntItems = 2, kCntRecH = 3, kCntRecG = 4, kCntSegH = 5, kCntSegG = 6,
-       kCntAccd = 7, kCntZero = 8, kCntEvalQueue = 16, kCntScreened = 15, kCntDedup = 17, kCntUnitsH = 18,
+       kCntAccd = 7, kCntZero = 8, kCntEvalQueue = 16, kCntScreened = 15, kCntDedup = 17,
        kCntMollBad = 20, kCntCcdQueue = 21, kCntCcdList = 22, kCntMollList = 23,
        kCntEvalRest = 24, /* two entries */
        kCntHvpTicket = 26,
+       kCntGroups = 27, kCntRecords = 18,
        kCntN = 28 };
 
 // device counters a kernel zeroes before the launches that count (null: none)

@@ -355,9 +355,7 @@ __global__ void __launch_bounds__(256) k_seg_heads_partial(const uint64_t* __res
 // exclusive partial
 __global__ void __launch_bounds__(256) k_seg_heads_write(const uint64_t* __restrict__ keys, const int64_t* n_dev,
                                                          int64_t cap, const int64_t* __restrict__ partial,
-                                                         int64_t* __restrict__ start, const uint32_t* __restrict__ perm,
-                                                         const uint64_t* __restrict__ src,
-                                                         uint64_t* __restrict__ src_sorted) {
+                                                         int64_t* __restrict__ start) {
   pdl_entry();
   __shared__ int32_t wsum[8];
   int64_t n = *n_dev;
@@ -368,7 +366,6 @@ __global__ void __launch_bounds__(256) k_seg_heads_write(const uint64_t* __restr
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   for (int64_t tile = beg; tile < end; tile += 256) {
     const int64_t i = tile + t;
-    if (src && i < end) src_sorted[i] = src[perm[i]];
     const bool h = i < end && seg_head(keys, i);
     const unsigned m = __ballot_sync(0xffffffffu, h);
     if (lane == 0) wsum[warp] = __popc(m);
@@ -446,11 +443,13 @@ void exclusive_scan2_i64(const int64_t* in_a, int64_t* out_a, int64_t* total_a, 
   launch(k_scan2_apply, kScanBlocks, 256, 0, s, in_a, out_a, in_b, out_b, n, cap, static_cast<const int64_t*>(partial));
 }
 
+void scan_partials(int64_t* partial, int64_t* total, cudaStream_t s) { launch(k_scan_partials, 1, 32, 0, s, partial, total); }
+
 void segment_starts(const uint64_t* keys, const int64_t* n, int64_t cap, int64_t* start, int64_t* n_seg,
-                    int64_t* partial, cudaStream_t s, const uint32_t* perm, const uint64_t* src, uint64_t* src_sorted) {
+                    int64_t* partial, cudaStream_t s) {
   launch(k_seg_heads_partial, kScanBlocks, 256, 0, s, keys, n, cap, partial);
   launch(k_scan_partials, 1, 32, 0, s, partial, n_seg);
-  launch(k_seg_heads_write, kScanBlocks, 256, 0, s, keys, n, cap, static_cast<const int64_t*>(partial), start, perm, src, src_sorted);
+  launch(k_seg_heads_write, kScanBlocks, 256, 0, s, keys, n, cap, static_cast<const int64_t*>(partial), start);
 }
 
 }  // namespace eipc

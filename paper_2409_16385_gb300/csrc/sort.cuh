@@ -34,13 +34,14 @@ void exclusive_scan_i64(const int64_t* in, int64_t* out, const int64_t* n, int64
 void exclusive_scan2_i64(const int64_t* in_a, int64_t* out_a, int64_t* total_a, const int64_t* in_b, int64_t* out_b,
                          int64_t* total_b, const int64_t* n, int64_t cap, int64_t* partial, cudaStream_t s);
 
+// Exclusive scan of kScanBlocks per-block counts in place, their sum to *total.
+void scan_partials(int64_t* partial, int64_t* total, cudaStream_t s);
+
 // Segments of a sorted key array keys[0 .. min(*n, cap)), a segment being a run of equal
 // keys: start[s] = position of segment s's first element, *n_seg = the number of segments.
-// With perm (the sort's values: the original index of each sorted element) and src, also
-// src_sorted[i] = src[perm[i]].  partial needs kScanBlocks + 1 entries.
+// partial needs kScanBlocks + 1 entries.
 void segment_starts(const uint64_t* keys, const int64_t* n, int64_t cap, int64_t* start, int64_t* n_seg,
-                    int64_t* partial, cudaStream_t s, const uint32_t* perm = nullptr, const uint64_t* src = nullptr,
-                    uint64_t* src_sorted = nullptr);
+                    int64_t* partial, cudaStream_t s);
 
 // Zeroes up to kZeroRanges byte ranges in one launch (each range 4-byte aligned, its
 // length a multiple of 4 bytes).  The library resets its counters and accumulators with
