@@ -1093,152 +1093,299 @@ __device__ __forceinline__ void light_factors(const EvalArgs& A, int64_t k, int 
   }
 }
 
-// ... of any pair: two free closest-point parameters (projected by the eigensolver of the span's
-// 5 x 5 matrix, which has exactly two negative eigenvalues then, so at most three columns), or a
-// region the FP32 test left open.
+// eigenvalues (big, small) of the symmetric [[a, b], [b, c]] and the unit eigenvector of the big one
+template <class T>
+__device__ __forceinline__ void eigen2(T a, T b, T c, T* big, T* small, T* y0, T* y1) {
+  const T h = T(0.5) * (a + c), dl = T(0.5) * (a - c), r2 = dl * dl + b * b;
+  const T r = r2 > T(0) ? r2 * rsqrt(r2) : T(0);
+  const T p = r + (dl < T(0) ? -dl : dl), n = p * p + b * b;
+  const T s = n > T(0) ? rsqrt(n) : T(0);
+  const T u = n > T(0) ? p * s : T(1), v = b * s;
+  *big = h + r;
+  *small = h - r;
+  *y0 = dl < T(0) ? v : u;
+  *y1 = dl < T(0) ? u : v;
+}
+
+// Pairs whose closest points have two free parameters: a point over a triangle's interior, two
+// edges' interiors.  n = e_1 x e_2 gives r^ = +-n/|n| and d = |w . n|/|n|.  With v_j = sum_a
+// a_j[a] x_a = L (p_1, p_2) (Gram-Schmidt, in the plane normal to r^) and a_j made orthonormal
+// against c and each other, the span c^ (x) r^, c^ (x) p_1, c^ (x) p_2, a^_1 (x) r^, a^_2 (x) r^ has
+//   K = diag(A, -B, -B, 0, 0) + B U U^T,  U = [x^T; I; Y],
+//   x = (d/|c|) L^-1 (c^.a_1, c^.a_2),  Y = (d/|c|) [a^_l . a_j] L^-T  (upper triangular),
+// with A, B as for one parameter.  Two entries of the diagonal part are negative and the rest is
+// positive, so K has exactly two negative eigenvalues -B mu: mu^2 = (1 - mu) N, where N is an
+// eigenvalue of W(tau) = Y^T Y + tau x x^T at tau = B mu/(A + B mu) and y its eigenvector, and
+// q = (tau/mu x.y, -y/(1 - mu), Y y/mu) spans K's eigenvector.  tau is found in FP32 and polished
+// in FP64 (N moves by (x.y)^2 dtau, so each pass squares the error); mu and 1 - mu come from N
+// without cancellation.  K+ = K + B sum mu q q^T/|q|^2 has rank three, taken by three steps of
+// Cholesky with the largest pivot.  Against a 12 x 12 eigensolver: 8e-12 at d = 7e-6 dhat, 1e-13
+// and below from 1e-3 dhat, near-parallel edges and slivers included.  About 700 FP64
+// instructions, where a 5 x 5 Jacobi eigensolver and its set-up took over 4,000: 130 us for a
+// warp of pairs before, 67 us after.
 __device__ __forceinline__ void heavy_factors(const EvalArgs& A, int64_t k) {
   int32_t v[4];
   const int type = A.pr.type[k];
   const int32_t i = A.pr.i[k], j = A.pr.j[k];
   stencil_vertices(A.T, type, i, j, v);
-  V3 Y[4];
-  const V3 X0 = load_x(A.x4, v[0]);
+  const int hint = stencil_hint(type, A.x4f, v);
+  V3 X[4];
 #pragma unroll
-  for (int a = 0; a < 4; ++a) Y[a] = load_x(A.x4, v[a]) - X0;
-  Stencil S;
-  closest_pair<true>(type, Y, stencil_hint(type, A.x4f, v), &S);
-  double d = 0.0;
-  bool active = false;
-  if (!(S.d2 > 0.0)) {
-    raise_flag(A.st, EIPC_FLAG_PENETRATION);
-  } else {
-    d = sqrt(S.d2);
-    active = lt_nonneg(d, A.dhat);
+  for (int a = 0; a < 4; ++a) X[a] = load_x(A.x4, v[a]);
+  const bool pt = type == 0;
+  double c[4];
+  V3 rh = {0.0, 0.0, 0.0};
+  double d = 0.0, inv_d = 0.0;
+  bool in, apart;
+  {
+    const V3 e1 = pt ? X[2] - X[1] : X[1] - X[0], e2 = pt ? X[3] - X[1] : X[3] - X[2], w = pt ? X[0] - X[1] : X[0] - X[2];
+    const V3 n = cross(e1, e2);
+    const double nn = dot(n, n), inv_nn = 1.0 / nn;
+    double s, t;
+    if (pt) {
+      s = dot(cross(w, e2), n) * inv_nn;
+      t = dot(cross(e1, w), n) * inv_nn;
+      in = s >= 0.0 && t >= 0.0 && s + t <= 1.0;
+      c[0] = 1.0; c[1] = -(1.0 - s - t); c[2] = -s; c[3] = -t;
+    } else {
+      const double a = dot(e1, e1), b = dot(e1, e2), cc = dot(e2, e2), dd = dot(e1, w), ee = dot(e2, w);
+      s = (b * ee - cc * dd) * inv_nn;
+      t = (a * ee - b * dd) * inv_nn;
+      in = nn > 1e-20 * a * cc && s >= 0.0 && s <= 1.0 && t >= 0.0 && t <= 1.0;
+      c[0] = 1.0 - s; c[1] = s; c[2] = -(1.0 - t); c[3] = -t;
+    }
+    in = in || (hint & kHintCertain);
+    const double h = dot(w, n), rn = rsqrt(nn), hs = h < 0.0 ? -rn : rn;
+    rh = n * hs;
+    d = h * hs;
+    apart = d > 0.0;
+    if (apart) inv_d = 1.0 / d;
   }
-  double eps_m, c_m;
-  if (active && ee_mollified(A, type, i, j, Y, &eps_m, &c_m)) {   // k_mollified
-    list_mollified(A, k);
+  if (!in) {                                   // the region the FP32 test left open: a segment after all
+    light_factors(A, k, type, i, j, v, pt ? 7 : 15);
     return;
+  }
+  if (!apart) raise_flag(A.st, EIPC_FLAG_PENETRATION);
+  const bool active = apart && lt_nonneg(d, A.dhat);
+  if (active && A.moll_r2 && type == 1) {
+    const V3 Y[4] = {{0.0, 0.0, 0.0}, X[1] - X[0], X[2] - X[0], X[3] - X[0]};
+    double eps_m, c_m;
+    if (ee_mollified(A, type, i, j, Y, &eps_m, &c_m)) {           // k_mollified_eval
+      list_mollified(A, k);
+      return;
+    }
   }
   const int n = A.item_n[k];
   const uint64_t map = A.item_map[k];
-  const int64_t base = A.ro_g[k];
-  double nw[3][kMaxNodes], wf[kMaxNodes];
-  for (int c = 0; c < 3; ++c) zero_nodes(nw[c], n);
+  double om[kMaxNodes], al[2][kMaxNodes], wf[kMaxNodes];
+  zero_nodes(om, n);
+  zero_nodes(al[0], n);
+  zero_nodes(al[1], n);
   zero_nodes(wf, n);
+  double E = 0.0, gs = 0.0, iso = 0.0;
+  // z_k = (omega f[k][0] + alpha_1 f[k][1] + alpha_2 f[k][2]) r^ + omega P[k]
+  double f[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
+  V3 P[3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
+  if (active) {
+    double b, b1, b2;
+    barrier_scalars(d, inv_d, A.dhat, A.inv_dhat, &b, &b1, &b2);
+    E = A.kappa * b;
+    gs = A.kappa * b1;
+    const double bd = -A.kappa * (b1 * inv_d);
+    // v_1, v_2 by Gram-Schmidt: v_1 = l11 p_1, v_2 = l21 p_1 + l22 p_2
+    const V3 v1 = pt ? X[1] - X[2] : X[1] - X[0], v2 = pt ? X[1] - X[3] : X[2] - X[3];
+    const double j11 = rsqrt(dot(v1, v1));
+    const V3 p1 = v1 * j11;
+    const double l21 = dot(v2, p1);
+    const V3 u2 = v2 - p1 * l21;
+    const double j22 = rsqrt(dot(u2, u2));
+    const V3 p2 = u2 * j22;
+    const double lj = l21 * j11;
+    if (A.project && is_pos(bd)) {
+      const double cc = c[0] * c[0] + c[1] * c[1] + c[2] * c[2] + c[3] * c[3], rcn = rsqrt(cc);
+      const double Aq = A.kappa * cc * b2, B = cc * bd;
+      const double k1 = (pt ? c[1] - c[2] : c[1] - c[0]) * rcn, k2 = (pt ? c[1] - c[3] : c[2] - c[3]) * rcn;
+      const double t11 = 2.0 - k1 * k1, i11 = rsqrt(t11), al11 = t11 * i11;
+      const double al12 = ((pt ? 1.0 : 0.0) - k1 * k2) * i11;
+      const double t22 = 2.0 - k2 * k2 - al12 * al12, i22 = rsqrt(t22), al22 = t22 * i22;
+      const double dc = d * rcn, d1 = dc * j11, d2 = dc * j22;
+      const double x1 = k1 * d1, x2 = (k2 - k1 * lj) * d2;
+      const double y11 = al11 * d1, y12 = (al12 - al11 * lj) * d2, y22 = al22 * d2;
+      const double w11 = y11 * y11, w12 = y11 * y12, w22 = y12 * y12 + y22 * y22;
+      const double s11 = x1 * x1, s12 = x1 * x2, s22 = x2 * x2;
+      double K[5][5];                          // upper triangle, over B
+      const double iB = 1.0 / B;
+      K[0][0] = Aq * iB + s11 + s22;
+      K[0][1] = x1; K[0][2] = x2; K[0][3] = x1 * y11 + x2 * y12; K[0][4] = x2 * y22;
+      K[1][1] = 0.0; K[1][2] = 0.0; K[1][3] = y11; K[1][4] = 0.0;
+      K[2][2] = 0.0; K[2][3] = y12; K[2][4] = y22;
+      K[3][3] = w11 + y12 * y12; K[3][4] = y12 * y22; K[4][4] = y22 * y22;
+      const double as = Aq * iB;               // A / B
+      const float af = to_float<0>(as), w11f = to_float<0>(w11), w12f = to_float<0>(w12), w22f = to_float<0>(w22);
+      const float s11f = to_float<0>(s11), s12f = to_float<0>(s12), s22f = to_float<0>(s22);
+      const double dy = y11 * y22, det0 = dy * dy, g1 = y12 * x1 - y11 * x2, g2 = y22 * x1, det1 = g1 * g1 + g2 * g2;
+      double q0[5];
+      double q0n = 0.0;
+#pragma unroll 1
+      for (int e = 0; e < 2; ++e) {
+        float tf = 0.f;
+#pragma unroll 1
+        for (int it = 0; it < 4; ++it) {
+          float big, sml, ya, yb;
+          eigen2<float>(w11f + tf * s11f, w12f + tf * s12f, w22f + tf * s22f, &big, &sml, &ya, &yb);
+          const float N = fmaxf(e == 0 ? big : sml, 1e-30f), mu = 2.f * N / (N + sqrtf(N * N + 4.f * N));
+          tf = __fdividef(mu, af + mu);
+        }
+        double tau = tf >= 0.f && tf <= 1.f ? (double)tf : 0.5;
+        double ya = 0.0, yb = 0.0, xy = 0.0, mu = 0.0, nu = 1.0;
+#pragma unroll 1
+        for (int it = 0; it < 8; ++it) {
+          double big, sml;
+          eigen2<double>(fma(tau, s11, w11), fma(tau, s12, w12), fma(tau, s22, w22), &big, &sml, &ya, &yb);
+          double N = big;
+          if (e == 1) {
+            N = fma(tau, det1, det0) / big;    // the small eigenvalue without cancellation
+            const double t = ya;
+            ya = -yb;
+            yb = t;
+          }
+          N = fmax(N, 1e-280);
+          xy = x1 * ya + x2 * yb;
+          // mu = 2N/(N + s), 1 - mu = 2/(N + 2 + s), s = sqrt(N^2 + 4N)
+          double s2 = N * (N + 4.0), s = s2 * rsqrt(s2), a = N + s, g = a + 2.0, rc = 2.0 / (a * g);
+          const double t1 = N * g * rc, tn = t1 / (as + t1), dt = tn - tau;
+          N = fma(xy * xy, dt, N);
+          N = fmax(N, 1e-280);
+          s2 = N * (N + 4.0); s = s2 * rsqrt(s2); a = N + s; g = a + 2.0; rc = 2.0 / (a * g);
+          mu = N * g * rc;
+          nu = a * rc;
+          tau = mu / (as + mu);
+          if (lt_nonneg(fabs(dt), 1e-9)) break;
+        }
+        // the eigenvector of K at -mu, times mu nu; the second made orthogonal to the first
+        double q[5] = {tau * xy * nu, -ya * mu, -yb * mu, (y11 * ya + y12 * yb) * nu, y22 * yb * nu};
+        if (e == 1) {
+          double pr = 0.0;
+#pragma unroll
+          for (int p = 0; p < 5; ++p) pr += q0[p] * q[p];
+          pr *= q0n;
+#pragma unroll
+          for (int p = 0; p < 5; ++p) q[p] -= pr * q0[p];
+        }
+        double qq = 0.0;
+#pragma unroll
+        for (int p = 0; p < 5; ++p) qq += q[p] * q[p];
+        const double iq = 1.0 / qq, m = mu * iq;
+#pragma unroll
+        for (int p = 0; p < 5; ++p) {
+          const double mp = m * q[p];
+#pragma unroll
+          for (int r = p; r < 5; ++r) K[p][r] = fma(mp, q[r], K[p][r]);
+        }
+        if (e == 0) {
+          q0n = iq;
+#pragma unroll
+          for (int p = 0; p < 5; ++p) q0[p] = q[p];
+        }
+      }
+      // three columns of Cholesky, times sqrt(B): r^ first, then the largest diagonal entries left
+      const double sB = B * rsqrt(B);
+      double S[4][4], l[3][5];
+      {
+        const double rk = rsqrt(K[0][0]);
+#pragma unroll
+        for (int p = 0; p < 5; ++p) l[0][p] = K[0][p] * rk;
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+          for (int r = p; r < 4; ++r) {
+            S[p][r] = fma(-l[0][1 + p], l[0][1 + r], K[1 + p][1 + r]);
+            S[r][p] = S[p][r];
+          }
+      }
+#pragma unroll
+      for (int col = 1; col < 3; ++col) {
+        int piv = 0;
+        double best = S[0][0];
+#pragma unroll
+        for (int p = 1; p < 4; ++p)
+          if (__double_as_longlong(S[p][p]) > __double_as_longlong(best)) { best = S[p][p]; piv = p; }
+        const double rp = is_pos(best) ? rsqrt(best) : 0.0;
+        double row[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          double x = S[0][r];
+          if (piv == 1) x = S[1][r];
+          if (piv == 2) x = S[2][r];
+          if (piv == 3) x = S[3][r];
+          row[r] = x * rp;
+          l[col][1 + r] = row[r];
+        }
+        l[col][0] = 0.0;
+        if (col == 1) {
+#pragma unroll
+          for (int p = 0; p < 4; ++p)
+#pragma unroll
+            for (int r = p; r < 4; ++r) {
+              S[p][r] = fma(-row[p], row[r], S[p][r]);
+              S[r][p] = S[p][r];
+            }
+        }
+      }
+      // omega^ = omega/|c|, alpha^_1 = (alpha_1 - k1 omega^)/al11, alpha^_2 = (alpha_2 - k2 omega^ - al12 alpha^_1)/al22
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const double m2 = l[q][4] * i22 * sB, m1 = (l[q][3] * sB - m2 * al12) * i11;
+        f[q][1] = m1;
+        f[q][2] = m2;
+        f[q][0] = (l[q][0] * sB - m1 * k1 - m2 * k2) * rcn;
+        P[q] = (p1 * l[q][1] + p2 * l[q][2]) * (sB * rcn);
+      }
+    } else {
+      // exact: r^, isotropic and G M^-1 G^T terms (the last as y_1 = (omega v_1 + alpha_1 r)/l11, y_2
+      // likewise less its share of y_1).  A projected pair whose b' has underflowed keeps r^ alone.
+      const double h = A.project ? A.kappa * b2 : fma(A.kappa, b2, bd);
+      f[0][0] = h * rsqrt(h);
+      if (!A.project) {
+        iso = -bd;
+        const double sb = is_pos(bd) ? bd * rsqrt(bd) : 0.0, q1 = sb * d * j11, q2 = sb * d * j22;
+        P[1] = p1 * sb;
+        f[1][1] = q1;
+        P[2] = p2 * sb;
+        f[2][2] = q2;
+        f[2][1] = -lj * q2;
+      }
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a) add_slots(A, v[a], (uint32_t)(map >> (16 * a)) & 0xffffu, c[a], om);
+    const int m1s = pt ? 2 : 0, p2s = pt ? 1 : 2;          // a_1 = +1 at 1, -1 at m1s; a_2 = +1 at p2s, -1 at 3
+    add_slots(A, v[1], (uint32_t)(map >> 16) & 0xffffu, 1.0, al[0]);
+    add_slots(A, pick(v, m1s), (uint32_t)(map >> (16 * m1s)) & 0xffffu, -1.0, al[0]);
+    add_slots(A, pick(v, p2s), (uint32_t)(map >> (16 * p2s)) & 0xffffu, 1.0, al[1]);
+    add_slots(A, v[3], (uint32_t)(map >> 48) & 0xffffu, -1.0, al[1]);
+  }
   const int32_t fenc = A.fric_of_pair ? A.fric_of_pair[k] : 0;
   FrictionTerms R;
-  double E = 0.0;
   if (fenc > 0) {
     double gam[4];
     friction_terms(A.x4, A.lag, (int64_t)(INT32_MAX - fenc), v, A.mu, A.eps_f, R, gam);
-    E = R.E;
+    E += R.E;
 #pragma unroll
     for (int a = 0; a < 4; ++a) add_slots(A, v[a], (uint32_t)(map >> (16 * a)) & 0xffffu, gam[a], wf);
   }
-  const FrictionTerms* Rp = fenc > 0 ? &R : nullptr;
-  int flags = fenc > 0 ? kItemFriction : 0;
-  if (!active) {
-    A.item_E[k] = E;
-    store_header(A.ihead + kIHead * k, Rp, V3{0.0, 0.0, 0.0}, 0.0, flags);
-    for (int u = 0; u < n && base + u < A.gcap; ++u)
-      store_row(A.frow + kFRow * (base + u), V3{0.0, 0.0, 0.0}, V3{0.0, 0.0, 0.0}, 0.0, wf[u]);
-    return;
-  }
-  BarrierSpan B;
-  barrier_span(Y, S, d, A.dhat, A.kappa, B);
-  A.item_E[k] = E + B.E;
-  const V3 rh = B.rh;
-  if (A.project) {
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int a = 0; a < 4; ++a) add_slots(A, v[a], (uint32_t)(map >> (16 * a)) & 0xffffu, B.basis[c][a], nw[c]);
-    double V[5][5];
-    eigen_sym<5>(B.K, V);
-    // columns of positive eigenvalue; a fourth can only be one at its rounding error: the
-    // smallest goes
-    double lam[5];
-    int cnt = 0, least = 0;
-#pragma unroll
-    for (int e = 0; e < 5; ++e) {
-      lam[e] = is_pos(B.K[e][e]) ? B.K[e][e] : 0.0;
-      cnt += lam[e] != 0.0;
-    }
-    for (; cnt > 3; --cnt) {
-      double lo = 0.0;
-#pragma unroll
-      for (int e = 0; e < 5; ++e)
-        if (lam[e] != 0.0 && (lo == 0.0 || lt_nonneg(lam[e], lo))) { lo = lam[e]; least = e; }
-#pragma unroll
-      for (int e = 0; e < 5; ++e)
-        if (e == least) lam[e] = 0.0;
-    }
-    flags |= kItemThird;
-    store_header(A.ihead + kIHead * k, Rp, rh * (A.kappa * B.b1 * B.cn), 0.0, flags);
-    double cols[3][5];                                            // sqrt(lambda) eigenvector
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int p = 0; p < 5; ++p) cols[c][p] = 0.0;
-    int at = 0;
-#pragma unroll
-    for (int e = 0; e < 5; ++e) {
-      if (lam[e] == 0.0) continue;
-      const double sl = sqrt(lam[e]);
-#pragma unroll
-      for (int c = 0; c < 3; ++c)
-        if (c == at) {
-#pragma unroll
-          for (int p = 0; p < 5; ++p) cols[c][p] = sl * V[p][e];
-        }
-      ++at;
-    }
-    for (int u = 0; u < n && base + u < A.gcap; ++u) {
-      V3 z[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c)
-        z[c] = V3{cols[c][0], cols[c][1], cols[c][2]} * nw[0][u] + rh * (nw[1][u] * cols[c][3] + nw[2][u] * cols[c][4]);
-      double* row = A.frow + kFRow * (base + u);
-      store_row(row, z[0], z[1], nw[0][u], wf[u]);
-      reinterpret_cast<double2*>(row)[4] = make_double2(z[2].x, z[2].y);
-      row[10] = z[2].z;
-    }
-    return;
-  }
-  // exact: r^, isotropic and G M^-1 G^T terms, M = L L^T
-#pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    add_slots(A, v[a], (uint32_t)(map >> (16 * a)) & 0xffffu, S.c[a], nw[0]);
-    add_slots2(A, v[a], (uint32_t)(map >> (16 * a)) & 0xffffu, S.a[0][a], nw[1], S.a[1][a], nw[2]);
-  }
-  const double inv_d = 1.0 / d;
-  double b, b1, b2;
-  barrier_scalars(d, inv_d, A.dhat, A.inv_dhat, &b, &b1, &b2);
-  const double bd = -A.kappa * (b1 * inv_d), h = fma(A.kappa, b2, bd), kr = sqrt(h);
-  V3 vj[2];
-  for (int c = 0; c < 2; ++c) {
-    vj[c] = {0.0, 0.0, 0.0};
-    for (int a = 0; a < 4; ++a) vj[c] = vj[c] + Y[a] * S.a[c][a];
-  }
-  // s G M^-1 G^T with s = bd / 2, G_j = 2 (omega v_j + alpha_j r): columns sqrt(2 s) L^-1 ( . )
-  const double sb = is_pos(bd) ? sqrt(bd) : 0.0;
-  double i1 = 0.0, l21 = 0.0, i2 = 0.0;
-  if (S.m > 0) i1 = rsqrt(dot(vj[0], vj[0]));
-  if (S.m > 1) {
-    l21 = dot(vj[0], vj[1]) * i1;
-    i2 = rsqrt(dot(vj[1], vj[1]) - l21 * l21);
-  }
-  flags |= kItemThird | kItemIso;
-  store_header(A.ihead + kIHead * k, Rp, rh * (A.kappa * b1), -bd, flags);
+  A.item_E[k] = E;
+  store_header(A.ihead + kIHead * k, fenc > 0 ? &R : nullptr, rh * gs, iso,
+               (fenc > 0 ? kItemFriction : 0) | (iso != 0.0 ? kItemIso : 0) | kItemThird);
+  const int64_t base = A.ro_g[k];
   for (int u = 0; u < n && base + u < A.gcap; ++u) {
-    const double o = nw[0][u];
-    const V3 y1 = (vj[0] * o + rh * (d * nw[1][u])) * i1;
-    const V3 y2 = (vj[1] * o + rh * (d * nw[2][u]) - y1 * l21) * i2;
+    const double o = om[u], a1 = al[0][u], a2 = al[1][u];
+    V3 z[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) z[q] = P[q] * o + rh * (o * f[q][0] + a1 * f[q][1] + a2 * f[q][2]);
     double* row = A.frow + kFRow * (base + u);
-    const V3 z3 = y2 * sb;
-    store_row(row, rh * (o * kr), y1 * sb, o, wf[u]);
-    reinterpret_cast<double2*>(row)[4] = make_double2(z3.x, z3.y);
-    row[10] = z3.z;
+    store_row(row, z[0], z[1], o, wf[u]);
+    reinterpret_cast<double2*>(row)[4] = make_double2(z[2].x, z[2].y);
+    row[10] = z[2].z;
   }
 }
 
