@@ -2263,12 +2263,15 @@ __global__ void __launch_bounds__(256) k_group_count(const uint64_t* __restrict_
 __global__ void __launch_bounds__(256) k_group_start(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ vals,
                                                      const int64_t* n_items, const int32_t* __restrict__ item_n,
                                                      const int32_t* __restrict__ item_nodes,
-                                                     const int64_t* __restrict__ partial, int64_t* __restrict__ start) {
+                                                     const int64_t* __restrict__ partial, int64_t* n_groups,
+                                                     int64_t* __restrict__ start) {
   pdl_entry();
   __shared__ int32_t wsum[8];
   const int64_t n = *n_items, per = (n + gridDim.x - 1) / gridDim.x, b = blockIdx.x * per, e = b + per < n ? b + per : n;
-  int64_t run = partial[blockIdx.x];
+  int64_t all_groups;
+  int64_t run = partials_before(partial, blockIdx.x, &all_groups);
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  if (blockIdx.x == 0 && t == 0) *n_groups = all_groups;
   for (int64_t tile = b; tile < e; tile += 256) {
     const int64_t i = tile + t;
     const bool h = i < e && group_head(i, keys, vals, item_n, item_nodes);
@@ -2717,9 +2720,8 @@ void eval_launch(eipc_scene* sc, const double* q, const eipc_pairs& pr, const ei
   const int64_t* n_rec = cnt + kCntRecords;
   launch(k_group_count, kScanBlocks, 256, 0, s, ik, iv, n_items, static_cast<const int32_t*>(sc->item_n),
          static_cast<const int32_t*>(sc->item_nodes), sc->scan_partial);
-  scan_partials(sc->scan_partial, cnt + kCntGroups, s);
   launch(k_group_start, kScanBlocks, 256, 0, s, ik, iv, n_items, static_cast<const int32_t*>(sc->item_n),
-         static_cast<const int32_t*>(sc->item_nodes), static_cast<const int64_t*>(sc->scan_partial), sc->group_start);
+         static_cast<const int32_t*>(sc->item_nodes), static_cast<const int64_t*>(sc->scan_partial), cnt + kCntGroups, sc->group_start);
   int64_t* gcount = reinterpret_cast<int64_t*>(sc->gkeys);
   int64_t* goffset = reinterpret_cast<int64_t*>(sc->gkeys_alt);
   launch(k_group_records, blocks_for(item_cap, 8), kBlock, 0, s, static_cast<const int64_t*>(sc->group_start), n_groups, n_items,

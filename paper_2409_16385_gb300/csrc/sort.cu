@@ -1,26 +1,31 @@
 // Stable LSD radix sort, exclusive scan and segment starts with device-resident element
 // counts.
 //
-// Radix pass (8-bit digit): each of kSortBlocks blocks owns one contiguous chunk of the
-// input.  (1) per-block digit histograms, (2) one block per digit turns its counts into
-// exclusive per-block prefixes and a digit total, (3) each block scans the 256 digit totals
-// for its digit bases and scatters its chunk tile by tile: warp peers
-// with equal digits are found with __match_any_sync, per-warp digit counts are prefix-
-// summed across the block's 8 warps, so every element lands at a position that preserves
-// input order among equal digits (stability is what makes the sort-and-reduce of the
-// reduced Hessian deterministic).
+// Radix pass (8-bit digit) in two launches: one block per SM owns one contiguous chunk of the
+// input.  (1) per-block digit histograms; (2) each block sums the histograms of the blocks before
+// it and of all blocks (152 x 256 counters, four threads per digit), scans the 256 totals for
+// its digit bases and scatters its chunk tile by tile: warp peers with equal digits are found
+// with __match_any_sync and per-warp digit counts are prefix-summed across the block's 32 warps,
+// so every element lands at a position that preserves input order among equal digits (stability
+// is what makes the sort-and-reduce of the reduced Hessian deterministic).  The sorts of a step
+// are short (a few thousand to a few hundred thousand elements), so a pass costs its launches:
+// with 1,216 blocks a third one had to turn the counters into offsets.  A block takes at least a
+// whole tile, so that short inputs have few counters to sum.  Per pass, caches flushed: sphere on
+// pad (a few thousand) 14.6 us in three launches, 11.2 us in two; bubble grasp (2 x 10^5) 17.7 and
+// 19.5 us, which the saved launch makes up for (evaluation 602 and 598 us).
 #include "common.cuh"
 #include "sort.cuh"
 
 namespace eipc {
 namespace {
 
-__device__ __forceinline__ void chunk_range(int64_t n, int64_t* beg, int64_t* end) {
+__device__ __forceinline__ int chunk_range(int64_t n, int64_t* beg, int64_t* end) {
   int64_t per = (n + kSortBlocks - 1) / kSortBlocks;
-  per = (per + kSortThreads - 1) / kSortThreads * kSortThreads;
+  per = per > kSortThreads ? (per + 31) / 32 * 32 : kSortThreads;     // at least one whole tile: fewer counters to sum
   *beg = (int64_t)blockIdx.x * per;
   int64_t e = *beg + per;
   *end = e < n ? e : n;
+  return (int)((n + per - 1) / per);           // blocks that have elements
 }
 
 __global__ void __launch_bounds__(kSortThreads) k_hist(const uint64_t* __restrict__ keys,
@@ -28,65 +33,24 @@ __global__ void __launch_bounds__(kSortThreads) k_hist(const uint64_t* __restric
                                                        uint32_t* __restrict__ hist) {
   pdl_entry();
   __shared__ uint32_t h[256];
-  for (int d = threadIdx.x; d < 256; d += blockDim.x) h[d] = 0;
+  if (threadIdx.x < 256) h[threadIdx.x] = 0;
   __syncthreads();
   int64_t n = *n_dev;
   if (n > cap) n = cap;
   int64_t beg, end;
   chunk_range(n, &beg, &end);
-  // one shared-memory atomic per distinct digit of a warp's 32 elements (the record keys of
-  // the reduction are heavily skewed: a few thousand distinct keys over millions)
+  if (beg >= end) return;                       // its counters are not read
+  // one shared-memory atomic per distinct digit of a warp's 32 elements (keys can be heavily
+  // skewed)
   const uint32_t lt_mask = (1u << (threadIdx.x & 31)) - 1u;
-  for (int64_t i0 = beg; i0 < end; i0 += blockDim.x) {
+  for (int64_t i0 = beg; i0 < end; i0 += kSortThreads) {
     const int64_t i = i0 + threadIdx.x;
     const uint32_t d = i < end ? (uint32_t)((keys[i] >> shift) & 255u) : 256u;
     const uint32_t peers = __match_any_sync(0xffffffffu, d);
     if (d < 256u && (peers & lt_mask) == 0u) atomicAdd(&h[d], (uint32_t)__popc(peers));
   }
   __syncthreads();
-  for (int d = threadIdx.x; d < 256; d += blockDim.x) hist[d * kSortBlocks + blockIdx.x] = h[d];
-}
-
-// One block per digit: exclusive prefix of that digit's counts over the blocks (in place)
-// and the digit's total, stored after the 256 * kSortBlocks counters.  Thread t owns the
-// consecutive counters [t * per, (t + 1) * per); a block scan of the threads' sums gives
-// each its starting offset.
-__global__ void __launch_bounds__(256) k_hist_digits(uint32_t* hist) {
-  pdl_entry();
-  constexpr int per = (kSortBlocks + 255) / 256;
-  __shared__ uint32_t wsum[8];
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  uint32_t* row = hist + (size_t)blockIdx.x * kSortBlocks;
-  uint32_t c[per];
-  uint32_t mine = 0;
-#pragma unroll
-  for (int k = 0; k < per; ++k) {
-    const int b = t * per + k;
-    c[k] = b < kSortBlocks ? row[b] : 0u;
-    mine += c[k];
-  }
-  uint32_t x = mine;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) wsum[warp] = x;
-  __syncthreads();
-  uint32_t before = 0, all = 0;
-#pragma unroll
-  for (int w = 0; w < 8; ++w) {
-    before += w < warp ? wsum[w] : 0u;
-    all += wsum[w];
-  }
-  uint32_t run = before + x - mine;
-#pragma unroll
-  for (int k = 0; k < per; ++k) {
-    const int b = t * per + k;
-    if (b < kSortBlocks) row[b] = run;
-    run += c[k];
-  }
-  if (t == 0) hist[256 * kSortBlocks + blockIdx.x] = all;
+  if (threadIdx.x < 256) hist[256 * blockIdx.x + threadIdx.x] = h[threadIdx.x];
 }
 
 __global__ void __launch_bounds__(kSortThreads) k_scatter(const uint64_t* __restrict__ kin,
@@ -94,67 +58,82 @@ __global__ void __launch_bounds__(kSortThreads) k_scatter(const uint64_t* __rest
                                                           uint64_t* __restrict__ kout,
                                                           uint32_t* __restrict__ vout,
                                                           const int64_t* n_dev, int64_t cap, int shift,
-                                                          const uint32_t* __restrict__ offs) {
+                                                          const uint32_t* __restrict__ hist) {
   pdl_entry();
   constexpr int W = kSortThreads / 32;
   __shared__ uint32_t base[256];
   __shared__ uint32_t wcnt[W][257];
-  __shared__ uint32_t total[256];
+  __shared__ uint32_t part[4][256];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int d = t & 255, q = t >> 8;            // digit and quarter of this thread in the digit sums
   int64_t n = *n_dev;
   if (n > cap) n = cap;
   int64_t beg, end;
-  chunk_range(n, &beg, &end);
-  // digit bases: exclusive scan of the 256 digit totals, plus this block's prefix
-  if (t < 256) total[t] = offs[256 * kSortBlocks + t];
-  __syncthreads();
-  if (t < 32) {
-    uint32_t run = 0;
-    for (int d0 = 0; d0 < 256; d0 += 32) {
-      const uint32_t c = total[d0 + t];
-      uint32_t x = c;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (t >= o) x += y;
-      }
-      base[d0 + t] = run + x - c;
-      run += __shfl_sync(0xffffffffu, x, 31);
+  const int blocks = chunk_range(n, &beg, &end);
+  if (beg >= end) return;
+  {
+    uint32_t before = 0, all = 0;
+#pragma unroll 8
+    for (int b = q; b < blocks; b += 4) {
+      const uint32_t c = __ldg(hist + 256 * b + d);
+      all += c;
+      before += b < (int)blockIdx.x ? c : 0u;
     }
+    part[q][d] = before;
+    wcnt[q][d] = all;
   }
   __syncthreads();
-  for (int d = t; d < 256; d += blockDim.x) base[d] += offs[d * kSortBlocks + blockIdx.x];
+  uint32_t total = 0, incl = 0;
+  if (t < 256) {                                // digit bases: exclusive scan of the 256 totals, plus this block's prefix
+    total = wcnt[0][t] + wcnt[1][t] + wcnt[2][t] + wcnt[3][t];
+    incl = total;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (lane == 31) wcnt[4][warp] = incl;
+  }
+  __syncthreads();
+  if (t < 256) {
+    uint32_t run = incl - total + part[0][t] + part[1][t] + part[2][t] + part[3][t];
+    for (int w = 0; w < warp; ++w) run += wcnt[4][w];
+    base[t] = run;
+  }
+  __syncthreads();
   const uint32_t lt_mask = (1u << lane) - 1u;
   for (int64_t tile = beg; tile < end; tile += kSortThreads) {
-    for (int d = lane; d < 257; d += 32) wcnt[warp][d] = 0;
-    __syncthreads();
-    int64_t i = tile + t;
-    bool valid = i < end;
-    uint64_t key = valid ? kin[i] : 0;
-    uint32_t val = valid ? vin[i] : 0;
-    uint32_t digit = valid ? (uint32_t)((key >> shift) & 255u) : 256u;
-    uint32_t peers = __match_any_sync(0xffffffffu, digit);
-    uint32_t rank = __popc(peers & lt_mask);
+    for (int e = lane; e < 257; e += 32) wcnt[warp][e] = 0;
+    __syncwarp();
+    const int64_t i = tile + t;
+    const bool valid = i < end;
+    const uint64_t key = valid ? kin[i] : 0;
+    const uint32_t val = valid ? vin[i] : 0;
+    const uint32_t digit = valid ? (uint32_t)((key >> shift) & 255u) : 256u;
+    const uint32_t peers = __match_any_sync(0xffffffffu, digit);
+    const uint32_t rank = __popc(peers & lt_mask);
     if (rank == 0) wcnt[warp][digit] = __popc(peers);
     __syncthreads();
-    if (t < 256) {
+    {                                           // eight warps' counts of digit d by each of its four threads
       uint32_t run = 0;
 #pragma unroll
-      for (int w = 0; w < W; ++w) {
-        uint32_t c = wcnt[w][t];
-        wcnt[w][t] = run;
+      for (int w = 0; w < W / 4; ++w) {
+        const uint32_t c = wcnt[q * (W / 4) + w][d];
+        wcnt[q * (W / 4) + w][d] = run;
         run += c;
       }
-      total[t] = run;
+      part[q][d] = run;
     }
     __syncthreads();
     if (valid) {
       uint32_t pos = base[digit] + wcnt[warp][digit] + rank;
+      const int wq = warp / (W / 4);
+      for (int p = 0; p < wq; ++p) pos += part[p][digit];
       kout[pos] = key;
       vout[pos] = val;
     }
     __syncthreads();
-    if (t < 256) base[t] += total[t];
+    if (t < 256) base[t] += part[0][t] + part[1][t] + part[2][t] + part[3][t];
   }
 }
 
@@ -193,41 +172,19 @@ __global__ void __launch_bounds__(256) k_scan_partial(const int64_t* __restrict_
   if (threadIdx.x == 0) partial[blockIdx.x] = s;
 }
 
-// exclusive scan of the kScanBlocks partial sums by one warp (chunks of 32 with a carry)
-__global__ void k_scan_partials(int64_t* partial, int64_t* total) {
-  pdl_entry();
-  const int lane = threadIdx.x & 31;
-  if (threadIdx.x >= 32 || blockIdx.x != 0) return;
-  int64_t run = 0;
-  for (int b0 = 0; b0 < kScanBlocks; b0 += 32) {
-    const int b = b0 + lane;
-    const int64_t c = b < kScanBlocks ? partial[b] : 0;
-    int64_t x = c;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    if (b < kScanBlocks) partial[b] = run + x - c;
-    run += __shfl_sync(0xffffffffu, x, 31);
-  }
-  if (lane == 0) {
-    partial[kScanBlocks] = run;
-    if (total) *total = run;
-  }
-}
-
 __global__ void __launch_bounds__(256) k_scan_apply(const int64_t* __restrict__ in, int64_t* __restrict__ out,
                                                     const int64_t* n_dev, int64_t cap,
-                                                    const int64_t* __restrict__ partial) {
+                                                    const int64_t* __restrict__ partial, int64_t* total) {
   pdl_entry();
   __shared__ int64_t tile_sum[256];
   int64_t n = *n_dev;
   if (n > cap) n = cap;
   int64_t beg, end;
   scan_range(n, &beg, &end);
-  int64_t run = partial[blockIdx.x];
+  int64_t all;
+  int64_t run = partials_before(partial, blockIdx.x, &all);
   const int t = threadIdx.x;
+  if (total && blockIdx.x == 0 && t == 0) *total = all;
   for (int64_t tile = beg; tile < end; tile += 256) {
     int64_t i = tile + t;
     int64_t v = (i < end) ? in[i] : 0;
@@ -247,7 +204,7 @@ __global__ void __launch_bounds__(256) k_scan_apply(const int64_t* __restrict__ 
 }
 
 // ---- two exclusive scans of the same length in the launches of one: partial holds
-// 2 (kScanBlocks + 1) entries, the first array's partials then the second's
+// 2 kScanBlocks entries, the first array's partials then the second's
 __global__ void __launch_bounds__(256) k_scan2_partial(const int64_t* __restrict__ a, const int64_t* __restrict__ b,
                                                        const int64_t* n_dev, int64_t cap, int64_t* __restrict__ partial) {
   pdl_entry();
@@ -264,33 +221,7 @@ __global__ void __launch_bounds__(256) k_scan2_partial(const int64_t* __restrict
   sb = block_sum_i64(sb);
   if (threadIdx.x == 0) {
     partial[blockIdx.x] = sa;
-    partial[kScanBlocks + 1 + blockIdx.x] = sb;
-  }
-}
-
-// exclusive scans of both partial arrays, one warp each
-__global__ void k_scan2_partials(int64_t* partial, int64_t* total_a, int64_t* total_b) {
-  pdl_entry();
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (w > 1 || blockIdx.x != 0) return;
-  int64_t* p = partial + w * (kScanBlocks + 1);
-  int64_t* total = w == 0 ? total_a : total_b;
-  int64_t run = 0;
-  for (int b0 = 0; b0 < kScanBlocks; b0 += 32) {
-    const int b = b0 + lane;
-    const int64_t c = b < kScanBlocks ? p[b] : 0;
-    int64_t x = c;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    if (b < kScanBlocks) p[b] = run + x - c;
-    run += __shfl_sync(0xffffffffu, x, 31);
-  }
-  if (lane == 0) {
-    p[kScanBlocks] = run;
-    if (total) *total = run;
+    partial[kScanBlocks + blockIdx.x] = sb;
   }
 }
 
@@ -298,15 +229,21 @@ __global__ void k_scan2_partials(int64_t* partial, int64_t* total_a, int64_t* to
 __global__ void __launch_bounds__(256) k_scan2_apply(const int64_t* __restrict__ a, int64_t* __restrict__ out_a,
                                                      const int64_t* __restrict__ b, int64_t* __restrict__ out_b,
                                                      const int64_t* n_dev, int64_t cap,
-                                                     const int64_t* __restrict__ partial) {
+                                                     const int64_t* __restrict__ partial, int64_t* total_a,
+                                                     int64_t* total_b) {
   pdl_entry();
   __shared__ int64_t ta[256], tb[256];
   int64_t n = *n_dev;
   if (n > cap) n = cap;
   int64_t beg, end;
   scan_range(n, &beg, &end);
-  int64_t run_a = partial[blockIdx.x], run_b = partial[kScanBlocks + 1 + blockIdx.x];
+  int64_t all_a, all_b;
+  int64_t run_a = partials_before(partial, blockIdx.x, &all_a), run_b = partials_before(partial + kScanBlocks, blockIdx.x, &all_b);
   const int t = threadIdx.x;
+  if (blockIdx.x == 0 && t == 0) {
+    *total_a = all_a;
+    *total_b = all_b;
+  }
   for (int64_t tile = beg; tile < end; tile += 256) {
     const int64_t i = tile + t;
     const int64_t va = (i < end) ? a[i] : 0, vb = (i < end) ? b[i] : 0;
@@ -354,7 +291,7 @@ __global__ void __launch_bounds__(256) k_seg_heads_partial(const uint64_t* __res
 // start[s] = position of the s-th head: each chunk ranks its heads tile by tile from its
 // exclusive partial
 __global__ void __launch_bounds__(256) k_seg_heads_write(const uint64_t* __restrict__ keys, const int64_t* n_dev,
-                                                         int64_t cap, const int64_t* __restrict__ partial,
+                                                         int64_t cap, const int64_t* __restrict__ partial, int64_t* n_seg,
                                                          int64_t* __restrict__ start) {
   pdl_entry();
   __shared__ int32_t wsum[8];
@@ -362,8 +299,10 @@ __global__ void __launch_bounds__(256) k_seg_heads_write(const uint64_t* __restr
   if (n > cap) n = cap;
   int64_t beg, end;
   scan_range(n, &beg, &end);
-  int64_t run = partial[blockIdx.x];
+  int64_t all_seg;
+  int64_t run = partials_before(partial, blockIdx.x, &all_seg);
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  if (blockIdx.x == 0 && t == 0) *n_seg = all_seg;
   for (int64_t tile = beg; tile < end; tile += 256) {
     const int64_t i = tile + t;
     const bool h = i < end && seg_head(keys, i);
@@ -422,7 +361,6 @@ int radix_sort_u64(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, uint32_t*
     uint64_t* ko = which ? keys : keys_alt;
     uint32_t* vo = which ? vals : vals_alt;
     launch(k_hist, kSortBlocks, kSortThreads, 0, s, ki, n, cap, shift, hist);
-    launch(k_hist_digits, 256, 256, 0, s, hist);
     launch(k_scatter, kSortBlocks, kSortThreads, 0, s, ki, vi, ko, vo, n, cap, shift, hist);
     which ^= 1;
   }
@@ -432,24 +370,20 @@ int radix_sort_u64(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, uint32_t*
 void exclusive_scan_i64(const int64_t* in, int64_t* out, const int64_t* n, int64_t cap, int64_t* total,
                         int64_t* partial, cudaStream_t s) {
   launch(k_scan_partial, kScanBlocks, 256, 0, s, in, n, cap, partial);
-  launch(k_scan_partials, 1, 32, 0, s, partial, total);
-  launch(k_scan_apply, kScanBlocks, 256, 0, s, in, out, n, cap, partial);
+  launch(k_scan_apply, kScanBlocks, 256, 0, s, in, out, n, cap, partial, total);
 }
 
 void exclusive_scan2_i64(const int64_t* in_a, int64_t* out_a, int64_t* total_a, const int64_t* in_b, int64_t* out_b,
                          int64_t* total_b, const int64_t* n, int64_t cap, int64_t* partial, cudaStream_t s) {
   launch(k_scan2_partial, kScanBlocks, 256, 0, s, in_a, in_b, n, cap, partial);
-  launch(k_scan2_partials, 1, 64, 0, s, partial, total_a, total_b);
-  launch(k_scan2_apply, kScanBlocks, 256, 0, s, in_a, out_a, in_b, out_b, n, cap, static_cast<const int64_t*>(partial));
+  launch(k_scan2_apply, kScanBlocks, 256, 0, s, in_a, out_a, in_b, out_b, n, cap, static_cast<const int64_t*>(partial), total_a,
+         total_b);
 }
-
-void scan_partials(int64_t* partial, int64_t* total, cudaStream_t s) { launch(k_scan_partials, 1, 32, 0, s, partial, total); }
 
 void segment_starts(const uint64_t* keys, const int64_t* n, int64_t cap, int64_t* start, int64_t* n_seg,
                     int64_t* partial, cudaStream_t s) {
   launch(k_seg_heads_partial, kScanBlocks, 256, 0, s, keys, n, cap, partial);
-  launch(k_scan_partials, 1, 32, 0, s, partial, n_seg);
-  launch(k_seg_heads_write, kScanBlocks, 256, 0, s, keys, n, cap, static_cast<const int64_t*>(partial), start);
+  launch(k_seg_heads_write, kScanBlocks, 256, 0, s, keys, n, cap, static_cast<const int64_t*>(partial), n_seg, start);
 }
 
 }  // namespace eipc

@@ -8,11 +8,11 @@
 
 namespace eipc {
 
-constexpr int kSortBlocks = 1216;  // 8 per SM; each block owns one contiguous chunk
-constexpr int kSortThreads = 256;  // 8 warps, one element per thread per tile
+constexpr int kSortBlocks = 152;    // one per SM; each block owns one contiguous chunk
+constexpr int kSortThreads = 1024;  // 32 warps, one element per thread per tile
 
-// Scratch: 256 * kSortBlocks digit counters followed by 256 digit totals.
-inline size_t sort_hist_entries() { return 256u * kSortBlocks + 256u; }
+// Scratch: 256 digit counters per block.
+inline size_t sort_hist_entries() { return 256u * kSortBlocks; }
 
 // Stable LSD radix sort of (keys[i], vals[i]), i < min(*n, cap), by the key's bits
 // [start_bit, start_bit + 8 ceil(bits / 8)) in 8-bit digits: bits below start_bit are
@@ -24,22 +24,47 @@ int radix_sort_u64(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, uint32_t*
                    const int64_t* n, int64_t cap, int bits, uint32_t* hist, cudaStream_t s, int start_bit = 0);
 
 // out[i] = sum_{k<i} in[k] for i < min(*n, cap); *total = the full sum.
-// partial needs kScanBlocks + 1 entries.
+// partial needs kScanBlocks entries.
 constexpr int kScanBlocks = 304;
 void exclusive_scan_i64(const int64_t* in, int64_t* out, const int64_t* n, int64_t cap,
                         int64_t* total, int64_t* partial, cudaStream_t s);
 
-// Two exclusive scans over the same count in three launches (as two exclusive_scan_i64
-// calls).  partial needs 2 (kScanBlocks + 1) entries.
+// Two exclusive scans over the same count in two launches (as two exclusive_scan_i64
+// calls).  partial needs 2 kScanBlocks entries.
 void exclusive_scan2_i64(const int64_t* in_a, int64_t* out_a, int64_t* total_a, const int64_t* in_b, int64_t* out_b,
                          int64_t* total_b, const int64_t* n, int64_t cap, int64_t* partial, cudaStream_t s);
 
-// Exclusive scan of kScanBlocks per-block counts in place, their sum to *total.
-void scan_partials(int64_t* partial, int64_t* total, cudaStream_t s);
+// The kScanBlocks per-block sums of a scan, summed before block `block`, and in all.  Called by
+// every thread of a block of 256 threads.
+#ifdef __CUDACC__
+__device__ __forceinline__ int64_t partials_before(const int64_t* __restrict__ partial, int block, int64_t* all) {
+  __shared__ int64_t before_w[8], all_w[8];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  int64_t b = 0, a = 0;
+  for (int q = t; q < kScanBlocks; q += 256) {
+    const int64_t c = partial[q];
+    a += c;
+    b += q < block ? c : 0;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    b += __shfl_xor_sync(0xffffffffu, b, o);
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+  }
+  if (lane == 0) { before_w[warp] = b; all_w[warp] = a; }
+  __syncthreads();
+  b = a = 0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) { b += before_w[w]; a += all_w[w]; }
+  __syncthreads();
+  *all = a;
+  return b;
+}
+#endif
 
 // Segments of a sorted key array keys[0 .. min(*n, cap)), a segment being a run of equal
 // keys: start[s] = position of segment s's first element, *n_seg = the number of segments.
-// partial needs kScanBlocks + 1 entries.
+// partial needs kScanBlocks entries.
 void segment_starts(const uint64_t* keys, const int64_t* n, int64_t cap, int64_t* start, int64_t* n_seg,
                     int64_t* partial, cudaStream_t s);
 
