@@ -304,23 +304,44 @@ __device__ __forceinline__ bool box_overlap(const float* lo, const float* hi, co
 }
 
 // ---------------------------------------------------------------- traversal
-// A warp answers 32 queries that are neighbours in Morton order.  (1) It walks the nodes above the
-// treelets once for all of them, depth first: the node is one 64-byte broadcast read, each lane
-// tests its own query against both children, and a child is followed if any lane meets it.  33
-// nodes per warp on the 256-scene batch, where a walk per query visited 31 and a warp of such
-// walks took 47 steps with 13 of 32 lanes active.  Stack and treelet list are spread over the
-// lanes' registers.  (2) Each treelet reached is tested a lane per leaf: its leaf boxes arrive in
-// one coalesced read, fetched one treelet ahead, and each query that met the treelet is compared
-// with all its leaves at once.  Candidates go to a buffer of the warp and out with one global
-// atomic per flush.  Contact
-// set of the bubble grasp: 180 us, with a walk per query 215 us.
+// A warp answers 32 queries that are neighbours in Morton order.  Instructions bound it, then the
+// chain of dependent node reads.  (1) It walks the nodes above the treelets with two boxes, the
+// unions of its queries before and after their largest jump, sixteen waiting nodes at a time, a
+// lane per child box: nearly always a level of the tree per step, 17 steps on the 256-scene
+// batch.  The two meet 11 treelets there and the queries themselves 9, while tests of every node
+// by every query (one node a step) took 33 steps of more instructions each.  (With one union a
+// percent of the warps met hundreds of nodes and held up the kernel; queries so scattered that
+// two do not do go on in the one-node form.)  (2) Each query tests the boxes of those treelets;
+// the ballot is the set of queries that the treelet concerns.  (3) A treelet is tested a lane per
+// leaf: its leaf boxes arrive in one coalesced read, fetched one treelet ahead, and each query
+// that met the treelet is compared with all its leaves at once.  Candidates go to a buffer of
+// the warp and out with one global atomic per flush.  256-scene batch 2,230 us with every query
+// testing every node, 2,036 us so; bubble grasp's contact set 181 and 157 us; sphere on pad 53 and
+// 41 us.
 constexpr int kQueryBuf = 128;         // candidates; flushed when a treelet's 32 might not fit
+constexpr int kNear = 64;              // treelets; handled when a step's 32 might not fit
+constexpr int kWaiting = 128;          // nodes to visit
+constexpr int kWaitingWide = 48;       // past this the queries are taken as scattered: one node at a time from then on
 
 struct QueryWarp {
-  float4 box[32][2];                   // lo xyz, hi x | hi yz, id, -
-  int4 info[32];                       // vertices a, b (PT: both the vertex), own leaf position, kin | group << 1
+  float4 box[32][2];                   // lo xyz, hi x | hi yz, id, own leaf position
+  int4 info[32];                       // vertices a, b (PT: both the vertex), -, kin | group << 1
+  float4 near[kNear][2];               // lo xyz, hi x | hi yz, first leaf, leaves | kin << 8
   uint64_t cand[kQueryBuf];
+  int32_t waiting[kWaiting];
 };
+
+// min and max over the warp (no NaN reaches a box)
+__device__ __forceinline__ float warp_fmin(float v) {
+  float r;
+  asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
+}
+__device__ __forceinline__ float warp_fmax(float v) {
+  float r;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
+}
 
 __device__ __forceinline__ void flush_candidates(QueryWarp& W, int count, uint64_t* cand, int64_t* n_cand, int64_t cap,
                                                  DevStatus* st, int lane) {
@@ -376,120 +397,160 @@ __global__ void __launch_bounds__(256, 4) k_query(Bvh tt, Bvh te, Topo T, const 
         qpos = (int32_t)qi;                // each EE pair is found once, from the edge earlier in Morton order
       }
       verts_box(vbox_q, a, pt ? -1 : b, -1, qlo, qhi);
-      W.info[lane] = make_int4(a, b, qpos, (kin ? 1 : 0) | (T.vgroup[a] << 1));
+      W.info[lane] = make_int4(a, b, 0, (kin ? 1 : 0) | (T.vgroup[a] << 1));
       W.box[lane][0] = make_float4(qlo[0], qlo[1], qlo[2], qhi[0]);
-      W.box[lane][1] = make_float4(qhi[1], qhi[2], __int_as_float(id), 0.f);
+      W.box[lane][1] = make_float4(qhi[1], qhi[2], __int_as_float(id), __int_as_float(qpos));
     }
+    // the queries from `cut` on, whose box with its predecessor's is the longest, have a union of
+    // their own
+    float jump = 0.f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const float plo = __shfl_up_sync(0xffffffffu, qlo[k], 1), phi = __shfl_up_sync(0xffffffffu, qhi[k], 1);
+      jump = fmaxf(jump, fmaxf(qhi[k], phi) - fminf(qlo[k], plo));
+    }
+    if (lane == 0 || !(jump < INFINITY)) jump = 0.f;
+    const int cut = __ffs(__ballot_sync(0xffffffffu, jump == warp_max(jump))) - 1;
+    float ulo[2][3], uhi[2][3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      ulo[0][k] = warp_min(lane < cut ? qlo[k] : INFINITY);
+      uhi[0][k] = warp_max(lane < cut ? qhi[k] : -INFINITY);
+      ulo[1][k] = warp_min(lane < cut ? INFINITY : qlo[k]);
+      uhi[1][k] = warp_max(lane < cut ? -INFINITY : qhi[k]);
+    }
+    const int32_t upos = __reduce_min_sync(0xffffffffu, qpos);
+    const bool ukin = __all_sync(0xffffffffu, kin);
     __syncwarp();
-    int kept = 0;                            // candidates in the buffer (the same in all lanes)
-    int listed = 0, l_first = 0, l_count = 0;      // treelet t of the list is lane t's
-    unsigned l_mask = 0;
-    auto list = [&](int first, int count, unsigned mask) {
-      if (lane == listed) { l_first = first; l_count = count; l_mask = mask; }
-      ++listed;
-    };
-    // the listed treelets, their leaf boxes fetched one ahead
+    int kept = 0, listed = 0;                // candidates and treelets in the buffers (the same in all lanes)
     auto handle = [&]() {
-      float4 nb0 = make_float4(0.f, 0.f, 0.f, 0.f), nb1 = nb0;
-      int nfirst = __shfl_sync(0xffffffffu, l_first, 0), ncount = __shfl_sync(0xffffffffu, l_count, 0);
-      auto fetch = [&]() {
-        if (lane < ncount) {
-          const float4* p = reinterpret_cast<const float4*>(leaf_box + 8 * ((int64_t)nfirst + lane));
-          nb0 = __ldg(p);
-          nb1 = __ldg(p + 1);
+      for (int base = 0; base < listed; base += 32) {
+        const int m = listed - base < 32 ? listed - base : 32;
+        unsigned mask = 0;                   // lane t: the queries that meet treelet t
+        for (int t = 0; t < m; ++t) {
+          const float4 b0 = W.near[base + t][0], b1 = W.near[base + t][1];
+          const float lo[3] = {b0.x, b0.y, b0.z}, hi[3] = {b0.w, b1.x, b1.y};
+          const int tail = __float_as_int(b1.w), last = __float_as_int(b1.z) + (tail & 255) - 1;
+          const unsigned meet = __ballot_sync(0xffffffffu, box_overlap(lo, hi, qlo, qhi) && last > qpos && !(kin && tail > 255));
+          if (lane == t) mask = meet;
         }
-      };
-      if (listed > 0) fetch();
-      for (int t = 0; t < listed; ++t) {
-        const float llo[3] = {nb0.x, nb0.y, nb0.z}, lhi[3] = {nb0.w, nb1.x, nb1.y};
-        const int32_t m = ncount, lpos = nfirst + lane;
-        unsigned mask = __shfl_sync(0xffffffffu, l_mask, t);
-        if (t + 1 < listed) {
-          nfirst = __shfl_sync(0xffffffffu, l_first, t + 1);
-          ncount = __shfl_sync(0xffffffffu, l_count, t + 1);
-          fetch();
-        }
-        int4 li = make_int4(0, 0, 0, 0);
-        bool loaded = false;
-        while (mask) {
-          const int q = __ffs(mask) - 1;
-          mask &= mask - 1;
-          const float4 q0 = W.box[q][0], q1 = W.box[q][1];
-          const float blo[3] = {q0.x, q0.y, q0.z}, bhi[3] = {q0.w, q1.x, q1.y};
-          const int4 qn = W.info[q];
-          bool hit = lane < m && lpos > qn.z && box_overlap(llo, lhi, blo, bhi);
-          if (!__any_sync(0xffffffffu, hit)) continue;
-          if (!loaded) {
-            loaded = true;
-            if (lane < m) li = __ldg(leaf_info + lpos);
+        unsigned live = __ballot_sync(0xffffffffu, mask != 0);
+        float4 nb0 = make_float4(0.f, 0.f, 0.f, 0.f), nb1 = nb0;
+        int4 nli = make_int4(0, 0, 0, 0);
+        int nfirst = 0, ncount = 0;
+        auto fetch = [&](int t) {
+          nfirst = __float_as_int(W.near[base + t][1].z);
+          ncount = __float_as_int(W.near[base + t][1].w) & 255;
+          if (lane < ncount) {
+            const float4* p = reinterpret_cast<const float4*>(leaf_box + 8 * ((int64_t)nfirst + lane));
+            nb0 = __ldg(p);
+            nb1 = __ldg(p + 1);
+            nli = __ldg(leaf_info + nfirst + lane);
           }
-          hit = hit && li.x != qn.x && li.y != qn.x && li.z != qn.x && li.x != qn.y && li.y != qn.y && li.z != qn.y &&
-                !(qn.w & li.w & 1) && (qn.w >> 1) == (li.w >> 1);
-          const unsigned mh = __ballot_sync(0xffffffffu, hit);
-          if (!mh) continue;
-          if (hit) {
-            const uint32_t id = (uint32_t)__float_as_int(q1.z), prim = __ldg(leaf_prim + lpos);
-            const uint32_t lo32 = pt ? id : (id < prim ? id : prim), hi32 = pt ? prim : (id < prim ? prim : id);
-            W.cand[kept + __popc(mh & below)] = pair_key(pt ? 0 : 1, lo32, hi32, T.bits_i, T.bits_j);
-          }
-          kept += __popc(mh);
-          if (kept > kQueryBuf - 32) {
-            flush_candidates(W, kept, cand, n_cand, cap, st, lane);
-            kept = 0;
+        };
+        if (live) fetch(__ffs(live) - 1);
+        while (live) {
+          unsigned todo = __shfl_sync(0xffffffffu, mask, __ffs(live) - 1);
+          live &= live - 1;
+          const float llo[3] = {nb0.x, nb0.y, nb0.z}, lhi[3] = {nb0.w, nb1.x, nb1.y};
+          const int4 li = nli;
+          const int32_t lpos = lane < ncount ? nfirst + lane : -2;       // -2: below every query's position
+          if (live) fetch(__ffs(live) - 1);
+          while (todo) {
+            const int q = __ffs(todo) - 1;
+            todo &= todo - 1;
+            const float4 q0 = W.box[q][0], q1 = W.box[q][1];
+            const float blo[3] = {q0.x, q0.y, q0.z}, bhi[3] = {q0.w, q1.x, q1.y};
+            bool hit = lpos > __float_as_int(q1.w) && box_overlap(llo, lhi, blo, bhi);
+            if (!__any_sync(0xffffffffu, hit)) continue;
+            // not a candidate if the two share a vertex, are both kinematic or of different scenes
+            const int4 qn = W.info[q];
+            hit = hit && li.x != qn.x && li.y != qn.x && li.z != qn.x && li.x != qn.y && li.y != qn.y &&
+                  !(qn.w & li.w & 1) && (qn.w >> 1) == (li.w >> 1);
+            const unsigned mh = __ballot_sync(0xffffffffu, hit);
+            if (!mh) continue;
+            if (hit) {
+              const uint32_t id = (uint32_t)__float_as_int(q1.z), prim = __ldg(leaf_prim + lpos);
+              const uint32_t lo32 = pt ? id : (id < prim ? id : prim), hi32 = pt ? prim : (id < prim ? prim : id);
+              W.cand[kept + __popc(mh & below)] = pair_key(pt ? 0 : 1, lo32, hi32, T.bits_i, T.bits_j);
+            }
+            kept += __popc(mh);
+            if (kept > kQueryBuf - 32) {
+              flush_candidates(W, kept, cand, n_cand, cap, st, lane);
+              kept = 0;
+            }
           }
         }
       }
       listed = 0;
+      __syncwarp();
     };
-    if (n_leaves <= kTreelet) {
-      list(0, n_leaves, __ballot_sync(0xffffffffu, qpos != INT32_MAX));
+    if (n_leaves <= kTreelet) {              // one treelet, met by every query
+      if (lane == 0) {
+        W.near[0][0] = make_float4(-INFINITY, -INFINITY, -INFINITY, INFINITY);
+        W.near[0][1] = make_float4(INFINITY, INFINITY, __int_as_float(0), __int_as_float(n_leaves));
+      }
+      listed = 1;
     } else {
-      int32_t node = 0, stack0 = 0, stack1 = 0;     // entries 0-31 and 32-63, one per lane
-      int held = 0;
+      if (lane == 0) W.waiting[0] = 0;
+      int held = 1;
+      bool wide = true;
       int64_t visits = 0;                    // a tree of n leaves has n-1 internal nodes, each fetched at most once
-      while (true) {
-        if (++visits > n_leaves) {
+      __syncwarp();
+      while (held > 0) {
+        wide = wide && held <= kWaitingWide;
+        const int take = wide ? (held < 16 ? held : 16) : 1;
+        const bool mine = (lane >> 1) < take;
+        const int side = lane & 1;
+        const int32_t node = mine ? W.waiting[held - 1 - (lane >> 1)] : 0;
+        held -= take;
+        visits += take;
+        if (visits > n_leaves) {
           if (lane == 0) raise_flag(st, EIPC_FLAG_STACK_OVERFLOW);
           break;
         }
-        const float4* np = reinterpret_cast<const float4*>(&nodes[node]);
-        const float4 f0 = __ldg(np), f1 = __ldg(np + 1), f2 = __ldg(np + 2);
-        const int4 tail = __ldg(reinterpret_cast<const int4*>(np + 3));      // first, last, kin, split
-        const float lo0[3] = {f0.x, f0.y, f0.z}, hi0[3] = {f0.w, f1.x, f1.y};
-        const float lo1[3] = {f1.z, f1.w, f2.x}, hi1[3] = {f2.y, f2.z, f2.w};
-        const unsigned m0 = __ballot_sync(0xffffffffu, box_overlap(lo0, hi0, qlo, qhi) && tail.w > qpos && !(kin && (tail.z & 1)));
-        const unsigned m1 = __ballot_sync(0xffffffffu, box_overlap(lo1, hi1, qlo, qhi) && tail.y > qpos && !(kin && (tail.z & 2)));
-        const int n0 = tail.w - tail.x + 1, n1 = tail.y - tail.w;
-        int32_t next = -1;
-        if (m0) {
-          if (n0 <= kTreelet) list(tail.x, n0, m0);
-          else next = tail.w;
-        }
-        if (m1) {
-          if (n1 <= kTreelet) {
-            list(tail.w + 1, n1, m1);
-          } else if (next < 0) {
-            next = tail.w + 1;
-          } else if (held < 64) {
-            if (lane == (held & 31)) {
-              if (held < 32) stack0 = tail.w + 1;
-              else stack1 = tail.w + 1;
+        __syncwarp();                        // the entries are read before new ones take their places
+        const float2* bp = reinterpret_cast<const float2*>(nodes[node].box[side]);
+        const float2 c0 = __ldg(bp), c1 = __ldg(bp + 1), c2 = __ldg(bp + 2);
+        const int4 tail = __ldg(reinterpret_cast<const int4*>(&nodes[node].first));       // first, last, kin, split
+        const float lo[3] = {c0.x, c0.y, c1.x}, hi[3] = {c1.y, c2.x, c2.y};
+        const int32_t first = side ? tail.w + 1 : tail.x, last = side ? tail.y : tail.w;
+        const int child_kin = (tail.z >> side) & 1;
+        bool meet = mine && last > upos && !(ukin && child_kin);
+        if (wide) {
+          meet = meet && (box_overlap(lo, hi, ulo[0], uhi[0]) || box_overlap(lo, hi, ulo[1], uhi[1]));
+        } else {                             // lanes 0 and 1 hold the two children
+          unsigned met = 0;
+          for (int c = 0; c < 2; ++c) {
+            float clo[3], chi[3];
+            for (int k = 0; k < 3; ++k) {
+              clo[k] = __shfl_sync(0xffffffffu, lo[k], c);
+              chi[k] = __shfl_sync(0xffffffffu, hi[k], c);
             }
-            ++held;
-          } else if (lane == 0) {
-            raise_flag(st, EIPC_FLAG_STACK_OVERFLOW);
+            const int32_t clast = __shfl_sync(0xffffffffu, last, c);
+            if (__any_sync(0xffffffffu, box_overlap(clo, chi, qlo, qhi) && clast > qpos)) met |= 1u << c;
           }
+          meet = meet && (met >> side & 1u);
         }
-        if (listed > 30) handle();
-        if (next >= 0) {
-          node = next;
-        } else {
-          if (held == 0) break;
-          --held;
-          node = __shfl_sync(0xffffffffu, held < 32 ? stack0 : stack1, held & 31);
+        const bool leafy = last - first < kTreelet;
+        const unsigned m_near = __ballot_sync(0xffffffffu, meet && leafy), m_next = __ballot_sync(0xffffffffu, meet && !leafy);
+        if (meet && leafy) {
+          const int k = listed + __popc(m_near & below);
+          W.near[k][0] = make_float4(lo[0], lo[1], lo[2], hi[0]);
+          W.near[k][1] = make_float4(hi[1], hi[2], __int_as_float(first), __int_as_float((last - first + 1) | (child_kin << 8)));
+        } else if (meet) {
+          const int k = held + __popc(m_next & below);
+          if (k < kWaiting) W.waiting[k] = tail.w + side;
+          else raise_flag(st, EIPC_FLAG_STACK_OVERFLOW);
         }
+        listed += __popc(m_near);
+        held += __popc(m_next);
+        if (held > kWaiting) held = kWaiting;
+        __syncwarp();
+        if (listed > kNear - 32) handle();
       }
     }
+    __syncwarp();
     handle();
     flush_candidates(W, kept, cand, n_cand, cap, st, lane);
   }
