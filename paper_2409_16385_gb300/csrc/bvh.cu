@@ -12,15 +12,24 @@ __device__ __forceinline__ int32_t f2ord(float f) {
 }
 __device__ __forceinline__ float ord2f(int32_t i) { return __int_as_float(i >= 0 ? i : i ^ 0x7fffffff); }
 
-__device__ __forceinline__ float warp_min(float x) { return ord2f(__reduce_min_sync(0xffffffffu, f2ord(x))); }
-__device__ __forceinline__ float warp_max(float x) { return ord2f(__reduce_max_sync(0xffffffffu, f2ord(x))); }
+// min and max over the warp (no NaN reaches a primitive's box)
+__device__ __forceinline__ float warp_min(float x) {
+  float r;
+  asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float warp_max(float x) {
+  float r;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+  return r;
+}
 
 __global__ void k_bounds_init(int32_t* b, int32_t* n_tri, int32_t* n_edge) {
   pdl_entry();
   if (threadIdx.x < 3) b[threadIdx.x] = 0x7fffffff;
   else if (threadIdx.x < 6) b[threadIdx.x] = (int32_t)0x80000000;
-  else if (threadIdx.x == 6) *n_tri = 0;
-  else if (threadIdx.x == 7) *n_edge = 0;
+  else if (threadIdx.x < 9) n_tri[threadIdx.x - 6] = 0;
+  else if (threadIdx.x < 12) n_edge[threadIdx.x - 9] = 0;
 }
 
 // scene box over all per-vertex boxes
@@ -118,8 +127,14 @@ struct TreeView {
   float* leaf_box;
   int32_t* flag;
   int4* treelet;
-  float* treelet_box;
-  int32_t* n_treelets;
+  int4* cluster;
+  float* part_box;
+  int2* upper;
+  int32_t* cluster_up;
+  int32_t* n_lists;
+  // build only: per leaf, the leaves of the treelet that starts there (0: none) and that treelet's
+  // parent << 1 | slot; in leaf_box, which the first refit overwrites
+  __device__ int2* head() const { return reinterpret_cast<int2*>(leaf_box); }
 };
 
 // Karras 2012: internal node i covers a key range; its split is the highest differing bit.
@@ -146,6 +161,8 @@ __device__ __forceinline__ void internal_node(const TreeView& T, int64_t i) {
   int4* tail = reinterpret_cast<int4*>(&T.nodes[i].first);
   *tail = make_int4((int32_t)lo, (int32_t)hi, 0, (int32_t)split);
   T.flag[i] = 0;
+  T.head()[i] = make_int2(0, 0);
+  if (i == 0) T.head()[n - 1] = make_int2(0, 0);
   T.parent[lo == split ? n - 1 + split : split] = (int32_t)(i << 1);
   T.parent[hi == split + 1 ? n + split : split + 1] = (int32_t)(i << 1) | 1;
 }
@@ -159,13 +176,14 @@ __global__ void __launch_bounds__(kBlock) k_internal(TreeView A, TreeView B) {
   }
 }
 
-// Leaf records, and the treelets: the largest subtrees of at most kTreelet leaves (single leaves
-// directly under a larger node among them).  Their order in the list has no meaning.
-__device__ __forceinline__ void treelet_lists(const TreeView& T, PrimKind kind, const Topo& topo, int64_t wbase) {
+// Leaf records, treelets and clusters: the largest subtrees of at most kTreelet and kCluster leaves
+// (single leaves directly under a larger node among them).  The order of the clusters in their
+// list has no meaning.  The nodes above the clusters are numbered, in any order; a node's flag
+// holds twice its number (even: no arrival).
+__device__ __forceinline__ void tree_parts(const TreeView& T, PrimKind kind, const Topo& topo, int64_t wbase) {
   const int lane = threadIdx.x & 31;
   const int64_t n = T.n, i = wbase + lane;
-  bool is = false;
-  int4 en = make_int4(0, 0, -1, 0);
+  int32_t first = 0, size = 0, ps = -1, above = 0;       // above: leaves of the parent
   auto size_of = [&](int32_t node) { return T.nodes[node].last - T.nodes[node].first + 1; };
   if (i < n) {                                    // leaf i
     const int64_t p = T.prim[i];
@@ -176,39 +194,96 @@ __device__ __forceinline__ void treelet_lists(const TreeView& T, PrimKind kind, 
       const int32_t v0 = topo.edges[2 * p];
       T.leaf_info[i] = make_int4(v0, topo.edges[2 * p + 1], -1, topo.ekin[p] | (topo.vgroup[v0] << 1));
     }
-    const int32_t ps = n > 1 ? T.parent[n - 1 + i] : -1;
-    if (ps < 0 || size_of(ps >> 1) > kTreelet) {
-      is = true;
-      en = make_int4((int32_t)i, 1, ps, 0);
-    }
+    first = (int32_t)i;
+    size = 1;
+    if (n > 1) ps = T.parent[n - 1 + i];
   } else if (i < 2 * n - 1) {                     // internal node i - n
     const int32_t node = (int32_t)(i - n);
-    const int32_t size = size_of(node);
-    if (size <= kTreelet) {
-      const int32_t ps = node == 0 ? -1 : T.parent[node];
-      if (ps < 0 || size_of(ps >> 1) > kTreelet) {
-        is = true;
-        en = make_int4(T.nodes[node].first, size, ps, 0);
-      }
-    }
+    first = T.nodes[node].first;
+    size = size_of(node);
+    if (node) ps = T.parent[node];
   }
+  above = ps < 0 ? INT32_MAX : size_of(ps >> 1);
+  if (size > 0 && size <= kTreelet && above > kTreelet) T.head()[first] = make_int2(size, ps);
+  const bool is = size > 0 && size <= kCluster && above > kCluster;
   const unsigned m = __ballot_sync(0xffffffffu, is);
   if (m) {
     int base = 0;
-    if (lane == 0) base = atomicAdd(T.n_treelets, __popc(m));
+    if (lane == 0) base = atomicAdd(T.n_lists + 1, __popc(m));
     base = __shfl_sync(0xffffffffu, base, 0);
-    if (is) T.treelet[base + __popc(m & ((1u << lane) - 1u))] = en;
+    if (is) T.cluster[base + __popc(m & ((1u << lane) - 1u))] = make_int4(first, size, ps, 0);
+  }
+  const unsigned u = __ballot_sync(0xffffffffu, size > kCluster);
+  if (u) {
+    int base = 0;
+    if (lane == 0) base = atomicAdd(T.n_lists + 2, __popc(u));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (size > kCluster) {
+      const int id = base + __popc(u & ((1u << lane) - 1u));
+      T.flag[i - n] = 2 * id;
+      if (id < kUpper) T.upper[id].x = (int32_t)(i - n);
+    }
   }
 }
 
-__global__ void __launch_bounds__(kBlock) k_treelet_lists(TreeView A, TreeView B, Topo topo) {
+__global__ void __launch_bounds__(kBlock) k_tree_parts(TreeView A, TreeView B, Topo topo) {
   pdl_entry();
   // whole warps per tree
   const int64_t nA = (2 * A.n + 30) / 32, nB = (2 * B.n + 30) / 32;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < nA + nB; w += nw) {
-    if (w < nA) treelet_lists(A, kTri, topo, 32 * w);
-    else treelet_lists(B, kEdge, topo, 32 * (w - nA));
+    if (w < nA) tree_parts(A, kTri, topo, 32 * w);
+    else tree_parts(B, kEdge, topo, 32 * (w - nA));
+  }
+}
+
+// Each cluster's treelets, in leaf order, into consecutive entries of the treelet list; where the
+// nodes above the clusters are few, the parents among them by number.
+__global__ void __launch_bounds__(kBlock) k_cluster_treelets(TreeView A, TreeView B) {
+  static_assert(kBlock * 2 == kCluster, "a thread takes two leaves");
+  pdl_entry();
+  __shared__ int32_t count[kCluster / 32], base;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int64_t nA = A.n > 0 ? A.n_lists[1] : 0, nB = B.n > 0 ? B.n_lists[1] : 0;
+  for (int64_t g = blockIdx.x * (int64_t)kBlock + t; g < 2 * (2 * kUpper + 1); g += grid_stride()) {
+    const bool inA = g < 2 * kUpper + 1;
+    const int32_t k = (int32_t)(inA ? g : g - (2 * kUpper + 1)), clusters = (int32_t)(inA ? nA : nB);
+    const int32_t* flag = inA ? A.flag : B.flag;
+    if (clusters > kUpper + 1) continue;
+    auto numbered = [&](int32_t ps) { return ps < 0 ? -1 : (flag[ps >> 1] & ~1) | (ps & 1); };
+    if (k < clusters) {
+      (inA ? A.cluster_up : B.cluster_up)[k] = numbered((inA ? A.cluster : B.cluster)[k].z);
+    } else if (k >= kUpper + 1 && k - (kUpper + 1) < clusters - 1) {
+      int2* up = (inA ? A.upper : B.upper) + (k - (kUpper + 1));
+      up->y = up->x ? numbered((inA ? A.parent : B.parent)[up->x]) : -1;
+    }
+  }
+  for (int64_t c = blockIdx.x; c < nA + nB; c += gridDim.x) {
+    const TreeView& T = c < nA ? A : B;
+    int4* entry = T.cluster + (c < nA ? c : c - nA);
+    const int32_t first = entry->x, leaves = entry->y;
+    int2 h[2];
+    unsigned m[2];
+    for (int r = 0; r < 2; ++r) {
+      const int l = r * kBlock + t;
+      h[r] = l < leaves ? T.head()[first + l] : make_int2(0, 0);
+      m[r] = __ballot_sync(0xffffffffu, h[r].x > 0);
+      if (lane == 0) count[r * (kBlock / 32) + warp] = __popc(m[r]);
+    }
+    __syncthreads();
+    if (t == 0) {
+      int sum = 0;
+      for (int k = 0; k < kCluster / 32; ++k) { const int v = count[k]; count[k] = sum; sum += v; }
+      base = atomicAdd(T.n_lists, sum);
+      entry->y = leaves | (sum << 16);
+      entry->w = base;
+    }
+    __syncthreads();
+    for (int r = 0; r < 2; ++r)
+      if (h[r].x > 0)
+        T.treelet[base + count[r * (kBlock / 32) + warp] + __popc(m[r] & ((1u << lane) - 1u))] =
+            make_int4(first + r * kBlock + t, h[r].x, h[r].y, 0);
+    __syncthreads();
   }
 }
 
@@ -222,20 +297,24 @@ __device__ __forceinline__ bool arrive_first(int32_t* f) {
   return (old & 1) == 0;
 }
 
-// Refit of both trees in two launches.  Leaves: one warp per treelet, a lane per leaf taking the
-// leaf's box from the per-vertex boxes and storing it, and six warp reductions giving the
-// treelet's box.  Nothing is kept below the treelets: the traversal reads their leaf boxes
-// directly.  Climb: a thread per treelet carries its box upward, the second child to arrive at a
-// node taking the union on; no thread waits on another.  (One kernel for both, lane 0 climbing,
-// took twice as long on the 256-scene batch: the climbs' round trips stood between a warp's
-// treelets.)  On a build (`first`) the kinematic bits climb with the boxes.  The first is bound by
-// memory (16 B record and 32 B box per leaf), the second by dependent L2 round trips.  256-scene
-// batch (10.5 M leaves): 211 + 150 us per refit, where treelets refitted node by node in shared
-// memory and the same climb took 533 + 224 us; bubble grasp 11 + 33 us, before 28 + 34 us.
+// Refit of both trees in two launches: leaves to subtree roots, then from there to the root.
+// Nothing is kept below the treelets: the traversal reads their leaf boxes directly.  A climb goes
+// up with a box; the second child to arrive at a node takes the union on, and no thread waits on
+// another.  On a build (`first`) the kinematic bits climb with the boxes.  A level costs two
+// device-scope round trips, 2 us, in L2 and about a twentieth of that in shared memory, so up to
+// kClusterPrims primitives the subtrees are clusters, climbed in shared memory by a block each,
+// and the nodes above them are climbed in shared memory by a block per tree (beyond kUpper
+// nodes: in L2).  Sphere on pad 31.7 us with the treelets climbed in L2, 18.5 us so; bubble grasp
+// (454,550 triangles and edges) 46.3 and 32.5 us.  On larger scenes the chip is full with a warp
+// per treelet, and blocks that wait between a cluster's phases keep fewer reads in flight: the
+// subtrees are the treelets and the climb is in L2.  256-scene batch (10.5 M) 129 + 99 us, by
+// clusters 519 + 35 us; 211 + 150 us with shuffled integer reductions and 256-thread blocks.
+constexpr int64_t kClusterPrims = 1 << 20;
+
 __global__ void __launch_bounds__(kBlock) k_refit_leaves(TreeView A, TreeView B, const float* __restrict__ vbox) {
   pdl_entry();
   const int lane = threadIdx.x & 31;
-  const int64_t nA = A.n > 0 ? *A.n_treelets : 0, nB = B.n > 0 ? *B.n_treelets : 0;
+  const int64_t nA = A.n > 0 ? *A.n_lists : 0, nB = B.n > 0 ? *B.n_lists : 0;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < nA + nB; w += nw) {
     const bool inA = w < nA;
@@ -255,22 +334,175 @@ __global__ void __launch_bounds__(kBlock) k_refit_leaves(TreeView A, TreeView B,
     for (int k = 0; k < 3; ++k) { lo[k] = warp_min(lo[k]); hi[k] = warp_max(hi[k]); }
     kin = __all_sync(0xffffffffu, kin);
     if (lane == 0) {
-      float4* o = reinterpret_cast<float4*>(inA ? A.treelet_box + 8 * w : B.treelet_box + 8 * (w - nA));
+      float4* o = reinterpret_cast<float4*>(inA ? A.part_box + 8 * w : B.part_box + 8 * (w - nA));
       o[0] = make_float4(lo[0], lo[1], lo[2], hi[0]);
       o[1] = make_float4(hi[1], hi[2], __int_as_float(kin), 0.f);
     }
   }
 }
 
+struct ClusterTree {
+  float box[kCluster][2][6];           // of an internal node's children, by node - first leaf
+  float treelet[kCluster][6];
+  uint8_t kin[kCluster];               // treelet: all leaves kinematic
+  int32_t parent[kCluster];
+  int32_t flag[kCluster];              // arrivals | child 0, 1 kinematic << 8
+};
+
 template <bool first>
-__global__ void __launch_bounds__(kBlock) k_refit_climb(TreeView A, TreeView B) {
+__global__ void __launch_bounds__(kBlock, 5) k_refit_clusters(TreeView A, TreeView B, const float* __restrict__ vbox) {
   pdl_entry();
-  const int64_t nA = A.n > 0 ? *A.n_treelets : 0, nB = B.n > 0 ? *B.n_treelets : 0;
+  __shared__ ClusterTree S;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int64_t nA = A.n > 0 ? A.n_lists[1] : 0, nB = B.n > 0 ? B.n_lists[1] : 0;
+  for (int64_t c = blockIdx.x; c < nA + nB; c += gridDim.x) {
+    const bool inA = c < nA;
+    const int64_t cl = inA ? c : c - nA, n = inA ? A.n : B.n;
+    const int4 entry = __ldg((inA ? A.cluster : B.cluster) + cl);
+    const int32_t begin = entry.x, leaves = entry.y & 0xffff, treelets = entry.y >> 16;
+    const int4* list = (inA ? A.treelet : B.treelet) + entry.w;
+    const int4* leaf_info = inA ? A.leaf_info : B.leaf_info;
+    float* leaf_box = inA ? A.leaf_box : B.leaf_box;
+    const int32_t* parent = inA ? A.parent : B.parent;
+    BvhNode* nodes = inA ? A.nodes : B.nodes;
+    for (int l = t; l < leaves; l += kBlock) {
+      const int64_t node = (int64_t)begin + l;
+      S.parent[l] = node > 0 && node < n - 1 ? __ldg(parent + node) : -1;
+      S.flag[l] = 0;
+    }
+    int4 en = make_int4(0, 0, 0, 0);
+    if (warp < treelets) en = __ldg(list + warp);
+    for (int k = warp; k < treelets; k += kBlock / 32) {
+      const int64_t l = en.x + (int64_t)lane;
+      const bool have = lane < en.y;
+      if (k + kBlock / 32 < treelets) en = __ldg(list + k + kBlock / 32);
+      float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+      int kin = 1;
+      if (have) {
+        const int4 li = __ldg(leaf_info + l);
+        verts_box(vbox, li.x, li.y, li.z, lo, hi);
+        kin = li.w & 1;
+        float4* o = reinterpret_cast<float4*>(leaf_box + 8 * l);
+        o[0] = make_float4(lo[0], lo[1], lo[2], hi[0]);
+        o[1] = make_float4(hi[1], hi[2], 0.f, 0.f);
+      }
+#pragma unroll
+      for (int q = 0; q < 3; ++q) { lo[q] = warp_min(lo[q]); hi[q] = warp_max(hi[q]); }
+      if (first) kin = __all_sync(0xffffffffu, kin);
+      if (lane == 0) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) { S.treelet[k][q] = lo[q]; S.treelet[k][3 + q] = hi[q]; }
+        if (first) S.kin[k] = (uint8_t)kin;
+      }
+    }
+    __syncthreads();
+    for (int k = t; k < treelets; k += kBlock) {
+      float b[6];
+#pragma unroll
+      for (int q = 0; q < 6; ++q) b[q] = S.treelet[k][q];
+      int kin = first ? S.kin[k] : 0;
+      int32_t ps = __ldg(&list[k].z);
+      for (int step = 0; step < kCluster; ++step) {      // a path within the cluster has fewer nodes
+        if (ps == entry.z) {                     // the cluster's root
+          float4* o = reinterpret_cast<float4*>((inA ? A.part_box : B.part_box) + 8 * cl);
+          o[0] = make_float4(b[0], b[1], b[2], b[3]);
+          o[1] = make_float4(b[4], b[5], __int_as_float(kin), 0.f);
+          break;
+        }
+        const int32_t node = ps >> 1, slot = ps & 1, at = node - begin;
+        float2* mine = reinterpret_cast<float2*>(nodes[node].box[slot]);
+        mine[0] = make_float2(b[0], b[1]);
+        mine[1] = make_float2(b[2], b[3]);
+        mine[2] = make_float2(b[4], b[5]);
+#pragma unroll
+        for (int q = 0; q < 6; ++q) S.box[at][slot][q] = b[q];
+        __threadfence_block();
+        const int old = atomicAdd(&S.flag[at], 1 + (kin << (8 + slot)));
+        if ((old & 255) == 0) break;
+        __threadfence_block();
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          b[q] = fminf(b[q], S.box[at][slot ^ 1][q]);
+          b[3 + q] = fmaxf(b[3 + q], S.box[at][slot ^ 1][3 + q]);
+        }
+        if (first) {
+          const int sib = (old >> (8 + (slot ^ 1))) & 1;
+          nodes[node].kin = (kin << slot) | (sib << (slot ^ 1));
+          kin &= sib;
+        }
+        ps = S.parent[at];
+      }
+    }
+    __syncthreads();                             // before the next cluster takes the shared arrays
+  }
+}
+
+struct TopTree {
+  float box[kUpper][2][6];             // of the children of the nodes above the clusters, by number
+  int32_t flag[kUpper];                // arrivals | child 0, 1 kinematic << 8
+  int2 node[kUpper];                   // node, numbered parent << 1 | slot (-1: the root)
+};
+
+template <bool first>
+__device__ __forceinline__ void climb_in_shared(const TreeView& T, int clusters, TopTree& S) {
+  for (int k = threadIdx.x; k < clusters - 1; k += blockDim.x) {
+    S.node[k] = T.upper[k];
+    S.flag[k] = 0;
+  }
+  __syncthreads();
+  for (int c = threadIdx.x; c < clusters; c += blockDim.x) {
+    int32_t ps = T.cluster_up[c];
+    const float4* tb = reinterpret_cast<const float4*>(T.part_box + 8 * (int64_t)c);
+    const float4 t0 = __ldg(tb), t1 = __ldg(tb + 1);
+    float b[6] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y};
+    int kin = first ? __float_as_int(t1.z) : 0;
+    for (int step = 0; step < kUpper && ps >= 0; ++step) {     // a path has fewer nodes
+      const int32_t at = ps >> 1, slot = ps & 1;
+      const int2 node = S.node[at];
+      float2* mine = reinterpret_cast<float2*>(T.nodes[node.x].box[slot]);
+      mine[0] = make_float2(b[0], b[1]);
+      mine[1] = make_float2(b[2], b[3]);
+      mine[2] = make_float2(b[4], b[5]);
+#pragma unroll
+      for (int q = 0; q < 6; ++q) S.box[at][slot][q] = b[q];
+      __threadfence_block();
+      const int old = atomicAdd(&S.flag[at], 1 + (kin << (8 + slot)));
+      if ((old & 255) == 0) break;
+      __threadfence_block();
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        b[q] = fminf(b[q], S.box[at][slot ^ 1][q]);
+        b[3 + q] = fmaxf(b[3 + q], S.box[at][slot ^ 1][3 + q]);
+      }
+      if (first) {
+        const int sib = (old >> (8 + (slot ^ 1))) & 1;
+        T.nodes[node.x].kin = (kin << slot) | (sib << (slot ^ 1));
+        kin &= sib;
+      }
+      ps = node.y;
+    }
+  }
+}
+
+template <bool first>
+__global__ void __launch_bounds__(kTopThreads) k_refit_climb(TreeView A, TreeView B, bool clusters) {
+  pdl_entry();
+  extern __shared__ __align__(16) unsigned char top_smem[];
+  const int list = clusters ? 1 : 0;
+  int64_t nA = A.n > 0 ? A.n_lists[list] : 0, nB = B.n > 0 ? B.n_lists[list] : 0;
+  if (clusters) {                                    // blocks 0 and 1: a tree each in shared memory
+    TopTree& S = *reinterpret_cast<TopTree*>(top_smem);
+    const int64_t wA = nA, wB = nB;
+    if (wA <= kUpper + 1) nA = 0;
+    if (wB <= kUpper + 1) nB = 0;
+    if (blockIdx.x == 0 && nA == 0) climb_in_shared<first>(A, (int)wA, S);
+    if (blockIdx.x == 1 && nB == 0) climb_in_shared<first>(B, (int)wB, S);
+  }
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nA + nB; k += grid_stride()) {
     const bool inA = k < nA;
-    int32_t ps = (inA ? A.treelet + k : B.treelet + (k - nA))->z;
-    if (ps < 0) continue;                            // the whole tree is this treelet
-    const float4* tb = reinterpret_cast<const float4*>(inA ? A.treelet_box + 8 * k : B.treelet_box + 8 * (k - nA));
+    int32_t ps = (clusters ? (inA ? A.cluster + k : B.cluster + (k - nA)) : (inA ? A.treelet + k : B.treelet + (k - nA)))->z;
+    if (ps < 0) continue;                            // the whole tree is this subtree
+    const float4* tb = reinterpret_cast<const float4*>(inA ? A.part_box + 8 * k : B.part_box + 8 * (k - nA));
     const float4 t0 = __ldg(tb), t1 = __ldg(tb + 1);
     float lo[3] = {t0.x, t0.y, t0.z}, hi[3] = {t0.w, t1.x, t1.y};
     int kin = __float_as_int(t1.z);
@@ -330,18 +562,6 @@ struct QueryWarp {
   uint64_t cand[kQueryBuf];
   int32_t waiting[kWaiting];
 };
-
-// min and max over the warp (no NaN reaches a box)
-__device__ __forceinline__ float warp_fmin(float v) {
-  float r;
-  asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
-  return r;
-}
-__device__ __forceinline__ float warp_fmax(float v) {
-  float r;
-  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
-  return r;
-}
 
 __device__ __forceinline__ void flush_candidates(QueryWarp& W, int count, uint64_t* cand, int64_t* n_cand, int64_t cap,
                                                  DevStatus* st, int lane) {
@@ -557,14 +777,31 @@ __global__ void __launch_bounds__(256, 4) k_query(Bvh tt, Bvh te, Topo T, const 
 }
 
 TreeView view(const Bvh& t, const uint64_t* keys) {
-  return TreeView{t.n, keys, t.prim, t.nodes, t.parent, t.leaf_info, t.leaf_box, t.flag, t.treelet, t.treelet_box, t.n_treelets};
+  return TreeView{t.n, keys, t.prim, t.nodes, t.parent, t.leaf_info, t.leaf_box, t.flag, t.treelet, t.cluster, t.part_box, t.upper,
+                  t.cluster_up, t.n_lists};
+}
+
+template <bool first>
+void refit(const TreeView& A, const TreeView& B, const float* vbox, cudaStream_t s) {
+  const int64_t n = A.n + B.n;
+  const bool clusters = n <= kClusterPrims;
+  if (clusters) launch(k_refit_clusters<first>, blocks_for(n, 5), kBlock, 0, s, A, B, vbox);
+  else launch(k_refit_leaves, blocks_for(n), kBlock, 0, s, A, B, vbox);
+  const int blocks = blocks_for(n / (clusters ? 64 : 8), 4, kTopThreads);
+  launch(k_refit_climb<first>, blocks < 2 ? 2 : blocks, kTopThreads, clusters ? sizeof(TopTree) : 0, s, A, B, clusters);
 }
 
 }  // namespace
 
+cudaError_t bvh_prepare() {
+  const cudaError_t e = cudaFuncSetAttribute(k_refit_climb<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(TopTree));
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_refit_climb<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(TopTree));
+}
+
 void bvh_build(Broad& b, const Topo& topo, const float* vbox, uint32_t* sort_hist, cudaStream_t s) {
   const int64_t n = topo.nf + topo.ne + topo.nv;
-  launch(k_bounds_init, 1, 32, 0, s, b.bounds, b.tri.n_treelets, b.edge.n_treelets);
+  launch(k_bounds_init, 1, 32, 0, s, b.bounds, b.tri.n_lists, b.edge.n_lists);
   launch(k_bounds, blocks_for(topo.nv, 4), kBlock, 0, s, vbox, topo.nv, b.bounds);
   launch(k_morton_keys, blocks_for(n), kBlock, 0, s, topo, vbox, static_cast<const int32_t*>(b.bounds), b.keys, b.vals);
   const int which = radix_sort_u64(b.keys, b.vals, b.keys_alt, b.vals_alt, b.n_dev, n, 32, sort_hist, s);
@@ -575,16 +812,14 @@ void bvh_build(Broad& b, const Topo& topo, const float* vbox, uint32_t* sort_his
   b.vertex_order = sv + topo.nf + topo.ne;
   const TreeView A = view(b.tri, sk), B = view(b.edge, sk + topo.nf);
   launch(k_internal, blocks_for(topo.nf + topo.ne), kBlock, 0, s, A, B);
-  launch(k_treelet_lists, blocks_for(2 * (topo.nf + topo.ne)), kBlock, 0, s, A, B, topo);
-  launch(k_refit_leaves, blocks_for(topo.nf + topo.ne), kBlock, 0, s, A, B, vbox);
-  launch(k_refit_climb<true>, blocks_for((topo.nf + topo.ne) / 8), kBlock, 0, s, A, B);
+  launch(k_tree_parts, blocks_for(2 * (topo.nf + topo.ne)), kBlock, 0, s, A, B, topo);
+  launch(k_cluster_treelets, blocks_for(topo.nf + topo.ne), kBlock, 0, s, A, B);
+  refit<true>(A, B, vbox, s);
   b.built = true;
 }
 
 void bvh_refit(Broad& b, const float* vbox, cudaStream_t s) {
-  const TreeView A = view(b.tri, nullptr), B = view(b.edge, nullptr);
-  launch(k_refit_leaves, blocks_for(A.n + B.n), kBlock, 0, s, A, B, vbox);
-  launch(k_refit_climb<false>, blocks_for((A.n + B.n) / 8), kBlock, 0, s, A, B);
+  refit<false>(view(b.tri, nullptr), view(b.edge, nullptr), vbox, s);
 }
 
 void bvh_query(const Broad& b, const Topo& topo, const float* vbox_q, uint64_t* cand, int64_t* n_cand, int64_t cap,

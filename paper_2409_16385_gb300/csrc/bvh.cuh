@@ -28,12 +28,20 @@ struct Bvh {
   float* leaf_box;       // [8n] per leaf: lo xyz, hi xyz, two unused
   int32_t* flag;         // [n] arrivals at each internal node (two per refit)
   int4* treelet;         // [n] first leaf, leaves, parent << 1 | slot (-1: none) of each treelet
-  float* treelet_box;    // [8n] lo xyz, hi xyz, all kinematic, one unused
-  int32_t* n_treelets;   // [1]
+  int4* cluster;         // [n] first leaf, leaves | treelets << 16, parent << 1 | slot (-1: none), first treelet
+  float* part_box;       // [8n] of each cluster (large scenes: treelet): lo xyz, hi xyz, all kinematic, one unused
+  int2* upper;           // [kUpper] the nodes above the clusters: node, numbered parent << 1 | slot (-1: none)
+  int32_t* cluster_up;   // [kUpper + 1] each cluster's numbered parent << 1 | slot
+  int32_t* n_lists;      // [3] treelets, clusters, nodes above the clusters
 };
 
 // leaves per treelet: one warp refits one, and tests one against a query with a lane per leaf
 constexpr int kTreelet = 32;
+// leaves per cluster: one block refits one in shared memory
+constexpr int kCluster = 512;
+// nodes above the clusters that one block climbs in shared memory
+constexpr int kUpper = 2048;
+constexpr int kTopThreads = 512;
 
 enum PrimKind { kVertex = 0, kEdge = 1, kTri = 2 };
 
@@ -66,6 +74,9 @@ struct Broad {
   int32_t* bounds;               // [6]
   bool built;
 };
+
+// Lets the refit's climb use its shared memory; once per scene, on the scene's device.
+cudaError_t bvh_prepare();
 
 // Builds both trees from the per-vertex boxes vbox (swept ones for CCD).
 void bvh_build(Broad& b, const Topo& topo, const float* vbox, uint32_t* sort_hist, cudaStream_t s);
