@@ -531,12 +531,12 @@ __global__ void __launch_bounds__(kTopThreads) k_refit_climb(TreeView A, TreeVie
 }
 
 __device__ __forceinline__ bool box_overlap(const float* lo, const float* hi, const float qlo[3], const float qhi[3]) {
-  return !(lo[0] > qhi[0] || qlo[0] > hi[0] || lo[1] > qhi[1] || qlo[1] > hi[1] || lo[2] > qhi[2] ||
-           qlo[2] > hi[2]);
+  return !((lo[0] > qhi[0]) | (qlo[0] > hi[0]) | (lo[1] > qhi[1]) | (qlo[1] > hi[1]) | (lo[2] > qhi[2]) |
+           (qlo[2] > hi[2]));
 }
 
 // ---------------------------------------------------------------- traversal
-// A warp answers 32 queries that are neighbours in Morton order.  Instructions bound it, then the
+// A warp answers up to 32 queries that are neighbours in Morton order.  Instructions bound it, then the
 // chain of dependent node reads.  (1) It walks the nodes above the treelets with two boxes, the
 // unions of its queries before and after their largest jump, sixteen waiting nodes at a time, a
 // lane per child box: nearly always a level of the tree per step, 17 steps on the 256-scene
@@ -547,17 +547,20 @@ __device__ __forceinline__ bool box_overlap(const float* lo, const float* hi, co
 // the ballot is the set of queries that the treelet concerns.  (3) A treelet is tested a lane per
 // leaf: its leaf boxes arrive in one coalesced read, fetched one treelet ahead, and each query
 // that met the treelet is compared with all its leaves at once.  Candidates go to a buffer of
-// the warp and out with one global atomic per flush.  256-scene batch 2,230 us with every query
-// testing every node, 2,036 us so; bubble grasp's contact set 181 and 157 us; sphere on pad 53 and
-// 41 us.
+// the warp and out with one global atomic per flush.  Bubble grasp's
+// contact set 181 us with every query testing every node, 157 us with the unions, 120 us with the
+// leaf tests free of branches and the unions in shared memory; sphere on pad 53, 41 and 22 us (with
+// 8 queries a warp).  Four blocks of 256 an SM: with five, spilled registers and a smaller L1 cost
+// 9 % of the contact set.
 constexpr int kQueryBuf = 128;         // candidates; flushed when a treelet's 32 might not fit
 constexpr int kNear = 64;              // treelets; handled when a step's 32 might not fit
 constexpr int kWaiting = 128;          // nodes to visit
 constexpr int kWaitingWide = 48;       // past this the queries are taken as scattered: one node at a time from then on
 
 struct QueryWarp {
-  float4 box[32][2];                   // lo xyz, hi x | hi yz, id, own leaf position
-  int4 info[32];                       // vertices a, b (PT: both the vertex), -, kin | group << 1
+  float4 box[32][2];                   // lo xyz, hi x | hi yz, -, own leaf position
+  float4 walk[3];                      // the two unions' lo xyz, hi xyz
+  int4 info[32];                       // vertices a, b (PT: both the vertex), id, kin | group << 1
   float4 near[kNear][2];               // lo xyz, hi x | hi yz, first leaf, leaves | kin << 8
   uint64_t cand[kQueryBuf];
   int32_t waiting[kWaiting];
@@ -582,7 +585,7 @@ __device__ __forceinline__ void flush_candidates(QueryWarp& W, int count, uint64
   __syncwarp();
 }
 
-__global__ void __launch_bounds__(256, 4) k_query(Bvh tt, Bvh te, Topo T, const uint32_t* __restrict__ vertex_order,
+__global__ void __launch_bounds__(256, 4) k_query(Bvh tt, Bvh te, Topo T, int per, const uint32_t* __restrict__ vertex_order,
                                                const float* __restrict__ vbox_q, uint64_t* cand, int64_t* n_cand,
                                                int64_t cap, DevStatus* st) {
   pdl_entry();
@@ -590,7 +593,7 @@ __global__ void __launch_bounds__(256, 4) k_query(Bvh tt, Bvh te, Topo T, const 
   QueryWarp& W = reinterpret_cast<QueryWarp*>(query_smem)[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
   const unsigned below = (1u << lane) - 1u;
-  const int64_t pt_warps = tt.n > 0 ? (T.nv + 31) / 32 : 0, ee_warps = te.n > 0 ? (T.ne + 31) / 32 : 0;
+  const int64_t pt_warps = tt.n > 0 ? (T.nv + per - 1) / per : 0, ee_warps = te.n > 0 ? (T.ne + per - 1) / per : 0;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < pt_warps + ee_warps; w += nw) {
     const bool pt = w < pt_warps;
@@ -599,12 +602,12 @@ __global__ void __launch_bounds__(256, 4) k_query(Bvh tt, Bvh te, Topo T, const 
     const int4* leaf_info = pt ? tt.leaf_info : te.leaf_info;
     const uint32_t* leaf_prim = pt ? tt.prim : te.prim;
     const int32_t n_leaves = (int32_t)(pt ? tt.n : te.n);
-    const int64_t qi = 32 * (pt ? w : w - pt_warps) + lane;
+    const int64_t qi = per * (pt ? w : w - pt_warps) + lane;
     // the lane's query; a lane past the end has an empty box
     float qlo[3] = {INFINITY, INFINITY, INFINITY}, qhi[3] = {-INFINITY, -INFINITY, -INFINITY};
     int32_t qpos = INT32_MAX;
     bool kin = true;
-    if (qi < (pt ? T.nv : T.ne)) {
+    if (lane < per && qi < (pt ? T.nv : T.ne)) {
       const int32_t id = (int32_t)(pt ? vertex_order[qi] : leaf_prim[qi]);
       int32_t a = id, b = id;
       if (pt) {
@@ -617,9 +620,9 @@ __global__ void __launch_bounds__(256, 4) k_query(Bvh tt, Bvh te, Topo T, const 
         qpos = (int32_t)qi;                // each EE pair is found once, from the edge earlier in Morton order
       }
       verts_box(vbox_q, a, pt ? -1 : b, -1, qlo, qhi);
-      W.info[lane] = make_int4(a, b, 0, (kin ? 1 : 0) | (T.vgroup[a] << 1));
+      W.info[lane] = make_int4(a, b, id, (kin ? 1 : 0) | (T.vgroup[a] << 1));
       W.box[lane][0] = make_float4(qlo[0], qlo[1], qlo[2], qhi[0]);
-      W.box[lane][1] = make_float4(qhi[1], qhi[2], __int_as_float(id), __int_as_float(qpos));
+      W.box[lane][1] = make_float4(qhi[1], qhi[2], 0.f, __int_as_float(qpos));
     }
     // the queries from `cut` on, whose box with its predecessor's is the longest, have a union of
     // their own
@@ -631,13 +634,18 @@ __global__ void __launch_bounds__(256, 4) k_query(Bvh tt, Bvh te, Topo T, const 
     }
     if (lane == 0 || !(jump < INFINITY)) jump = 0.f;
     const int cut = __ffs(__ballot_sync(0xffffffffu, jump == warp_max(jump))) - 1;
-    float ulo[2][3], uhi[2][3];
+    {
+      float u[12];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      ulo[0][k] = warp_min(lane < cut ? qlo[k] : INFINITY);
-      uhi[0][k] = warp_max(lane < cut ? qhi[k] : -INFINITY);
-      ulo[1][k] = warp_min(lane < cut ? INFINITY : qlo[k]);
-      uhi[1][k] = warp_max(lane < cut ? -INFINITY : qhi[k]);
+      for (int k = 0; k < 3; ++k) {
+        u[k] = warp_min(lane < cut ? qlo[k] : INFINITY);
+        u[3 + k] = warp_max(lane < cut ? qhi[k] : -INFINITY);
+        u[6 + k] = warp_min(lane < cut ? INFINITY : qlo[k]);
+        u[9 + k] = warp_max(lane < cut ? -INFINITY : qhi[k]);
+      }
+      if (lane == 0)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) W.walk[k] = make_float4(u[4 * k], u[4 * k + 1], u[4 * k + 2], u[4 * k + 3]);
     }
     const int32_t upos = __reduce_min_sync(0xffffffffu, qpos);
     const bool ukin = __all_sync(0xffffffffu, kin);
@@ -676,24 +684,30 @@ __global__ void __launch_bounds__(256, 4) k_query(Bvh tt, Bvh te, Topo T, const 
           const int4 li = nli;
           const int32_t lpos = lane < ncount ? nfirst + lane : -2;       // -2: below every query's position
           if (live) fetch(__ffs(live) - 1);
+          // every query against the lane's leaf without a branch, then the lane's candidates one by
+          // one, each lane at its own query
+          unsigned hits = 0;
           while (todo) {
             const int q = __ffs(todo) - 1;
-            todo &= todo - 1;
             const float4 q0 = W.box[q][0], q1 = W.box[q][1];
-            const float blo[3] = {q0.x, q0.y, q0.z}, bhi[3] = {q0.w, q1.x, q1.y};
-            bool hit = lpos > __float_as_int(q1.w) && box_overlap(llo, lhi, blo, bhi);
-            if (!__any_sync(0xffffffffu, hit)) continue;
-            // not a candidate if the two share a vertex, are both kinematic or of different scenes
             const int4 qn = W.info[q];
-            hit = hit && li.x != qn.x && li.y != qn.x && li.z != qn.x && li.x != qn.y && li.y != qn.y &&
-                  !(qn.w & li.w & 1) && (qn.w >> 1) == (li.w >> 1);
+            const float blo[3] = {q0.x, q0.y, q0.z}, bhi[3] = {q0.w, q1.x, q1.y};
+            // not a candidate if the two share a vertex, are both kinematic or of different scenes
+            const bool hit = (lpos > __float_as_int(q1.w)) & box_overlap(llo, lhi, blo, bhi) & (li.x != qn.x) & (li.y != qn.x) &
+                             (li.z != qn.x) & (li.x != qn.y) & (li.y != qn.y) & ((unsigned)(li.w ^ qn.w) < 2u) & !(qn.w & li.w & 1);
+            if (hit) hits |= todo & (0u - todo);
+            todo &= todo - 1;
+          }
+          while (true) {
+            const bool hit = hits != 0;
             const unsigned mh = __ballot_sync(0xffffffffu, hit);
-            if (!mh) continue;
+            if (!mh) break;
             if (hit) {
-              const uint32_t id = (uint32_t)__float_as_int(q1.z), prim = __ldg(leaf_prim + lpos);
+              const uint32_t id = (uint32_t)W.info[__ffs(hits) - 1].z, prim = __ldg(leaf_prim + lpos);
               const uint32_t lo32 = pt ? id : (id < prim ? id : prim), hi32 = pt ? prim : (id < prim ? prim : id);
               W.cand[kept + __popc(mh & below)] = pair_key(pt ? 0 : 1, lo32, hi32, T.bits_i, T.bits_j);
             }
+            hits &= hits - 1;
             kept += __popc(mh);
             if (kept > kQueryBuf - 32) {
               flush_candidates(W, kept, cand, n_cand, cap, st, lane);
@@ -715,7 +729,7 @@ __global__ void __launch_bounds__(256, 4) k_query(Bvh tt, Bvh te, Topo T, const 
       if (lane == 0) W.waiting[0] = 0;
       int held = 1;
       bool wide = true;
-      int64_t visits = 0;                    // a tree of n leaves has n-1 internal nodes, each fetched at most once
+      int visits = 0;                        // a tree of n leaves has n-1 internal nodes, each fetched at most once
       __syncwarp();
       while (held > 0) {
         wide = wide && held <= kWaitingWide;
@@ -738,11 +752,15 @@ __global__ void __launch_bounds__(256, 4) k_query(Bvh tt, Bvh te, Topo T, const 
         const int child_kin = (tail.z >> side) & 1;
         bool meet = mine && last > upos && !(ukin && child_kin);
         if (wide) {
-          meet = meet && (box_overlap(lo, hi, ulo[0], uhi[0]) || box_overlap(lo, hi, ulo[1], uhi[1]));
+          const float4 w0 = W.walk[0], w1 = W.walk[1], w2 = W.walk[2];
+          const float ulo[2][3] = {{w0.x, w0.y, w0.z}, {w1.z, w1.w, w2.x}}, uhi[2][3] = {{w0.w, w1.x, w1.y}, {w2.y, w2.z, w2.w}};
+          meet = meet & (box_overlap(lo, hi, ulo[0], uhi[0]) | box_overlap(lo, hi, ulo[1], uhi[1]));
         } else {                             // lanes 0 and 1 hold the two children
           unsigned met = 0;
+#pragma unroll
           for (int c = 0; c < 2; ++c) {
             float clo[3], chi[3];
+#pragma unroll
             for (int k = 0; k < 3; ++k) {
               clo[k] = __shfl_sync(0xffffffffu, lo[k], c);
               chi[k] = __shfl_sync(0xffffffffu, hi[k], c);
@@ -824,10 +842,16 @@ void bvh_refit(Broad& b, const float* vbox, cudaStream_t s) {
 
 void bvh_query(const Broad& b, const Topo& topo, const float* vbox_q, uint64_t* cand, int64_t* n_cand, int64_t cap,
                DevStatus* st, cudaStream_t s, int threads, int bps) {
-  const int64_t warps = (b.tri.n > 0 ? (topo.nv + 31) / 32 : 0) + (b.edge.n > 0 ? (topo.ne + 31) / 32 : 0);
-  if (warps <= 0) return;
+  // queries per warp: 32, but 16 or 8 where that still leaves the warps room on the chip at once (4
+  // blocks of 8 an SM): a small scene's time is its slowest warp's.  Sphere
+  // on pad 41 us with 32, 25 us with 8
+  const int64_t queries = (b.tri.n > 0 ? topo.nv : 0) + (b.edge.n > 0 ? topo.ne : 0);
+  const int64_t room = (int64_t)kSMs * 32;
+  const int per = queries <= 8 * room ? 8 : (queries <= 16 * room ? 16 : 32);
+  const int64_t warps = queries / per + 2;
+  if (queries <= 0) return;
   const size_t smem = (size_t)(threads / 32) * sizeof(QueryWarp);
-  launch(k_query, blocks_for(32 * warps, bps, threads), threads, smem, s, b.tri, b.edge, topo, b.vertex_order, vbox_q, cand,
+  launch(k_query, blocks_for(32 * warps, bps, threads), threads, smem, s, b.tri, b.edge, topo, per, b.vertex_order, vbox_q, cand,
          n_cand, cap, st);
 }
 
