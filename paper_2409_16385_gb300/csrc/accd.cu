@@ -187,8 +187,8 @@ __global__ void __launch_bounds__(kBlock) k_ccd_screen(Topo T, const double* __r
 // Conservative advancement of the listed candidates in FP64.  Each step costs about 50 FP64
 // instructions: the closest feature is chosen in FP32 (closest_hint, from the FP32 positions at
 // the same t) and only its distance is taken in FP64.  A warp claims `tile` candidates at a
-// time from a queue -- the first claim is its own, and a list shorter than the warps' first
-// claims is taken 32 at a time, so that a short list spreads over the chip.
+// time from a queue -- the first claim is its own.  A list shorter than the warps' first claims is
+// taken by items_per_warp.
 __global__ void __launch_bounds__(kAccdThreads) k_ccd_advance(Topo T, const double* __restrict__ x4,
                                                               const double* __restrict__ dx4, const float* __restrict__ x4f,
                                                               const float* __restrict__ dx4f,
@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(kAccdThreads) k_ccd_advance(Topo T, const doub
   const int lane = threadIdx.x & 31;
   const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   int tile = tile_req >= 32 ? (tile_req & ~31) : 32;
-  if (n < warps * tile) tile = 32;
+  if (n < warps * tile) tile = items_per_warp(n, 4);
   int64_t base = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * tile;
   // every claim takes `tile` candidates, so n / tile + 2 claims cover all a warp can make
   const int64_t max_rounds = n / tile + 2;
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(kAccdThreads) k_ccd_advance(Topo T, const doub
     for (int o = 0; o < tile; o += 32) {
       const int64_t k = base + o + lane;
       int iters = 0;
-      if (k < n) {
+      if (k < n && lane < tile) {
         int type;
         int32_t v[4];
         decode_pair(T, list[k], &type, v);

@@ -100,6 +100,20 @@ inline int blocks_for(int64_t n_max, int per_sm = 8, int block = kBlock) {
   return (int)b;
 }
 
+// Items that a warp takes at a time of a list bound by its FP64 chains: 32, but less where the
+// list would give the chip fewer than `per_sm` warps an SM.  An FP64 instruction holds an SM
+// quarter's pipe for 64 cycles however many lanes are active, so a warp's time is that of every
+// branch and iteration that any of its lanes needs, and an idle quarter takes some of them for
+// nothing.  Four warps an SM where the chains' lengths differ widely (CCD advancement, sphere on
+// pad: 45 us with 32 items a warp, 38 with four warps an SM, 43 with two), two where they are
+// alike, since blocks that share an SM then double the time (interior pairs, bubble grasp: 95 us
+// with two, 125 with four; sphere on pad 67 us with 32 items a warp, 55 with two warps an SM).
+__device__ __forceinline__ int items_per_warp(int64_t n, int per_sm = 2) {
+  int w = 1;
+  while (w < 32 && n > (int64_t)w * (per_sm * kSMs)) w *= 2;
+  return w;
+}
+
 // clamp a device-side count to a capacity (the producer flagged the overflow)
 __device__ __forceinline__ int64_t clamp_count(const int64_t* count, int64_t cap) {
   int64_t n = *count;

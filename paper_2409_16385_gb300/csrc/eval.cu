@@ -1422,12 +1422,13 @@ __global__ void __launch_bounds__(kEvalThreads, 4) k_eval_factors(EvalArgs A) {
   const int64_t P = clamp_count(A.pr.count, A.pr.capacity);
   const int64_t nit = *A.n_items;
   const int64_t np = P < nit ? P : nit;
-  const int tile = A.tile >= 32 ? (A.tile & ~31) : 32;
+  const int width = items_per_warp(nit);
+  const int tile = width < 32 ? width : (A.tile >= 32 ? (A.tile & ~31) : 32);
   const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   int64_t base = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * tile;
   int left = tile;
-  // a warp takes 32 items a round: nit / 32 + 2 rounds cover every claim it can make
-  const int64_t max_rounds = nit / 32 + 2;
+  // a warp takes `width` items a round: nit / width + 2 rounds cover every claim it can make
+  const int64_t max_rounds = nit / width + 2;
   for (int64_t round = 0;; ++round) {
     if (round > max_rounds) {
       raise_flag(A.st, EIPC_FLAG_STACK_OVERFLOW);
@@ -1442,7 +1443,8 @@ __global__ void __launch_bounds__(kEvalThreads, 4) k_eval_factors(EvalArgs A) {
     if (base >= nit) break;
     const int64_t k = base + lane;
     int later = -1;
-    if (k < np) {
+    const bool mine = lane < width;
+    if (mine && k < np) {
       int32_t v[4];
       const int type = A.pr.type[k];
       const int32_t i = A.pr.i[k], j = A.pr.j[k];
@@ -1450,7 +1452,7 @@ __global__ void __launch_bounds__(kEvalThreads, 4) k_eval_factors(EvalArgs A) {
       const int hint = stencil_hint(type, A.x4f, v);
       if (hint & kHintInterior) later = 0;
       else light_factors(A, k, type, i, j, v, hint);
-    } else if (k < nit) {
+    } else if (mine && k < nit) {
       if (friction_merged(A.fric_of_pair, A.pair_of_fric, k - P)) A.item_E[k] = 0.0;   // with its contact pair
       else later = 1;
     }
@@ -1470,8 +1472,8 @@ __global__ void __launch_bounds__(kEvalThreads, 4) k_eval_factors(EvalArgs A) {
         }
       }
     }
-    base += 32;
-    left -= 32;
+    base += width;
+    left -= width;
   }
 }
 
@@ -1481,14 +1483,16 @@ __global__ void __launch_bounds__(kEvalThreads, 2) k_eval_rest(EvalArgs A) {
   const int lane = threadIdx.x & 31;
   const int64_t P = clamp_count(A.pr.count, A.pr.capacity);
   const int64_t n0 = A.n_rest[0], n1 = A.n_rest[1];
-  const int64_t w0 = (n0 + 31) / 32, w1 = (n1 + 31) / 32;
+  const int width = items_per_warp(n0 + n1);
+  const int64_t w0 = (n0 + width - 1) / width, w1 = (n1 + width - 1) / width;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < w0 + w1; w += nw) {
+    if (lane >= width) continue;
     if (w < w0) {
-      const int64_t q = 32 * w + lane;
+      const int64_t q = width * w + lane;
       if (q < n0) heavy_factors(A, A.rest[q]);
     } else {
-      const int64_t q = 32 * (w - w0) + lane;
+      const int64_t q = width * (w - w0) + lane;
       if (q < n1) {
         const int64_t k = A.rest[A.item_cap - 1 - q];
         friction_factors(A, k, k - P);
@@ -2023,11 +2027,13 @@ __global__ void __launch_bounds__(kEvalThreads, 4) k_hvp_items(HvpArgs A) {
   const int64_t n = P + L < A.item_cap ? P + L : A.item_cap;
   if (P + L > A.item_cap && blockIdx.x == 0 && threadIdx.x == 0) raise_flag(A.st, EIPC_FLAG_REC_OVERFLOW);
   const int64_t np = P < n ? P : n;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t base = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
+  const int width = items_per_warp(n);
+  const int64_t stride = (int64_t)gridDim.x * (blockDim.x >> 5) * width;
+  for (int64_t base = (blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5)) * width; base < n; base += stride) {
     const int64_t k = base + lane;
     bool rest = false, moll = false;
-    if (k < np) {
+    const bool mine = lane < width;
+    if (mine && k < np) {
       int32_t v[4];
       const int type = A.pr.type[k];
       const int32_t i = A.pr.i[k], j = A.pr.j[k];
@@ -2040,7 +2046,7 @@ __global__ void __launch_bounds__(kEvalThreads, 4) k_hvp_items(HvpArgs A) {
         if (hint & kHintInterior) rest = true;
         else hvp_light(A, k, type, v, hint);
       }
-    } else if (k < n) {
+    } else if (mine && k < n) {
       hvp_friction(A, k, k - P);
     }
     list_append(rest, k, A.rest, A.n_rest);
@@ -2051,7 +2057,12 @@ __global__ void __launch_bounds__(kEvalThreads, 4) k_hvp_items(HvpArgs A) {
 __global__ void __launch_bounds__(kEvalThreads) k_hvp_rest(HvpArgs A) {
   pdl_entry();
   const int64_t n = *A.n_rest;
-  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += grid_stride()) hvp_heavy(A, A.rest[q]);
+  const int lane = threadIdx.x & 31, width = items_per_warp(n);
+  const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t w = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); w * width < n; w += nw) {
+    const int64_t q = w * width + lane;
+    if (lane < width && q < n) hvp_heavy(A, A.rest[q]);
+  }
 }
 
 __global__ void __launch_bounds__(kEvalThreads) k_hvp_mollified(HvpArgs A) {
