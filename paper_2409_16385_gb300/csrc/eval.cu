@@ -266,140 +266,6 @@ __global__ void __launch_bounds__(kBlock) k_item_nodes(Topo T, eipc_pairs pr, co
   }
 }
 
-// One Jacobi rotation J (c, s = t c in rows/columns p, q) of the symmetric A held in full,
-// A <- J^T A J, and V <- V J.  The entries outside rows and columns p, q are unchanged; the
-// (p, q) block takes the closed form of the rotation that zeroes a_pq (a_pp - t a_pq,
-// a_qq + t a_pq, 0), so each pair of mirrored entries is computed once.
-template <class T, int N>
-__device__ __forceinline__ void rotate_sym(T A[N][N], T V[N][N], int p, int q, T c, T s, T t, T apq) {
-#pragma unroll
-  for (int k = 0; k < N; ++k) {
-    if (k == p || k == q) continue;
-    const T akp = A[k][p], akq = A[k][q];
-    const T np = c * akp - s * akq, nq = s * akp + c * akq;
-    A[k][p] = np; A[p][k] = np;
-    A[k][q] = nq; A[q][k] = nq;
-  }
-  A[p][p] -= t * apq;
-  A[q][q] += t * apq;
-  A[p][q] = T(0);
-  A[q][p] = T(0);
-#pragma unroll
-  for (int k = 0; k < N; ++k) {
-    const T vkp = V[k][p], vkq = V[k][q];
-    V[k][p] = c * vkp - s * vkq;
-    V[k][q] = s * vkp + c * vkq;
-  }
-}
-
-// Sweep orders of the Jacobi solvers: rounds of two rotations in disjoint planes covering
-// every index pair once (a round-robin schedule: 5 rounds for N = 5, 3 for N = 4).  The
-// rotations of a round commute, so their order inside the round does not matter.
-__device__ constexpr int kRound5[5][2][2] = {{{1, 4}, {2, 3}}, {{0, 4}, {1, 2}}, {{0, 3}, {2, 4}},
-                                             {{0, 2}, {1, 3}}, {{0, 1}, {3, 4}}};
-__device__ constexpr int kRound4[3][2][2] = {{{0, 1}, {2, 3}}, {{0, 2}, {1, 3}}, {{0, 3}, {1, 2}}};
-template <int N>
-__device__ __forceinline__ int round_entry(int r, int h, int w) {
-  return N == 5 ? kRound5[r][h][w] : kRound4[r][h][w];
-}
-template <int N>
-constexpr int kRounds = N == 5 ? 5 : 3;
-
-// FP32 rotation angle zeroing a_pq: t = tan, c = cos, s = sin; false when a_pq is negligible
-__device__ __forceinline__ bool angle_f32(float app, float aqq, float apq, float* t, float* c, float* s) {
-  if (!(fabsf(apq) > 1e-30f)) return false;
-  const float theta = (aqq - app) / (2.f * apq);
-  const float at = fabsf(theta);
-  float tt = at > 1e18f ? 0.5f / at : 1.f / (at + sqrtf(at * at + 1.f));
-  tt = theta < 0.f ? -tt : tt;
-  *t = tt;
-  *c = 1.f / sqrtf(tt * tt + 1.f);
-  *s = tt * *c;
-  return true;
-}
-
-// Fixed number of Jacobi sweeps in FP32 (62x the FP64 rate on this part): a cheap
-// approximate eigenbasis V of the symmetric N x N matrix A (scaled to unit norm beforehand).
-template <int N>
-__device__ __forceinline__ void jacobi_f32(float A[N][N], float V[N][N], int sweeps) {
-#pragma unroll
-  for (int i = 0; i < N; ++i)
-#pragma unroll
-    for (int j = 0; j < N; ++j) V[i][j] = (i == j) ? 1.f : 0.f;
-  for (int sweep = 0; sweep < sweeps; ++sweep) {
-#pragma unroll
-    for (int r = 0; r < kRounds<N>; ++r)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int p = round_entry<N>(r, h, 0), q = round_entry<N>(r, h, 1);
-        const float apq = A[p][q];
-        float t, c, sn;
-        if (angle_f32(A[p][p], A[q][q], apq, &t, &c, &sn)) rotate_sym<float, N>(A, V, p, q, c, sn, t, apq);
-      }
-  }
-}
-
-// FP64 rotation angle zeroing a_pq (t, c), false when a_pq is exactly zero.  The zero test
-// and the small-angle test read the exponent fields with integer instructions, keeping them
-// off the FP64 pipe.
-__device__ __forceinline__ bool angle_f64(double app, double aqq, double apq, double* t_out, double* c_out) {
-  const int hi_a = __double2hiint(apq);
-  if (((hi_a & 0x7fffffff) | __double2loint(apq)) == 0) return false;
-  const double gap = aqq - app;
-  const int ea = (hi_a >> 20) & 0x7ff, eg = (__double2hiint(gap) >> 20) & 0x7ff;
-  double t, c;
-  if (eg - ea >= 21 && eg > 1023 - 120 && eg < 1023 + 120) {
-    // small angle, |apq| < 2^-20 |gap| (the usual case after the FP32
-    // pre-diagonalisation): t = apq / gap to relative O(t^2) <= 2^-40, with 1/gap to FP32
-    // precision (the exponent range check keeps gap a normal float).  Any t gives an exact
-    // rotation (c = 1 - t^2 / 2 and s = t c are orthonormal to O(t^4)); the approximate t
-    // leaves an off-diagonal residual of about 2^-24 |apq|, far below the sweep's stopping
-    // threshold
-    t = apq * (double)__frcp_rn((float)gap);
-    c = 1.0 - 0.5 * t * t;
-  } else {
-    const double theta = gap / (2.0 * apq);
-    const double at = fabs(theta);
-    t = at > 1e150 ? 0.5 / at : 1.0 / (at + sqrt(at * at + 1.0));
-    t = theta < 0.0 ? -t : t;
-    c = rsqrt(t * t + 1.0);
-  }
-  *t_out = t;
-  *c_out = c;
-  return true;
-}
-
-// Jacobi on the symmetric N x N A held in registers, from the basis V the caller has
-// already rotated A into; A becomes diagonal (eigenvalues), V accumulates the rotations
-// (columns = eigenvectors).
-template <int N>
-__device__ __forceinline__ void jacobi(double A[N][N], double V[N][N]) {
-  double fro = 0.0;
-#pragma unroll
-  for (int i = 0; i < N; ++i)
-#pragma unroll
-    for (int j = 0; j < N; ++j) fro += A[i][j] * A[i][j];
-  // stop once the off-diagonal norm is below 1e-13 of the matrix norm
-  const double tol = 1e-26 * fro;
-  for (int sweep = 0; sweep < 12; ++sweep) {
-    double off = 0.0;
-#pragma unroll
-    for (int p = 0; p < N; ++p)
-#pragma unroll
-      for (int q = p + 1; q < N; ++q) off += A[p][q] * A[p][q];
-    if (off <= tol) break;
-#pragma unroll
-    for (int r = 0; r < kRounds<N>; ++r)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int p = round_entry<N>(r, h, 0), q = round_entry<N>(r, h, 1);
-        const double apq = A[p][q];
-        double t, c;
-        if (angle_f64(A[p][p], A[q][q], apq, &t, &c)) rotate_sym<double, N>(A, V, p, q, c, t * c, t, apq);
-      }
-  }
-}
-
 struct EvalArgs {
   Topo T;
   eipc_pairs pr;
@@ -493,80 +359,6 @@ __device__ __forceinline__ void friction_terms(const double* __restrict__ x4, co
       R.F[p][q] = s;
       R.F[q][p] = s;
     }
-}
-
-// Eigen-decomposition of the symmetric N x N K (N = 5, or 4 when the span has four
-// dimensions): an FP32 Jacobi pre-diagonalisation of K/|K|, its eigenvectors
-// re-orthonormalised in FP64 (modified Gram-Schmidt), K rotated into that basis in FP64,
-// then FP64 Jacobi sweeps to full precision (quadratic convergence from the ~1e-7 residual
-// leaves one or two sweeps).  On return K is diagonal, V its eigenvectors.
-template <int N>
-__device__ __forceinline__ void eigen_sym(double K[N][N], double V[N][N]) {
-  double fro = 0.0;
-#pragma unroll
-  for (int p = 0; p < N; ++p)
-#pragma unroll
-    for (int q = 0; q < N; ++q) fro += K[p][q] * K[p][q];
-  if (fro == 0.0) {
-#pragma unroll
-    for (int p = 0; p < N; ++p)
-#pragma unroll
-      for (int q = 0; q < N; ++q) V[p][q] = (p == q) ? 1.0 : 0.0;
-    return;
-  }
-  // 1/|K| only scales the FP32 stage: FP32 precision is enough when |K|^2 is a normal float
-  const double inv = (fro > 1e-36 && fro < 1e36) ? (double)rsqrtf((float)fro) : rsqrt(fro);
-  float Af[N][N], Vf[N][N];
-#pragma unroll
-  for (int p = 0; p < N; ++p)
-#pragma unroll
-    for (int q = 0; q < N; ++q) Af[p][q] = (float)(K[p][q] * inv);
-  jacobi_f32<N>(Af, Vf, 4);
-  // FP64 orthonormal basis from the FP32 eigenvectors (columns)
-#pragma unroll
-  for (int j = 0; j < N; ++j) {
-#pragma unroll
-    for (int p = 0; p < N; ++p) V[p][j] = (double)Vf[p][j];
-#pragma unroll
-    for (int i = 0; i < j; ++i) {
-      double pr = 0.0;
-#pragma unroll
-      for (int p = 0; p < N; ++p) pr += V[p][i] * V[p][j];
-#pragma unroll
-      for (int p = 0; p < N; ++p) V[p][j] -= pr * V[p][i];
-    }
-    double nn = 0.0;
-#pragma unroll
-    for (int p = 0; p < N; ++p) nn += V[p][j] * V[p][j];
-    // the FP32 eigenvectors are orthonormal to FP32 precision, so |nn - 1| is about 1e-7:
-    // two Newton steps for 1/sqrt(nn) from 1 leave an error of order (nn - 1)^4
-    double r = 1.5 - 0.5 * nn;
-    r = r * (1.5 - 0.5 * nn * r * r);
-#pragma unroll
-    for (int p = 0; p < N; ++p) V[p][j] *= r;
-  }
-  // K <- V^T K V
-  double T[N][N];
-#pragma unroll
-  for (int p = 0; p < N; ++p)
-#pragma unroll
-    for (int j = 0; j < N; ++j) {
-      double s = 0.0;
-#pragma unroll
-      for (int q = 0; q < N; ++q) s += K[p][q] * V[q][j];
-      T[p][j] = s;
-    }
-#pragma unroll
-  for (int i = 0; i < N; ++i)
-#pragma unroll
-    for (int j = i; j < N; ++j) {
-      double s = 0.0;
-#pragma unroll
-      for (int p = 0; p < N; ++p) s += V[p][i] * T[p][j];
-      K[i][j] = s;
-      K[j][i] = s;
-    }
-  jacobi<N>(K, V);
 }
 
 // Explicit records (mollified pairs): record pos of the item holds its upper block, of nodes
