@@ -1,27 +1,33 @@
 // Stable LSD radix sort, exclusive scan and segment starts with device-resident element
 // counts.
 //
-// Radix pass (8-bit digit) in two launches: one block per SM owns one contiguous chunk of the
-// input.  (1) per-block digit histograms; (2) each block sums the histograms of the blocks before
-// it and of all blocks (152 x 256 counters, four threads per digit), scans the 256 totals for
-// its digit bases and scatters its chunk tile by tile: warp peers with equal digits are found
+// A radix pass (8-bit digit) is one launch, a sort one more: one block per SM owns one contiguous
+// chunk of the input.  (1) Before the first pass, per-block digit histograms.  (2) A pass: each
+// block sums the histograms of the blocks before it and of all blocks (152 x 256 counters, four
+// threads per digit), scans the 256 totals for its digit bases and scatters its chunk tile by tile: warp peers with equal digits are found
 // with __match_any_sync and per-warp digit counts are prefix-summed across the block's 32 warps,
 // so every element lands at a position that preserves input order among equal digits (stability
 // is what makes the sort-and-reduce of the reduced Hessian deterministic).  The sorts of a step
 // are short (a few thousand to a few hundred thousand elements), so a pass costs its launches:
-// with 1,216 blocks a third one had to turn the counters into offsets.  A block takes at least a
-// whole tile, so that short inputs have few counters to sum.  Per pass, caches flushed: sphere on
-// pad (a few thousand) 14.6 us in three launches, 11.2 us in two; bubble grasp (2 x 10^5) 17.7 and
-// 19.5 us, which the saved launch makes up for (evaluation 602 and 598 us).
+// with 1,216 blocks a third one had to turn the counters into offsets.  An element's next digit is
+// counted for the chunk that it is scattered to, so later passes need no histograms of their
+// own (integer atomics: the counts do not depend on their order).  A block takes at least a
+// whole tile, so that short inputs have few counters to sum.  Caches flushed, a
+// pass of the sphere on pad (a few thousand) took 14.6 us in three launches, 11 us in two, 6.5 us
+// and 5 us once a sort so; of the bubble grasp (2 x 10^5) 17.7, 19.5, and 15.8 us and 6.4 us once.
 #include "common.cuh"
 #include "sort.cuh"
 
 namespace eipc {
 namespace {
 
+__device__ __forceinline__ uint32_t chunk_size(int64_t n) {
+  const int64_t per = (n + kSortBlocks - 1) / kSortBlocks;
+  return (uint32_t)(per > kSortThreads ? (per + 31) / 32 * 32 : kSortThreads);     // at least one whole tile: fewer counters to sum
+}
+
 __device__ __forceinline__ int chunk_range(int64_t n, int64_t* beg, int64_t* end) {
-  int64_t per = (n + kSortBlocks - 1) / kSortBlocks;
-  per = per > kSortThreads ? (per + 31) / 32 * 32 : kSortThreads;     // at least one whole tile: fewer counters to sum
+  const int64_t per = chunk_size(n);
   *beg = (int64_t)blockIdx.x * per;
   int64_t e = *beg + per;
   *end = e < n ? e : n;
@@ -30,7 +36,7 @@ __device__ __forceinline__ int chunk_range(int64_t n, int64_t* beg, int64_t* end
 
 __global__ void __launch_bounds__(kSortThreads) k_hist(const uint64_t* __restrict__ keys,
                                                        const int64_t* n_dev, int64_t cap, int shift,
-                                                       uint32_t* __restrict__ hist) {
+                                                       uint32_t* __restrict__ hist, uint32_t* __restrict__ hist_next) {
   pdl_entry();
   __shared__ uint32_t h[256];
   if (threadIdx.x < 256) h[threadIdx.x] = 0;
@@ -50,7 +56,10 @@ __global__ void __launch_bounds__(kSortThreads) k_hist(const uint64_t* __restric
     if (d < 256u && (peers & lt_mask) == 0u) atomicAdd(&h[d], (uint32_t)__popc(peers));
   }
   __syncthreads();
-  if (threadIdx.x < 256) hist[256 * blockIdx.x + threadIdx.x] = h[threadIdx.x];
+  if (threadIdx.x < 256) {
+    hist[256 * blockIdx.x + threadIdx.x] = h[threadIdx.x];
+    hist_next[256 * blockIdx.x + threadIdx.x] = 0;
+  }
 }
 
 __global__ void __launch_bounds__(kSortThreads) k_scatter(const uint64_t* __restrict__ kin,
@@ -58,7 +67,9 @@ __global__ void __launch_bounds__(kSortThreads) k_scatter(const uint64_t* __rest
                                                           uint64_t* __restrict__ kout,
                                                           uint32_t* __restrict__ vout,
                                                           const int64_t* n_dev, int64_t cap, int shift,
-                                                          const uint32_t* __restrict__ hist) {
+                                                          const uint32_t* __restrict__ hist,
+                                                          uint32_t* hist_next, uint32_t* __restrict__ hist_clear,
+                                                          bool more) {
   pdl_entry();
   constexpr int W = kSortThreads / 32;
   __shared__ uint32_t base[256];
@@ -71,6 +82,8 @@ __global__ void __launch_bounds__(kSortThreads) k_scatter(const uint64_t* __rest
   int64_t beg, end;
   const int blocks = chunk_range(n, &beg, &end);
   if (beg >= end) return;
+  const uint32_t per = chunk_size(n);
+  if (t < 256) hist_clear[256 * blockIdx.x + t] = 0;
   {
     uint32_t before = 0, all = 0;
 #pragma unroll 8
@@ -131,6 +144,7 @@ __global__ void __launch_bounds__(kSortThreads) k_scatter(const uint64_t* __rest
       for (int p = 0; p < wq; ++p) pos += part[p][digit];
       kout[pos] = key;
       vout[pos] = val;
+      if (more) atomicAdd(hist_next + 256 * (pos / per) + (uint32_t)((key >> (shift + 8)) & 255u), 1u);
     }
     __syncthreads();
     if (t < 256) base[t] += part[0][t] + part[1][t] + part[2][t] + part[3][t];
@@ -354,15 +368,20 @@ void zero_ranges(cudaStream_t s, std::initializer_list<ZeroRange> ranges) {
 
 int radix_sort_u64(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, uint32_t* vals_alt,
                    const int64_t* n, int64_t cap, int bits, uint32_t* hist, cudaStream_t s, int start_bit) {
-  int which = 0;
+  int which = 0, pass = 0;
   for (int shift = start_bit; shift < start_bit + bits; shift += 8) {
     uint64_t* ki = which ? keys_alt : keys;
     uint32_t* vi = which ? vals_alt : vals;
     uint64_t* ko = which ? keys : keys_alt;
     uint32_t* vo = which ? vals : vals_alt;
-    launch(k_hist, kSortBlocks, kSortThreads, 0, s, ki, n, cap, shift, hist);
-    launch(k_scatter, kSortBlocks, kSortThreads, 0, s, ki, vi, ko, vo, n, cap, shift, hist);
+    // counters of this pass, of the next, and those that this pass clears for the one after it
+    uint32_t* h[3];
+    for (int k = 0; k < 3; ++k) h[k] = hist + (size_t)((pass + k) % 3) * (256u * kSortBlocks);
+    if (pass == 0) launch(k_hist, kSortBlocks, kSortThreads, 0, s, ki, n, cap, shift, h[0], h[1]);
+    launch(k_scatter, kSortBlocks, kSortThreads, 0, s, ki, vi, ko, vo, n, cap, shift, h[0], h[1], h[2],
+           shift + 8 < start_bit + bits);
     which ^= 1;
+    ++pass;
   }
   return which;
 }

@@ -11,8 +11,8 @@ namespace eipc {
 constexpr int kSortBlocks = 152;    // one per SM; each block owns one contiguous chunk
 constexpr int kSortThreads = 1024;  // 32 warps, one element per thread per tile
 
-// Scratch: 256 digit counters per block.
-inline size_t sort_hist_entries() { return 256u * kSortBlocks; }
+// Scratch: 256 digit counters per block, for three passes.
+inline size_t sort_hist_entries() { return 3u * 256u * kSortBlocks; }
 
 // Stable LSD radix sort of (keys[i], vals[i]), i < min(*n, cap), by the key's bits
 // [start_bit, start_bit + 8 ceil(bits / 8)) in 8-bit digits: bits below start_bit are
