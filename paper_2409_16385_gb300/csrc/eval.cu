@@ -914,8 +914,14 @@ __device__ __forceinline__ void eigen2(T a, T b, T c, T* big, T* small, T* y0, T
 // Cholesky with the largest pivot.  Against a 12 x 12 eigensolver: 8e-12 at d = 7e-6 dhat, 1e-13
 // and below from 1e-3 dhat, near-parallel edges and slivers included.  About 700 FP64
 // instructions, where a 5 x 5 Jacobi eigensolver and its set-up took over 4,000: 130 us for a
-// warp of pairs before, 67 us after.
+// warp of pairs before, 67 us after, 55 us with few pairs a warp.
+//
+// Two neighbouring lanes take a pair: each finds one of the two eigenvectors and writes every
+// other row, and both do the rest alike, so that they stay together: 45 us for a
+// short list where one lane a pair took 55, plate in rack 93 and 113 us.
 __device__ __forceinline__ void heavy_factors(const EvalArgs& A, int64_t k) {
+  const int half = threadIdx.x & 1;
+  const unsigned both = 3u << (threadIdx.x & 30);
   int32_t v[4];
   const int type = A.pr.type[k];
   const int32_t i = A.pr.i[k], j = A.pr.j[k];
@@ -954,7 +960,7 @@ __device__ __forceinline__ void heavy_factors(const EvalArgs& A, int64_t k) {
     if (apart) inv_d = 1.0 / d;
   }
   if (!in) {                                   // the region the FP32 test left open: a segment after all
-    light_factors(A, k, type, i, j, v, pt ? 7 : 15);
+    if (half == 0) light_factors(A, k, type, i, j, v, pt ? 7 : 15);
     return;
   }
   if (!apart) raise_flag(A.st, EIPC_FLAG_PENETRATION);
@@ -963,7 +969,7 @@ __device__ __forceinline__ void heavy_factors(const EvalArgs& A, int64_t k) {
     const V3 Y[4] = {{0.0, 0.0, 0.0}, X[1] - X[0], X[2] - X[0], X[3] - X[0]};
     double eps_m, c_m;
     if (ee_mollified(A, type, i, j, Y, &eps_m, &c_m)) {           // k_mollified_eval
-      list_mollified(A, k);
+      if (half == 0) list_mollified(A, k);
       return;
     }
   }
@@ -1016,10 +1022,9 @@ __device__ __forceinline__ void heavy_factors(const EvalArgs& A, int64_t k) {
       const float af = to_float<0>(as), w11f = to_float<0>(w11), w12f = to_float<0>(w12), w22f = to_float<0>(w22);
       const float s11f = to_float<0>(s11), s12f = to_float<0>(s12), s22f = to_float<0>(s22);
       const double dy = y11 * y22, det0 = dy * dy, g1 = y12 * x1 - y11 * x2, g2 = y22 * x1, det1 = g1 * g1 + g2 * g2;
-      double q0[5];
-      double q0n = 0.0;
-#pragma unroll 1
-      for (int e = 0; e < 2; ++e) {
+      double mine[5], mu_mine;                 // this lane's eigenvector of K, times mu nu, and mu
+      {
+        const int e = half;
         float tf = 0.f;
 #pragma unroll 1
         for (int it = 0; it < 4; ++it) {
@@ -1054,31 +1059,44 @@ __device__ __forceinline__ void heavy_factors(const EvalArgs& A, int64_t k) {
           tau = mu / (as + mu);
           if (lt_nonneg(fabs(dt), 1e-9)) break;
         }
-        // the eigenvector of K at -mu, times mu nu; the second made orthogonal to the first
-        double q[5] = {tau * xy * nu, -ya * mu, -yb * mu, (y11 * ya + y12 * yb) * nu, y22 * yb * nu};
-        if (e == 1) {
+        mine[0] = tau * xy * nu; mine[1] = -ya * mu; mine[2] = -yb * mu;
+        mine[3] = (y11 * ya + y12 * yb) * nu; mine[4] = y22 * yb * nu;
+        mu_mine = mu;
+      }
+      double q[2][5], mus[2];
+#pragma unroll
+      for (int p = 0; p < 5; ++p) {
+        const double other = __shfl_xor_sync(both, mine[p], 1);
+        q[0][p] = half ? other : mine[p];
+        q[1][p] = half ? mine[p] : other;
+      }
+      {
+        const double other = __shfl_xor_sync(both, mu_mine, 1);
+        mus[0] = half ? other : mu_mine;
+        mus[1] = half ? mu_mine : other;
+      }
+      double q0n = 0.0;
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        if (e == 1) {                          // the second made orthogonal to the first
           double pr = 0.0;
 #pragma unroll
-          for (int p = 0; p < 5; ++p) pr += q0[p] * q[p];
+          for (int p = 0; p < 5; ++p) pr += q[0][p] * q[1][p];
           pr *= q0n;
 #pragma unroll
-          for (int p = 0; p < 5; ++p) q[p] -= pr * q0[p];
+          for (int p = 0; p < 5; ++p) q[1][p] -= pr * q[0][p];
         }
         double qq = 0.0;
 #pragma unroll
-        for (int p = 0; p < 5; ++p) qq += q[p] * q[p];
-        const double iq = 1.0 / qq, m = mu * iq;
+        for (int p = 0; p < 5; ++p) qq += q[e][p] * q[e][p];
+        const double iq = 1.0 / qq, m = mus[e] * iq;
 #pragma unroll
         for (int p = 0; p < 5; ++p) {
-          const double mp = m * q[p];
+          const double mp = m * q[e][p];
 #pragma unroll
-          for (int r = p; r < 5; ++r) K[p][r] = fma(mp, q[r], K[p][r]);
+          for (int r = p; r < 5; ++r) K[p][r] = fma(mp, q[e][r], K[p][r]);
         }
-        if (e == 0) {
-          q0n = iq;
-#pragma unroll
-          for (int p = 0; p < 5; ++p) q0[p] = q[p];
-        }
+        if (e == 0) q0n = iq;
       }
       // three columns of Cholesky, times sqrt(B): r^ first, then the largest diagonal entries left
       const double sB = B * rsqrt(B);
@@ -1165,11 +1183,13 @@ __device__ __forceinline__ void heavy_factors(const EvalArgs& A, int64_t k) {
 #pragma unroll
     for (int a = 0; a < 4; ++a) add_slots(A, v[a], (uint32_t)(map >> (16 * a)) & 0xffffu, gam[a], wf);
   }
-  A.item_E[k] = E;
-  store_header(A.ihead + kIHead * k, fenc > 0 ? &R : nullptr, rh * gs, iso,
-               (fenc > 0 ? kItemFriction : 0) | (iso != 0.0 ? kItemIso : 0) | kItemThird);
+  if (half == 0) {
+    A.item_E[k] = E;
+    store_header(A.ihead + kIHead * k, fenc > 0 ? &R : nullptr, rh * gs, iso,
+                 (fenc > 0 ? kItemFriction : 0) | (iso != 0.0 ? kItemIso : 0) | kItemThird);
+  }
   const int64_t base = A.ro_g[k];
-  for (int u = 0; u < n && base + u < A.gcap; ++u) {
+  for (int u = half; u < n && base + u < A.gcap; u += 2) {
     const double o = om[u], a1 = al[0][u], a2 = al[1][u];
     V3 z[3];
 #pragma unroll
@@ -1275,15 +1295,14 @@ __global__ void __launch_bounds__(kEvalThreads, 2) k_eval_rest(EvalArgs A) {
   const int lane = threadIdx.x & 31;
   const int64_t P = clamp_count(A.pr.count, A.pr.capacity);
   const int64_t n0 = A.n_rest[0], n1 = A.n_rest[1];
-  const int width = items_per_warp(n0 + n1);
-  const int64_t w0 = (n0 + width - 1) / width, w1 = (n1 + width - 1) / width;
+  const int width = items_per_warp(2 * n0 + n1), pairs = width > 1 ? width / 2 : 1;       // two lanes a pair
+  const int64_t w0 = (n0 + pairs - 1) / pairs, w1 = (n1 + width - 1) / width;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < w0 + w1; w += nw) {
-    if (lane >= width) continue;
     if (w < w0) {
-      const int64_t q = width * w + lane;
-      if (q < n0) heavy_factors(A, A.rest[q]);
-    } else {
+      const int64_t q = pairs * w + (lane >> 1);
+      if (lane < 2 * pairs && q < n0) heavy_factors(A, A.rest[q]);
+    } else if (lane < width) {
       const int64_t q = width * (w - w0) + lane;
       if (q < n1) {
         const int64_t k = A.rest[A.item_cap - 1 - q];
@@ -1819,7 +1838,7 @@ __global__ void __launch_bounds__(kEvalThreads, 4) k_hvp_items(HvpArgs A) {
   const int64_t n = P + L < A.item_cap ? P + L : A.item_cap;
   if (P + L > A.item_cap && blockIdx.x == 0 && threadIdx.x == 0) raise_flag(A.st, EIPC_FLAG_REC_OVERFLOW);
   const int64_t np = P < n ? P : n;
-  const int width = items_per_warp(n);
+  const int width = items_per_warp(n, 4);
   const int64_t stride = (int64_t)gridDim.x * (blockDim.x >> 5) * width;
   for (int64_t base = (blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5)) * width; base < n; base += stride) {
     const int64_t k = base + lane;
