@@ -20,6 +20,11 @@ SHIM = r"""
 #include <cstring>
 static inline long long __double_as_longlong(double x) { long long r; memcpy(&r, &x, 8); return r; }
 static inline int __double2hiint(double x) { return (int)(__double_as_longlong(x) >> 32); }
+static inline int __double2loint(double x) { return (int)__double_as_longlong(x); }
+static inline float __int_as_float(int x) { float r; memcpy(&r, &x, 4); return r; }
+static inline float __double2float_rn(double x) { return (float)x; }
+static inline float __double2float_rd(double x) { float f = (float)x; return f > x ? std::nextafter(f, -INFINITY) : f; }
+static inline float __double2float_ru(double x) { float f = (float)x; return f < x ? std::nextafter(f, INFINITY) : f; }
 static inline float __fdividef(float a, float b) { return a / b; }
 template <class T> static inline T __ldg(const T* p) { return *p; }
 static inline int __ffs(int x) { return __builtin_ffs(x); }
@@ -30,6 +35,13 @@ static Dim gridDim, blockDim;
 using std::fmaxf; using std::fminf; using std::isfinite;
 #include "geometry.cuh"
 using namespace eipc;
+extern "C" void convert(long n, const double* x, float* rn, float* rd, float* ru) {
+  for (long k = 0; k < n; ++k) {
+    rn[k] = to_float<0>(x[k]);
+    rd[k] = to_float<-1>(x[k]);
+    ru[k] = to_float<1>(x[k]);
+  }
+}
 extern "C" int compare(long n, const int* type, const double* x, int* features) {
   int bad = 0;
   for (long k = 0; k < n; ++k) {
@@ -69,6 +81,12 @@ def compare(tmp_path_factory):
                            str(d / "hint.cpp"), "-o", str(so)])
     lib = ctypes.CDLL(str(so))
 
+    def convert(x):
+        x = np.ascontiguousarray(x, np.float64)
+        r = np.zeros((3, len(x)), np.float32)
+        lib.convert(ctypes.c_long(len(x)), x.ctypes.data_as(ctypes.c_void_p), *(r[k].ctypes.data_as(ctypes.c_void_p) for k in range(3)))
+        return r
+
     def run(ty, X):
         ty, X = np.ascontiguousarray(ty, np.int32), np.ascontiguousarray(X, np.float64)
         f = np.zeros(len(ty), np.int32)
@@ -76,6 +94,7 @@ def compare(tmp_path_factory):
                           f.ctypes.data_as(ctypes.c_void_p))
         return bad, f
 
+    run.convert = convert
     return run
 
 
@@ -129,3 +148,24 @@ def test_ties_boundaries_and_degenerate_stencils(compare, offset):
     X = np.array(X) + offset
     bad, _ = compare(np.array(ty), X)
     assert bad == 0
+
+
+def test_integer_conversions_round_like_the_instructions(compare):
+    """to_float's three roundings against numpy's conversion and its neighbours: exact values, ties,
+    both sides of them, the ends of FP32's normal range, subnormals, zeros, infinities and NaN."""
+    rng = np.random.default_rng(7)
+    f = np.ldexp(rng.uniform(0.5, 1.0, 4000), rng.integers(-148, 128, 4000)).astype(np.float32)
+    up = np.nextafter(f, np.float32(np.inf)).astype(np.float64)
+    f = f.astype(np.float64)
+    tie = 0.5 * (f + up)
+    x = np.concatenate([f, tie, np.nextafter(tie, 0.0), np.nextafter(tie, np.inf), np.ldexp(rng.uniform(0.5, 1.0, 4000), -150),
+                        np.ldexp(rng.uniform(0.5, 1.0, 4000), rng.integers(-300, 300, 4000)),
+                        [0.0, np.inf, np.finfo(np.float32).max, 3.4028235677973366e38, 1e39, np.finfo(np.float32).tiny]])
+    x = np.concatenate([x, -x, [np.nan]])
+    with np.errstate(over="ignore"):
+        rn = x.astype(np.float32)
+    rd = np.where(rn.astype(np.float64) > x, np.nextafter(rn, np.float32(-np.inf)), rn)
+    ru = np.where(rn.astype(np.float64) < x, np.nextafter(rn, np.float32(np.inf)), rn)
+    got = compare.convert(x)
+    for g, want in zip(got, (rn, rd, ru)):
+        np.testing.assert_array_equal(g, want)
