@@ -24,7 +24,7 @@ void free_scene(eipc_scene* s) {
   if (!s) return;
   void* ptrs[] = {s->tris, s->edges, s->cage_idx, s->w, s->x_kin4, s->inc_ptr, s->inc, s->hvp_part, s->edge_key, s->edge_id, s->moll_r2, s->vkin, s->ekin, s->fkin, s->vgroup, s->group_alpha_bits, s->group_count, s->item_group, s->fric_of_pair, s->pair_of_fric, s->lag_key, s->x4, s->dx4, s->x4f, s->dx4f, s->vbox, s->vbox_pad, s->cand2,
                   s->broad.tri.nodes, s->broad.tri.parent, s->broad.tri.leaf_info, s->broad.tri.leaf_box, s->broad.tri.flag,
-                  s->broad.tri.treelet, s->broad.tri.n_lists, s->broad.tri.cluster, s->broad.tri.part_box, s->broad.tri.upper, s->broad.tri.cluster_up, s->broad.edge.part_box, s->broad.edge.upper, s->broad.edge.cluster_up, s->broad.edge.nodes, s->broad.edge.parent,
+                  s->broad.tri.treelet, s->broad.tri.n_lists, s->broad.tri.cluster, s->broad.tri.part_box, s->broad.tri.upper, s->broad.tri.cluster_up, s->broad.tri.top, s->broad.edge.part_box, s->broad.edge.upper, s->broad.edge.cluster_up, s->broad.edge.top, s->broad.edge.nodes, s->broad.edge.parent,
                   s->broad.edge.leaf_info, s->broad.edge.leaf_box, s->broad.edge.flag, s->broad.edge.treelet,
                   s->broad.edge.n_lists, s->broad.edge.cluster, s->broad.keys, s->broad.keys_alt, s->broad.vals, s->broad.vals_alt,
                   s->broad.n_dev, s->broad.bounds,
@@ -58,7 +58,7 @@ cudaError_t alloc_bvh(Bvh& t, int64_t n) {
   ok(dalloc(&t.treelet, n));
   ok(dalloc(&t.cluster, n));
   ok(dalloc(&t.part_box, 8 * n));
-  ok(dalloc(&t.upper, kUpper)); ok(dalloc(&t.cluster_up, kUpper + 1));
+  ok(dalloc(&t.upper, kUpper)); ok(dalloc(&t.cluster_up, kUpper + 1)); ok(dalloc(&t.top, kWalkStarts + 1));
   ok(dalloc(&t.n_lists, 3));
   return e;
 }

@@ -131,6 +131,7 @@ struct TreeView {
   float* part_box;
   int2* upper;
   int32_t* cluster_up;
+  int32_t* top;
   int32_t* n_lists;
   // build only: per leaf, the leaves of the treelet that starts there (0: none) and that treelet's
   // parent << 1 | slot; in leaf_box, which the first refit overwrites
@@ -238,13 +239,41 @@ __global__ void __launch_bounds__(kBlock) k_tree_parts(TreeView A, TreeView B, T
 }
 
 // Each cluster's treelets, in leaf order, into consecutive entries of the treelet list; where the
-// nodes above the clusters are few, the parents among them by number.
+// nodes above the clusters are few, the parents among them by number.  One warp per tree also finds
+// the nodes that a walk starts from: from the root, four times every node whose children are both
+// above the treelets is replaced by them.
+__device__ __forceinline__ void walk_starts(const TreeView& T, int lane) {
+  int count = T.n > kTreelet ? 1 : 0;
+  int32_t node = 0;
+  for (int level = 0; level < 4; ++level) {
+    const bool mine = lane < count;
+    const int4 tail = mine ? *reinterpret_cast<const int4*>(&T.nodes[node].first) : make_int4(0, 0, 0, 0);   // first, last, kin, split
+    const bool open = mine && tail.w - tail.x + 1 > kTreelet && tail.y - tail.w > kTreelet;
+    const unsigned m_open = __ballot_sync(0xffffffffu, open), below = (1u << lane) - 1u;
+    const int at = lane + __popc(m_open & below);          // an opened node takes two places
+    int32_t from = 0, next = 0;
+    for (int l = 0; l < count; ++l) {
+      const int32_t l_at = __shfl_sync(0xffffffffu, at, l), l_node = __shfl_sync(0xffffffffu, node, l);
+      const int32_t l_split = __shfl_sync(0xffffffffu, tail.w, l);
+      const bool l_open = m_open >> l & 1u;
+      from = l_open ? l_split : l_node;
+      if (lane == l_at) next = from;
+      if (l_open && lane == l_at + 1) next = l_split + 1;
+    }
+    node = next;
+    count += __popc(m_open);
+  }
+  if (lane < count) T.top[lane] = node;
+  if (lane == 0) T.top[kWalkStarts] = count;
+}
+
 __global__ void __launch_bounds__(kBlock) k_cluster_treelets(TreeView A, TreeView B) {
   static_assert(kBlock * 2 == kCluster, "a thread takes two leaves");
   pdl_entry();
   __shared__ int32_t count[kCluster / 32], base;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int64_t nA = A.n > 0 ? A.n_lists[1] : 0, nB = B.n > 0 ? B.n_lists[1] : 0;
+  if (blockIdx.x == gridDim.x - 1 && warp < 2) walk_starts(warp == 0 ? A : B, lane);
   for (int64_t g = blockIdx.x * (int64_t)kBlock + t; g < 2 * (2 * kUpper + 1); g += grid_stride()) {
     const bool inA = g < 2 * kUpper + 1;
     const int32_t k = (int32_t)(inA ? g : g - (2 * kUpper + 1)), clusters = (int32_t)(inA ? nA : nB);
@@ -539,8 +568,8 @@ __device__ __forceinline__ bool box_overlap(const float* lo, const float* hi, co
 // A warp answers up to 32 queries that are neighbours in Morton order.  Instructions bound it, then the
 // chain of dependent node reads.  (1) It walks the nodes above the treelets with two boxes, the
 // unions of its queries before and after their largest jump, sixteen waiting nodes at a time, a
-// lane per child box: nearly always a level of the tree per step, 17 steps on the 256-scene
-// batch.  The two meet 11 treelets there and the queries themselves 9, while tests of every node
+// lane per child box: nearly always a level of the tree per step, from the (up to sixteen) nodes
+// four levels below the root: 13 steps on the 256-scene batch.  The two meet 11 treelets there and the queries themselves 9, while tests of every node
 // by every query (one node a step) took 33 steps of more instructions each.  (With one union a
 // percent of the warps met hundreds of nodes and held up the kernel; queries so scattered that
 // two do not do go on in the one-node form.)  (2) Each query tests the boxes of those treelets;
@@ -726,8 +755,9 @@ __global__ void __launch_bounds__(256, 4) k_query(Bvh tt, Bvh te, Topo T, int pe
       }
       listed = 1;
     } else {
-      if (lane == 0) W.waiting[0] = 0;
-      int held = 1;
+      const int32_t* top = pt ? tt.top : te.top;
+      int held = __ldg(top + kWalkStarts);
+      if (lane < held) W.waiting[lane] = __ldg(top + lane);
       bool wide = true;
       int visits = 0;                        // a tree of n leaves has n-1 internal nodes, each fetched at most once
       __syncwarp();
@@ -796,7 +826,7 @@ __global__ void __launch_bounds__(256, 4) k_query(Bvh tt, Bvh te, Topo T, int pe
 
 TreeView view(const Bvh& t, const uint64_t* keys) {
   return TreeView{t.n, keys, t.prim, t.nodes, t.parent, t.leaf_info, t.leaf_box, t.flag, t.treelet, t.cluster, t.part_box, t.upper,
-                  t.cluster_up, t.n_lists};
+                  t.cluster_up, t.top, t.n_lists};
 }
 
 template <bool first>

@@ -32,6 +32,7 @@ struct Bvh {
   float* part_box;       // [8n] of each cluster (large scenes: treelet): lo xyz, hi xyz, all kinematic, one unused
   int2* upper;           // [kUpper] the nodes above the clusters: node, numbered parent << 1 | slot (-1: none)
   int32_t* cluster_up;   // [kUpper + 1] each cluster's numbered parent << 1 | slot
+  int32_t* top;          // [kWalkStarts + 1] the nodes a walk starts from, and their number
   int32_t* n_lists;      // [3] treelets, clusters, nodes above the clusters
 };
 
@@ -42,6 +43,8 @@ constexpr int kCluster = 512;
 // nodes above the clusters that one block climbs in shared memory
 constexpr int kUpper = 2048;
 constexpr int kTopThreads = 512;
+// nodes that a traversal's walk starts from, at most: one step of a warp
+constexpr int kWalkStarts = 16;
 
 enum PrimKind { kVertex = 0, kEdge = 1, kTri = 2 };
 
