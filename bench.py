@@ -186,13 +186,13 @@ def measured_peaks():
 #                 friction of the pairs that carry it included
 #   ccd_advance   FP64 flops per advanced CCD candidate (box test, advancement distances)
 #   others        DRAM bytes per unit of their minimum input + output traffic
-# eval_barrier: 345.20e6 flops over the 115,699 pairs of bubble-grasp iterate 2 (ncu, the
-# autotuned shape 64 threads, 170-register variant); see profiles/
-FP64_FLOPS_PER_PAIR = 2983.6
+# eval_barrier: 71.08e6 flops of k_eval_factors and k_eval_rest over the 115,699 pairs of
+# bubble-grasp iterate 2 (ncu); see profiles/
+FP64_FLOPS_PER_PAIR = 614.3
 FP64_FLOPS_PER_CCD_CAND = 420.0
 # DRAM bytes (read + write) per unit from one ncu capture of the same kernel code and shape
-# (eval_barrier: 112.4 MB + 239.7 MB for the same 115,699 pairs)
-NCU_TRAFFIC_PER_UNIT = {"eval_barrier": 3043.1}
+# (eval_barrier: 36.0 MB + 24.9 MB for the same 115,699 pairs)
+NCU_TRAFFIC_PER_UNIT = {"eval_barrier": 526.5}
 
 
 def query_bytes(sc, n_cand):
@@ -220,9 +220,7 @@ def roofline_figure(name, total_ms, launches, steps, per_step, sc, fp64_probe=No
         per = FP64_FLOPS_PER_CCD_CAND if name == "ccd_advance" else FP64_FLOPS_PER_PAIR
         tr = NCU_TRAFFIC_PER_UNIT.get(name)
         if name == "eval_kernels":
-            # barrier evaluation (with the friction of the pairs that carry it) and the
-            # friction items without a contact pair beside it on a second stream, from the
-            # fork to the join; the latter's few flops are not counted
+            # the same kernels, with mollified pairs' where the mollifier is on
             tr = NCU_TRAFFIC_PER_UNIT["eval_barrier"]
         ach = units * per / avg_s / 1e12
         peak = FP64_PEAK_TFLOPS
@@ -561,7 +559,7 @@ def run_eval_by_type(args, ws, rank, local):
     feature class (PAIR_CLASSES): one list per class, evaluated without friction; device
     time per class from the kernel's event timer.  With --profile-once each class is
     evaluated exactly once, in PAIR_CLASSES order, so that an ncu launch list of
-    k_eval_barrier gives each class's FP64 instruction counts (launch k = class k)."""
+    k_eval_factors and k_eval_rest gives each class's FP64 instruction counts (launch k = class k)."""
     import torch
     from paper_2409_16385_gb300 import ContactScene, PairList
     dev = torch.device("cuda", local)
@@ -598,7 +596,7 @@ def run_eval_by_type(args, ws, rank, local):
     if st["flags"] & ~64:
         raise RuntimeError(f"eval by type: device status {st}")
     line = dict(workload=sc.name, iterate=t0, classes=out, reps=reps,
-                note="k_eval_barrier time per class (no friction items); FP64 instruction counts per class "
+                note="k_eval_factors + k_eval_rest time per class (no friction items); FP64 instruction counts per class "
                      "come from an ncu launch list of the --profile-once run")
     if rank == 0:
         print(json.dumps(line), flush=True)
@@ -670,12 +668,13 @@ def run_ours(args, ws, rank, local):
         step(t, Q[t], DQ[t])
     torch.cuda.synchronize()
     warm = cs.timing_read()
-    # the barrier and friction kernels run inside eval_kernels' span (the friction kernel on
-    # a second stream, its own span stretched by the barrier kernel beside it).  Timed inside
+    # the pair kernels (eval_barrier) run inside eval_kernels' span, on a second stream.  Timed inside
     # the timed steps: the largest of the other timers and eval_barrier (for its own
     # roofline); no more, since every timer's events sit between two launches of the stream
     # and cut their programmatic overlap
-    ranked = sorted((k for k in warm if k not in ("eval_barrier", "eval_friction")), key=lambda k: -warm[k][0])
+    # (hessian_reduce's span, beside them, ends with the wait for them: it has no rate of its own)
+    ranked = sorted((k for k in warm if k not in ("eval_barrier", "eval_friction", "hessian_reduce")),
+                    key=lambda k: -warm[k][0])
     timed = ranked[:1] + ["eval_barrier"]
     cs.timing_enable(timed)
     st = cs.status()

@@ -180,7 +180,8 @@ eipc_status eipc_accd_toi(eipc_scene* scene, const double* x, const double* dx,
  *   out_kin[3]   (device, may be NULL) <- the sum of y over the kinematic vertices, i.e.
  *                 the derivative of the contact force on the kinematic set along v.
  * v: device [Ns*3]; kin_dir: HOST array of 3 doubles, or NULL for zero.  The reduction
- * is deterministic (sort by node, fixed-order warp sums), like eipc_eval_contact's. */
+ * is deterministic: the pairs' shares are added per vertex as fixed-point integers, whose sum
+ * has no order, and the vertices' per node in a fixed order. */
 eipc_status eipc_contact_hvp(eipc_scene* scene, const double* q, const eipc_pairs* pairs, const eipc_lag* lag,
                              const eipc_params* params, const double* v, const double* kin_dir, double* out_r,
                              double* out_kin, eipc_stream stream);
@@ -189,8 +190,8 @@ eipc_status eipc_contact_hvp(eipc_scene* scene, const double* q, const eipc_pair
  * with factor > 0, an edge-edge pair (i, j) with c = |e_i x e_j|^2 below
  * eps_x = factor * rest_len2[i] * rest_len2[j] carries kappa m(c) b(d), m(c) = c (2/eps_x
  * - c/eps_x^2), in every later eval_contact, contact_hvp and friction_lag (whose lambda is
- * scaled by m at x^n); such pairs take a full 12 x 12 Hessian (PSD-projected by Jacobi for
- * eval_contact).  IPC's factor is 1e-3.  x_rest: DEVICE [Nv*3] (caller-owned, read
+ * scaled by m at x^n); such pairs take a full 12 x 12 Hessian (PSD-projected by Jacobi
+ * rotations for eval_contact).  IPC's factor is 1e-3.  x_rest: DEVICE [Nv*3] (caller-owned, read
  * during the call only), the rest positions the edge lengths |e|^2 are taken from; the
  * library computes and keeps the squared rest length of every edge.  Returns
  * EIPC_ERR_INVALID (and leaves the mollifier off) if any edge has a zero or non-finite
@@ -248,9 +249,11 @@ eipc_status eipc_candidates_read(eipc_scene* scene, int32_t* type, int32_t* i, i
 /* Tracing: per-kernel CUDA-event timers.  Bit k of mask enables timer k (0 embed,
  * 1 bvh_build, 2 bvh_query, 3 narrow_phase, 4 pair_sort, 5 friction_lag, 6 stencil_nodes,
  * 7 eval_barrier, 8 eval_friction, 9 hessian_reduce, 10 gradient_reduce, 11 energy_sum,
- * 12 ccd_advance, 13 eval_kernels -- the barrier and friction evaluations together, which
- * run side by side on two streams; eipc_kernel_name(k) names them): each launch is
- * bracketed by two events on its stream.  eipc_timing_read synchronises, writes the summed milliseconds and launch
+ * 12 ccd_advance, 13 eval_kernels -- the pair evaluations together, which run on a second
+ * stream; eipc_kernel_name(k) names them): each launch, or run of launches, is bracketed by two
+ * events on its stream.  Friction is evaluated by the pairs' kernels and the gradient is carried
+ * in the Hessian's records, so timer 8 stays at zero and timer 10 counts only the reduction of
+ * eipc_contact_hvp.  eipc_timing_read synchronises, writes the summed milliseconds and launch
  * counts of the first n timers and resets them. */
 eipc_status eipc_timing_enable(eipc_scene* scene, uint32_t mask);
 eipc_status eipc_timing_read(eipc_scene* scene, double* total_ms, int64_t* launches, int32_t n);
@@ -286,12 +289,10 @@ eipc_status eipc_group_alpha(eipc_scene* scene, double* alpha_groups, eipc_strea
  * of items a warp claims from the kernel's work queue at a time (32, 64, 128 or 256;
  * defaults 32 and 128), and the other two arguments are ignored.  blocks_per_sm: cap on the
  * grid as a multiple of the 152 SMs (1..64; ignored by the refit); variant: eval 2, 3 or 4
- * (accepted; one register budget is compiled, since others round differently);
- * traversal 2 = no register cap, 3 = at most 40
- * registers (6 blocks of 256 per SM); refit 0 = arrival counters behind full device
- * fences, 1 = release-acquire arrival counters, 2 = treelets of up to 32 leaves refitted per
- * warp in shared memory below release-acquire counters, for the refits and for the
- * rebuilds' own bottom-up pass (default).  Results never depend on the shape. */
+ * (accepted; one register budget is compiled, since others round differently); traversal 2 or
+ * 3, refit 0, 1 or 2 (accepted; one form of each is compiled).  A list too short to give every
+ * SM quarter a warp is taken in smaller pieces than the tile asks for.  Results never depend on
+ * the shape. */
 eipc_status eipc_set_launch(eipc_scene* scene, int32_t kernel, int32_t threads, int32_t blocks_per_sm,
                             int32_t variant);
 
