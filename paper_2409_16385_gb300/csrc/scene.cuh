@@ -91,15 +91,15 @@ struct eipc_scene {
   struct {
     int eval_threads = 128, eval_bps = 16, eval_variant = 2, eval_tile = 32;
     int ccd_tile = 128;
-    int query_threads = 128, query_bps = 24, query_variant = 2;
+    int query_threads = 128, query_bps = 64, query_variant = 2;
     int refit_variant = 2;
   } tune;                // launch shapes of the tunable kernels (eipc_set_launch)
   int contact_refits;    // refits since the last full rebuild
   eipc::DevStatus* status;
   eipc::Timers* timers;   // host-side event timers (off unless enabled)
-  // a second stream of the scene's device: the friction evaluation runs on it beside the
-  // barrier evaluation (they write disjoint records), forked from and joined back to the
-  // caller's stream with two events, which also works inside a graph capture
+  // a second stream of the scene's device: the items' factors and the records' sums run on it beside
+  // the pattern's sorts and scans, forked from and joined back to the caller's stream with events,
+  // which also works inside a graph capture
   cudaStream_t aux;
   cudaEvent_t ev_fork, ev_mid, ev_join;
 };
