@@ -576,11 +576,11 @@ __device__ __forceinline__ bool box_overlap(const float* lo, const float* hi, co
 // the ballot is the set of queries that the treelet concerns.  (3) A treelet is tested a lane per
 // leaf: its leaf boxes arrive in one coalesced read, fetched one treelet ahead, and each query
 // that met the treelet is compared with all its leaves at once.  Candidates go to a buffer of
-// the warp and out with one global atomic per flush.  Bubble grasp's
-// contact set 181 us with every query testing every node, 157 us with the unions, 120 us with the
-// leaf tests free of branches and the unions in shared memory; sphere on pad 53, 41 and 22 us (with
-// 8 queries a warp).  Four blocks of 256 an SM: with five, spilled registers and a smaller L1 cost
-// 9 % of the contact set.
+// the warp and out with one global atomic per flush.  With every query testing every node, with the
+// unions, and with branch-free leaf tests, unions in shared memory and the start below the root:
+// bubble grasp's contact set 181, 157 and 118 us, 256-scene batch 2,230, 2,036 and 1,581 us, sphere
+// on pad 53, 41 and 20 us (with 8 queries a warp).  Four blocks of 256 an SM: with five, spilled
+// registers and a smaller L1 cost 9 % of the contact set; with three, 2 %.
 constexpr int kQueryBuf = 128;         // candidates; flushed when a treelet's 32 might not fit
 constexpr int kNear = 64;              // treelets; handled when a step's 32 might not fit
 constexpr int kWaiting = 128;          // nodes to visit

@@ -4,10 +4,10 @@
 // A radix pass (8-bit digit) is one launch, a sort one more: one block per SM owns one contiguous
 // chunk of the input.  (1) Before the first pass, per-block digit histograms.  (2) A pass: each
 // block sums the histograms of the blocks before it and of all blocks (152 x 256 counters, four
-// threads per digit), scans the 256 totals for its digit bases and scatters its chunk tile by tile: warp peers with equal digits are found
-// with __match_any_sync and per-warp digit counts are prefix-summed across the block's 32 warps,
-// so every element lands at a position that preserves input order among equal digits (stability
-// is what makes the sort-and-reduce of the reduced Hessian deterministic).  The sorts of a step
+// threads per digit), scans the 256 totals for its digit bases and scatters its chunk tile by
+// tile: warp peers with equal digits are found with __match_any_sync and per-warp digit counts are
+// prefix-summed across the block's 32 warps, so every element lands at a position that preserves
+// input order among equal digits (stability is what makes the sort-and-reduce of the reduced Hessian deterministic).  The sorts of a step
 // are short (a few thousand to a few hundred thousand elements), so a pass costs its launches:
 // with 1,216 blocks a third one had to turn the counters into offsets.  An element's next digit is
 // counted for the chunk that it is scattered to, so later passes need no histograms of their
