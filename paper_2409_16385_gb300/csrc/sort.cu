@@ -7,8 +7,9 @@
 // threads per digit), scans the 256 totals for its digit bases and scatters its chunk tile by
 // tile: warp peers with equal digits are found with __match_any_sync and per-warp digit counts are
 // prefix-summed across the block's 32 warps, so every element lands at a position that preserves
-// input order among equal digits (stability is what makes the sort-and-reduce of the reduced Hessian deterministic).  The sorts of a step
-// are short (a few thousand to a few hundred thousand elements), so a pass costs its launches:
+// input order among equal digits (stability is what makes the sort-and-reduce of the reduced
+// Hessian deterministic).  The sorts of a step are short (a few thousand to a few hundred
+// thousand elements), so a pass costs its launches:
 // with 1,216 blocks a third one had to turn the counters into offsets.  An element's next digit is
 // counted for the chunk that it is scattered to, so later passes need no histograms of their
 // own (integer atomics: the counts do not depend on their order).  A block takes at least a
