@@ -1343,9 +1343,10 @@ __device__ __forceinline__ double select_d(const double (&x)[N], int k) {
   return r;
 }
 
-// one round of rotations on the columns T, V of lane `me` of the nine from lane `first` on
+// one round of rotations on the columns T, V of lane `me` of the nine from lane `first` on; by no
+// angle, which leaves the values as they are, where `on` (the same in all nine) is not set
 template <int R>
-__device__ __forceinline__ void jacobi9_round(double (&T)[9], double (&V)[9], int me, int first) {
+__device__ __forceinline__ void jacobi9_round(double (&T)[9], double (&V)[9], int me, int first, bool on) {
   int other = R - me;
   if (other < 0) other += 9;
   const bool bye = other == me;
@@ -1360,7 +1361,7 @@ __device__ __forceinline__ void jacobi9_round(double (&T)[9], double (&V)[9], in
     tf = at > 1e18f ? 0.5f / at : 1.f / (at + sqrtf(at * at + 1.f));
     tf = th < 0.f ? -tf : tf;
   }
-  if (bye) tf = 0.f;
+  if (bye || !on) tf = 0.f;
   const double t = (double)tf, c = rsqrt(fma(t, t, 1.0)), s = t * c, sg = low ? -s : s;
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
@@ -1484,10 +1485,13 @@ __global__ void __launch_bounds__(32 * kMollWarps) k_mollified_eval(EvalArgs A, 
         double all = 0.0;
 #pragma unroll
         for (int q = 0; q < 9; ++q) all += shfl_d(off, first + q);
-        if (!__any_sync(0xffffffffu, 0.5 * all > tol)) break;
-        jacobi9_round<0>(T, V, m_e, first); jacobi9_round<1>(T, V, m_e, first); jacobi9_round<2>(T, V, m_e, first);
-        jacobi9_round<3>(T, V, m_e, first); jacobi9_round<4>(T, V, m_e, first); jacobi9_round<5>(T, V, m_e, first);
-        jacobi9_round<6>(T, V, m_e, first); jacobi9_round<7>(T, V, m_e, first); jacobi9_round<8>(T, V, m_e, first);
+        // each pair stops by itself: the list's order, and so its neighbours in the warp, differ from
+        // call to call
+        const bool on = 0.5 * all > tol;
+        if (!__any_sync(0xffffffffu, on)) break;
+        jacobi9_round<0>(T, V, m_e, first, on); jacobi9_round<1>(T, V, m_e, first, on); jacobi9_round<2>(T, V, m_e, first, on);
+        jacobi9_round<3>(T, V, m_e, first, on); jacobi9_round<4>(T, V, m_e, first, on); jacobi9_round<5>(T, V, m_e, first, on);
+        jacobi9_round<6>(T, V, m_e, first, on); jacobi9_round<7>(T, V, m_e, first, on); jacobi9_round<8>(T, V, m_e, first, on);
       }
       // column me of V max(Lambda, 0) V^T: sum over e of V[:, e] lambda_e V[me][e]
       const double lam = select_d(T, m_e), lp = lam > 0.0 ? lam : 0.0;

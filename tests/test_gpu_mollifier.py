@@ -107,3 +107,22 @@ def test_mollifier_rest_lengths_are_checked_in_the_library():
     cs.set_mollifier(xr)
     E_on, _, _ = cs.eval_contact(q1, pairs)
     assert E_on.item() != E_off.item()
+
+
+@pytest.mark.parametrize("project", [True, False])
+def test_mollified_evaluation_repeats_bit_for_bit(project):
+    """The kernel takes its pairs three to a warp, in an order that differs from call to call: what a
+    pair gives may not depend on its neighbours."""
+    from paper_2409_16385_gb300 import ContactScene
+    sc = scenes.parallel_sheets()
+    cs = ContactScene(sc, pair_capacity=1 << 14, bsr_capacity=1 << 16, rec_capacity=1 << 18)
+    cs.set_mollifier(oracle.embed(sc, sc.q_rest))
+    q = _t(sc.iterate(1))
+    pairs = cs.build_candidates(q)
+    first = None
+    for _ in range(8):
+        E, g, H = cs.eval_contact(q, pairs, project=project)
+        got = E.item(), g.cpu().numpy().tobytes(), H.host()["val"].tobytes()
+        first = first or got
+        assert got == first
+    assert cs.status()["flags"] == 0
