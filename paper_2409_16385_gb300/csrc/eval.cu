@@ -36,6 +36,7 @@ namespace {
 
 constexpr int kMaxNodes = 16;
 constexpr int kEvalThreads = 128;
+constexpr int kRecCheckThreads = 512;
 
 // Key of the upper block (I, J), I <= J < ns: its row-major position in the upper triangle,
 // I ns - I (I - 1) / 2 + (J - I).  Ordered like (I, J), and below ns (ns + 1) / 2, so the
@@ -1994,18 +1995,32 @@ __global__ void __launch_bounds__(kBlock) k_hvp_gather(int64_t ns, const int64_t
   }
 }
 
-// record totals -> overflow flags and clamped sort counts
-__global__ void k_rec_check(const int64_t* rh_total, const int64_t* rg_total, int64_t rec_cap, int64_t gcap,
-                            int64_t* n_rh, int64_t* n_rg, DevStatus* st) {
+// Record totals -> overflow flags and clamped counts.  After an overflow the items whose factor rows
+// end past gcap, or whose explicit records (mollifier) would end past rec_cap, are taken as items
+// without nodes: no kernel writes rows or records for them and none sums any, so the flag and their
+// missing shares are all that is left of them (their energies are still summed).  Decided here,
+// before the items are read, rather than at each of k_chunk_sums' reads, which it would slow down.
+__global__ void __launch_bounds__(kRecCheckThreads) k_rec_check(const int64_t* rh_total, const int64_t* rg_total,
+                                                                int64_t rec_cap, int64_t gcap, int64_t* n_rh,
+                                                                int64_t* n_rg, DevStatus* st, const int64_t* n_items,
+                                                                const int64_t* __restrict__ ro_h,
+                                                                const int64_t* __restrict__ ro_g,
+                                                                int32_t* __restrict__ item_n, bool records) {
   pdl_entry();
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    int64_t a = *rh_total, b = *rg_total;
+  const int64_t a = *rh_total, b = *rg_total;
+  if (threadIdx.x == 0) {
     if (a > rec_cap || b > gcap) {
       raise_flag(st, EIPC_FLAG_REC_OVERFLOW);
       raise_need(st, &st->need_rec, a > b ? a : b);
     }
     *n_rh = a < rec_cap ? a : rec_cap;
     *n_rg = b < gcap ? b : gcap;
+  }
+  if (b <= gcap && (!records || a <= rec_cap)) return;
+  const int64_t n = *n_items;
+  for (int64_t k = threadIdx.x; k < n; k += kRecCheckThreads) {
+    const int64_t m = item_n[k];
+    if (ro_g[k] + m > gcap || (records && ro_h[k] + m * (m + 1) / 2 > rec_cap)) item_n[k] = 0;
   }
 }
 
@@ -2491,7 +2506,9 @@ void eval_launch(eipc_scene* sc, const double* q, const eipc_pairs& pr, const ei
   int64_t* tot_g = cnt + 10;
   exclusive_scan2_i64(sc->rc_h, sc->ro_h, tot_h, sc->rc_g, sc->ro_g, tot_g, cnt + kCntItems, item_cap,
                       sc->scan_partial, s);
-  launch(k_rec_check, 1, 32, 0, s, tot_h, tot_g, sc->rec_cap, sc->gcap, cnt + kCntRecH, cnt + kCntRecG, sc->status);
+  launch(k_rec_check, 1, kRecCheckThreads, 0, s, tot_h, tot_g, sc->rec_cap, sc->gcap, cnt + kCntRecH, cnt + kCntRecG, sc->status,
+         static_cast<const int64_t*>(cnt + kCntItems), static_cast<const int64_t*>(sc->ro_h),
+         static_cast<const int64_t*>(sc->ro_g), sc->item_n, sc->moll_factor > 0.0);
   sc->timers->stop(kKItems, s);
 
   EvalArgs A{};
