@@ -295,8 +295,10 @@ __device__ __forceinline__ bool ee_far_f32(F3 a0, F3 a1, F3 b0, F3 b1, float r2m
 // parameters (sizes up to W E^3) are off by at most (16 u W E + 8 ec (E + 3 W)) E^2 to first
 // order, taken as 64 (u E + ec)(W + E) E^2; a segment's FP32 distance is off by 8 u (W + E) + 4 ec,
 // taken as 32 u (W + E) + 8 ec (its parameter enters in second order).  Where |e1 x e2|^2 is
-// below 1e-6 |e1|^2 |e2|^2 or close to FP32's smallest numbers nothing is concluded, and any
-// NaN leaves every feature in.
+// below 1e-6 |e1|^2 |e2|^2 or close to FP32's smallest numbers nothing is concluded.  Where the bound
+// 64 (u E + ec)(W + E) E^2 is not below 1e30 -- lengths whose products may overflow FP32, infinite
+// and NaN coordinates -- every feature is left in; below it W E^3 and E^4 are under 3e35, and every
+// product here is finite.
 constexpr int kHintInterior = 16, kHintCertain = 32;
 
 __device__ __forceinline__ float fmax_abs(F3 a) { return fmaxf(fabsf(a.x), fmaxf(fabsf(a.y), fabsf(a.z))); }
@@ -315,6 +317,7 @@ __device__ __forceinline__ int closest_hint(int type, F3 p0, F3 p1, F3 p2, F3 p3
   const float Em = sqrtf(fmaxf(A, C)), W = sqrtf(ww);
   const float u = 5.9604645e-8f;
   const float tol = 64.f * (u * Em + ec) * (W + Em) * Em * Em;
+  if (!(tol < 1e30f)) return kHintInterior | (pt ? 7 : 15);
   float lo;                                    // signed room inside the parameter region (times nn)
   float d2[4];
   if (pt) {

@@ -169,3 +169,17 @@ def test_integer_conversions_round_like_the_instructions(compare):
     got = compare.convert(x)
     for g, want in zip(got, (rn, rd, ru)):
         np.testing.assert_array_equal(g, want)
+
+
+@pytest.mark.parametrize("edge,gap,offset", [(1e8, 1e7, 0.0), (1e9, 1e9, 0.0), (2e9, 1e8, 1e9), (1e10, 1e10, 0.0), (1e12, 1e11, 0.0),
+                                             (1e19, 1e18, 0.0), (1e21, 1e21, 0.0), (1e36, 1e36, 0.0), (1e40, 1e40, 0.0),
+                                             (1e-3, 1e20, 0.0), (1e-3, 1e-3, 1e25), (1e19, 1e-3, 0.0), (1e6, 1e18, 0.0)])
+def test_stencils_beyond_fp32s_range_keep_every_feature(compare, edge, gap, offset):
+    """Lengths whose products, squares or selves overflow FP32: nothing may be concluded from what did."""
+    rng = np.random.default_rng(8)
+    ty, X = _stencils(rng, 50000, edge, gap, offset)
+    bad, _ = compare(ty, X)
+    assert bad == 0
+    X = X * 10.0 ** rng.uniform(-12, 0, (len(X), 4, 1))           # ... and mixed with short ones
+    bad, _ = compare(ty, X)
+    assert bad == 0
