@@ -191,8 +191,10 @@ __device__ __forceinline__ double ee_distance(V3 a0, V3 a1, V3 b0, V3 b1, Stenci
 // curvature times the squared parameter error.  Stencils whose parameter solve is not
 // well conditioned (|n|^2 <= 0.1 |e1|^2 |e2|^2) are screened by a bound that needs no
 // parameter solve: edges within 18 degrees of parallel by their segment-to-line distances
-// (seg_line_far_f32); skinny triangles not at all.  Every pair not screened goes through
-// the exact FP64 test, so the kept set is unchanged.
+// (seg_line_far_f32); skinny triangles not at all.  Nor is a stencil whose products leave FP32's range
+// (with dhat as large as the edges, at 1e5 units and more and at 1e-6 and less): an infinite, NaN or
+// subnormal one proves nothing.  Every pair not screened goes through the exact FP64 test, so the
+// kept set is unchanged.
 struct F3 {
   float x, y, z;
 };
@@ -214,17 +216,22 @@ __device__ __forceinline__ float fseg_d2(F3 w, F3 e) {
   return fdot(r, r);
 }
 
+// a product that neither overflowed nor lost more than 2^-12 of itself as a subnormal
+__device__ __forceinline__ bool in_f32_range(float x) { return x > 1e-41f && x < INFINITY; }
+
 __device__ __forceinline__ bool pt_far_f32(F3 p, F3 t0, F3 t1, F3 t2, float r2m) {
   const F3 e1 = t1 - t0, e2 = t2 - t0, w = p - t0;
   const F3 n = fcross(e1, e2);
-  const float nn = fdot(n, n);
-  if (!(nn > 0.1f * fdot(e1, e1) * fdot(e2, e2))) return false;
+  const float nn = fdot(n, n), A = fdot(e1, e1), C = fdot(e2, e2);
+  if (!(nn > 0.1f * A * C && nn > 1e-38f && A + C < 1e38f)) return false;
   const float b1 = fdot(fcross(w, e2), n) / nn;
   const float b2 = fdot(fcross(e1, w), n) / nn;
+  if (!(fabsf(b1) + fabsf(b2) < INFINITY)) return false;
   float d2;
   if (b1 >= 0.f && b2 >= 0.f && b1 + b2 <= 1.f) {
-    const float h = fdot(w, n);
-    d2 = h * h / nn;
+    const float h = fdot(w, n), hh = h * h;
+    if (!in_f32_range(hh)) return false;
+    d2 = hh / nn;
   } else {
     d2 = fminf(fseg_d2(w, e1), fminf(fseg_d2(w - e1, e2 - e1), fseg_d2(w, e2)));
   }
@@ -243,6 +250,7 @@ __device__ __forceinline__ bool pt_far_f32(F3 p, F3 t0, F3 t1, F3 t2, float r2m)
 // else nothing is proven.
 __device__ __forceinline__ bool seg_line_far_f32(F3 U, F3 V, float Lseg, float L, float r2m) {
   const float uv = fdot(U, V), vv = fdot(V, V);
+  if (!(vv + fabsf(uv) < INFINITY)) return false;
   float g;
   if (uv >= 0.f) {
     g = fdot(U, U);
@@ -250,11 +258,13 @@ __device__ __forceinline__ bool seg_line_far_f32(F3 U, F3 V, float Lseg, float L
     const F3 W = {U.x + V.x, U.y + V.y, U.z + V.z};
     g = fdot(W, W);
   } else {
-    if (!(vv > 1e-12f * Lseg * L)) return false;
+    if (!(vv > 1e-12f * Lseg * L && vv > 1e-38f)) return false;
     const F3 X = fcross(U, V);
-    g = fdot(X, X) / vv;
+    const float xx = fdot(X, X);
+    if (!in_f32_range(xx)) return false;
+    g = xx / vv;
   }
-  return g > r2m * L;
+  return g > r2m * L && g > 1e-41f;
 }
 
 __device__ __forceinline__ bool ee_far_f32(F3 a0, F3 a1, F3 b0, F3 b1, float r2m) {
@@ -262,17 +272,19 @@ __device__ __forceinline__ bool ee_far_f32(F3 a0, F3 a1, F3 b0, F3 b1, float r2m
   const float A = fdot(ea, ea), C = fdot(eb, eb);
   const F3 n = fcross(ea, eb);
   const float nn = fdot(n, n);
-  if (!(nn > 0.1f * A * C)) {
+  if (!(nn > 0.1f * A * C && nn > 1e-38f)) {
     // near-parallel: segment a against line b, segment b against line a
     const F3 wb = b0 - a0;
     return seg_line_far_f32(fcross(w, eb), n, A, C, r2m) || seg_line_far_f32(fcross(wb, ea), n * -1.f, C, A, r2m);
   }
   const float B = fdot(ea, eb), D = fdot(ea, w), E = fdot(eb, w);
   const float s = (B * E - C * D) / nn, t = (A * E - B * D) / nn;
+  if (!(fabsf(s) + fabsf(t) < INFINITY)) return false;
   float d2;
   if (s >= 0.f && s <= 1.f && t >= 0.f && t <= 1.f) {
-    const float h = fdot(w, n);
-    d2 = h * h / nn;
+    const float h = fdot(w, n), hh = h * h;
+    if (!in_f32_range(hh)) return false;
+    d2 = hh / nn;
   } else {
     d2 = fminf(fminf(fseg_d2(w, eb), fseg_d2(a1 - b0, eb)), fminf(fseg_d2(b0 - a0, ea), fseg_d2(b1 - a0, ea)));
   }
