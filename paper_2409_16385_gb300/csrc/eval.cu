@@ -1589,15 +1589,18 @@ __device__ __forceinline__ void warp_tree_sum(double acc[W]) {
 // Each item's y = H_k u is twelve numbers on its four vertices, in closed form (no 12 x 12 matrix,
 // no eigensolve, about 110 FP64 instructions); they are added per vertex, and J^T is applied once
 // per vertex instead of once per item and cage node.  The sum over items has to be the same bits
-// on every run without sorting records: every vertex keeps the largest exponent E among its
-// contributions (an integer maximum), and each contribution is added to the vertex as a fixed-point
-// number of 80 bits below 2^(E+1), in two 64-bit integers of 40 bits each (headroom for 2^22
-// items).  Integer sums do not depend on their order, and 80 bits lose less than adding in FP64.
-// The sums then become doubles where the static lists of each node's vertices gather them, a
+// on every run without sorting records: every component of every vertex keeps the largest exponent
+// E among its contributions (an integer maximum), and each contribution is added to it as a
+// fixed-point number of 2 kFix = 68 bits below 2^(E+1), in two 64-bit integers of 34 bits each
+// (headroom for 2^29 items, the most a scene takes).  Integer sums do not depend on their order, and
+// a contribution loses less than 2^-67 of the component's largest, where an addition in FP64 loses up
+// to 2^-53 of the sum.  Infinite and NaN contributions (whose sum has no order either) are added as
+// they are.  The sums then become doubles where the static lists of each node's vertices gather them, a
 // warp per node in a fixed order.  Before: 1.24 M keyed records of the bubble grasp written,
 // radix-sorted and summed, 23 launches, 443 us; now 6 launches, 162 us.
 constexpr int kKinSlots = 64;          // partial sums over the kinematic vertices
 constexpr int kFix = 34;               // bits per fixed-point limb
+static_assert(kFix + 29 <= 63, "2^29 contributions below 2^kFix fit a limb's sum");
 
 __device__ __forceinline__ V3 load_dir(const double* __restrict__ v, int32_t node) {
   return {v[3 * (int64_t)node], v[3 * (int64_t)node + 1], v[3 * (int64_t)node + 2]};
@@ -1625,7 +1628,7 @@ __global__ void __launch_bounds__(kBlock) k_hvp_direction(int64_t nv, const int3
     }
     reinterpret_cast<double2*>(u4)[2 * v] = make_double2(r.x, r.y);
     reinterpret_cast<double2*>(u4)[2 * v + 1] = make_double2(r.z, 0.0);
-    vexp[v] = 0;
+    reinterpret_cast<int4*>(vexp)[v] = make_int4(0, 0, 0, 0);
     reinterpret_cast<ulonglong2*>(hi)[2 * v] = make_ulonglong2(0, 0);
     reinterpret_cast<ulonglong2*>(hi)[2 * v + 1] = make_ulonglong2(0, 0);
     reinterpret_cast<ulonglong2*>(lo)[2 * v] = make_ulonglong2(0, 0);
@@ -1646,7 +1649,7 @@ struct HvpArgs {
   double moll_factor;
   int64_t item_cap;
   double* y;                 // [12 * items]
-  int32_t* vexp;             // [nv] largest biased exponent of the vertex's contributions
+  int32_t* vexp;             // [4 nv] largest exponent_of the contributions to each component of a vertex
   unsigned long long* hi;    // [4 nv] fixed-point sums, upper and lower limbs
   unsigned long long* lo;
   uint32_t* rest;            // pairs left to k_hvp_rest, mollified pairs left to k_hvp_mollified
@@ -1656,13 +1659,21 @@ struct HvpArgs {
   DevStatus* st;
 };
 
-__device__ __forceinline__ int32_t exponent_of(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+// biased exponent of x, 1 where x is subnormal, 0 for zeros, 0x7ff for infinities and NaN
+__device__ __forceinline__ int32_t exponent_of(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  return (int32_t)max((hi >> 20) & 0x7ffu, min((hi << 1) | lo, 1u));
+}
 
 __device__ __forceinline__ void hvp_store(const HvpArgs& A, int64_t k, int slot, int32_t v, V3 y) {
   double* row = A.y + 12 * k + 3 * slot;
   row[0] = y.x; row[1] = y.y; row[2] = y.z;
-  const int32_t e = max(exponent_of(y.x), max(exponent_of(y.y), exponent_of(y.z)));
-  if (e > 0 && e > __ldcg(A.vexp + v)) atomicMax(A.vexp + v, e);
+  int32_t* held = A.vexp + 4 * (int64_t)v;
+  const int4 h = __ldcg(reinterpret_cast<const int4*>(held));
+  const int32_t ex = exponent_of(y.x), ey = exponent_of(y.y), ez = exponent_of(y.z);
+  if (ex > h.x) atomicMax(held, ex);
+  if (ey > h.y) atomicMax(held + 1, ey);
+  if (ez > h.z) atomicMax(held + 2, ez);
 }
 
 // y of a pair whose closest feature is a segment of `hint`
@@ -1887,9 +1898,14 @@ __global__ void __launch_bounds__(kEvalThreads) k_hvp_mollified(HvpArgs A) {
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += grid_stride()) hvp_mollified(A, A.moll_list[q]);
 }
 
-// adds y / 2^(E - 1022) as a fixed-point number: kFix bits in hi, the next kFix in lo
+// adds y / 2^(E - 1022) as a fixed-point number: kFix bits in hi, the next kFix in lo; where a
+// contribution is not finite, those that are not as they are, in hi as a double
 __device__ __forceinline__ void add_fixed(unsigned long long* hi, unsigned long long* lo, double y, int32_t E) {
   const long long b = __double_as_longlong(y);
+  if (E == 0x7ff) {
+    if (!finite_bits(y)) atomicAdd(reinterpret_cast<double*>(hi), y);
+    return;
+  }
   int32_t e = (int32_t)((b >> 52) & 0x7ff);
   unsigned long long m = (unsigned long long)b & 0xfffffffffffffull;
   if (e > 0) m |= 1ull << 52;
@@ -1918,16 +1934,19 @@ __global__ void __launch_bounds__(kBlock) k_hvp_accumulate(HvpArgs A) {
     const int32_t va = pick(v, a);
     const double* y = A.y + 3 * t;
     const double y0 = y[0], y1 = y[1], y2 = y[2];
-    const int32_t E = A.vexp[va];
-    if (E == 0 || E == 0x7ff) continue;        // nothing but zeros; a NaN or infinity (the gather says so)
-    add_fixed(A.hi + 4 * (int64_t)va, A.lo + 4 * (int64_t)va, y0, E);
-    add_fixed(A.hi + 4 * (int64_t)va + 1, A.lo + 4 * (int64_t)va + 1, y1, E);
-    add_fixed(A.hi + 4 * (int64_t)va + 2, A.lo + 4 * (int64_t)va + 2, y2, E);
+    const int4 E = reinterpret_cast<const int4*>(A.vexp)[va];
+    add_fixed(A.hi + 4 * (int64_t)va, A.lo + 4 * (int64_t)va, y0, E.x);
+    add_fixed(A.hi + 4 * (int64_t)va + 1, A.lo + 4 * (int64_t)va + 1, y1, E.y);
+    add_fixed(A.hi + 4 * (int64_t)va + 2, A.lo + 4 * (int64_t)va + 2, y2, E.z);
   }
 }
 
-// a fixed-point sum as a double
-__device__ __forceinline__ double from_fixed(long long hi, long long lo, double scale) {
+// a fixed-point sum of contributions of largest exponent E as a double
+__device__ __forceinline__ double from_fixed(long long hi, long long lo, int32_t E) {
+  if (E == 0) return 0.0;
+  if (E == 0x7ff) return __longlong_as_double(hi);
+  // 2^(E - 1022 - kFix), subnormal below E = kFix
+  const double scale = E >= kFix ? __hiloint2double((E - kFix + 1) << 20, 0) : __longlong_as_double(1ll << (E + 52 - kFix));
   const long long t = hi + (lo >> kFix), f = lo & ((1ll << kFix) - 1);
   return fma((double)f, 1.0 / (double)(1ll << kFix), (double)t) * scale;
 }
@@ -1955,16 +1974,13 @@ __global__ void __launch_bounds__(kBlock) k_hvp_gather(int64_t ns, const int64_t
     for (int64_t q = b + lane; q < e; q += 32) {
       const uint32_t t = inc[q];
       const int64_t v = t >> 2;
-      const int32_t E = vexp[v];
-      if (E == 0) continue;
-      // 2^(E - 1022 - kFix), or NaN where a contribution was not finite
-      const double sc = E == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
-                                   : (E >= kFix ? __hiloint2double((E - kFix + 1) << 20, 0) : ldexp(1.0, E - 1022 - kFix));
+      const int4 E = reinterpret_cast<const int4*>(vexp)[v];
+      if ((E.x | E.y | E.z) == 0) continue;
       const longlong2 h01 = *reinterpret_cast<const longlong2*>(hi + 4 * v), l01 = *reinterpret_cast<const longlong2*>(lo + 4 * v);
       const double ww = kin ? 1.0 : w[t];
-      a0 = fma(ww, from_fixed(h01.x, l01.x, sc), a0);
-      a1 = fma(ww, from_fixed(h01.y, l01.y, sc), a1);
-      a2 = fma(ww, from_fixed(hi[4 * v + 2], lo[4 * v + 2], sc), a2);
+      a0 = fma(ww, from_fixed(h01.x, l01.x, E.x), a0);
+      a1 = fma(ww, from_fixed(h01.y, l01.y, E.y), a1);
+      a2 = fma(ww, from_fixed(hi[4 * v + 2], lo[4 * v + 2], E.z), a2);
     }
     if (__any_sync(0xffffffffu, a0 != 0.0 || a1 != 0.0 || a2 != 0.0)) {
       double acc[3] = {a0, a1, a2};

@@ -138,3 +138,54 @@ def test_set_kinematic_equals_a_scene_built_with_the_new_positions():
         assert cs.status()["flags"] == 0
     assert outs[0] == outs[1]
     assert len(a.build_candidates(q).host()["i"]) > 0
+
+
+def _point_over_triangle():
+    """One contact pair whose Hessian is diagonal in exact arithmetic: a cage node's own vertex over the
+    middle of a kinematic triangle, every coordinate a multiple of a power of two."""
+    verts = np.array([[0, 0, 0], [2.0**-4, 0, 0], [0, 2.0**-4, 0],
+                      [2.0**-6, 2.0**-6, 2.0**-11], [2.0**-6, 2.0**-5, 2.0**-4], [2.0**-5, 2.0**-6, 2.0**-4]])
+    idx = np.full((6, 4), -1, np.int32)
+    w = np.zeros((6, 4))
+    for v in range(3, 6):
+        idx[v] = v - 3
+        w[v] = 0.25                # no zero weight: its product with an infinity is a NaN
+    xk = verts.copy()
+    xk[3:] = 0
+    tris = np.array([[0, 1, 2], [3, 4, 5]], np.int32)
+    return scenes.Scene(name="point_over_triangle", tris=tris, edges=scenes.edges_of(tris), cage_idx=idx, w=w, x_kin=xk, Ns=3,
+                        cage_tets=np.zeros((0, 4), np.int32), q_rest=verts[3:].copy(),
+                        body=np.array([0, 0, 0, 1, 1, 1], np.int32), params=dict(scenes.DEFAULT_PARAMS))
+
+
+def test_hvp_components_keep_their_own_precision():
+    """A vertex's small components are not held relative to its largest one: with friction along x and
+    y and the barrier along z, out's x and y do not change when v's z is raised from 0 to 1, however
+    small they are (1e-14: the FP64 operations are the same, the sums lose less)."""
+    from paper_2409_16385_gb300 import ContactScene
+    sc = _point_over_triangle()
+    cs = ContactScene(sc, pair_capacity=64, bsr_capacity=64)
+    q = _t(sc.q_rest)
+    pairs = cs.build_candidates(q)
+    assert pairs.n() == 1
+    lag = cs.friction_lag(q, pairs)
+
+    def hvp(x, y, z):
+        v = np.zeros((3, 3))
+        v[0] = x, y, z
+        out, kin = cs.contact_hvp(q, pairs, _t(v), lag=lag)
+        return out.cpu().numpy()[0], kin.cpu().numpy()
+
+    one = hvp(0.0, 0.0, 1.0)[0]
+    assert one[2] > 0
+    for e in (-10, -30, -50, -100, -400):
+        a, b = 2.0**e, 3 * 2.0 ** (e - 1)
+        alone, beside = hvp(a, b, 0.0)[0], hvp(a, b, 1.0)[0]
+        assert alone[0] > 0 and alone[1] > 0 and beside[2] == one[2]
+        np.testing.assert_allclose(beside[:2], alone[:2], rtol=1e-14, atol=0)
+    # subnormal sums are kept, and a sum beyond FP64's range is infinite
+    tiny = hvp(0.0, 0.0, 2.0**-1060)[0]
+    np.testing.assert_allclose(tiny[2], one[2] * 2.0**-1060, rtol=2.0**-20, atol=0)
+    out, kin = hvp(0.0, 0.0, 4e303)
+    assert out[2] == np.inf and kin[2] == -np.inf
+    assert cs.status()["flags"] == 0
