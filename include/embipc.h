@@ -314,8 +314,9 @@ void eipc_set_programmatic_launch(int32_t on);
  * cannot afford the implicit device synchronisation of an allocation -- and so cannot
  * create an eipc_scene, whose workspace is allocated at creation.
  *
- * Same arithmetic as eipc_accd_toi, over a candidate list the caller supplies instead of
- * the LBVH search: for k < n_cand, pair (cand_type[k], cand_i[k], cand_j[k]) is a PT pair
+ * The kernels of eipc_accd_toi, hence its arithmetic bit for bit, over a candidate list the
+ * caller supplies instead of the LBVH search: for k < n_cand, pair (cand_type[k], cand_i[k],
+ * cand_j[k]) is a PT pair
  * (type 0: vertex i, triangle j) or an EE pair (type 1: edges i, j).  Candidates whose
  * closed FP64 swept boxes over [x, x + dx] do not overlap, and incident ones, are skipped,
  * so any superset of the overlapping pairs gives the same alpha.  This call has no
@@ -325,10 +326,10 @@ void eipc_set_programmatic_launch(int32_t on);
  * owned): x[Nv*3], dx[Nv*3], tris[F*3], edges[E*2], the three candidate arrays.  Outputs
  * (device, caller-owned): *alpha; *flags (EIPC_FLAG_PENETRATION / NONFINITE / ACCD_CAP /
  * BAD_INDEX, may be NULL); *n_advanced (candidates whose boxes overlap, may be NULL).
- * Scratch: a fixed device array inside the library holding two padded copies of the
- * positions, for at most eipc_accd_static_max_vertices() = 131,072 vertices (8 MiB plus a
- * 256-byte header, resident on every device that loads the library until the process
- * exits).  Nv above that returns EIPC_ERR_TOO_LARGE before anything is enqueued.
+ * Scratch: a fixed device array inside the library holding padded copies of the positions
+ * and displacements, for at most eipc_accd_static_max_vertices() = 131,072 vertices, and lists
+ * of candidates, which are taken 2^18 at a time (16 MiB plus a 256-byte header, resident on every
+ * device that loads the library until the process exits).  Nv above that returns EIPC_ERR_TOO_LARGE before anything is enqueued.
  * The first call on a device looks up that array's device address with the device
  * current (cudaGetSymbolAddress); make that first call before any stream capture.  The
  * address is kept for the life of the process: after cudaDeviceReset the library's module

@@ -68,8 +68,9 @@ __device__ __forceinline__ void decode_pair(const Topo& T, uint64_t key, int* ty
     v[0] = i;
     v[1] = T.tris[3 * (int64_t)j]; v[2] = T.tris[3 * (int64_t)j + 1]; v[3] = T.tris[3 * (int64_t)j + 2];
   } else {
-    const int2 a = reinterpret_cast<const int2*>(T.edges)[i], b = reinterpret_cast<const int2*>(T.edges)[j];
-    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+    // by single words: eipc_accd_toi_static's edges are the caller's, of any alignment
+    v[0] = T.edges[2 * (int64_t)i]; v[1] = T.edges[2 * (int64_t)i + 1];
+    v[2] = T.edges[2 * (int64_t)j]; v[3] = T.edges[2 * (int64_t)j + 1];
   }
 }
 
@@ -277,8 +278,10 @@ __global__ void __launch_bounds__(kAccdThreads) k_ccd_advance(Topo T, const doub
         if (t < 1.0) {
           // exact minimum, scene (of a batch) and whole; the plain read only saves atomics
           const unsigned long long tb = (unsigned long long)__double_as_longlong(t * kMargin);
-          unsigned long long* gb = group_bits + T.vgroup[v[0]];
-          if (tb < __ldcg(gb)) atomicMin(gb, tb);
+          if (group_bits) {
+            unsigned long long* gb = group_bits + T.vgroup[v[0]];
+            if (tb < __ldcg(gb)) atomicMin(gb, tb);
+          }
           if (tb < __ldcg(alpha_bits)) atomicMin(alpha_bits, tb);
         }
       }
@@ -301,6 +304,14 @@ __global__ void k_alpha_out(const unsigned long long* bits, double* alpha, const
 
 }  // namespace
 
+void ccd_bound_launch(const CcdBound& b, cudaStream_t s) {
+  launch(k_ccd_screen, blocks_for(b.cap, 8), kBlock, 0, s, b.topo, b.x4, b.dx4, b.x4f, b.dx4f, b.cand, b.n_cand, b.cap, b.s, b.list,
+         b.n_list, b.n_adv);
+  launch(k_ccd_advance, blocks_for(b.cap, 8, kAccdThreads), kAccdThreads, 0, s, b.topo, b.x4, b.dx4, b.x4f, b.dx4f,
+         static_cast<const uint64_t*>(b.list), static_cast<const int64_t*>(b.n_list), b.s, b.max_iter, b.alpha_bits, b.group_bits,
+         b.status, b.queue, b.tile);
+}
+
 void accd_launch(eipc_scene* sc, const double* x, const double* dx, const eipc_params& p, double* alpha,
                  int64_t* n_candidates, cudaStream_t s) {
   int64_t* n_cand = sc->counters + kCntCand;
@@ -321,14 +332,9 @@ void accd_launch(eipc_scene* sc, const double* x, const double* dx, const eipc_p
                        sc->tune.query_threads, sc->tune.query_bps));
   // cand2 is free here (the contact search's screened list)
   sc->timers->start(kKCa, s);
-  launch(k_ccd_screen, blocks_for(sc->cand_cap, 8), kBlock, 0, s, sc->topo, static_cast<const double*>(sc->x4),
-         static_cast<const double*>(sc->dx4), static_cast<const float*>(sc->x4f), static_cast<const float*>(sc->dx4f),
-         static_cast<const uint64_t*>(sc->cand), static_cast<const int64_t*>(n_cand), sc->cand_cap, p.accd_s, sc->cand2, n_list,
-         n_adv);
-  launch(k_ccd_advance, blocks_for(sc->cand_cap, 8, kAccdThreads), kAccdThreads, 0, s, sc->topo,
-         static_cast<const double*>(sc->x4), static_cast<const double*>(sc->dx4), static_cast<const float*>(sc->x4f),
-         static_cast<const float*>(sc->dx4f), static_cast<const uint64_t*>(sc->cand2), static_cast<const int64_t*>(n_list),
-         p.accd_s, p.accd_max_iter, abits, sc->group_alpha_bits, sc->status, queue, sc->tune.ccd_tile);
+  ccd_bound_launch(CcdBound{sc->topo, sc->x4, sc->dx4, sc->x4f, sc->dx4f, sc->cand, n_cand, sc->cand_cap, sc->cand2, n_list, n_adv,
+                            queue, p.accd_s, p.accd_max_iter, abits, sc->group_alpha_bits, sc->status, sc->tune.ccd_tile},
+                   s);
   sc->timers->stop(kKCa, s);
   launch(k_alpha_out, 1, 32, 0, s, abits, alpha, n_adv, n_candidates);
 }

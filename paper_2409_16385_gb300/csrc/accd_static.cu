@@ -2,179 +2,138 @@
 // its scratch memory in a fixed-size device array compiled into the library, so the call
 // allocates no device memory at all.
 //
-// The advancement arithmetic is the same as the scene-based eipc_accd_toi (accd.cu): exact
-// FP64 closed swept-box test, mean displacement removed, L = largest relative speed on
-// each side, advance by (1 - s) d(t) / L until d <= s d(0), t >= 1 or max_iter advances;
-// the pair's t is scaled by (1 - 2^-30) and alpha is the exact minimum over pairs.
-// Incident candidates (sharing a vertex) are skipped here because the caller builds the
-// list.
+// The caller's candidates are checked and packed into pair keys, kStaticChunk at a time, and go
+// through the kernels of the scene-based eipc_accd_toi (ccd_bound_launch): one compiled arithmetic,
+// hence the same bits.  (With kernels of its own, whose distances and advances were written
+// differently, a third of the advances rounded differently.)  Incident candidates (sharing a vertex)
+// are skipped here because the caller builds the list.
 #include <mutex>
 
 #include "geometry.cuh"
+#include "scene.cuh"
 
 namespace eipc {
 namespace {
 
 constexpr int64_t kStaticMaxVertices = 1 << 17;   // 131,072 vertices
-constexpr int kStaticThreads = 128;
-constexpr double kStaticMargin = 1.0 - 9.313225746154785e-10;   // 1 - 2^-30
+constexpr int64_t kStaticChunk = 1 << 18;         // candidates taken at a time
 
-// Layout: [0, 256): alpha bits (u64) at 0, flags (i32) at 8, advanced count (u64) at 16;
-// then padded x (32 B per vertex), then padded dx.
+// Layout: a header, then padded x and dx (32 B per vertex each), their FP32 copies (16 B each), and
+// two lists of pair keys.
+struct StaticHeader {
+  DevStatus status;
+  unsigned long long alpha_bits;
+  int64_t n_adv, n_keys, n_list, queue;
+};
 constexpr size_t kStaticHeader = 256;
-constexpr size_t kStaticBytes = kStaticHeader + 2 * (size_t)kStaticMaxVertices * 32;
+static_assert(sizeof(StaticHeader) <= kStaticHeader, "the header has its room");
+constexpr size_t kStaticBytes = kStaticHeader + (size_t)kStaticMaxVertices * (2 * 32 + 2 * 16) + 2 * (size_t)kStaticChunk * 8;
 
 static __device__ __align__(256) unsigned char g_accd_scratch[kStaticBytes];
 
 struct StaticView {
-  unsigned long long* alpha_bits;
-  int32_t* flags;
-  unsigned long long* n_adv;
+  StaticHeader* head;
   double* x4;
   double* dx4;
+  float* x4f;
+  float* dx4f;
+  uint64_t* keys;
+  uint64_t* list;
 };
 
-__host__ __device__ inline StaticView view_of(unsigned char* base) {
+StaticView view_of(unsigned char* base) {
   StaticView v;
-  v.alpha_bits = reinterpret_cast<unsigned long long*>(base);
-  v.flags = reinterpret_cast<int32_t*>(base + 8);
-  v.n_adv = reinterpret_cast<unsigned long long*>(base + 16);
-  v.x4 = reinterpret_cast<double*>(base + kStaticHeader);
-  v.dx4 = reinterpret_cast<double*>(base + kStaticHeader + (size_t)kStaticMaxVertices * 32);
+  v.head = reinterpret_cast<StaticHeader*>(base);
+  unsigned char* p = base + kStaticHeader;
+  v.x4 = reinterpret_cast<double*>(p);
+  v.dx4 = v.x4 + 4 * kStaticMaxVertices;
+  v.x4f = reinterpret_cast<float*>(v.dx4 + 4 * kStaticMaxVertices);
+  v.dx4f = v.x4f + 4 * kStaticMaxVertices;
+  v.keys = reinterpret_cast<uint64_t*>(v.dx4f + 4 * kStaticMaxVertices);
+  v.list = v.keys + kStaticChunk;
   return v;
 }
 
-// every call starts from alpha = 1, no flags, no advanced pairs
-__global__ void k_static_init(unsigned char* base) {
+// every call starts from alpha = 1, no flags, no advanced pairs; every chunk from empty lists
+__global__ void k_static_init(StaticHeader* h, bool first) {
   pdl_entry();
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    StaticView v = view_of(base);
-    *v.alpha_bits = (unsigned long long)__double_as_longlong(1.0);
-    *v.flags = 0;
-    *v.n_adv = 0ull;
+  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+  if (first) {
+    h->status = DevStatus{};
+    h->alpha_bits = (unsigned long long)__double_as_longlong(1.0);
+    h->n_adv = 0;
   }
+  h->n_keys = h->n_list = h->queue = 0;
 }
 
 __global__ void __launch_bounds__(256) k_static_pad(const double* __restrict__ x, const double* __restrict__ dx,
-                                                    int64_t nv, unsigned char* base) {
+                                                    int64_t nv, StaticView sv) {
   pdl_entry();
-  StaticView sv = view_of(base);
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < nv; v += gridDim.x * blockDim.x) {
     const double a = x[3 * v], b = x[3 * v + 1], c = x[3 * v + 2];
     const double e = dx[3 * v], f = dx[3 * v + 1], g = dx[3 * v + 2];
     if (!(isfinite(a) && isfinite(b) && isfinite(c) && isfinite(e) && isfinite(f) && isfinite(g)))
-      atomicOr(sv.flags, EIPC_FLAG_NONFINITE);
+      raise_flag(&sv.head->status, EIPC_FLAG_NONFINITE);
     reinterpret_cast<double2*>(sv.x4)[2 * v] = make_double2(a, b);
     reinterpret_cast<double2*>(sv.x4)[2 * v + 1] = make_double2(c, 0.0);
     reinterpret_cast<double2*>(sv.dx4)[2 * v] = make_double2(e, f);
     reinterpret_cast<double2*>(sv.dx4)[2 * v + 1] = make_double2(g, 0.0);
+    reinterpret_cast<float4*>(sv.x4f)[v] = make_float4(to_float<0>(a), to_float<0>(b), to_float<0>(c), 0.f);
+    reinterpret_cast<float4*>(sv.dx4f)[v] = make_float4(to_float<0>(e), to_float<0>(f), to_float<0>(g), 0.f);
   }
 }
 
-__device__ __forceinline__ double static_pair_distance(int type, const V3 p[4]) {
-  const V3 o = p[0];
-  if (type == 0) return sqrt(pt_distance<false>(p[0] - o, p[1] - o, p[2] - o, p[3] - o, nullptr));
-  return sqrt(ee_distance<false>(p[0] - o, p[1] - o, p[2] - o, p[3] - o, nullptr));
-}
-
-__global__ void __launch_bounds__(kStaticThreads) k_static_ca(int64_t nv, int64_t nf, int64_t ne,
-                                                              const int32_t* __restrict__ tris,
-                                                              const int32_t* __restrict__ edges, int64_t nc,
-                                                              const int32_t* __restrict__ ctype,
-                                                              const int32_t* __restrict__ ci,
-                                                              const int32_t* __restrict__ cj, double s, int max_iter,
-                                                              unsigned char* base) {
+// candidates [0, nc) whose ids are in range and that share no vertex, as pair keys
+__global__ void __launch_bounds__(kBlock) k_static_keys(Topo T, int64_t nc, const int32_t* __restrict__ ctype,
+                                                        const int32_t* __restrict__ ci, const int32_t* __restrict__ cj,
+                                                        StaticView sv) {
   pdl_entry();
-  StaticView sv = view_of(base);
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nc; k += gridDim.x * blockDim.x) {
-    const int type = ctype[k];
-    const int32_t i = ci[k], j = cj[k];
-    const bool ids_ok = (type == 0) ? (i >= 0 && i < nv && j >= 0 && j < nf)
-                                    : (type == 1 && i >= 0 && i < ne && j >= 0 && j < ne);
-    if (!ids_ok) {
-      atomicOr(sv.flags, EIPC_FLAG_BAD_INDEX);
-      continue;
-    }
-    int32_t v[4];
-    if (type == 0) {
-      v[0] = i;
-      v[1] = tris[3 * (int64_t)j]; v[2] = tris[3 * (int64_t)j + 1]; v[3] = tris[3 * (int64_t)j + 2];
-    } else {
-      v[0] = edges[2 * (int64_t)i]; v[1] = edges[2 * (int64_t)i + 1];
-      v[2] = edges[2 * (int64_t)j]; v[3] = edges[2 * (int64_t)j + 1];
-    }
-    bool bad_id = false;
-    for (int a = 0; a < 4; ++a) bad_id |= (v[a] < 0 || v[a] >= nv);
-    if (bad_id) {
-      atomicOr(sv.flags, EIPC_FLAG_BAD_INDEX);
-      continue;
-    }
-    const int na = type == 0 ? 1 : 2;
-    bool incident = false;
-    for (int a = 0; a < na; ++a)
-      for (int b = na; b < 4; ++b) incident |= (v[a] == v[b]);
-    if (incident) continue;
-    V3 X[4], D[4];
-    for (int a = 0; a < 4; ++a) { X[a] = load_x(sv.x4, v[a]); D[a] = load_x(sv.dx4, v[a]); }
-    double lo[2][3], hi[2][3];
-    for (int sd = 0; sd < 2; ++sd)
-      for (int c = 0; c < 3; ++c) { lo[sd][c] = INFINITY; hi[sd][c] = -INFINITY; }
-    for (int a = 0; a < 4; ++a) {
-      const int sd = a < na ? 0 : 1;
-      const double p0[3] = {X[a].x, X[a].y, X[a].z};
-      const double p1[3] = {X[a].x + D[a].x, X[a].y + D[a].y, X[a].z + D[a].z};
-      for (int c = 0; c < 3; ++c) {
-        lo[sd][c] = fmin(lo[sd][c], fmin(p0[c], p1[c]));
-        hi[sd][c] = fmax(hi[sd][c], fmax(p0[c], p1[c]));
-      }
-    }
-    bool ov = true;
-    for (int c = 0; c < 3; ++c) ov &= !(lo[0][c] > hi[1][c] || lo[1][c] > hi[0][c]);
-    if (!ov) continue;
-    atomicAdd(sv.n_adv, 1ull);
-    const V3 mean = (D[0] + D[1] + D[2] + D[3]) * 0.25;
-    V3 R[4];
-    double la = 0.0, lb = 0.0;
-    for (int a = 0; a < 4; ++a) {
-      R[a] = D[a] - mean;
-      const double sp = sqrt(dot(R[a], R[a]));
-      if (a < na) la = fmax(la, sp); else lb = fmax(lb, sp);
-    }
-    const double L = la + lb;
-    double t = 1.0;
-    if (L > 0.0) {
-      const double d0 = static_pair_distance(type, X);
-      if (!(d0 > 0.0)) {
-        atomicOr(sv.flags, EIPC_FLAG_PENETRATION);
-        t = 0.0;
-      } else {
-        double d = d0;
-        int iters = 0;
-        t = 0.0;
-        while (true) {
-          const double tn = t + (1.0 - s) * d / L;
-          if (tn >= 1.0) { t = 1.0; break; }
-          t = tn;
-          V3 P[4];
-          for (int a = 0; a < 4; ++a) P[a] = X[a] + R[a] * t;
-          d = static_pair_distance(type, P);
-          ++iters;
-          if (d <= s * d0) break;
-          if (iters >= max_iter) { atomicOr(sv.flags, EIPC_FLAG_ACCD_CAP); break; }
+  const int lane = threadIdx.x & 31;
+  for (int64_t base = blockIdx.x * (int64_t)blockDim.x; base < nc; base += grid_stride()) {
+    const int64_t k = base + threadIdx.x;
+    bool keep = false;
+    uint64_t key = 0;
+    if (k < nc) {
+      const int type = ctype[k];
+      const int32_t i = ci[k], j = cj[k];
+      bool ids_ok = (type == 0) ? (i >= 0 && i < T.nv && j >= 0 && j < T.nf)
+                                : (type == 1 && i >= 0 && i < T.ne && j >= 0 && j < T.ne);
+      if (ids_ok) {
+        int32_t v[4];
+        if (type == 0) {
+          v[0] = i;
+          v[1] = T.tris[3 * (int64_t)j]; v[2] = T.tris[3 * (int64_t)j + 1]; v[3] = T.tris[3 * (int64_t)j + 2];
+        } else {
+          v[0] = T.edges[2 * (int64_t)i]; v[1] = T.edges[2 * (int64_t)i + 1];
+          v[2] = T.edges[2 * (int64_t)j]; v[3] = T.edges[2 * (int64_t)j + 1];
         }
+        for (int a = 0; a < 4; ++a) ids_ok = ids_ok && v[a] >= 0 && v[a] < T.nv;
+        const int na = type == 0 ? 1 : 2;
+        bool incident = false;
+        for (int a = 0; a < na; ++a)
+          for (int b = na; b < 4; ++b) incident |= (v[a] == v[b]);
+        keep = ids_ok && !incident;
+        key = pair_key(type, (uint32_t)i, (uint32_t)j, T.bits_i, T.bits_j);
       }
+      if (!ids_ok) raise_flag(&sv.head->status, EIPC_FLAG_BAD_INDEX);
     }
-    if (t < 1.0) atomicMin(sv.alpha_bits, (unsigned long long)__double_as_longlong(t * kStaticMargin));
+    const uint32_t mask = __ballot_sync(0xffffffffu, keep);
+    if (mask) {
+      unsigned long long b = 0;
+      if (lane == 0) b = atomicAdd(reinterpret_cast<unsigned long long*>(&sv.head->n_keys), (unsigned long long)__popc(mask));
+      b = __shfl_sync(0xffffffffu, b, 0);
+      // keys never outnumber the chunk's candidates
+      if (keep) sv.keys[(int64_t)b + __popc(mask & ((1u << lane) - 1u))] = key;
+    }
   }
 }
 
-__global__ void k_static_out(const unsigned char* base, double* alpha, int32_t* flags, int64_t* n_adv) {
+__global__ void k_static_out(const StaticHeader* h, double* alpha, int32_t* flags, int64_t* n_adv) {
   pdl_entry();
   if (threadIdx.x == 0 && blockIdx.x == 0) {
-    StaticView v = view_of(const_cast<unsigned char*>(base));
-    *alpha = __longlong_as_double((long long)*v.alpha_bits);
-    if (flags) *flags = *v.flags;
-    if (n_adv) *n_adv = (int64_t)*v.n_adv;
+    *alpha = __longlong_as_double((long long)h->alpha_bits);
+    if (flags) *flags = h->status.flags;
+    if (n_adv) *n_adv = h->n_adv;
   }
 }
 
@@ -218,16 +177,25 @@ extern "C" eipc_status eipc_accd_toi_static(int64_t Nv, int64_t F, int64_t E, co
   unsigned char* base = nullptr;
   if (scratch_address(&base) != cudaSuccess) return EIPC_ERR_CUDA;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  launch(k_static_init, 1, 32, 0, s, base);
-  int pb = (int)((Nv + 255) / 256);
-  if (pb > kSMs * 4) pb = kSMs * 4;
-  launch(k_static_pad, pb, 256, 0, s, x, dx, Nv, base);
-  if (n_cand > 0) {
-    int cb = (int)((n_cand + kStaticThreads - 1) / kStaticThreads);
-    if (cb > kSMs * 16) cb = kSMs * 16;
-    launch(k_static_ca, cb, kStaticThreads, 0, s, Nv, F, E, tris, edges, n_cand, cand_type, cand_i, cand_j, p->accd_s,
-           (int)p->accd_max_iter, base);
+  const StaticView sv = view_of(base);
+  launch(k_static_init, 1, 32, 0, s, sv.head, true);
+  launch(k_static_pad, blocks_for(Nv, 4), kBlock, 0, s, x, dx, Nv, sv);
+  Topo T{};
+  T.nv = Nv; T.ne = E; T.nf = F;
+  T.tris = tris; T.edges = edges;
+  constexpr int64_t kMaxId = (1ll << 31) - 1;        // ids are 32 bits wide, whatever the counts
+  const int64_t most_i = Nv > E ? Nv : E, most_j = F > E ? F : E;
+  T.bits_i = bits_for((uint64_t)(most_i < kMaxId ? most_i : kMaxId));
+  T.bits_j = bits_for((uint64_t)(most_j < kMaxId ? most_j : kMaxId));
+  for (int64_t k = 0; k < n_cand; k += kStaticChunk) {
+    const int64_t n = n_cand - k < kStaticChunk ? n_cand - k : kStaticChunk;
+    if (k > 0) launch(k_static_init, 1, 32, 0, s, sv.head, false);
+    launch(k_static_keys, blocks_for(n, 8), kBlock, 0, s, T, n, cand_type + k, cand_i + k, cand_j + k, sv);
+    ccd_bound_launch(CcdBound{T, sv.x4, sv.dx4, sv.x4f, sv.dx4f, sv.keys, &sv.head->n_keys, n, sv.list, &sv.head->n_list,
+                              &sv.head->n_adv, &sv.head->queue, p->accd_s, (int)p->accd_max_iter, &sv.head->alpha_bits, nullptr,
+                              &sv.head->status, 32},
+                     s);
   }
-  launch(k_static_out, 1, 32, 0, s, static_cast<const unsigned char*>(base), alpha, flags, n_advanced);
+  launch(k_static_out, 1, 32, 0, s, static_cast<const StaticHeader*>(sv.head), alpha, flags, n_advanced);
   return cudaPeekAtLastError() == cudaSuccess ? EIPC_OK : EIPC_ERR_CUDA;
 }

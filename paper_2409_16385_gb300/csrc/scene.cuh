@@ -169,4 +169,29 @@ void bsr_spmv_launch(int64_t nrows, const int32_t* row_ptr, const int32_t* col, 
 void group_alpha_launch(eipc_scene* sc, double* alpha_groups, cudaStream_t s);
 void accd_launch(eipc_scene* sc, const double* x, const double* dx, const eipc_params& p, double* alpha,
                  int64_t* n_candidates, cudaStream_t s);
+
+// The step bound over a list of pair keys: the kernels of eipc_accd_toi and of
+// eipc_accd_toi_static alike, so that both give the same bits.  The counters of `list`, `n_adv` and
+// `queue` are reset by the caller, alpha_bits (and group_bits, null: none) to one.
+struct CcdBound {
+  Topo topo;
+  const double* x4;          // positions and displacements, padded, and their FP32 copies
+  const double* dx4;
+  const float* x4f;
+  const float* dx4f;
+  const uint64_t* cand;      // [cap] pair keys, and their number
+  const int64_t* n_cand;
+  int64_t cap;
+  uint64_t* list;            // [cap] scratch: those that need the advancement, and their number
+  int64_t* n_list;
+  int64_t* n_adv;            // + candidates whose swept boxes overlap
+  int64_t* queue;
+  double s;
+  int max_iter;
+  unsigned long long* alpha_bits;
+  unsigned long long* group_bits;
+  DevStatus* status;
+  int tile;
+};
+void ccd_bound_launch(const CcdBound& b, cudaStream_t s);
 }  // namespace eipc
