@@ -8,9 +8,10 @@ Results never depend on the shape: every kernel is a grid-stride loop over a dev
 count, and every reduction order is fixed by sort keys, not by the launch.  So the tuner
 is free to pick on time alone.  It times each candidate with the library's per-kernel
 CUDA-event timers on the caller's own stage (one call of `stage()` runs the workload once),
-takes the median of a few repetitions, and keeps the fastest.  Choices are cached in a
-JSON file keyed by device name, compute capability and a workload key chosen by the
-caller, so later runs on the same kind of GPU and workload skip the search.
+takes the median of a few repetitions, and keeps the fastest, which is the library's default
+unless another is faster.  Choices are cached in a JSON file keyed by device name, compute
+capability and a workload key chosen by the caller, so later runs on the same kind of GPU
+and workload skip the search.
 """
 from __future__ import annotations
 
@@ -23,12 +24,15 @@ EVAL_SPACE: Tuple[Tuple[int, int, int], ...] = tuple(
 # items a warp claims from the evaluation's / CCD advancement's work queue at a time
 TILE_SPACE: Tuple[Tuple[int, int, int], ...] = tuple((items, 1, 0) for items in (32, 64, 128, 256))
 QUERY_SPACE: Tuple[Tuple[int, int, int], ...] = tuple(
-    (threads, bps, variant) for threads in (64, 128, 256) for bps in (2, 4, 8, 12, 16, 24, 32) for variant in (2, 3))
+    (threads, bps, variant) for threads in (64, 128, 256) for bps in (2, 4, 8, 12, 16, 24, 32, 64) for variant in (2, 3))
 
 REFIT_SPACE: Tuple[Tuple[int, int, int], ...] = ((256, 8, 0), (256, 8, 1), (256, 8, 2))
 
 SPACES = {"eval_barrier": EVAL_SPACE, "bvh_query": QUERY_SPACE, "bvh_refit": REFIT_SPACE, "eval_tile": TILE_SPACE,
           "ccd_tile": TILE_SPACE}
+# the shapes a scene is created with, each in its space
+DEFAULTS = {"eval_barrier": (128, 16, 2), "bvh_query": (128, 64, 2), "bvh_refit": (256, 8, 2), "eval_tile": (32, 1, 0),
+            "ccd_tile": (128, 1, 0)}
 # the library timer that brackets each tunable kernel's launches
 TIMERS = {"eval_barrier": "eval_barrier", "bvh_query": "bvh_query", "bvh_refit": "bvh_build",
           "eval_tile": "eval_barrier", "ccd_tile": "ccd_advance"}
@@ -97,10 +101,14 @@ def tune(cs, stage: Callable[[], None], workload_key: str,
             out[kernel] = dict(entry[kernel], cached=True)
             continue
         timer = TIMERS[kernel]
+        best = DEFAULTS[kernel]
+        cs.set_launch(kernel, *best)
         stage()                                   # warm: hierarchies built, caches primed
-        default_ms = time_kernel(cs, stage, timer, reps)
-        best, best_ms, seen = None, float("inf"), {}
+        default_ms = best_ms = time_kernel(cs, stage, timer, reps)
+        seen = {"x".join(map(str, best)): default_ms}
         for shape in SPACES[kernel]:
+            if shape == DEFAULTS[kernel]:
+                continue
             cs.set_launch(kernel, *shape)
             stage()
             ms = time_kernel(cs, stage, timer, reps)

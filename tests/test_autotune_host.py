@@ -91,3 +91,18 @@ def test_unreadable_cache_is_ignored(tmp_path):
     res = autotune.tune(cs, lambda: None, "w", kernels=("bvh_refit",), cache_path=str(cache))
     assert res["bvh_refit"]["shape"] == [256, 8, 1]
     assert json.loads(cache.read_text())["fake|sm_103|152sm|w"]["bvh_refit"]["shape"] == [256, 8, 1]
+
+
+@pytest.mark.parametrize("kernel", sorted(autotune.SPACES))
+def test_the_default_is_kept_unless_another_shape_is_faster(tmp_path, kernel):
+    default = autotune.DEFAULTS[kernel]
+    assert default in autotune.SPACES[kernel]
+    for faster in [default] + [s for s in autotune.SPACES[kernel] if s != default][:1]:
+        cs = FakeScene(lambda k, shape: 1.0 if shape == faster else 2.0)
+        cs.shape[kernel] = autotune.SPACES[kernel][-1]          # a scene that was given another shape before
+        res = autotune.tune(cs, lambda: None, "w", kernels=(kernel,), cache_path=str(tmp_path / "t.json"), force=True)
+        assert cs.shape[kernel] == faster and res[kernel]["shape"] == list(faster)
+        assert res[kernel]["default_ms"] == (1.0 if faster == default else 2.0)
+    cs = FakeScene(lambda k, shape: 2.0)
+    autotune.tune(cs, lambda: None, "w", kernels=(kernel,), cache_path=str(tmp_path / "t.json"), force=True)
+    assert cs.shape[kernel] == default
