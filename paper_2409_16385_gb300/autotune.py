@@ -1,8 +1,7 @@
 """Launch-shape autotuner for the kernels whose best shape depends on the workload: the
-per-pair barrier evaluation (threads per block, grid cap in blocks per SM, register
-budget), the pair tile of its work queue and of the CCD advancement's (items a warp claims
-at a time), the BVH traversal (threads per block, grid cap, register budget) and the BVH
-refit (how its bottom-up arrival counters are ordered).
+per-pair evaluation (threads per block, grid cap in blocks per SM), the pair tile of its work
+queue and of the CCD advancement's (items a warp claims at a time) and the BVH traversal
+(threads per block, grid cap).  Of the BVH refit one shape is left.
 
 Results never depend on the shape: every kernel is a grid-stride loop over a device-side
 count, and every reduction order is fixed by sort keys, not by the launch.  So the tuner
@@ -19,19 +18,20 @@ import json
 import os
 from typing import Callable, Dict, Iterable, Optional, Tuple
 
+# (threads, blocks per SM, variant).  One form of each kernel is compiled, so every variant the
+# library accepts is the same launch: each shape is listed, and timed, once.
 EVAL_SPACE: Tuple[Tuple[int, int, int], ...] = tuple(
-    (threads, bps, variant) for threads in (64, 128) for bps in (2, 3, 4, 6, 8, 16) for variant in (2, 3, 4))
+    (threads, bps, 3) for threads in (64, 128) for bps in (2, 3, 4, 6, 8, 16))
 # items a warp claims from the evaluation's / CCD advancement's work queue at a time
 TILE_SPACE: Tuple[Tuple[int, int, int], ...] = tuple((items, 1, 0) for items in (32, 64, 128, 256))
 QUERY_SPACE: Tuple[Tuple[int, int, int], ...] = tuple(
-    (threads, bps, variant) for threads in (64, 128, 256) for bps in (2, 4, 8, 12, 16, 24, 32, 64) for variant in (2, 3))
-
-REFIT_SPACE: Tuple[Tuple[int, int, int], ...] = ((256, 8, 0), (256, 8, 1), (256, 8, 2))
+    (threads, bps, 2) for threads in (64, 128, 256) for bps in (2, 4, 8, 12, 16, 24, 32, 64))
+REFIT_SPACE: Tuple[Tuple[int, int, int], ...] = ((256, 8, 1),)
 
 SPACES = {"eval_barrier": EVAL_SPACE, "bvh_query": QUERY_SPACE, "bvh_refit": REFIT_SPACE, "eval_tile": TILE_SPACE,
           "ccd_tile": TILE_SPACE}
 # the shapes a scene is created with, each in its space
-DEFAULTS = {"eval_barrier": (128, 16, 2), "bvh_query": (128, 64, 2), "bvh_refit": (256, 8, 2), "eval_tile": (32, 1, 0),
+DEFAULTS = {"eval_barrier": (128, 16, 3), "bvh_query": (128, 64, 2), "bvh_refit": (256, 8, 1), "eval_tile": (32, 1, 0),
             "ccd_tile": (128, 1, 0)}
 # the library timer that brackets each tunable kernel's launches
 TIMERS = {"eval_barrier": "eval_barrier", "bvh_query": "bvh_query", "bvh_refit": "bvh_build",

@@ -238,11 +238,11 @@ eipc_status eipc_scene_create(int64_t Nv, int64_t F, int64_t E, int64_t Ns, cons
   }
   s->rebuild_interval = 8;
   // the scene was zero-filled after construction: every launch-shape default is set here
-  s->tune.eval_threads = 128; s->tune.eval_bps = 16; s->tune.eval_variant = 2; s->tune.eval_tile = 32;
+  s->tune.eval_threads = 128; s->tune.eval_bps = 16; s->tune.eval_tile = 32;
   s->tune.ccd_tile = 128;
   // the traversal's warps differ widely in work: up to 64 blocks an SM leave it to the chip to even
   // them out (256-scene batch 5,116 us a step with 24, 4,970 with 64; smaller scenes need fewer)
-  s->tune.query_threads = 128; s->tune.query_bps = 64; s->tune.query_variant = 2; s->tune.refit_variant = 2;
+  s->tune.query_threads = 128; s->tune.query_bps = 64;
   s->contact_refits = 0;
   *out = s;
   return EIPC_OK;
@@ -457,25 +457,22 @@ eipc_status eipc_group_alpha(eipc_scene* sc, double* alpha_groups, eipc_stream s
 
 eipc_status eipc_set_launch(eipc_scene* sc, int32_t kernel, int32_t threads, int32_t blocks_per_sm,
                             int32_t variant) {
+  // one form of each kernel is compiled: the variants that are accepted have no effect
   if (!sc || blocks_per_sm < 1 || blocks_per_sm > 64) return EIPC_ERR_INVALID;
   if (kernel == 0) {
     if ((threads != 64 && threads != 128) || variant < 2 || variant > 4) return EIPC_ERR_INVALID;
     sc->tune.eval_threads = threads;
     sc->tune.eval_bps = blocks_per_sm;
-    sc->tune.eval_variant = variant;
     return EIPC_OK;
   }
   if (kernel == 1) {
     if ((threads != 64 && threads != 128 && threads != 256) || (variant != 2 && variant != 3)) return EIPC_ERR_INVALID;
     sc->tune.query_threads = threads;
     sc->tune.query_bps = blocks_per_sm;
-    sc->tune.query_variant = variant;
     return EIPC_OK;
   }
   if (kernel == 2) {
-    if (threads != 256 || variant < 0 || variant > 2) return EIPC_ERR_INVALID;
-    sc->tune.refit_variant = variant;
-    return EIPC_OK;
+    return threads != 256 || variant < 0 || variant > 2 ? EIPC_ERR_INVALID : EIPC_OK;
   }
   if (kernel == 3 || kernel == 4) {
     // work-queue tiles: `threads` = items a warp claims at a time (32, 64, 128 or 256)

@@ -89,10 +89,9 @@ struct eipc_scene {
   int bits_h, bits_g;    // key widths of the reduction sorts
   int rebuild_interval;  // contact LBVH: full rebuild every this many build_candidates calls
   struct {
-    int eval_threads = 128, eval_bps = 16, eval_variant = 2, eval_tile = 32;
+    int eval_threads = 128, eval_bps = 16, eval_tile = 32;
     int ccd_tile = 128;
-    int query_threads = 128, query_bps = 64, query_variant = 2;
-    int refit_variant = 2;
+    int query_threads = 128, query_bps = 64;
   } tune;                // launch shapes of the tunable kernels (eipc_set_launch)
   int contact_refits;    // refits since the last full rebuild
   eipc::DevStatus* status;

@@ -106,3 +106,15 @@ def test_the_default_is_kept_unless_another_shape_is_faster(tmp_path, kernel):
     cs = FakeScene(lambda k, shape: 2.0)
     autotune.tune(cs, lambda: None, "w", kernels=(kernel,), cache_path=str(tmp_path / "t.json"), force=True)
     assert cs.shape[kernel] == default
+
+
+def test_defaults_are_the_librarys_and_no_launch_is_listed_twice():
+    import os
+    import re
+    src = open(os.path.join(os.path.dirname(autotune.__file__), "csrc", "api.cu")).read()
+    tune = {k: int(v) for k, v in re.findall(r"s->tune\.(\w+) = (\d+);", src)}
+    assert autotune.DEFAULTS["eval_barrier"][:2] == (tune["eval_threads"], tune["eval_bps"])
+    assert autotune.DEFAULTS["bvh_query"][:2] == (tune["query_threads"], tune["query_bps"])
+    assert autotune.DEFAULTS["eval_tile"][0] == tune["eval_tile"] and autotune.DEFAULTS["ccd_tile"][0] == tune["ccd_tile"]
+    for space in autotune.SPACES.values():
+        assert len({s[:2] for s in space}) == len(space)
