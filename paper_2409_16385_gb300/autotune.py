@@ -10,7 +10,7 @@ CUDA-event timers on the caller's own stage (one call of `stage()` runs the work
 takes the median of a few repetitions, and keeps the fastest, which is the library's default
 unless another is faster.  Choices are cached in a JSON file keyed by device name, compute
 capability and a workload key chosen by the caller, so later runs on the same kind of GPU
-and workload skip the search.
+and workload skip the search; a choice made for other kernels (KERNELS) is searched again.
 """
 from __future__ import annotations
 
@@ -33,6 +33,8 @@ SPACES = {"eval_barrier": EVAL_SPACE, "bvh_query": QUERY_SPACE, "bvh_refit": REF
 # the shapes a scene is created with, each in its space
 DEFAULTS = {"eval_barrier": (128, 16, 3), "bvh_query": (128, 64, 2), "bvh_refit": (256, 8, 1), "eval_tile": (32, 1, 0),
             "ccd_tile": (128, 1, 0)}
+# raised when the tunable kernels change so much that shapes timed before mean nothing
+KERNELS = 2
 # the library timer that brackets each tunable kernel's launches
 TIMERS = {"eval_barrier": "eval_barrier", "bvh_query": "bvh_query", "bvh_refit": "bvh_build",
           "eval_tile": "eval_barrier", "ccd_tile": "ccd_advance"}
@@ -95,7 +97,7 @@ def tune(cs, stage: Callable[[], None], workload_key: str,
     entry = table.get(key, {})
     out = {}
     for kernel in kernels:
-        if not force and kernel in entry:
+        if not force and entry.get(kernel, {}).get("kernels") == KERNELS:
             shape = entry[kernel]["shape"]
             cs.set_launch(kernel, *shape)
             out[kernel] = dict(entry[kernel], cached=True)
@@ -116,7 +118,7 @@ def tune(cs, stage: Callable[[], None], workload_key: str,
             if ms < best_ms:
                 best, best_ms = shape, ms
         cs.set_launch(kernel, *best)
-        entry[kernel] = dict(shape=list(best), ms=best_ms, default_ms=default_ms, candidates=seen)
+        entry[kernel] = dict(shape=list(best), ms=best_ms, default_ms=default_ms, candidates=seen, kernels=KERNELS)
         out[kernel] = dict(entry[kernel], cached=False)
     table[key] = entry
     _store(path, table)

@@ -118,3 +118,14 @@ def test_defaults_are_the_librarys_and_no_launch_is_listed_twice():
     assert autotune.DEFAULTS["eval_tile"][0] == tune["eval_tile"] and autotune.DEFAULTS["ccd_tile"][0] == tune["ccd_tile"]
     for space in autotune.SPACES.values():
         assert len({s[:2] for s in space}) == len(space)
+
+
+def test_shapes_cached_for_other_kernels_are_searched_again(tmp_path):
+    cache = tmp_path / "tune.json"
+    old = {"shape": [256, 8, 2], "ms": 1.0, "default_ms": 1.0, "candidates": {}}
+    cache.write_text(json.dumps({"fake|sm_103|152sm|w": {"bvh_query": old}}))
+    calls = []
+    res = autotune.tune(FakeScene(_cost), lambda: calls.append(1), "w", kernels=("bvh_query",), cache_path=str(cache))
+    assert calls and not res["bvh_query"]["cached"] and res["bvh_query"]["shape"] == [256, 12, 2]
+    res = autotune.tune(FakeScene(_cost), lambda: calls.append(1), "w", kernels=("bvh_query",), cache_path=str(cache))
+    assert res["bvh_query"]["cached"]
