@@ -184,12 +184,15 @@ def measured_peaks():
 #   eval_barrier  FP64 flops per contact pair, counted by ncu on the bubble-grasp workload
 #                 ((2 x DFMA + DMUL + DADD) thread instructions / pairs), the lagged
 #                 friction of the pairs that carry it included
-#   ccd_advance   FP64 flops per advanced CCD candidate (box test, advancement distances)
+#   ccd_advance   FP64 flops per counted CCD candidate: almost all of them are settled in FP32
+#                 (k_ccd_screen), so this FP64 fraction is small and not what bounds the stage
 #   others        DRAM bytes per unit of their minimum input + output traffic
 # eval_barrier: 71.08e6 flops of k_eval_factors and k_eval_rest over the 115,699 pairs of
 # bubble-grasp iterate 2 (ncu); see profiles/
 FP64_FLOPS_PER_PAIR = 614.3
-FP64_FLOPS_PER_CCD_CAND = 420.0
+# ccd_advance: 0.259e6 flops of k_ccd_screen and k_ccd_advance over the 187,823 candidates of a
+# bubble-grasp step bound (ncu)
+FP64_FLOPS_PER_CCD_CAND = 1.38
 # DRAM bytes (read + write) per unit from one ncu capture of the same kernel code and shape
 # (eval_barrier: 36.0 MB + 24.9 MB for the same 115,699 pairs)
 NCU_TRAFFIC_PER_UNIT = {"eval_barrier": 526.5}
@@ -226,7 +229,7 @@ def roofline_figure(name, total_ms, launches, steps, per_step, sc, fp64_probe=No
         peak = FP64_PEAK_TFLOPS
         out = dict(bound="alu", achieved=ach, peak=peak, unit="TFLOP/s", frac=ach / peak,
                    traffic=(tr * units if tr else None), kernel=name, launch_ms=avg_s * 1e3,
-                   units_per_launch=units, unit_cost=f"{per:.0f} FP64 flop per unit",
+                   units_per_launch=units, unit_cost=f"{per:.4g} FP64 flop per unit",
                    peak_source="derived: 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz (FP64)")
         if fp64_probe:
             out["peak_probe"] = fp64_probe["tflops"]
