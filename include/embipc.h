@@ -49,12 +49,15 @@ enum {
   EIPC_FLAG_PENETRATION = 1,  /* some pair has d <= 0: the configuration is infeasible  */
   EIPC_FLAG_PAIR_OVERFLOW = 2,/* more contact pairs than the caller's pair capacity     */
   EIPC_FLAG_CAND_OVERFLOW = 4,/* more broad-phase candidates than the scene workspace   */
-  EIPC_FLAG_REC_OVERFLOW = 8, /* more reduction records than the scene workspace        */
+  EIPC_FLAG_REC_OVERFLOW = 8, /* more reduction records than the scene workspace (n (n+1)/2 of
+                                 every item of n cage nodes, an upper bound where the mollifier is
+                                 off: the outputs may then be complete), or more items           */
   EIPC_FLAG_BSR_OVERFLOW = 16,/* more BSR blocks than the caller's block capacity       */
   EIPC_FLAG_NONFINITE = 32,   /* a non-finite position or displacement was read         */
   EIPC_FLAG_ACCD_CAP = 64,    /* a CCD pair reached accd_max_iter (alpha still safe)    */
   EIPC_FLAG_LAG_OVERFLOW = 128,/* more friction pairs than the lag buffer capacity      */
-  EIPC_FLAG_STACK_OVERFLOW = 256,/* a BVH traversal exceeded its 64-entry stack         */
+  EIPC_FLAG_STACK_OVERFLOW = 256,/* a BVH traversal exceeded its list of 128 nodes, or a work
+                                    queue more claims than its items can supply (a guard)       */
   EIPC_FLAG_BAD_INDEX = 512   /* a caller-supplied candidate names an out-of-range id   */
 };
 

@@ -337,7 +337,10 @@ __device__ __forceinline__ bool arrive_first(int32_t* f) {
 // (454,550 triangles and edges) 46.3 and 32.5 us.  On larger scenes the chip is full with a warp
 // per treelet, and blocks that wait between a cluster's phases keep fewer reads in flight: the
 // subtrees are the treelets and the climb is in L2.  256-scene batch (10.5 M) 129 + 99 us, by
-// clusters 519 + 35 us; 211 + 150 us with shuffled integer reductions and 256-thread blocks.
+// clusters 519 + 35 us; 211 + 150 us with shuffled integer reductions and 256-thread blocks.  Batches
+// of 8 to 96 scenes, caches flushed, by clusters and by treelets: 0.32 M primitives 30 and 40 us, 0.55 M
+// 39 and 46, 0.98 M 58 and 52, 1.31 M 105 and 59, 3.92 M 159 and 101: the two meet near 0.8 M, and the
+// line costs up to 6 us between there and 2^20.
 constexpr int64_t kClusterPrims = 1 << 20;
 
 __global__ void __launch_bounds__(kBlock) k_refit_leaves(TreeView A, TreeView B, const float* __restrict__ vbox) {

@@ -9,24 +9,26 @@
 //   hess E = kappa [(b'' - b'/d) (c c^T) (x) (r^ r^T) + (b'/d) (c c^T) (x) I3]
 //            - (kappa b' / (2d)) G M^-1 G^T.
 // Every term lies in the span of {c^ (x) e_x, c^ (x) e_y, c^ (x) e_z, a^_1 (x) r^, a^_2 (x) r^}
-// (a^_j: a_j orthonormalised against c), an orthonormal basis Q of at most 5 columns.  The
-// 12x12 Hessian is Q K Q^T with K (<= 5x5) in closed form; its projection onto the PSD cone
-// (projected Newton, Sec. III-C) is Q K+ Q^T with K+ from a 5x5 Jacobi eigensolve -- the
-// same matrix as projecting the 12x12 itself, because P+ acts on eigenpairs and the
-// complement of span(Q) is the zero eigenspace.
+// (a^_j: a_j orthonormalised against c), an orthonormal basis of at most 5 columns, so projecting
+// the 12x12 Hessian onto the PSD cone (projected Newton, Sec. III-C) is projecting a matrix of at
+// most 5x5: P+ acts on eigenpairs and the complement of the span is the zero eigenspace.  That
+// projection is closed form: its one or two negative eigenvectors are roots of small secular
+// equations, and what is left has rank two or three, P+ = sum_k z_k z_k^T (see "pair factors").
 //
 // Reduction (Eq. 17): g_r = J^T g, H_r = J^T H J.  J restricted to a stencil maps the
-// stencil's unique cage nodes I to the 4 vertices with weights w_aI, so Q's columns map to
-// per-node scalars omega_I = sum_a c^_a w_aI, alpha_jI = sum_a a^_j[a] w_aI, and
-//   block(I, J) = A_I K+ A_J^T,   A_I = [omega_I I3 | alpha_1I r^ | alpha_2I r^]  (3x5).
+// stencil's unique cage nodes I to the 4 vertices with weights w_aI, so an item leaves one row of
+// factors per node, z_kI with the scalars omega_I = sum_a c_a w_aI, and block(I, J) = sum_k z_kI
+// z_kJ^T.
 // Friction (Sec. III-B, lagged): D = mu lambda f0(|u|), u = (I - n n^T)(sum gamma_a x_a - anchor),
 //   grad = mu lambda f1(y)/y gamma (x) u,   hess = (gamma gamma^T) (x) F,
 //   F = mu lambda [(f1/y)(I - n n^T) + (f1' - f1/y) u^ u^T]   (PSD as written).
-// Records (key = I * Ns + J, 3x3 block): the keys depend only on each item's cage nodes, so
-// they are written and stably sorted before the evaluation, which then writes every block to
-// its sorted position; each key's records are summed in a fixed order that depends only on
-// that key's own records (32-record units, then a fixed warp tree), so the result is bitwise
-// repeatable and the same for a scene alone or inside a batch.
+// Records: items with the same nodes form a group, in the order of a stable sort by node set, and
+// a group is cut into chunks of 16 items from its own start; a record is one upper block of one
+// chunk, multiplied out of its items' rows in their order (k_chunk_sums).  The records are stably
+// sorted by block (key: its position in the upper triangle), and a block is the sum of its records
+// by three interleaved chains that start at its first one (k_segment_sums).  Groups, chunks and
+// chains depend on the scene's own items alone, so a result is bitwise repeatable and the same for
+// a scene alone or inside a batch.
 #include "geometry.cuh"
 #include "scene.cuh"
 #include "sort.cuh"
@@ -188,7 +190,11 @@ __global__ void __launch_bounds__(kBlock) k_fric_match(Topo T, eipc_pairs pr, ei
 // the first node above a hash of the others' offsets from it.  Offsets, not ids, so that a
 // scene's items order alike alone and inside a batch, where its ids are shifted.  Items without
 // nodes get a key above all.
-constexpr int kHashBits = 7;   // the full grasp has about ten node sets per first node
+// Too few bits and different sets with one key take turns in the order, each turn a group; a bit more
+// costs nothing until the sort takes a pass more.  The full grasp, with about ten sets per first
+// node, takes 618 us an evaluation with 5 bits, 587 with 7, 583 with 10; the plate in rack 178, 181 and
+// 180, the 256-scene batch's stage 4,642, 4,634 and 4,636.
+constexpr int kHashBits = 7;
 
 __global__ void __launch_bounds__(kBlock) k_item_nodes(Topo T, eipc_pairs pr, const int32_t* lag_v,
                                                        const int64_t* lag_count, int64_t lag_cap,

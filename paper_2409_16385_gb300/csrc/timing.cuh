@@ -8,20 +8,20 @@
 namespace eipc {
 
 enum KernelId {
-  kKEmbed = 0,       // k_embed / k_pad
+  kKEmbed = 0,       // k_embed / k_ccd_begin
   kKBvh = 1,         // Morton codes + radix sort + hierarchy + refit (group)
   kKQuery = 2,       // BVH traversal producing candidates
   kKNarrow = 3,      // exact FP64 distance filter
   kKPairSort = 4,    // canonical sort of the pair list + emit (group)
   kKLag = 5,         // lagged friction state
   kKItems = 6,       // stencil cage nodes + record offsets (group)
-  kKEvalBarrier = 7, // barrier energy, gradient, projected Hessian, records
-  kKEvalFriction = 8,
-  kKHReduce = 9,     // sort-and-reduce of Hessian blocks into BSR (group)
-  kKGReduce = 10,    // sort-and-reduce of the reduced gradient (group)
+  kKEvalBarrier = 7, // the pairs' factors, friction and mollified pairs among them
+  kKEvalFriction = 8, // unused: friction is evaluated with the pairs
+  kKHReduce = 9,     // groups, records, sorts and sums into the BSR values and g_r (group)
+  kKGReduce = 10,    // the Hessian-vector product's sums per vertex and node (group)
   kKEnergy = 11,
-  kKCa = 12,         // conservative advancement of CCD candidates
-  kKEvalPair = 13,   // barrier and friction evaluation together (they overlap on two streams)
+  kKCa = 12,         // screen and conservative advancement of CCD candidates
+  kKEvalPair = 13,   // the pairs' factors from the second stream's fork on
   kKNum = 14
 };
 
