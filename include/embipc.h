@@ -43,7 +43,7 @@ enum {
   EIPC_OK = 0,
   EIPC_ERR_INVALID = -1,      /* bad argument (null pointer, size, capacity)            */
   EIPC_ERR_CUDA = -2,         /* a CUDA runtime call failed                             */
-  EIPC_ERR_NOMEM = -3,        /* workspace allocation failed at scene creation          */
+  EIPC_ERR_NOMEM = -3,        /* workspace allocation failed (scene creation, mollifier) */
   EIPC_ERR_TOO_LARGE = -4,    /* a size exceeds a fixed maximum of the call             */
   /* device status bits (eipc_status_read) */
   EIPC_FLAG_PENETRATION = 1,  /* some pair has d <= 0: the configuration is infeasible  */
@@ -51,7 +51,8 @@ enum {
   EIPC_FLAG_CAND_OVERFLOW = 4,/* more broad-phase candidates than the scene workspace   */
   EIPC_FLAG_REC_OVERFLOW = 8, /* more reduction records than the scene workspace (n (n+1)/2 of
                                  every item of n cage nodes, an upper bound where the mollifier is
-                                 off: the outputs may then be complete), or more items           */
+                                 off: the outputs may then be complete), more items, or more pairs
+                                 to deduplicate                                                  */
   EIPC_FLAG_BSR_OVERFLOW = 16,/* more BSR blocks than the caller's block capacity       */
   EIPC_FLAG_NONFINITE = 32,   /* a non-finite position or displacement was read         */
   EIPC_FLAG_ACCD_CAP = 64,    /* a CCD pair reached accd_max_iter (alpha still safe)    */
@@ -198,7 +199,8 @@ eipc_status eipc_contact_hvp(eipc_scene* scene, const double* q, const eipc_pair
  * during the call only), the rest positions the edge lengths |e|^2 are taken from; the
  * library computes and keeps the squared rest length of every edge.  Returns
  * EIPC_ERR_INVALID (and leaves the mollifier off) if any edge has a zero or non-finite
- * rest length.  factor = 0 turns it off (x_rest may then be NULL).  Synchronises `stream`
+ * rest length, EIPC_ERR_NOMEM (and changes nothing) if the workspace of mollified pairs, 80 B per
+ * record and allocated by the first call that turns the mollifier on, cannot be had.  factor = 0 turns it off (x_rest may then be NULL).  Synchronises `stream`
  * (the length check is read back). */
 eipc_status eipc_scene_set_mollifier(eipc_scene* scene, const double* x_rest, double factor, eipc_stream stream);
 

@@ -197,6 +197,10 @@ __global__ void __launch_bounds__(kBlock) k_feature_keys(Topo T, const double* _
                                                          DevStatus* st) {
   pdl_entry();
   const int64_t n = clamp_count(n_surv, cap);
+  if (blockIdx.x == 0 && threadIdx.x == 0 && n < *n_surv) {        // the pairs beyond are left out
+    raise_flag(st, EIPC_FLAG_REC_OVERFLOW);
+    raise_need(st, &st->need_rec, *n_surv);
+  }
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += grid_stride()) {
     int type; int32_t i, j;
     unpack(keys[k], T.bits_i, T.bits_j, &type, &i, &j);

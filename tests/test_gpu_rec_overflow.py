@@ -47,3 +47,20 @@ def test_overflow_is_reported_and_a_scene_of_the_size_needed_is_whole(moll, lagg
     np.testing.assert_array_equal(g2, g0)
     for k in ("row_ptr", "col", "val"):
         np.testing.assert_array_equal(H2[k], H0[k])
+
+
+def test_deduplication_reports_the_pairs_it_has_no_room_for():
+    from paper_2409_16385_gb300 import ContactScene
+    sc = scenes.parallel_sheets()
+    q, got = _t(sc.iterate(1)), {}
+    for rec in (1 << 22, 1000, 6628):
+        cs = ContactScene(sc, pair_capacity=1 << 13, bsr_capacity=1 << 16, cand_capacity=CAND, rec_capacity=rec)
+        cs.set_dedup()
+        h = cs.build_candidates(q).host()
+        st = cs.status()
+        if rec == 1000:
+            assert st["names"] == ["REC_OVERFLOW"] and st["needed"][2] == 6628
+        else:
+            assert st["flags"] == 0
+            got[rec] = [h[k].tobytes() for k in ("type", "i", "j", "d")]
+    assert got[1 << 22] == got[6628]
